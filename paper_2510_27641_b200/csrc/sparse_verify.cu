@@ -57,15 +57,11 @@ constexpr int kRec = 68 * 32;  // floats of one warp's (acc[64], m0, l0, m1, l1)
 constexpr int kCountersPerUnit = 4;
 constexpr int kAlignedMaxUnits = 256;  // the unit-aligned partition is tried up to this many units
 constexpr int kCandidates = 8;         // candidate target shares tried for it
-// A unit is not cut into parts of fewer than this many atoms (two 64-token tiles) even when
-// there are CTAs to spare: every part costs a record, an arrival and a share of the merge, which
-// on a small call (one short sequence) outweighs the streaming time saved.
-constexpr int kMinPartAtoms = 8;
-// With CTA pairs available (query blocks of up to 32 rows), a unit of up to this many atoms is cut
-// in two rather than in more parts: the pair's merge through shared memory (~1.7 us) beats the
-// merge of three or more records through global memory (~1 us per record) by more than the
-// longer parts cost.
-constexpr int kPairAtoms = 64;
+// Parts of one unit are at least one 64-token tile.
+constexpr int kMinPartAtoms = 4;
+// ... or twice that where the parts merge through global memory.
+constexpr int kMinGlobalAtoms = 8;
+constexpr int kMaxCluster = 8;
 constexpr size_t kCounterBytes = static_cast<size_t>(kMaxUnits) * kCountersPerUnit * sizeof(unsigned int);
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -93,8 +89,176 @@ struct VerifyParams {
   int tail_off;      // tail - T: query t may see tail tokens j <= t + tail_off
   const int* plan;   // precomputed work partition (specattn_verify_plan) or nullptr
   int test_lose;     // SPECATTN_VERIFY_TEST_LOSE_ARRIVAL: CTA 0 withholds one barrier arrival
-  int pairs;         // the launch runs as CTA pairs (clusters of two)
+  int cluster;       // CTAs per cluster of the launch (the parts of a unit merge inside one cluster)
 };
+
+// ---- work partition -----------------------------------------------------------------------------
+// Ways of dealing the N atoms of all units to the G CTAs of a launch:
+// - Aligned, inside clusters: every unit is cut into k equal parts, one CTA each, k a power of two up to the
+//   cluster size, the least that brings the part down to a target share; units are placed by descending k, so
+//   that none straddles a cluster, and the parts merge through shared memory.
+// - Aligned, anywhere: any number of parts of at least kMinGlobalAtoms atoms, merged through global memory.
+// - Ranges: the atoms of all units end to end, cut into G equal ranges.  It balances any mix of list
+//   lengths; but a CTA that straddles two units pays for two set-ups and merges.
+struct Partition {
+  int parts[2][kCandidates];    // inside clusters / anywhere, per candidate share: CTAs needed, largest part
+  int largest[2][kCandidates];
+  int unit_max;              // atoms of the largest unit
+  unsigned long long before[kAlignedMaxUnits / 32];  // units per class (16 bits each) before each group of 32 units
+  unsigned long long all;    // units per class
+  // this CTA's share, for the end of the kernel (kept out of registers meanwhile)
+  int mine[3];               // unit (-1: none), part and number of parts
+  int atoms, ctas, aligned;  // N, the number of CTAs with work, whether units are dealt in equal parts
+  int cluster;               // of the partition: 1 where parts merge through global memory
+};
+
+// Parts of a unit for a target share of `share` atoms, out of U units on G CTAs.  Inside clusters a part has at
+// least kMinPartAtoms atoms, half as many again where all the parts would take more than half of the GPU (32
+// units of 19 atoms: 8.5 us in four parts, 7.6 us in two; 8 such units: 6.3 us in four, 7.3 us in two).
+__device__ __forceinline__ int unit_parts(int atoms, int share, int cluster, int U, int G) {
+  if (cluster == 1) return max(1, min((atoms + share / 2) / share, atoms / kMinGlobalAtoms));
+  int k = cluster;
+  while (k > 1 && (2 * k * kMinPartAtoms > ((2 * U * k > G) ? atoms + atoms / 3 : 2 * atoms) || (k >> 1) * share >= atoms)) k >>= 1;
+  return k;
+}
+
+// Candidate share c: (N / G) (1 + c / 7), rounded up -- rounding part counts up to the chain can ask for
+// twice the CTAs.
+__device__ __forceinline__ int cand_share(long long N, int G, int c) {
+  // 32-bit: N <= 2048 * 12288
+  return static_cast<int>((static_cast<unsigned>(N) * (7u + c) + 7u * G - 1u) / (7u * G));
+}
+
+// Class of k parts: 0 for the cluster size, 1 for half of it, ...
+__device__ __forceinline__ int class_of(int k, int cluster) { return __ffs(cluster) - __ffs(k); }
+
+// Decides the partition (all NT threads of the CTA, after a barrier that follows unit_start[]): the candidate share, or -1 for ranges; `cluster` becomes 1 where parts are to merge through
+// global memory.  One barrier; warp 0 alone may go on to partition_locate() without another.
+template <int NT>
+__device__ __forceinline__ int partition_decide(Partition& pt, const int* unit_start, int U, int G, int& cluster) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int N = unit_start[U];
+  const bool try_aligned = U <= kAlignedMaxUnits && N > 0;
+  // Parts anywhere are worth a look where the cluster holds only two and the GPU has room for three.
+  const int way_lo = (cluster > 1) ? 0 : 1, way_hi = (cluster > 2 || (cluster == 2 && 3 * U > G)) ? 1 : 2;
+  if (try_aligned) {
+    // one warp per candidate: two divisions a lane, two reductions, no atomics
+#pragma unroll 1
+    for (int slot = way_lo * kCandidates + (tid >> 5); slot < way_hi * kCandidates; slot += NT / 32) {
+      const int way = slot / kCandidates, c = slot % kCandidates;
+      const int share = cand_share(N, G, c), cl = way ? 1 : cluster;
+      int sum = 0, big = 0, most = 0;
+#pragma unroll 1
+      for (int u = lane; u < U; u += 32) {
+        const int atoms = unit_start[u + 1] - unit_start[u];
+        if (atoms == 0) continue;
+        const int k = unit_parts(atoms, share, cl, U, G);
+        sum += k;
+        big = max(big, (atoms + k - 1) / k);
+        most = max(most, atoms);
+      }
+      sum = __reduce_add_sync(0xffffffffu, sum);
+      big = __reduce_max_sync(0xffffffffu, big);
+      most = __reduce_max_sync(0xffffffffu, most);
+      if (lane == 0) {
+        pt.parts[way][c] = sum;
+        pt.largest[way][c] = big;
+        pt.unit_max = most;  // (the same from every warp)
+      }
+    }
+  }
+  __syncthreads();
+  // Costs in atoms' time (~0.23 us): a straddling CTA ~24; a unit's merge through global memory ~6 and ~3 a record;
+  // inside a cluster ~3.
+  int cand = -1, way = 1;
+  if (try_aligned) {
+    int best = N / G + 24 + 3 * (pt.unit_max / (N / G + 1) + 1);
+    for (int w = way_lo; w < way_hi; ++w) {
+      for (int c = 0; c < kCandidates; ++c) {
+        if (pt.parts[w][c] > G) continue;
+        const int part = pt.largest[w][c];
+        const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : 6 + 3 * ((pt.unit_max + part - 1) / part));
+        if (cost <= best) {
+          best = cost;
+          cand = c;
+          way = w;
+        }
+        break;
+      }
+    }
+  }
+  if (way == 1) cluster = 1;
+  if (cand >= 0 && tid < 32) {  // units per class, 16 bits each, before every group of 32 units
+    const int share = cand_share(N, G, cand);
+    unsigned long long seen = 0ull;
+    for (int base = 0; base < U; base += 32) {
+      const int u = base + lane;
+      const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
+      // (without clusters: the units' CTAs, which lie in the order of the units)
+      const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+      const int at = (cluster == 1) ? 0 : 16 * class_of(k, cluster);
+      const unsigned one = (k == 0) ? 0u : (cluster == 1) ? static_cast<unsigned>(k) : 1u << (at & 31);
+      const unsigned long long hi = __reduce_add_sync(0xffffffffu, at < 32 ? 0u : one);
+      if (lane == 0) pt.before[base >> 5] = seen;
+      seen += (hi << 32) + __reduce_add_sync(0xffffffffu, at < 32 ? one : 0u);
+    }
+    if (lane == 0) pt.all = seen;
+    __syncwarp();
+  }
+  return cand;
+}
+
+// One warp, aligned partition: the unit of CTA `me` (-1: none), its part and the number of parts.
+__device__ __forceinline__ int partition_locate(const Partition& pt, const int* unit_start, int U, int G, int cluster,
+                                                int cand, int me, int& part, int& parts) {
+  const int lane = threadIdx.x & 31;
+  const int share = cand_share(unit_start[U], G, cand);
+  if (cluster == 1) {
+    for (int base = 0; base < U; base += 32) {
+      const int u = base + lane;
+      const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
+      const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+      int end = k;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += v;
+      }
+      const int start = static_cast<int>(pt.before[base >> 5]) + end - k;
+      const unsigned hit = __ballot_sync(0xffffffffu, me >= start && me < start + k);
+      if (hit != 0u) {
+        const int l = __ffs(hit) - 1;
+        part = me - __shfl_sync(0xffffffffu, start, l);
+        parts = __shfl_sync(0xffffffffu, k, l);
+        return base + l;
+      }
+    }
+    return -1;
+  }
+  // the CTA's class, its place among the class's units, the unit at that place
+  int first = 0, cls = 0, at = -1;
+  parts = cluster;
+  for (;; ++cls, parts >>= 1) {
+    const int n = static_cast<int>((pt.all >> (16 * cls)) & 0xffffull);
+    if (me < first + n * parts) {
+      at = (me - first) / parts;
+      break;
+    }
+    first += n * parts;
+    if (parts == 1) return -1;
+  }
+  part = me - first - at * parts;
+  for (int base = 0; base < U; base += 32) {
+    const int u = base + lane;
+    const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
+    const bool in = atoms > 0 && unit_parts(atoms, share, cluster, U, G) == parts;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    const int rank = static_cast<int>((pt.before[base >> 5] >> (16 * cls)) & 0xffffull) + __popc(m & ((1u << lane) - 1u));
+    const unsigned hit = __ballot_sync(0xffffffffu, in && rank == at);
+    if (hit != 0u) return base + __ffs(hit) - 1;
+  }
+  return -1;
+}
 
 // WPM = consumer warps per 16-row slab: 4 -> (stage parity, 32-key half), 2 -> (stage parity).
 template <int MT, int WPM>
@@ -107,18 +271,12 @@ struct VShared {
   unsigned long long q_full, q_empty;
   int unit_start[kMaxUnits + 1];
   int unit_cnt[kMaxUnits];
-  int part_start[kAlignedMaxUnits + 1];  // aligned partition: first CTA of each unit
-  int cand_parts[kCandidates];           // per candidate share: total parts, largest part
-  int cand_max[kCandidates];
-  int aligned;                           // 1: unit-aligned partition, 0: contiguous atoms
+  Partition part;
   volatile int abort_flag;
   // (kernels with two warps per slab) this CTA arrived last at the cut unit of its final segment:
   // both warps of the slab merge half of the columns each; with the merge's arguments
   volatile int merge_last[MT];
   volatile int merge_arg[MT][5];
-  // cluster merge (two CTAs per unit): the odd CTA's records land here, in the even CTA
-  unsigned long long peer_full;
-  alignas(16) float peer_rec[(MT <= 2) ? MT : 1][(MT <= 2) ? kRec : 1];
 };
 
 __device__ __forceinline__ int unit_count(const VerifyParams& P, int u) {
@@ -146,6 +304,17 @@ __device__ __forceinline__ int cta_of_atom(long long x, long long n, long long n
   return static_cast<int>(i);
 }
 
+// The unit that holds atom a0 (empty units share the start of their successor and are skipped).
+__device__ __forceinline__ int unit_of_atom(const int* unit_start, int U, int a0) {
+  int lo = 0, hi = U - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (unit_start[mid] <= a0) lo = mid; else hi = mid - 1;
+  }
+  while (unit_start[lo + 1] <= a0) ++lo;
+  return lo;
+}
+
 // Scales that bring a running maximum m and an incoming maximum im to their common maximum.
 __device__ __forceinline__ void merge_scales(float m, float im, float& mn, float& a_old, float& a_in) {
   mn = fmaxf(m, im);
@@ -157,20 +326,19 @@ __device__ __forceinline__ void merge_scales(float m, float im, float& mn, float
 // ---- precomputed work partition ("plan") ------------------------------------------------------
 // The partition of a launch depends only on the list lengths, the shapes and the grid: target
 // layers that share a draft layer's lists share it.  A plan holds, as int32:
-//   [0] magic  [1] U  [2] grid  [3] aligned  [4] NP  [5] N (atoms)  [6] tail  [7] dense
-//   unit_start[U + 1], unit_cnt[U], part_start[U + 1], then (a0, a1, u_first) per CTA
+//   [0] magic  [1] U  [2] grid  [3] 0: ranges, else the partition's cluster size  [4] NP  [5] N (atoms)  [6] tail  [7] dense
+//   unit_start[U + 1], unit_cnt[U], then (a0, a1, u_first, part | parts << 8) per CTA
 // A kernel whose launch does not match the header ignores the plan and partitions itself.
 constexpr int kPlanMagic = 0x5a17a9e1;
 constexpr int kPlanHeader = 8;
 __host__ __device__ inline size_t plan_ints(int U, int grid) {
-  return static_cast<size_t>(kPlanHeader) + (U + 1) + U + (U + 1) + 3 * static_cast<size_t>(grid);
+  return static_cast<size_t>(kPlanHeader) + (U + 1) + U + 4 * static_cast<size_t>(grid);
 }
 
 // One CTA computes what every CTA of a verify launch would compute for itself at start-up.
 __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int G) {
   __shared__ int unit_start[kMaxUnits + 1];
-  __shared__ int part_start[kAlignedMaxUnits + 1];
-  __shared__ int cand_parts[kCandidates], cand_max[kCandidates];
+  __shared__ Partition pt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int U = P.B * P.Hkv;
   // The lists are the previous kernel's output.  No early trigger for the next kernel either:
@@ -179,15 +347,13 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   pdl_wait();
   int* const p_us = plan + kPlanHeader;
   int* const p_cnt = p_us + (U + 1);
-  int* const p_ps = p_cnt + U;
-  int* const p_cta = p_ps + (U + 1);
+  int* const p_cta = p_cnt + U;
   if (tid == 0) unit_start[0] = 0;
   for (int u = tid; u < U; u += 256) {
     const int c = unit_count(P, u);
     p_cnt[u] = c;
     unit_start[u + 1] = (c + kAtom - 1) / kAtom;
   }
-  if (tid < kCandidates) { cand_parts[tid] = 0; cand_max[tid] = 0; }
   __syncthreads();
   if (warp == 0) {
     int carry = 0;
@@ -205,99 +371,38 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   }
   __syncthreads();
   const long long N = unit_start[U];
-  const bool try_aligned = (U <= kAlignedMaxUnits) && (N > 0);
-  if (try_aligned && tid < U) {
-    const int atoms = unit_start[tid + 1] - unit_start[tid];
-    if (atoms > 0) {
-      for (int c = 0; c < kCandidates; ++c) {
-        const unsigned int num = static_cast<unsigned int>(atoms) * G * 16u;
-        const unsigned int den = static_cast<unsigned int>(N) * (16u + c);
-        int k = static_cast<int>((2u * num + den) / (2u * den));
-        if (k < 1) k = 1;
-        if (k > atoms) k = atoms;
-        if (k * kMinPartAtoms > atoms) k = max(1, atoms / kMinPartAtoms);  // no part shorter than that
-        if (P.pairs && k > 2 && atoms <= kPairAtoms) k = 2;  // short unit: two parts merge through shared memory
-        atomicAdd(&cand_parts[c], k);
-        atomicMax(&cand_max[c], (atoms + k - 1) / k);
-      }
-    }
-  }
+  int cluster = P.cluster;
+  const int cand = partition_decide<256>(pt, unit_start, U, G, cluster);
   __syncthreads();
-  int cand = -1;
-  if (try_aligned) {
-    for (int c = 0; c < kCandidates; ++c)
-      if (cand_parts[c] <= G) { cand = c; break; }
-    if (cand >= 0 && static_cast<long long>(cand_max[cand]) * G > N + 24ll * G) cand = -1;
-  }
   const bool aligned = cand >= 0;
-  if (aligned && warp == 0) {
-    int carry = 0;
-    for (int base = 0; base < U; base += 32) {
-      const int u = base + lane;
-      int k = 0;
-      if (u < U) {
+  const long long NP = aligned ? pt.parts[cluster > 1 ? 0 : 1][cand] : ((N < G) ? N : static_cast<long long>(G));
+  for (int u = tid; u <= U; u += 256) p_us[u] = unit_start[u];
+  for (int i = warp; i < G; i += 8) {
+    int a0 = 0, a1 = 0, u_first = 0, part = 0, parts = 0;
+    if (aligned) {
+      const int u = partition_locate(pt, unit_start, U, G, cluster, cand, i, part, parts);
+      if (u >= 0) {
         const int atoms = unit_start[u + 1] - unit_start[u];
-        if (atoms > 0) {
-          const unsigned int num = static_cast<unsigned int>(atoms) * G * 16u;
-          const unsigned int den = static_cast<unsigned int>(N) * (16u + cand);
-          k = static_cast<int>((2u * num + den) / (2u * den));
-          if (k < 1) k = 1;
-          if (k > atoms) k = atoms;
-        if (k * kMinPartAtoms > atoms) k = max(1, atoms / kMinPartAtoms);  // no part shorter than that
-        if (P.pairs && k > 2 && atoms <= kPairAtoms) k = 2;  // short unit: two parts merge through shared memory
-        }
+        a0 = unit_start[u] + part * atoms / parts;
+        a1 = unit_start[u] + (part + 1) * atoms / parts;
+        u_first = u;
       }
-      int v = k;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-      }
-      if (u < U) part_start[u + 1] = v + carry;
-      if (base == 0 && lane == 0) part_start[0] = 0;
-      carry += __shfl_sync(0xffffffffu, v, 31);
+    } else if (i < NP) {
+      a0 = cta_first_atom(i, N, NP);
+      a1 = cta_first_atom(i + 1, N, NP);
+      u_first = unit_of_atom(unit_start, U, a0);
     }
-  }
-  __syncthreads();
-  const long long NP = aligned ? part_start[U] : ((N < G) ? N : static_cast<long long>(G));
-  for (int u = tid; u <= U; u += 256) {
-    p_us[u] = unit_start[u];
-    p_ps[u] = aligned ? part_start[u] : 0;
-  }
-  for (int i = tid; i < G; i += 256) {
-    int a0 = 0, a1 = 0, u_first = 0;
-    if (i < NP) {
-      if (aligned) {
-        int lo = 0, hi = U - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (part_start[mid] <= i) lo = mid; else hi = mid - 1;
-        }
-        const int k = part_start[lo + 1] - part_start[lo];
-        const int j = i - part_start[lo];
-        const int atoms = unit_start[lo + 1] - unit_start[lo];
-        a0 = unit_start[lo] + j * atoms / k;
-        a1 = unit_start[lo] + (j + 1) * atoms / k;
-      } else {
-        a0 = cta_first_atom(i, N, NP);
-        a1 = cta_first_atom(i + 1, N, NP);
-      }
-      int lo = 0, hi = U - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (unit_start[mid] <= a0) lo = mid; else hi = mid - 1;
-      }
-      u_first = lo;
-      while (unit_start[u_first + 1] <= a0) ++u_first;
+    if (lane == 0) {
+      p_cta[4 * i] = a0;
+      p_cta[4 * i + 1] = a1;
+      p_cta[4 * i + 2] = u_first;
+      p_cta[4 * i + 3] = part | (parts << 8);
     }
-    p_cta[3 * i] = a0;
-    p_cta[3 * i + 1] = a1;
-    p_cta[3 * i + 2] = u_first;
   }
   if (tid == 0) {
     plan[1] = U;
     plan[2] = G;
-    plan[3] = aligned ? 1 : 0;
+    plan[3] = aligned ? cluster : 0;
     plan[4] = static_cast<int>(NP);
     plan[5] = static_cast<int>(N);
     plan[6] = P.tail;
@@ -316,10 +421,10 @@ constexpr int kPlanBatch = 8;
 struct PlanBatch {
   VerifyParams p[kPlanBatch];
   int* plan[kPlanBatch];
-  int G;
+  int grid[kPlanBatch];
 };
 __global__ void __launch_bounds__(256, 1) verify_plan_many_kernel(const __grid_constant__ PlanBatch B) {
-  plan_body(B.p[blockIdx.x], B.plan[blockIdx.x], B.G);
+  plan_body(B.p[blockIdx.x], B.plan[blockIdx.x], B.grid[blockIdx.x]);
 }
 
 // Online-softmax state of one warp: rows g and g+8 of its 16-row slab, 128 output columns.
@@ -449,8 +554,8 @@ __device__ __forceinline__ void attend_block32(WarpState& st, const uint32_t (&q
 // warps per slab, whose second warp has nothing left to do on a CTA's last segment; kept out of
 // line so that it costs the tile loop no registers.
 template <int MT>
-__device__ __noinline__ void merge_half(const VerifyParams& P, int mt, int half, int i_lo, int i_hi, bool aligned,
-                                        long long N, long long NP, int us, int b, int kvh) {
+__device__ __noinline__ void merge_half(const VerifyParams& P, int mt, int half, int i_lo, int i_hi, bool aligned, long long N,
+                                        long long NP, int us, int b, int kvh) {
   const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
   auto record = [&](int i) -> const float4* {
     return reinterpret_cast<const float4*>(P.partials +
@@ -528,6 +633,81 @@ __device__ __noinline__ void merge_half(const VerifyParams& P, int mt, int half,
   }
 }
 
+// Merge of a unit whose parts lie in one cluster: every CTA has left its slab records in its shared memory
+// (rec_addr: slab mt's, the same address in every CTA) and arrived at the cluster barrier; CTA `part` of
+// `parts` combines its share of the 128 output columns from all of them, in part order, and writes rows
+// g and g + 8 of the slab; its warps share the columns out (part 0 also writes the LSE).  Reading is spread over
+// all CTAs and nobody waits for more than that barrier.  (Pushing the slices to their writers instead,
+// with one remote arrival each, took 1.5 - 2.7 us longer: the addresses of 17 remote stores are code, and
+// this late in a kernel every 128 bytes of code not yet fetched cost ~70 ns.)
+// Out of line: it costs the tile loop no registers.  kParts is a template parameter for the sake of straight, short code.
+template <int MT, int WPM, int kParts>
+__device__ __noinline__ void merge_cluster(const VerifyParams& P, uint32_t rec_addr, int mt, int wr, int part, int u) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
+  const uint32_t rank0 = cluster_cta_rank() - static_cast<uint32_t>(part);
+  const int n_hi = 16 / kParts * (part + 1);
+  int n = 16 / kParts * part + wr;
+  cluster_wait();
+  if (n < n_hi) {
+    uint32_t addr[kParts];
+    float4 ml[kParts], x[kParts];
+#pragma unroll
+    for (int r = 0; r < kParts; ++r) {
+      addr[r] = map_to_cta(rec_addr, rank0 + r) + lane * 16;
+      ml[r] = ld_cluster_v4(addr[r] + 16 * 512);
+    }
+#pragma unroll
+    for (int r = 0; r < kParts; ++r) x[r] = ld_cluster_v4(addr[r] + n * 512);
+    float m0 = ml[0].x, m1 = ml[0].z;
+#pragma unroll
+    for (int r = 1; r < kParts; ++r) {
+      m0 = fmaxf(m0, ml[r].x);
+      m1 = fmaxf(m1, ml[r].z);
+    }
+    const float base0 = (m0 == -INFINITY) ? 0.f : m0, base1 = (m1 == -INFINITY) ? 0.f : m1;
+    float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+    for (int r = 0; r < kParts; ++r) {
+      ml[r].x = ex2(ml[r].x - base0);
+      ml[r].z = ex2(ml[r].z - base1);
+      l0 += ml[r].y * ml[r].x;
+      l1 += ml[r].w * ml[r].z;
+    }
+    const float inv0 = (l0 > 0.f) ? 1.f / l0 : 0.f;
+    const float inv1 = (l1 > 0.f) ? 1.f / l1 : 0.f;
+    const int b = u / P.Hkv, kvh = u - b * P.Hkv;
+    const int r0 = mt * 16 + g, r1 = r0 + 8;
+    const int t0 = r0 / P.grp, t1 = r1 / P.grp;
+    const long long row0 = (static_cast<long long>(b) * P.T + t0) * P.Hq + kvh * P.grp + r0 - t0 * P.grp;
+    const long long row1 = (static_cast<long long>(b) * P.T + t1) * P.Hq + kvh * P.grp + r1 - t1 * P.grp;
+    const bool w0 = r0 < P.M, w1 = r1 < P.M;
+    if (part == 0 && wr == 0 && tq == 0) {
+      if (w0) P.lse[row0] = (l0 > 0.f) ? (m0 + log2f(l0)) * kLn2 : -INFINITY;
+      if (w1) P.lse[row1] = (l1 > 0.f) ? (m1 + log2f(l1)) * kLn2 : -INFINITY;
+    }
+#pragma unroll 1
+    for (;;) {
+      float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int r = 0; r < kParts; ++r) {
+        o[0] += x[r].x * ml[r].x;
+        o[1] += x[r].y * ml[r].x;
+        o[2] += x[r].z * ml[r].z;
+        o[3] += x[r].w * ml[r].z;
+      }
+      if (w0) *reinterpret_cast<float2*>(P.out + row0 * kD + n * 8 + tq * 2) = make_float2(o[0] * inv0, o[1] * inv0);
+      if (w1) *reinterpret_cast<float2*>(P.out + row1 * kD + n * 8 + tq * 2) = make_float2(o[2] * inv1, o[3] * inv1);
+      n += WPM;
+      if (n >= n_hi) break;
+#pragma unroll
+      for (int r = 0; r < kParts; ++r) x[r] = ld_cluster_v4(addr[r] + n * 512);
+    }
+  }
+  __syncwarp();
+  cluster_arrive();  // (only reads precede it)
+  cluster_wait();    // nobody leaves while its records may still be read
+}
+
 template <int MT, int WPM>
 __global__ void __launch_bounds__((MT * WPM + kProdWarps) * 32, 1)
 sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
@@ -563,7 +743,6 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     }
     mbar_init(&sh.q_full, 1);
     mbar_init(&sh.q_empty, NC);
-    mbar_init(&sh.peer_full, MT);
     mbar_fence_init();
     sh.abort_flag = 0;
     sh.unit_start[0] = 0;
@@ -576,11 +755,9 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   if (planned) {
     const int* const p_us = plan + kPlanHeader;
     const int* const p_cnt = p_us + (U + 1);
-    const int* const p_ps = p_cnt + U;
     for (int u = tid; u <= U; u += NT) {
       sh.unit_start[u] = p_us[u];
       if (u < U) sh.unit_cnt[u] = p_cnt[u];
-      if (u <= kAlignedMaxUnits) sh.part_start[u] = p_ps[u];
     }
   } else {
     for (int u = tid; u < U; u += NT) {
@@ -591,25 +768,24 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   }
   fence_proxy_async();
   __syncthreads();
-  // Launched as CTA pairs: the peer's barrier must exist before anyone can arrive on it.  Only
-  // the arrival happens here; every thread waits for the peer's arrival where it first needs
-  // it (the consumers before their first combine, everybody else before leaving), so that the
-  // barrier costs nothing on the way to the first copy.
-  const bool paired = (MT <= 2) && (cluster_num_ctas() == 2);
-  if (paired) cluster_arrive();
   long long N;        // atoms of all units
   bool aligned;       // which of the two partitions
   long long NP;       // CTAs that get work
   int a0 = 0, a1 = 0, u_first = 0;  // this CTA's atom range and the unit holding its first atom
+  int part = 0, parts = 0;          // (aligned) which part of how many of the unit
+  int cluster;                      // 1: parts merge through global memory
   const int G = static_cast<int>(gridDim.x);
   if (planned) {
     N = plan[5];
     aligned = plan[3] != 0;
+    cluster = plan[3];
     NP = plan[4];
-    const int* const p_cta = plan + kPlanHeader + (U + 1) + U + (U + 1) + 3 * blockIdx.x;
+    const int* const p_cta = plan + kPlanHeader + (U + 1) + U + 4 * blockIdx.x;
     a0 = p_cta[0];
     a1 = p_cta[1];
     u_first = p_cta[2];
+    part = p_cta[3] & 0xff;
+    parts = p_cta[3] >> 8;
   } else {
   if (warp == 0) {  // inclusive scan of the atom counts, 32 at a time
     int carry = 0;
@@ -627,76 +803,34 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   }
   __syncthreads();
 
-  // ---- work partition ----------------------------------------------------------------------
-  // Two ways of dealing the N atoms to the CTAs.  "Aligned": every unit is cut into k_u equal
-  // parts, k_u = round(atoms_u / share), one part per CTA -- each CTA then touches one unit
-  // only and a unit is merged from k_u records; chosen when the parts fit in one wave and the
-  // largest exceeds the ideal share by no more than 24 atoms.  Otherwise "contiguous": the atoms of all units
-  // laid end to end and cut into gridDim equal ranges, which balances any mix of list lengths
-  // at the price of CTAs that straddle unit boundaries.
   N = sh.unit_start[U];
-  if (tid < kCandidates) { sh.cand_parts[tid] = 0; sh.cand_max[tid] = 0; }
-  if (tid == 0) sh.aligned = 0;
-  __syncthreads();
-  const bool try_aligned = (U <= kAlignedMaxUnits) && (N > 0);
-  if (try_aligned && tid < U) {
-    const int atoms = sh.unit_start[tid + 1] - sh.unit_start[tid];
-    if (atoms > 0) {
-#pragma unroll
-      for (int c = 0; c < kCandidates; ++c) {
-        // share_c = (N / G) * (1 + c / 16); 32-bit: atoms <= 12288, G ~ 148, N <= 2048 * 12288
-        const unsigned int num = static_cast<unsigned int>(atoms) * G * 16u;
-        const unsigned int den = static_cast<unsigned int>(N) * (16u + c);
-        int k = static_cast<int>((2u * num + den) / (2u * den));  // round to nearest
-        if (k < 1) k = 1;
-        if (k > atoms) k = atoms;
-        if (k * kMinPartAtoms > atoms) k = max(1, atoms / kMinPartAtoms);  // no part shorter than that
-        if (P.pairs && k > 2 && atoms <= kPairAtoms) k = 2;  // short unit: two parts merge through shared memory
-        atomicAdd(&sh.cand_parts[c], k);
-        atomicMax(&sh.cand_max[c], (atoms + k - 1) / k);
-      }
-    }
-  }
-  __syncthreads();
-  int cand = -1;
-  if (try_aligned) {
-    for (int c = 0; c < kCandidates; ++c)
-      if (sh.cand_parts[c] <= G) { cand = c; break; }
-    // worth it only while the parts stay close to the ideal share: a straddling CTA costs a
-    // fixed few microseconds of extra merging, an oversized part costs time per atom
-    if (cand >= 0 && static_cast<long long>(sh.cand_max[cand]) * G > N + 24ll * G) cand = -1;
-  }
+  cluster = P.cluster;
+  const int cand = partition_decide<NT>(sh.part, sh.unit_start, U, G, cluster);
   aligned = cand >= 0;
-  if (aligned && warp == 0) {  // first CTA of every unit: exclusive scan of k_u
-    int carry = 0;
-    for (int base = 0; base < U; base += 32) {
-      const int u = base + lane;
-      int k = 0;
-      if (u < U) {
-        const int atoms = sh.unit_start[u + 1] - sh.unit_start[u];
-        if (atoms > 0) {
-          const unsigned int num = static_cast<unsigned int>(atoms) * G * 16u;
-          const unsigned int den = static_cast<unsigned int>(N) * (16u + cand);
-          k = static_cast<int>((2u * num + den) / (2u * den));
-          if (k < 1) k = 1;
-          if (k > atoms) k = atoms;
-        if (k * kMinPartAtoms > atoms) k = max(1, atoms / kMinPartAtoms);  // no part shorter than that
-        if (P.pairs && k > 2 && atoms <= kPairAtoms) k = 2;  // short unit: two parts merge through shared memory
-        }
+  NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : ((N < G) ? N : static_cast<long long>(G));
+  if (aligned) {
+    if (warp == 0) {
+      const int u = partition_locate(sh.part, sh.unit_start, U, G, cluster, cand, blockIdx.x, part, parts);
+      if (lane == 0) {
+        sh.part.mine[0] = u;
+        sh.part.mine[1] = part;
+        sh.part.mine[2] = parts;
       }
-      int v = k;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-      }
-      if (u < U) sh.part_start[u + 1] = v + carry;
-      if (base == 0 && lane == 0) sh.part_start[0] = 0;
-      carry += __shfl_sync(0xffffffffu, v, 31);
     }
+    __syncthreads();
+    u_first = max(sh.part.mine[0], 0);
+    part = sh.part.mine[1];
+    parts = sh.part.mine[2];
+    if (static_cast<long long>(blockIdx.x) < NP) {
+      const int atoms = sh.unit_start[u_first + 1] - sh.unit_start[u_first];  // part < parts <= 8: fits 32 bits
+      a0 = sh.unit_start[u_first] + part * atoms / parts;
+      a1 = sh.unit_start[u_first] + (part + 1) * atoms / parts;
+    }
+  } else if (static_cast<long long>(blockIdx.x) < NP) {
+    a0 = cta_first_atom(blockIdx.x, N, NP);
+    a1 = cta_first_atom(blockIdx.x + 1, N, NP);
+    u_first = unit_of_atom(sh.unit_start, U, a0);
   }
-  __syncthreads();
-  NP = aligned ? sh.part_start[U] : ((N < G) ? N : static_cast<long long>(G));
   }  // !planned
   if (warp < NC) {
     // consumers are the only writers of global memory: from here on the previous kernel's
@@ -713,38 +847,17 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       }
     }
   }
-  if (static_cast<long long>(blockIdx.x) >= NP) {
-    if (paired) cluster_wait();
-    return;
+  if (static_cast<long long>(blockIdx.x) >= NP) return;
+  if (lane == 0) {  // (every warp leaves itself the same values)
+    sh.part.mine[0] = u_first;
+    sh.part.mine[1] = part;
+    sh.part.mine[2] = parts;
+    sh.part.atoms = static_cast<int>(N);
+    sh.part.ctas = static_cast<int>(NP);
+    sh.part.aligned = aligned ? 1 : 0;
+    sh.part.cluster = cluster;
   }
-  if (!planned) {
-  if (aligned) {
-    int lo = 0, hi = U - 1;  // unit whose CTA range holds this CTA
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (sh.part_start[mid] <= static_cast<int>(blockIdx.x)) lo = mid; else hi = mid - 1;
-    }
-    const int k = sh.part_start[lo + 1] - sh.part_start[lo];
-    const int j = static_cast<int>(blockIdx.x) - sh.part_start[lo];
-    const int atoms = sh.unit_start[lo + 1] - sh.unit_start[lo];  // j < k <= G: the products fit 32 bits
-    a0 = sh.unit_start[lo] + j * atoms / k;
-    a1 = sh.unit_start[lo] + (j + 1) * atoms / k;
-  } else {
-    a0 = cta_first_atom(blockIdx.x, N, NP);
-    a1 = cta_first_atom(blockIdx.x + 1, N, NP);
-  }
-
-  // unit holding atom a0
-  {
-    int lo = 0, hi = U - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (sh.unit_start[mid] <= a0) lo = mid; else hi = mid - 1;
-    }
-    u_first = lo;
-    while (sh.unit_start[u_first + 1] <= a0) ++u_first;  // skip empty units that share the start
-  }
-  }  // !planned
+  __syncwarp();
 
   if (warp >= NC) {
     // =========================== producer warps ===========================================
@@ -905,7 +1018,6 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       // give this warp's last copies a bounded chance to land before the CTA retires
       mbar_wait(&sh.full[last_it % kStages], (last_it / kStages) & 1u, nullptr);
     }
-    if (paired) cluster_wait();
     return;
   }
 
@@ -930,9 +1042,9 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   int it = 0, seg = 0;
   int a = a0, u = u_first;
   bool ok = true;
-  bool peer_seen = false;
   constexpr bool kShareMerge = (WPM == 2);  // the slab's second warp helps with a final merge
   bool final_global = false;                // the CTA's last segment ends in a merge through global memory
+  bool in_cluster = false;                  // the CTA's part is merged inside its cluster
   while (a < a1) {
     const int us = sh.unit_start[u], ue = sh.unit_start[u + 1];
     const int seg_hi = min(a1, ue);
@@ -1015,10 +1127,6 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       if (lane == 0) mbar_arrive(&sh.q_empty);   // the query tile was read for the last time
     }
     // ---- end of the segment: row sums across the quad, then combine the slab's warps ---------
-    if (paired && !peer_seen) {  // the peer's arrival at kernel start: long past by now
-      cluster_wait();
-      peer_seen = true;
-    }
     float m0 = st.m0, m1 = st.m1, l0 = st.l0, l1 = st.l1;
     float (&acc)[16][4] = st.acc;
     l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
@@ -1057,48 +1165,26 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       }
       named_bar_sync(1 + mt, WPM * 32);
     }
-    if (sh.abort_flag) { ok = false; break; }
-
-    if (kShareMerge && seg_hi == a1 && !((a == us) && (seg_hi == ue))) final_global = true;
+    if (sh.abort_flag) ok = false;
+    const bool whole = (a == us) && (seg_hi == ue);
+    // A part of a unit, this CTA's only segment, is merged inside the cluster (after a failed wait too:
+    // the peers read this CTA's memory, so it leaves with them, and the result is flagged).
+    if (!whole && sh.part.aligned && sh.part.cluster > 1) {
+      if (wr == 0) {
+        float4* rec = reinterpret_cast<float4*>(sh.scratch[mt][0]) + lane;
+#pragma unroll
+        for (int n = 0; n < 16; ++n) rec[n * 32] = make_float4(acc[n][0], acc[n][1], acc[n][2], acc[n][3]);
+        rec[16 * 32] = make_float4(m0, l0, m1, l1);
+      }
+      cluster_arrive_release();
+      in_cluster = true;
+      break;
+    }
+    if (!ok) break;
+    if (kShareMerge && seg_hi == a1 && !whole) final_global = true;
     if (wr == 0) {
-      const bool whole = (a == us) && (seg_hi == ue);
       bool finish = whole;
-      // A unit cut in exactly two parts whose CTAs form one cluster is merged through the even
-      // CTA's shared memory: the odd CTA stores its record there and arrives on a barrier.
-      const bool pair_merge = paired && aligned && !whole && (sh.part_start[u + 1] - sh.part_start[u] == 2) &&
-                              ((sh.part_start[u] & 1) == 0);
-      if (pair_merge) {
-        if (cluster_cta_rank() == 1) {
-          // 17 16-byte remote stores per lane (lane-major float4 records)
-          const uint32_t dst = map_to_cta(smem_u32(sh.peer_rec[mt]), 0) + lane * 16;
-#pragma unroll
-          for (int n = 0; n < 16; ++n) st_cluster_v4(dst + n * 512, acc[n][0], acc[n][1], acc[n][2], acc[n][3]);
-          st_cluster_v4(dst + 16 * 512, m0, l0, m1, l1);
-          __syncwarp();
-          if (lane == 0) mbar_arrive_remote(map_to_cta(smem_u32(&sh.peer_full), 0));
-        } else {
-          if (!mbar_wait_cluster(&sh.peer_full, 0u, &sh.abort_flag)) { sh.abort_flag = 1; ok = false; break; }
-          const float4* rec = reinterpret_cast<const float4*>(sh.peer_rec[mt]) + lane;
-          const float4 ml = rec[16 * 32];
-          float mn, ao, ai;
-          merge_scales(m0, ml.x, mn, ao, ai);
-          l0 = l0 * ao + ml.y * ai;
-          m0 = mn;
-          float mn1, ao1, ai1;
-          merge_scales(m1, ml.z, mn1, ao1, ai1);
-          l1 = l1 * ao1 + ml.w * ai1;
-          m1 = mn1;
-#pragma unroll
-          for (int n = 0; n < 16; ++n) {
-            const float4 r = rec[n * 32];
-            acc[n][0] = acc[n][0] * ao + r.x * ai;
-            acc[n][1] = acc[n][1] * ao + r.y * ai;
-            acc[n][2] = acc[n][2] * ao1 + r.z * ai1;
-            acc[n][3] = acc[n][3] * ao1 + r.w * ai1;
-          }
-          finish = true;
-        }
-      } else if (!whole) {
+      if (!whole) {
         // publish this CTA's share of the unit, then see whether it was the last to arrive
         // lane-major float4 records, as in shared memory
         float4* rec = reinterpret_cast<float4*>(
@@ -1108,8 +1194,10 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
         __stcg(rec + 16 * 32, make_float4(m0, l0, m1, l1));
         __threadfence();
         __syncwarp();
-        const int i_lo = aligned ? sh.part_start[u] : cta_of_atom(us, N, NP);
-        const int i_hi = aligned ? sh.part_start[u + 1] - 1 : cta_of_atom(ue - 1, N, NP);
+        const long long N = sh.part.atoms, NP = sh.part.ctas;
+        const bool aligned = sh.part.aligned != 0;
+        const int i_lo = aligned ? blockIdx.x - sh.part.mine[1] : cta_of_atom(us, N, NP);
+        const int i_hi = aligned ? i_lo + sh.part.mine[2] - 1 : cta_of_atom(ue - 1, N, NP);
         unsigned int old = 0;
         if (lane == 0) old = atomicAdd(P.counters + u * kCountersPerUnit + mt, 1u);
         old = __shfl_sync(0xffffffffu, old, 0);
@@ -1234,31 +1322,108 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     // the first warp, and nothing of the unit's state is needed any more)
     named_bar_sync(1 + mt, WPM * 32);
     if (sh.merge_last[mt])
-      merge_half<MT>(P, mt, wr, sh.merge_arg[mt][0], sh.merge_arg[mt][1], aligned, N, NP, sh.merge_arg[mt][2],
+      merge_half<MT>(P, mt, wr, sh.merge_arg[mt][0], sh.merge_arg[mt][1], sh.part.aligned != 0, sh.part.atoms, sh.part.ctas, sh.merge_arg[mt][2],
                      sh.merge_arg[mt][3], sh.merge_arg[mt][4]);
   }
-  if (paired && !peer_seen) cluster_wait();
+  if (in_cluster) {
+    const uint32_t rec = smem_u32(sh.scratch[mt][0]);
+    const int u = sh.part.mine[0], me = sh.part.mine[1], k = sh.part.mine[2];
+    if (k == 2) merge_cluster<MT, WPM, 2>(P, rec, mt, wr, me, u);
+    else if (k == 4) merge_cluster<MT, WPM, 4>(P, rec, mt, wr, me, u);
+    else merge_cluster<MT, WPM, 8>(P, rec, mt, wr, me, u);
+  }
   if (!ok && P.status && lane == 0) atomicOr(P.status, SPECATTN_ROW_TIMEOUT);
 }
 
+// CTAs per cluster for U units on n_sm SMs: as many parts per unit as there are SMs for, as a power of
+// two (clusters of three do not fill the GPCs: 48 of them do not run at once).  Pairs also serve calls with one
+// CTA per unit: they let a long list among short ones be cut.
+int want_cluster(long long units, int n_sm) {
+  const long long k = (units > 0) ? n_sm / units : 1;
+  if (k >= 8) return 8;
+  if (k >= 4) return 4;
+  return (units > n_sm) ? 1 : 2;
+}
+
 template <int MT, int WPM>
-cudaError_t launch(const VerifyParams& P, int n_ctas, cudaStream_t stream) {
-  const size_t smem = sizeof(VShared<MT, WPM>) + 128;
-  static std::atomic<unsigned long long> done_mask{0};  // per device: shared-memory opt-in done
-  int dev = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!((done_mask.load(std::memory_order_acquire) >> dev) & 1ull)) {
-    err = cudaFuncSetAttribute(sparse_verify_kernel<MT, WPM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(smem));
-    if (err != cudaSuccess) return err;
-    done_mask.fetch_or(1ull << dev, std::memory_order_release);
+constexpr size_t verify_smem() {
+  static_assert(sizeof(VShared<MT, WPM>) + 128 <= 227 * 1024, "shared memory of one CTA");
+  return sizeof(VShared<MT, WPM>) + 128;
+}
+
+const void* verify_kernel_of(int m_tiles, size_t* smem, int* threads) {
+  switch (m_tiles) {
+    case 1: *smem = verify_smem<1, 4>(); *threads = (4 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<1, 4>;
+    case 2: *smem = verify_smem<2, 4>(); *threads = (8 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<2, 4>;
+    case 3: *smem = verify_smem<3, 2>(); *threads = (6 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<3, 2>;
+    default: *smem = verify_smem<4, 2>(); *threads = (8 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<4, 2>;
   }
+}
+
+// Grid and cluster size of a launch: whole clusters, as many as run at once (GPCs do not hold a multiple of
+// every cluster size).  Opts the kernel in to its shared memory and asks the runtime once per device,
+// kernel and cluster size.  false: the runtime refused.
+bool verify_grid(int m_tiles, long long units, int n_sm, int* n_ctas, int* cluster) {
+  static std::atomic<int> known[64][4][kMaxCluster + 1];  // clusters that fit + 1, 0 = not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return false;
+  }
+  size_t smem;
+  int threads;
+  const void* fn = verify_kernel_of(m_tiles, &smem, &threads);
+  int cs = want_cluster(units, n_sm);
+  for (;;) {
+    std::atomic<int>& slot = known[dev][m_tiles - 1][cs];
+    int n = slot.load(std::memory_order_acquire);
+    if (n == 0) {
+      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+      }
+      int fit = n_sm;
+      if (cs > 1) {
+        cudaLaunchConfig_t q;
+        memset(&q, 0, sizeof(q));
+        q.gridDim = dim3(static_cast<unsigned>(n_sm / cs * cs), 1, 1);
+        q.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+        q.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(cs);
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        q.attrs = attr;
+        q.numAttrs = 1;
+        fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, fn, &q) != cudaSuccess) {
+          cudaGetLastError();
+          fit = 0;
+        }
+      }
+      n = fit + 1;
+      slot.store(n, std::memory_order_release);
+    }
+    const int ctas = (n - 1 < n_sm / cs ? n - 1 : n_sm / cs) * cs;
+    // a size that leaves too much of the GPU idle is not worth its merges
+    if (cs == 1 || ctas * 8 >= n_sm * 7 || (ctas > 0 && ctas >= units * cs)) {
+      *n_ctas = ctas;
+      *cluster = cs;
+      return ctas > 0;
+    }
+    cs = (cs > 4) ? 4 : (cs > 2) ? 2 : 1;
+  }
+}
+
+cudaError_t launch_verify(const VerifyParams& P, int m_tiles, int n_ctas, cudaStream_t stream) {
+  size_t smem;
+  int threads;
+  const void* fn = verify_kernel_of(m_tiles, &smem, &threads);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(static_cast<unsigned>(n_ctas), 1, 1);
-  cfg.blockDim = dim3((MT * WPM + kProdWarps) * 32, 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -1266,14 +1431,15 @@ cudaError_t launch(const VerifyParams& P, int n_ctas, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (MT <= 2 && n_ctas % 2 == 0) {  // CTA pairs: short units are merged through peer shared memory
+  if (P.cluster > 1) {
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(P.cluster);
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
   }
-  err = cudaLaunchKernelEx(&cfg, sparse_verify_kernel<MT, WPM>, P);
+  void* params[1] = {const_cast<VerifyParams*>(&P)};
+  const cudaError_t err = cudaLaunchKernelExC(&cfg, fn, params);
   if (err != cudaSuccess) cudaGetLastError();
   return err;
 }
@@ -1431,7 +1597,6 @@ VerifyParams make_params(const specattn_verify_args& A) {
 
   P.plan = static_cast<const int*>(A.plan);
   P.test_lose = (A.flags & SPECATTN_VERIFY_TEST_LOSE_ARRIVAL) ? 1 : 0;
-  P.pairs = (m_tiles(A) <= 2 && device_sm_count() % 2 == 0) ? 1 : 0;  // as launch() decides
   return P;
 }
 }  // namespace
@@ -1495,12 +1660,10 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
       }
     }
   } else {
-    switch (specattn::m_tiles(A)) {
-      case 1: err = specattn::launch<1, 4>(P, n_ctas, stream); break;
-      case 2: err = specattn::launch<2, 4>(P, n_ctas, stream); break;
-      case 3: err = specattn::launch<3, 2>(P, n_ctas, stream); break;
-      default: err = specattn::launch<4, 2>(P, n_ctas, stream); break;
-    }
+    int grid = 0;
+    if (!specattn::verify_grid(specattn::m_tiles(A), static_cast<long long>(A.batch) * A.n_kv_heads, n_ctas, &grid, &P.cluster))
+      return SPECATTN_ERR_CUDA;
+    err = specattn::launch_verify(P, specattn::m_tiles(A), grid, stream);
   }
   if (err != cudaSuccess) return SPECATTN_ERR_CUDA;
   specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
@@ -1528,6 +1691,9 @@ extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan
   if (plan_bytes < specattn::plan_ints(A.batch * A.n_kv_heads, n_ctas) * sizeof(int)) return SPECATTN_ERR_WORKSPACE;
   if (A.batch == 0) return SPECATTN_OK;
   VerifyParams P = specattn::make_params(A);
+  int grid = 0;
+  if (!specattn::verify_grid(specattn::m_tiles(A), static_cast<long long>(A.batch) * A.n_kv_heads, n_ctas, &grid, &P.cluster))
+    return SPECATTN_ERR_CUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(1, 1, 1);
@@ -1538,7 +1704,7 @@ extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, specattn::verify_plan_kernel, P, static_cast<int*>(plan), n_ctas) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, specattn::verify_plan_kernel, P, static_cast<int*>(plan), grid) != cudaSuccess) {
     cudaGetLastError();
     return SPECATTN_ERR_CUDA;
   }
@@ -1571,10 +1737,12 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
       if (args[i]->batch == 0) continue;
       B.p[m] = specattn::make_params(*args[i]);
       B.plan[m] = static_cast<int*>(plans[i]);
+      if (!specattn::verify_grid(specattn::m_tiles(*args[i]), static_cast<long long>(args[i]->batch) * args[i]->n_kv_heads,
+                                 n_ctas, &B.grid[m], &B.p[m].cluster))
+        return SPECATTN_ERR_CUDA;
       ++m;
     }
     if (m == 0) continue;
-    B.G = n_ctas;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(static_cast<unsigned>(m), 1, 1);

@@ -39,6 +39,7 @@
 constexpr int kTcTile = 128;                     // keys per tile
 constexpr int kTcTileBytes = kTcTile * 256;      // one K or V tile (32 KB)
 constexpr int kTcStages = 3;
+constexpr int kTcMinPartAtoms = 8;              // no part of a unit is shorter: every part costs a record and an arrival
 constexpr int kTcRec = 130 * 32;                 // floats of a record per 32 query rows
 constexpr float kTcRaise = 8.f;                  // raise the reference maximum beyond 2^8
 constexpr int kTcThreads = 13 * 32;
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sparse_verify_tc_kernel(const _
         int k = static_cast<int>((2 * num + den) / (2 * den));
         if (k < 1) k = 1;
         if (k > atoms) k = atoms;
-        if (k * kMinPartAtoms > atoms) k = max(1, atoms / kMinPartAtoms);  // no part shorter than that
+        if (k * kTcMinPartAtoms > atoms) k = max(1, atoms / kTcMinPartAtoms);  // no part shorter than that
         atomicAdd(&sh.cand_parts[c], k);
         atomicMax(&sh.cand_max[c], (atoms + k - 1) / k);
       }
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) sparse_verify_tc_kernel(const _
           k = static_cast<int>((2 * num + den) / (2 * den));
           if (k < 1) k = 1;
           if (k > atoms) k = atoms;
-        if (k * kMinPartAtoms > atoms) k = max(1, atoms / kMinPartAtoms);  // no part shorter than that
+        if (k * kTcMinPartAtoms > atoms) k = max(1, atoms / kTcMinPartAtoms);  // no part shorter than that
         }
       }
       int v = k;

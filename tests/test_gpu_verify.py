@@ -473,3 +473,32 @@ def test_page_granular_per_head_lists_tails_and_contiguous_cache():
             assert st[1] == sa.ROW_BAD_INDEX
     finally:
         _ENGINE["flags"] = flags0
+
+
+@pytest.mark.parametrize("hkv,counts", [
+    (2, [1200, 0, 33, 130, 64]),                       # up to eight parts a unit: 8, 4, 2, 1 and an empty list
+    (8, [65, 127, 513]),                               # up to four
+    (8, [900, 17, 260, 0, 1024, 700]),                 # pairs, or more parts through global memory
+    (8, [300] * 9 + [2048]),                           # one long list among short ones
+    (8, [40 + 16 * i for i in range(20)]),             # more units than CTAs
+])
+def test_mixed_list_lengths_cut_into_parts_of_one_cluster(hkv, counts):
+    """Units of one call cut into different numbers of parts (a power of two up to the cluster size),
+    with and without a precomputed partition: same results, within the oracle's tolerance."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    case = _make_case(95, len(counts), 5, 4 * hkv, hkv, 16, [max(2 * c, 50) for c in counts], counts=[[c] for c in counts])
+    out, lse, status = _run(case)
+    assert int(status.abs().sum()) == 0
+    check_attention(out, lse, *_oracle(case))
+    kv_d = case["kv"].to(dev())
+    o, l, st = torch.empty_like(out), torch.empty_like(lse), torch.zeros_like(status)
+    keep = [bf16_to_dev(case["q"]), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]), to_dev(case["cnt"])]
+    a = sa.make_verify_args(keep[0], kv_d, keep[1], block_table=keep[2], idx=keep[3], counts=keep[4], out=o, lse=l,
+                            status=st, flags=_ENGINE["flags"])
+    ws, plan = sa.verify_workspace(a), sa.verify_plan_buffer(a)
+    a.workspace, a.workspace_bytes, a.plan = ws.data_ptr(), ws.numel(), plan.data_ptr()
+    sa.verify_plan(a, plan)
+    assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(o, out) and torch.equal(l, lse)
