@@ -246,6 +246,14 @@ size_t specattn_select_workspace_bytes(const specattn_select_args* args);
  * results for its sequence (entries that are not multiples of 16 raise SPECATTN_ROW_BAD_INDEX),
  * never a fault.  Results are the same as without the flag. */
 #define SPECATTN_VERIFY_PAGE_LISTS 8u
+/* SPECATTN_VERIFY_INIT_WORKSPACE / SPECATTN_VERIFY_INIT_STATUS: the call itself clears, on the stream and
+ * ahead of its kernel, the workspace's arrival counters that it uses (the workspace needs no
+ * specattn_verify_workspace_init before this call; nor can another call rely on it afterwards
+ * unless that call has at most this one's batch * n_kv_heads) / the status words.  One small kernel for
+ * both, which the verify kernel overlaps: cheaper than two memsets in front of a call that allocates
+ * its workspace anew. */
+#define SPECATTN_VERIFY_INIT_WORKSPACE 16u
+#define SPECATTN_VERIFY_INIT_STATUS 32u
 /* TEST ONLY -- never set this in production.  Exercises the failure path of the kernels' bounded
  * device-side waits without faulting anything: one producer warp of CTA 0 withholds the
  * completion signal of its first tile, the waits on it give up after their poll limit (about

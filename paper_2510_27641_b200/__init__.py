@@ -7,6 +7,7 @@ is no fallback: if the shared library has not been built the first call raises.
 from __future__ import annotations
 
 import ctypes as C
+import threading
 from pathlib import Path
 from typing import Sequence
 
@@ -17,7 +18,7 @@ __all__ = ["select_topp", "sparse_verify", "sparse_verify_static", "verify_works
            "SelectArgs", "VerifyArgs", "StepHostArgs", "lib", "SpecAttnError",
            "ROW_OK", "ROW_INVALID_PROB", "ROW_OVERFLOW", "ROW_BAD_INDEX", "ROW_TIMEOUT",
            "VERIFY_LISTS_STABLE", "VERIFY_ENGINE_MMA_SYNC", "VERIFY_ENGINE_TCGEN05",
-           "VERIFY_TEST_LOSE_ARRIVAL", "VERIFY_PAGE_LISTS", "SELECT_FORM_AUTO", "SELECT_FORM_CLUSTER",
+           "VERIFY_TEST_LOSE_ARRIVAL", "VERIFY_PAGE_LISTS", "VERIFY_INIT_WORKSPACE", "VERIFY_INIT_STATUS", "SELECT_FORM_AUTO", "SELECT_FORM_CLUSTER",
            "SELECT_FORM_TWO_LAUNCH", "verify_plan",
            "verify_plan_buffer", "verify_plan_many"]
 
@@ -26,6 +27,7 @@ VERIFY_LISTS_STABLE = 1
 VERIFY_ENGINE_MMA_SYNC = 2
 VERIFY_ENGINE_TCGEN05 = 4
 VERIFY_PAGE_LISTS = 8
+VERIFY_INIT_WORKSPACE, VERIFY_INIT_STATUS = 16, 32
 SELECT_FORM_AUTO, SELECT_FORM_CLUSTER, SELECT_FORM_TWO_LAUNCH = 0, 1, 2
 VERIFY_TEST_LOSE_ARRIVAL = 0x80000000   # test only: see include/specattn.h
 
@@ -121,10 +123,34 @@ def kernel_launch_count() -> int:
     return int(lib().specattn_kernel_launch_count())
 
 
-def _stream_ptr(stream) -> C.c_void_p:
+def _stream_ptr(stream) -> int:
+    """The cudaStream_t of a torch stream; None = the current stream of the current device (asked of
+    torch's C layer: torch.cuda.current_stream() builds a Python object, ~4 us a call)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
+
+
+class _Calls(threading.local):
+    """Argument structs of the one-call entry points, kept per thread and per shape: filling the ~20
+    fields of a struct that a call shares with the previous one of its shape took most of the call's host time.  A
+    call overwrites every pointer before the library sees the struct."""
+
+    LIMIT = 64
+
+    def __init__(self):
+        self.made = {}
+
+    def get(self, key, make):
+        call = self.made.get(key)
+        if call is None:
+            if len(self.made) >= self.LIMIT:
+                self.made.clear()
+            call = self.made[key] = make()
+        return call
+
+
+_calls = _Calls()
 
 
 def _ptr(t: torch.Tensor | None):
@@ -189,28 +215,59 @@ def select_topp(draft_probs: Sequence[torch.Tensor | None], kv_len: torch.Tensor
     (idx [n_d,B,G,idx_stride] int32, counts [n_d,B,G], row_status [n_d,B,G], diag or None)."""
     n_d = len(draft_probs)
     ref = next(t for t in draft_probs if t is not None)
-    B, _, _, Ls = ref.shape
+    shape, layer_map = ref.shape, tuple(layer_map)
+    B, Ls = shape[0], shape[3]
     dev = ref.device
-    stride = int(Ls if idx_stride is None else idx_stride)
     if idx is None:
-        idx = torch.empty((n_d, B, n_groups, stride), dtype=torch.int32, device=dev)
+        idx = torch.empty((n_d, B, n_groups, int(Ls if idx_stride is None else idx_stride)), dtype=torch.int32, device=dev)
+    # the library leaves the entries of unmapped draft layers alone
+    new = torch.empty if set(layer_map).issuperset(range(n_d)) else _minus_one
     if counts is None:
-        counts = torch.full((n_d, B, n_groups), -1, dtype=torch.int32, device=dev)
+        counts = new((n_d, B, n_groups), dtype=torch.int32, device=dev)
     if row_status is None:
-        row_status = torch.full((n_d, B, n_groups), -1, dtype=torch.int32, device=dev)
+        row_status = new((n_d, B, n_groups), dtype=torch.int32, device=dev)
     if diag is None and want_diag:
         diag = torch.zeros((n_d, B, n_groups, 4), dtype=torch.float64, device=dev)
-    args, keep = make_select_args(draft_probs, kv_len, layer_map, p, n_groups=n_groups,
-                                  head_group=head_group, idx=idx, counts=counts,
-                                  row_status=row_status, diag=diag, per_step=per_step,
-                                  bisect_iters=bisect_iters, chunk=chunk, workspace=workspace, form=form)
-    rc = lib().specattn_select_topp(C.byref(args), _stream_ptr(stream))
+    held = tuple([t is not None for t in draft_probs])
+    groups = None if head_group is None else tuple(head_group)
+    key = (held, shape, layer_map, p, n_groups, groups, idx.shape, per_step, bisect_iters, chunk, form)
+
+    def make():
+        args, keep = make_select_args(draft_probs, kv_len, layer_map, p, n_groups=n_groups, head_group=head_group,
+                                      idx=idx, counts=counts, row_status=row_status, diag=diag, per_step=per_step,
+                                      bisect_iters=bisect_iters, chunk=chunk, workspace=None, form=form)
+        return args, C.byref(args), keep[:3], int(lib().specattn_select_workspace_bytes(C.byref(args)))
+
+    args, ref_args, (ptrs, _, _), need = _calls.get(key, make)
+    for u, t in enumerate(draft_probs):
+        if t is not None:
+            assert t.dtype is torch.float32 and t.is_contiguous() and t.shape == shape
+            ptrs[u] = t.data_ptr()
+    assert kv_len.dtype is torch.int32 and idx.dtype is torch.int32 and counts.dtype is torch.int32
+    assert idx.is_contiguous()
+    args.kv_len, args.idx = kv_len.data_ptr(), idx.data_ptr()
+    args.counts, args.row_status = counts.data_ptr(), row_status.data_ptr()
+    args.diag = None if diag is None else diag.data_ptr()
+    given = workspace
+    if workspace is True:
+        workspace = torch.empty((need,), dtype=torch.uint8, device=dev) if need > 0 else None
+    elif workspace is False:
+        workspace = None
+    if workspace is None:
+        args.workspace, args.workspace_bytes = None, 0
+    else:
+        assert workspace.dtype is torch.uint8 and workspace.is_contiguous()
+        args.workspace, args.workspace_bytes = workspace.data_ptr(), workspace.numel()
+    rc = lib().specattn_select_topp(ref_args, _stream_ptr(stream))
     if rc != 0:
         raise SpecAttnError(rc, "specattn_select_topp")
-    if keep[-1] is not None and stream is not None and workspace is True:
-        keep[-1].record_stream(stream)   # allocated here, used on the caller's stream
-    del keep
+    if workspace is not None and stream is not None and given is True:
+        workspace.record_stream(stream)   # allocated here, used on the caller's stream
     return idx, counts, row_status, diag
+
+
+def _minus_one(shape, dtype, device):
+    return torch.full(shape, -1, dtype=dtype, device=device)
 
 
 def make_verify_args(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor, *,
@@ -279,23 +336,49 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
                   flags: int = 0, tail_len: int = 0, stream=None):
     """specattn_sparse_verify for one target layer.  Returns (out f32 [B,T,H_q,d], lse f32
     [B,T,H_q], status int32 [B])."""
-    B, T, Hq, d = q.shape
+    B, T, Hq, d = shape = q.shape
+    dev = q.device
+    own = 0   # what the call has to clear: buffers that were made here
     if out is None:
-        out = torch.empty((B, T, Hq, d), dtype=torch.float32, device=q.device)
+        out = torch.empty(shape, dtype=torch.float32, device=dev)
     if lse is None:
-        lse = torch.empty((B, T, Hq), dtype=torch.float32, device=q.device)
+        lse = torch.empty((B, T, Hq), dtype=torch.float32, device=dev)
     if status is None:
-        status = torch.zeros((B,), dtype=torch.int32, device=q.device)
-    args = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq,
-                            idx=idx, counts=counts, n_groups=n_groups, dense=dense, sm_scale=sm_scale,
-                            out=out, lse=lse, status=status, workspace=workspace, flags=flags,
-                            tail_len=tail_len)
-    if workspace is None:
-        workspace = verify_workspace(args, q.device, stream)
-        args.workspace, args.workspace_bytes = workspace.data_ptr(), workspace.numel()
-    rc = lib().specattn_sparse_verify(C.byref(args), _stream_ptr(stream))
+        status = torch.empty((B,), dtype=torch.int32, device=dev)
+        own |= VERIFY_INIT_STATUS
+    made = workspace is None
+    if made:
+        own |= VERIFY_INIT_WORKSPACE
+    key = (shape, kv_pages.shape, kv_pages.stride(), None if block_table is None else block_table.stride(),
+           pages_per_seq, None if dense else (idx.shape, idx.stride()), n_groups, dense, sm_scale, flags, tail_len)
+
+    def make():
+        a = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq, idx=idx,
+                             counts=counts, n_groups=n_groups, dense=dense, sm_scale=sm_scale, out=out, lse=lse,
+                             flags=flags, tail_len=tail_len)
+        return a, C.byref(a), verify_workspace_bytes(a)
+
+    args, ref_args, need = _calls.get(key, make)
+    assert q.is_contiguous() and q.dtype is torch.bfloat16 and kv_pages.dtype is torch.bfloat16
+    if made:
+        if need == 0:
+            raise SpecAttnError(-6, "specattn_verify_workspace_bytes")
+        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
+    args.q, args.kv_pages, args.kv_len = q.data_ptr(), kv_pages.data_ptr(), kv_len.data_ptr()
+    if block_table is not None:
+        assert block_table.dtype is torch.int32
+        args.block_table = block_table.data_ptr()
+    if not dense:
+        assert idx.dtype is torch.int32 and counts.dtype is torch.int32 and counts.is_contiguous()
+        args.idx, args.counts = idx.data_ptr(), counts.data_ptr()
+    args.out, args.lse, args.status = out.data_ptr(), lse.data_ptr(), status.data_ptr()
+    args.workspace, args.workspace_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
+    args.flags = int(flags) | own
+    rc = lib().specattn_sparse_verify(ref_args, _stream_ptr(stream))
     if rc != 0:
         raise SpecAttnError(rc, "specattn_sparse_verify")
+    if made and stream is not None:
+        workspace.record_stream(stream)   # allocated here, used on the caller's stream
     return out, lse, status
 
 

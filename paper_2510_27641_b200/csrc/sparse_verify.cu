@@ -415,6 +415,15 @@ __global__ void __launch_bounds__(256, 1) verify_plan_kernel(const __grid_consta
   plan_body(P, plan, G);
 }
 
+// Clears the arrival counters of U units and / or the status words in front of a verify launch, whose CTAs
+// may take their places meanwhile (they wait for this grid's end before they read anything).
+__global__ void __launch_bounds__(256, 1) verify_init_kernel(unsigned int* counters, int n_counters, int* status, int n_status) {
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = threadIdx.x; i < n_counters; i += 256) counters[i] = 0u;
+  for (int i = threadIdx.x; i < n_status; i += 256) status[i] = 0;
+}
+
 // The plans of several launches (one per draft layer whose lists the step's layers share) in
 // one launch, one CTA each.
 constexpr int kPlanBatch = 8;
@@ -1591,7 +1600,11 @@ VerifyParams make_params(const specattn_verify_args& A) {
   P.out = A.out;
   P.lse = A.lse;
   P.status = A.status;
-  P.lists_stable = (A.flags & SPECATTN_VERIFY_LISTS_STABLE) ? 1 : 0;
+  // (after a clearing launch the kernel waits for that launch before anything else)
+  P.lists_stable = (A.flags & (SPECATTN_VERIFY_LISTS_STABLE | SPECATTN_VERIFY_INIT_WORKSPACE | SPECATTN_VERIFY_INIT_STATUS)) ==
+                           SPECATTN_VERIFY_LISTS_STABLE
+                       ? 1
+                       : 0;
   P.tail = A.tail_len;
   P.tail_off = A.tail_len - A.n_q;
 
@@ -1641,6 +1654,27 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t err;
+  const bool init_ws = (A.flags & SPECATTN_VERIFY_INIT_WORKSPACE) != 0;
+  const bool init_status = (A.flags & SPECATTN_VERIFY_INIT_STATUS) != 0 && A.status != nullptr;
+  if (init_ws || init_status) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(1, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, specattn::verify_init_kernel, P.counters,
+                           init_ws ? A.batch * A.n_kv_heads * specattn::kCountersPerUnit : 0, A.status,
+                           init_status ? A.batch : 0) != cudaSuccess) {
+      cudaGetLastError();
+      return SPECATTN_ERR_CUDA;
+    }
+    specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
+  }
   if (specattn::use_tcgen05(A)) {
     alignas(64) CUtensorMap kv_map;
     memset(&kv_map, 0, sizeof(kv_map));

@@ -502,3 +502,27 @@ def test_mixed_list_lengths_cut_into_parts_of_one_cluster(hkv, counts):
     assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
     torch.cuda.synchronize()
     assert torch.equal(o, out) and torch.equal(l, lse)
+
+
+@pytest.mark.parametrize("kept", [40, 2500])
+def test_a_call_that_clears_its_own_workspace_and_status(kept):
+    """Workspace and status full of ones: with the two flags the call clears what it uses itself; with a
+    given status and without its flag, earlier status bits stay."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    case = _make_case(96, 3, 5, 32, 8, 16, [3000] * 3, counts=[[kept], [kept // 2], [kept]])
+    keep = [bf16_to_dev(case["q"]), case["kv"].to(dev()), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]),
+            to_dev(case["cnt"])]
+    out, lse, status = _run(case)
+    for init_status in (True, False):
+        o, l = torch.empty_like(out), torch.empty_like(lse)
+        st = torch.full_like(status, 1)
+        a = sa.make_verify_args(keep[0], keep[1], keep[2], block_table=keep[3], idx=keep[4], counts=keep[5], out=o, lse=l,
+                                status=st, flags=_ENGINE["flags"] | sa.VERIFY_INIT_WORKSPACE |
+                                (sa.VERIFY_INIT_STATUS if init_status else 0) | sa.VERIFY_LISTS_STABLE)
+        ws = torch.full((sa.verify_workspace_bytes(a),), 255, dtype=torch.uint8, device=dev())
+        a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+        assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(o, out) and torch.equal(l, lse)
+        assert st.tolist() == ([0, 0, 0] if init_status else [1, 1, 1])
