@@ -104,8 +104,7 @@ struct Partition {
   int parts[2][kCandidates];    // inside clusters / anywhere, per candidate share: CTAs needed, largest part
   int largest[2][kCandidates];
   int unit_max;              // atoms of the largest unit
-  unsigned long long before[kAlignedMaxUnits / 32];  // units per class (16 bits each) before each group of 32 units
-  unsigned long long all;    // units per class
+  unsigned long long units[kAlignedMaxUnits / 32];  // units per class (16 bits each) of each group of 32 units
   // this CTA's share, for the end of the kernel (kept out of registers meanwhile)
   int mine[3];               // unit (-1: none), part and number of parts
   int atoms, ctas, aligned;  // N, the number of CTAs with work, whether units are dealt in equal parts
@@ -132,10 +131,12 @@ __device__ __forceinline__ int cand_share(long long N, int G, int c) {
 // Class of k parts: 0 for the cluster size, 1 for half of it, ...
 __device__ __forceinline__ int class_of(int k, int cluster) { return __ffs(cluster) - __ffs(k); }
 
-// Decides the partition (all NT threads of the CTA, after a barrier that follows unit_start[]): the candidate share, or -1 for ranges; `cluster` becomes 1 where parts are to merge through
-// global memory.  One barrier; warp 0 alone may go on to partition_locate() without another.
-template <int NT>
-__device__ __forceinline__ int partition_decide(Partition& pt, const int* unit_start, int U, int G, int& cluster) {
+// Decides the partition (all NT threads of the CTA, after a barrier that follows unit_start[]): the candidate
+// share, or -1 for ranges; `cluster` becomes 1 where parts are to merge through global memory.  Then calls
+// place(unit, first CTA, number of parts) for every unit of an aligned partition, each from one thread.  Two
+// barriers, none after the last place().
+template <int NT, class Place>
+__device__ __forceinline__ int partition_units(Partition& pt, const int* unit_start, int U, int G, int& cluster, Place place) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int N = unit_start[U];
   const bool try_aligned = U <= kAlignedMaxUnits && N > 0;
@@ -188,76 +189,52 @@ __device__ __forceinline__ int partition_decide(Partition& pt, const int* unit_s
     }
   }
   if (way == 1) cluster = 1;
-  if (cand >= 0 && tid < 32) {  // units per class, 16 bits each, before every group of 32 units
-    const int share = cand_share(N, G, cand);
-    unsigned long long seen = 0ull;
-    for (int base = 0; base < U; base += 32) {
-      const int u = base + lane;
-      const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-      // (without clusters: the units' CTAs, which lie in the order of the units)
-      const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
-      const int at = (cluster == 1) ? 0 : 16 * class_of(k, cluster);
-      const unsigned one = (k == 0) ? 0u : (cluster == 1) ? static_cast<unsigned>(k) : 1u << (at & 31);
-      const unsigned long long hi = __reduce_add_sync(0xffffffffu, at < 32 ? 0u : one);
-      if (lane == 0) pt.before[base >> 5] = seen;
-      seen += (hi << 32) + __reduce_add_sync(0xffffffffu, at < 32 ? one : 0u);
-    }
-    if (lane == 0) pt.all = seen;
-    __syncwarp();
+  if (cand < 0) return cand;
+  // A warp takes 32 units.  Inside clusters units are placed by class, so a unit's place is the CTAs of the
+  // classes before its own plus its rank in its class; otherwise units lie in their order.
+  const int share = cand_share(N, G, cand);
+  for (int base = (tid >> 5) * 32; base < U; base += NT) {
+    const int u = base + lane;
+    const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
+    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+    const int at = (cluster == 1) ? 0 : 16 * class_of(k, cluster);
+    const unsigned one = (k == 0) ? 0u : (cluster == 1) ? static_cast<unsigned>(k) : 1u << (at & 31);
+    const unsigned long long hi = __reduce_add_sync(0xffffffffu, at < 32 ? 0u : one);
+    const unsigned lo = __reduce_add_sync(0xffffffffu, at < 32 ? one : 0u);
+    if (lane == 0) pt.units[base >> 5] = (hi << 32) + lo;
   }
-  return cand;
-}
-
-// One warp, aligned partition: the unit of CTA `me` (-1: none), its part and the number of parts.
-__device__ __forceinline__ int partition_locate(const Partition& pt, const int* unit_start, int U, int G, int cluster,
-                                                int cand, int me, int& part, int& parts) {
-  const int lane = threadIdx.x & 31;
-  const int share = cand_share(unit_start[U], G, cand);
-  if (cluster == 1) {
-    for (int base = 0; base < U; base += 32) {
-      const int u = base + lane;
-      const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-      const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+  __syncthreads();
+  for (int base = (tid >> 5) * 32; base < U; base += NT) {
+    const int u = base + lane;
+    const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
+    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+    unsigned long long before = 0ull, all = 0ull;
+    for (int i = 0; i < (U + 31) / 32; ++i) {
+      if (32 * i < base) before += pt.units[i];
+      all += pt.units[i];
+    }
+    int first;
+    if (cluster == 1) {
       int end = k;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, end, o);
         if (lane >= o) end += v;
       }
-      const int start = static_cast<int>(pt.before[base >> 5]) + end - k;
-      const unsigned hit = __ballot_sync(0xffffffffu, me >= start && me < start + k);
-      if (hit != 0u) {
-        const int l = __ffs(hit) - 1;
-        part = me - __shfl_sync(0xffffffffu, start, l);
-        parts = __shfl_sync(0xffffffffu, k, l);
-        return base + l;
+      first = static_cast<int>(before) + end - k;
+    } else {
+      int cta = 0;
+      first = 0;
+      for (int cls = 0, c = cluster; c > 0; ++cls, c >>= 1) {
+        const unsigned m = __ballot_sync(0xffffffffu, k == c);
+        const int rank = static_cast<int>((before >> (16 * cls)) & 0xffffull) + __popc(m & ((1u << lane) - 1u));
+        if (k == c) first = cta + rank * c;
+        cta += static_cast<int>((all >> (16 * cls)) & 0xffffull) * c;
       }
     }
-    return -1;
+    if (k > 0) place(u, first, k);
   }
-  // the CTA's class, its place among the class's units, the unit at that place
-  int first = 0, cls = 0, at = -1;
-  parts = cluster;
-  for (;; ++cls, parts >>= 1) {
-    const int n = static_cast<int>((pt.all >> (16 * cls)) & 0xffffull);
-    if (me < first + n * parts) {
-      at = (me - first) / parts;
-      break;
-    }
-    first += n * parts;
-    if (parts == 1) return -1;
-  }
-  part = me - first - at * parts;
-  for (int base = 0; base < U; base += 32) {
-    const int u = base + lane;
-    const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-    const bool in = atoms > 0 && unit_parts(atoms, share, cluster, U, G) == parts;
-    const unsigned m = __ballot_sync(0xffffffffu, in);
-    const int rank = static_cast<int>((pt.before[base >> 5] >> (16 * cls)) & 0xffffull) + __popc(m & ((1u << lane) - 1u));
-    const unsigned hit = __ballot_sync(0xffffffffu, in && rank == at);
-    if (hit != 0u) return base + __ffs(hit) - 1;
-  }
-  return -1;
+  return cand;
 }
 
 // WPM = consumer warps per 16-row slab: 4 -> (stage parity, 32-key half), 2 -> (stage parity).
@@ -327,12 +304,12 @@ __device__ __forceinline__ void merge_scales(float m, float im, float& mn, float
 // The partition of a launch depends only on the list lengths, the shapes and the grid: target
 // layers that share a draft layer's lists share it.  A plan holds, as int32:
 //   [0] magic  [1] U  [2] grid  [3] 0: ranges, else the partition's cluster size  [4] NP  [5] N (atoms)  [6] tail  [7] dense
-//   unit_start[U + 1], unit_cnt[U], then (a0, a1, u_first, part | parts << 8) per CTA
+//   unit_start[U + 1], unit_cnt[U], a pad, then (a0, a1, u_first, part | parts << 8) per CTA
 // A kernel whose launch does not match the header ignores the plan and partitions itself.
 constexpr int kPlanMagic = 0x5a17a9e1;
 constexpr int kPlanHeader = 8;
 __host__ __device__ inline size_t plan_ints(int U, int grid) {
-  return static_cast<size_t>(kPlanHeader) + (U + 1) + U + 4 * static_cast<size_t>(grid);
+  return static_cast<size_t>(kPlanHeader) + 2 * (U + 1) + 4 * static_cast<size_t>(grid);
 }
 
 // One CTA computes what every CTA of a verify launch would compute for itself at start-up.
@@ -347,7 +324,7 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   pdl_wait();
   int* const p_us = plan + kPlanHeader;
   int* const p_cnt = p_us + (U + 1);
-  int* const p_cta = p_cnt + U;
+  int* const p_cta = p_cnt + U + 1;   // (whole 8-byte words: the header and 2 U + 2 ints precede it)
   if (tid == 0) unit_start[0] = 0;
   for (int u = tid; u < U; u += 256) {
     const int c = unit_count(P, u);
@@ -372,32 +349,25 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   __syncthreads();
   const long long N = unit_start[U];
   int cluster = P.cluster;
-  const int cand = partition_decide<256>(pt, unit_start, U, G, cluster);
-  __syncthreads();
+  auto entry = [&](int i, int a0, int a1, int u_first, int what) {
+    *reinterpret_cast<int2*>(p_cta + 4 * i) = make_int2(a0, a1);
+    *reinterpret_cast<int2*>(p_cta + 4 * i + 2) = make_int2(u_first, what);
+  };
+  const int cand = partition_units<256>(pt, unit_start, U, G, cluster, [&](int u, int first, int k) {
+    const int us = unit_start[u], atoms = unit_start[u + 1] - us;
+    for (int j = 0; j < k; ++j) entry(first + j, us + j * atoms / k, us + (j + 1) * atoms / k, u, j | (k << 8));
+  });
   const bool aligned = cand >= 0;
   const long long NP = aligned ? pt.parts[cluster > 1 ? 0 : 1][cand] : ((N < G) ? N : static_cast<long long>(G));
   for (int u = tid; u <= U; u += 256) p_us[u] = unit_start[u];
-  for (int i = warp; i < G; i += 8) {
-    int a0 = 0, a1 = 0, u_first = 0, part = 0, parts = 0;
-    if (aligned) {
-      const int u = partition_locate(pt, unit_start, U, G, cluster, cand, i, part, parts);
-      if (u >= 0) {
-        const int atoms = unit_start[u + 1] - unit_start[u];
-        a0 = unit_start[u] + part * atoms / parts;
-        a1 = unit_start[u] + (part + 1) * atoms / parts;
-        u_first = u;
-      }
-    } else if (i < NP) {
+  for (int i = (aligned ? static_cast<int>(NP) : 0) + tid; i < G; i += 256) {
+    int a0 = 0, a1 = 0, u_first = 0;
+    if (i < NP) {
       a0 = cta_first_atom(i, N, NP);
       a1 = cta_first_atom(i + 1, N, NP);
       u_first = unit_of_atom(unit_start, U, a0);
     }
-    if (lane == 0) {
-      p_cta[4 * i] = a0;
-      p_cta[4 * i + 1] = a1;
-      p_cta[4 * i + 2] = u_first;
-      p_cta[4 * i + 3] = part | (parts << 8);
-    }
+    entry(i, a0, a1, u_first, 0);
   }
   if (tid == 0) {
     plan[1] = U;
@@ -789,7 +759,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     aligned = plan[3] != 0;
     cluster = plan[3];
     NP = plan[4];
-    const int* const p_cta = plan + kPlanHeader + (U + 1) + U + 4 * blockIdx.x;
+    const int* const p_cta = plan + kPlanHeader + 2 * (U + 1) + 4 * blockIdx.x;
     a0 = p_cta[0];
     a1 = p_cta[1];
     u_first = p_cta[2];
@@ -814,24 +784,23 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
 
   N = sh.unit_start[U];
   cluster = P.cluster;
-  const int cand = partition_decide<NT>(sh.part, sh.unit_start, U, G, cluster);
+  const int cand = partition_units<NT>(sh.part, sh.unit_start, U, G, cluster, [&](int u, int first, int k) {
+    const int j = static_cast<int>(blockIdx.x) - first;
+    if (j >= 0 && j < k) {
+      sh.part.mine[0] = u;
+      sh.part.mine[1] = j;
+      sh.part.mine[2] = k;
+    }
+  });
   aligned = cand >= 0;
   NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : ((N < G) ? N : static_cast<long long>(G));
   if (aligned) {
-    if (warp == 0) {
-      const int u = partition_locate(sh.part, sh.unit_start, U, G, cluster, cand, blockIdx.x, part, parts);
-      if (lane == 0) {
-        sh.part.mine[0] = u;
-        sh.part.mine[1] = part;
-        sh.part.mine[2] = parts;
-      }
-    }
     __syncthreads();
-    u_first = max(sh.part.mine[0], 0);
-    part = sh.part.mine[1];
-    parts = sh.part.mine[2];
     if (static_cast<long long>(blockIdx.x) < NP) {
-      const int atoms = sh.unit_start[u_first + 1] - sh.unit_start[u_first];  // part < parts <= 8: fits 32 bits
+      u_first = sh.part.mine[0];
+      part = sh.part.mine[1];
+      parts = sh.part.mine[2];
+      const int atoms = sh.unit_start[u_first + 1] - sh.unit_start[u_first];  // part < parts: the products fit 32 bits
       a0 = sh.unit_start[u_first] + part * atoms / parts;
       a1 = sh.unit_start[u_first] + (part + 1) * atoms / parts;
     }
