@@ -62,6 +62,7 @@ constexpr int kMinPartAtoms = 4;
 // ... or twice that where the parts merge through global memory.
 constexpr int kMinGlobalAtoms = 8;
 constexpr int kMaxCluster = 8;
+constexpr int kSegAtoms = 16;      // a unit's fixed cost in a CTA that walks several, in atoms' time
 constexpr size_t kCounterBytes = static_cast<size_t>(kMaxUnits) * kCountersPerUnit * sizeof(unsigned int);
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -173,7 +174,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   // inside a cluster ~3.
   int cand = -1, way = 1;
   if (try_aligned) {
-    int best = N / G + 24 + 3 * (pt.unit_max / (N / G + 1) + 1);
+    int best = (N + kSegAtoms * U) / G + 24 + 3 * (pt.unit_max / (N / G + 1) + 1);
     for (int w = way_lo; w < way_hi; ++w) {
       for (int c = 0; c < kCandidates; ++c) {
         if (pt.parts[w][c] > G) continue;
@@ -281,15 +282,19 @@ __device__ __forceinline__ int cta_of_atom(long long x, long long n, long long n
   return static_cast<int>(i);
 }
 
-// The unit that holds atom a0 (empty units share the start of their successor and are skipped).
-__device__ __forceinline__ int unit_of_atom(const int* unit_start, int U, int a0) {
+// Ranges in which every unit counts kSegAtoms atoms more than it has: what a CTA spends on a unit whatever its
+// length (set-up, combine, output).  A range starts at atom a0 of unit u (a range inside those extra atoms starts at
+// the unit's first).
+__device__ __forceinline__ void range_start(const int* unit_start, int U, int N, long long i, long long np, int& a0, int& u) {
+  const int x = cta_first_atom(i, static_cast<long long>(N) + static_cast<long long>(kSegAtoms) * U, np);
   int lo = 0, hi = U - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (unit_start[mid] <= a0) lo = mid; else hi = mid - 1;
+    if (unit_start[mid] + kSegAtoms * mid <= x) lo = mid; else hi = mid - 1;
   }
-  while (unit_start[lo + 1] <= a0) ++lo;
-  return lo;
+  a0 = min(unit_start[lo] + max(x - unit_start[lo] - kSegAtoms * lo - kSegAtoms, 0), N);
+  while (lo + 1 < U && unit_start[lo + 1] <= a0) ++lo;  // (an empty unit's extra atoms: on to the next)
+  u = lo;
 }
 
 // Scales that bring a running maximum m and an incoming maximum im to their common maximum.
@@ -363,9 +368,10 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   for (int i = (aligned ? static_cast<int>(NP) : 0) + tid; i < G; i += 256) {
     int a0 = 0, a1 = 0, u_first = 0;
     if (i < NP) {
-      a0 = cta_first_atom(i, N, NP);
-      a1 = cta_first_atom(i + 1, N, NP);
-      u_first = unit_of_atom(unit_start, U, a0);
+      int next;
+      range_start(unit_start, U, static_cast<int>(N), i, NP, a0, u_first);
+      range_start(unit_start, U, static_cast<int>(N), i + 1, NP, a1, next);
+      if (i + 1 == NP) a1 = static_cast<int>(N);
     }
     entry(i, a0, a1, u_first, 0);
   }
@@ -534,11 +540,11 @@ __device__ __forceinline__ void attend_block32(WarpState& st, const uint32_t (&q
 // line so that it costs the tile loop no registers.
 template <int MT>
 __device__ __noinline__ void merge_half(const VerifyParams& P, int mt, int half, int i_lo, int i_hi, bool aligned, long long N,
-                                        long long NP, int us, int b, int kvh) {
+                                        long long NP, int vs, int b, int kvh) {
   const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
   auto record = [&](int i) -> const float4* {
     return reinterpret_cast<const float4*>(P.partials +
-        (static_cast<size_t>(2 * i + ((aligned || cta_first_atom(i, N, NP) >= us) ? 0 : 1)) * MT + mt) * kRec) + lane;
+        (static_cast<size_t>(2 * i + ((aligned || cta_first_atom(i, N, NP) >= vs) ? 0 : 1)) * MT + mt) * kRec) + lane;
   };
   float m0 = -INFINITY, m1 = -INFINITY;
   for (int i = i_lo; i <= i_hi; i += 4) {
@@ -805,9 +811,10 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       a1 = sh.unit_start[u_first] + (part + 1) * atoms / parts;
     }
   } else if (static_cast<long long>(blockIdx.x) < NP) {
-    a0 = cta_first_atom(blockIdx.x, N, NP);
-    a1 = cta_first_atom(blockIdx.x + 1, N, NP);
-    u_first = unit_of_atom(sh.unit_start, U, a0);
+    int next;
+    range_start(sh.unit_start, U, static_cast<int>(N), blockIdx.x, NP, a0, u_first);
+    range_start(sh.unit_start, U, static_cast<int>(N), blockIdx.x + 1, NP, a1, next);
+    if (static_cast<long long>(blockIdx.x) + 1 == NP) a1 = static_cast<int>(N);
   }
   }  // !planned
   if (warp < NC) {
@@ -1163,19 +1170,20 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     if (wr == 0) {
       bool finish = whole;
       if (!whole) {
+        const long long N = sh.part.atoms + static_cast<long long>(kSegAtoms) * U, NP = sh.part.ctas;
+        const bool aligned = sh.part.aligned != 0;
+        const int vs = us + kSegAtoms * u;  // (where the unit's range begins)
         // publish this CTA's share of the unit, then see whether it was the last to arrive
         // lane-major float4 records, as in shared memory
         float4* rec = reinterpret_cast<float4*>(
-                          P.partials + (static_cast<size_t>(2 * blockIdx.x + (a == a0 ? 0 : 1)) * MT + mt) * kRec) + lane;
+                          P.partials + (static_cast<size_t>(2 * blockIdx.x + ((aligned || cta_first_atom(blockIdx.x, N, NP) >= vs) ? 0 : 1)) * MT + mt) * kRec) + lane;
 #pragma unroll
         for (int n = 0; n < 16; ++n) __stcg(rec + n * 32, make_float4(acc[n][0], acc[n][1], acc[n][2], acc[n][3]));
         __stcg(rec + 16 * 32, make_float4(m0, l0, m1, l1));
         __threadfence();
         __syncwarp();
-        const long long N = sh.part.atoms, NP = sh.part.ctas;
-        const bool aligned = sh.part.aligned != 0;
-        const int i_lo = aligned ? blockIdx.x - sh.part.mine[1] : cta_of_atom(us, N, NP);
-        const int i_hi = aligned ? i_lo + sh.part.mine[2] - 1 : cta_of_atom(ue - 1, N, NP);
+        const int i_lo = aligned ? blockIdx.x - sh.part.mine[1] : cta_of_atom(vs + kSegAtoms, N, NP);
+        const int i_hi = aligned ? i_lo + sh.part.mine[2] - 1 : cta_of_atom(vs + kSegAtoms + (ue - us) - 1, N, NP);
         unsigned int old = 0;
         if (lane == 0) old = atomicAdd(P.counters + u * kCountersPerUnit + mt, 1u);
         old = __shfl_sync(0xffffffffu, old, 0);
@@ -1188,7 +1196,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
               P.counters[u * kCountersPerUnit + mt] = 0u;  // ready for the next call
               sh.merge_arg[mt][0] = i_lo;
               sh.merge_arg[mt][1] = i_hi;
-              sh.merge_arg[mt][2] = us;
+              sh.merge_arg[mt][2] = vs;
               sh.merge_arg[mt][3] = b;
               sh.merge_arg[mt][4] = kvh;
             }
@@ -1204,7 +1212,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
           // walking the records one round trip to L2 at a time took 6 - 8 us for four of them)
           auto record = [&](int i) -> const float4* {
             return reinterpret_cast<const float4*>(P.partials +
-                (static_cast<size_t>(2 * i + ((aligned || cta_first_atom(i, N, NP) >= us) ? 0 : 1)) * MT + mt) * kRec) + lane;
+                (static_cast<size_t>(2 * i + ((aligned || cta_first_atom(i, N, NP) >= vs) ? 0 : 1)) * MT + mt) * kRec) + lane;
           };
           m0 = m1 = -INFINITY;
           for (int i = i_lo; i <= i_hi; i += 4) {   // four records' maxima per round trip
@@ -1300,7 +1308,8 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     // the first warp, and nothing of the unit's state is needed any more)
     named_bar_sync(1 + mt, WPM * 32);
     if (sh.merge_last[mt])
-      merge_half<MT>(P, mt, wr, sh.merge_arg[mt][0], sh.merge_arg[mt][1], sh.part.aligned != 0, sh.part.atoms, sh.part.ctas, sh.merge_arg[mt][2],
+      merge_half<MT>(P, mt, wr, sh.merge_arg[mt][0], sh.merge_arg[mt][1], sh.part.aligned != 0,
+                     sh.part.atoms + static_cast<long long>(kSegAtoms) * U, sh.part.ctas, sh.merge_arg[mt][2],
                      sh.merge_arg[mt][3], sh.merge_arg[mt][4]);
   }
   if (in_cluster) {
