@@ -76,6 +76,45 @@ struct HostPipe {
 };
 HostPipe g_pipe[64];
 
+// Copies small blocks from or to host memory that the GPU can address (pinned or registered) in one launch: grid
+// row y copies block y with 16-byte accesses over the bus.  A copy-engine transfer of ~100 KB takes 7 us of which
+// 2 are transfer, and an engine serves one at a time: eight layers' queries delayed the draft rows by 57 us, their
+// outputs (two transfers a layer) came in 16 us apart.
+constexpr int kGatherBlocks = 64;
+constexpr size_t kGatherMost = 4u << 20;  // larger blocks are left to the copy engine
+struct HostBlocks {
+  const uint4* src[kGatherBlocks];
+  uint4* dst[kGatherBlocks];
+  unsigned int n16[kGatherBlocks];
+};
+__global__ void __launch_bounds__(256) copy_host_blocks(const __grid_constant__ HostBlocks B) {
+  const uint4* const src = B.src[blockIdx.y];
+  uint4* const dst = B.dst[blockIdx.y];
+  const unsigned int n = B.n16[blockIdx.y], step = gridDim.x * 256;
+  for (unsigned int i = blockIdx.x * 256 + threadIdx.x; i < n; i += 4 * step) {
+    uint4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k * step < n) v[k] = src[i + k * step];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k * step < n) dst[i + k * step] = v[k];
+  }
+}
+
+// The address at which the current device sees host memory `p`, or nullptr if it does not (pageable
+// memory) or if 16-byte accesses to the block, or its size, do not suit the kernel above.
+uint4* device_view(const void* p, const void* device_side, size_t bytes) {
+  if (bytes % 16 != 0 || bytes > kGatherMost || reinterpret_cast<uintptr_t>(device_side) % 16 != 0) return nullptr;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (at.type != cudaMemoryTypeHost || reinterpret_cast<uintptr_t>(at.devicePointer) % 16 != 0) return nullptr;
+  return static_cast<uint4*>(at.devicePointer);
+}
+
 bool make_event(cudaEvent_t* e) {
   if (*e != nullptr) return true;
   if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) {
@@ -118,8 +157,8 @@ bool prepare_pipe(HostPipe& pipe, int n_target_layers) {
 }  // namespace
 }  // namespace specattn
 
-// The step as a three-lane pipeline.  Lane "in" (a copy stream) uploads all query blocks, then
-// the draft rows one mapped draft layer at a time; the caller's stream runs the selection of a
+// The step as a three-lane pipeline.  Lane "in" (a copy stream) uploads the draft rows one mapped draft layer
+// at a time while a kernel fetches the query blocks; the caller's stream runs the selection of a
 // draft layer as soon as its rows have landed and then the verify launches of the target layers
 // mapped to it, while the next draft layer is still crossing PCIe; lane "out" (a second copy
 // stream) downloads a layer's results while later layers compute and later inputs upload.  The
@@ -172,15 +211,7 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
       !ok(cudaStreamWaitEvent(pipe.d2h, pipe.start, 0)))
     return SPECATTN_ERR_CUDA;
 
-  // lane "in": query blocks first (small), then the draft rows in the order the layers need them
-  for (int j = 0; j < S.n_target_layers; ++j) {
-    const specattn_verify_args& v = S.verify[j];
-    const size_t rows = static_cast<size_t>(v.batch) * v.n_q * v.n_q_heads;
-    if (!ok(cudaMemcpyAsync(const_cast<void*>(v.q), S.q_host[j], rows * v.head_dim * 2, cudaMemcpyHostToDevice,
-                            pipe.h2d)))
-      return SPECATTN_ERR_CUDA;
-  }
-  if (!ok(cudaEventRecord(pipe.q_in, pipe.h2d))) return SPECATTN_ERR_CUDA;
+  // lane "in": the draft rows in the order the layers need them.  They bound the step (a PCIe link's ~53 GB/s).
   const size_t layer_bytes = static_cast<size_t>(sel.batch) * sel.n_draft_heads * sel.gamma *
                              static_cast<size_t>(sel.L_stride) * sizeof(float);
   bool uploaded[SPECATTN_MAX_DRAFT_LAYERS] = {false};
@@ -193,10 +224,44 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
   };
   for (int j = 0; j < S.n_target_layers; ++j)
     if (sel.layer_map[j] >= 0 && !upload(sel.layer_map[j])) return SPECATTN_ERR_CUDA;
+  // The query blocks: one kernel on the caller's stream, which has nothing else to do until the first
+  // draft layer is in, reads those that the GPU can read; the others follow the draft rows.
+  {
+    bool copied = false;
+    specattn::HostBlocks blocks;
+    int n_blocks = 0;
+    auto launch = [&]() {
+      if (n_blocks == 0) return true;
+      specattn::copy_host_blocks<<<dim3(8, static_cast<unsigned>(n_blocks)), 256, 0, stream>>>(blocks);
+      n_blocks = 0;
+      specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
+      return ok(cudaGetLastError());
+    };
+    for (int j = 0; j < S.n_target_layers; ++j) {
+      const specattn_verify_args& v = S.verify[j];
+      const size_t bytes = static_cast<size_t>(v.batch) * v.n_q * v.n_q_heads * v.head_dim * 2;
+      if (bytes == 0) continue;
+      const uint4* src = specattn::device_view(S.q_host[j], v.q, bytes);
+      if (src != nullptr) {
+        blocks.src[n_blocks] = src;
+        blocks.dst[n_blocks] = static_cast<uint4*>(const_cast<void*>(v.q));
+        blocks.n16[n_blocks] = static_cast<unsigned int>(bytes / 16);
+        if (++n_blocks == specattn::kGatherBlocks && !launch()) return SPECATTN_ERR_CUDA;
+      } else {
+        copied = true;
+        if (!ok(cudaMemcpyAsync(const_cast<void*>(v.q), S.q_host[j], bytes, cudaMemcpyHostToDevice, pipe.h2d)))
+          return SPECATTN_ERR_CUDA;
+      }
+    }
+    if (!launch()) return SPECATTN_ERR_CUDA;
+    if (copied && (!ok(cudaEventRecord(pipe.q_in, pipe.h2d)) || !ok(cudaStreamWaitEvent(stream, pipe.q_in, 0))))
+      return SPECATTN_ERR_CUDA;
+  }
 
   // the caller's stream: selection per draft layer when first needed, then the verify launches
-  if (!ok(cudaStreamWaitEvent(stream, pipe.q_in, 0))) return SPECATTN_ERR_CUDA;
   bool selected[SPECATTN_MAX_DRAFT_LAYERS] = {false};
+  int to_select = 0;  // draft layers whose selection is still to be enqueued
+  for (int u = 0; u < sel.n_draft_layers; ++u) to_select += used[u] ? 1 : 0;
   const void* planned[SPECATTN_MAX_DRAFT_LAYERS + 1];
   int n_planned = 0;
   // A verify launch may skip its wait for the preceding kernel (SPECATTN_VERIFY_LISTS_STABLE)
@@ -207,6 +272,7 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
     const int u = sel.layer_map[j];
     if (u >= 0 && !selected[u]) {
       selected[u] = true;
+      --to_select;
       fresh = true;
       if (!ok(cudaStreamWaitEvent(stream, pipe.layer_in[u], 0))) return SPECATTN_ERR_CUDA;
       specattn_select_args one = sel;  // the lists of draft layer u only
@@ -235,11 +301,29 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
     if (rc != SPECATTN_OK) return rc;
     // lane "out"
     const size_t rows = static_cast<size_t>(v.batch) * v.n_q * v.n_q_heads;
-    if (!ok(cudaEventRecord(pipe.layer_out[j], stream)) || !ok(cudaStreamWaitEvent(pipe.d2h, pipe.layer_out[j], 0)) ||
-        !ok(cudaMemcpyAsync(S.out_host[j], v.out, rows * v.head_dim * sizeof(float), cudaMemcpyDeviceToHost,
-                            pipe.d2h)) ||
-        !ok(cudaMemcpyAsync(S.lse_host[j], v.lse, rows * sizeof(float), cudaMemcpyDeviceToHost, pipe.d2h)))
+    if (!ok(cudaEventRecord(pipe.layer_out[j], stream)) || !ok(cudaStreamWaitEvent(pipe.d2h, pipe.layer_out[j], 0)))
       return SPECATTN_ERR_CUDA;
+    if (rows == 0) continue;
+    const size_t out_bytes = rows * v.head_dim * sizeof(float), lse_bytes = rows * sizeof(float);
+    // The kernel, whose stores crawl while draft rows still come in (27 us instead of 7, and its CTAs hold up
+    // the attention's), serves the layers after the last selection; the copy engine's way is hidden before it.
+    uint4* const out_view = (to_select == 0) ? specattn::device_view(S.out_host[j], v.out, out_bytes) : nullptr;
+    uint4* const lse_view = (to_select == 0) ? specattn::device_view(S.lse_host[j], v.lse, lse_bytes) : nullptr;
+    if (out_view != nullptr && lse_view != nullptr) {
+      specattn::HostBlocks blocks;
+      blocks.src[0] = reinterpret_cast<const uint4*>(v.out);
+      blocks.dst[0] = out_view;
+      blocks.n16[0] = static_cast<unsigned int>(out_bytes / 16);
+      blocks.src[1] = reinterpret_cast<const uint4*>(v.lse);
+      blocks.dst[1] = lse_view;
+      blocks.n16[1] = static_cast<unsigned int>(lse_bytes / 16);
+      specattn::copy_host_blocks<<<dim3(8, 2), 256, 0, pipe.d2h>>>(blocks);
+      specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
+      if (!ok(cudaGetLastError())) return SPECATTN_ERR_CUDA;
+    } else if (!ok(cudaMemcpyAsync(S.out_host[j], v.out, out_bytes, cudaMemcpyDeviceToHost, pipe.d2h)) ||
+               !ok(cudaMemcpyAsync(S.lse_host[j], v.lse, lse_bytes, cudaMemcpyDeviceToHost, pipe.d2h))) {
+      return SPECATTN_ERR_CUDA;
+    }
   }
   // join: later work on the caller's stream sees the inputs consumed and the results delivered
   if (!ok(cudaEventRecord(pipe.done, pipe.d2h)) || !ok(cudaStreamWaitEvent(stream, pipe.done, 0)))

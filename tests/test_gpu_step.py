@@ -347,3 +347,25 @@ def test_graft_entry_smoke_runs():
     if root not in sys.path:
         sys.path.insert(0, root)
     importlib.import_module("__graft_entry__").smoke()
+
+
+@pytest.mark.parametrize("pinned,layers", [(False, 3), (True, 3), (True, 70)])
+def test_host_buffer_step_from_pageable_memory_and_with_many_layers(pinned, layers):
+    """Query and result blocks move by a kernel where the GPU can address them and by copy-engine transfers
+    elsewhere (pageable memory); more layers than one launch of that kernel takes."""
+    cfg = wl.config1().scaled(n_target_layers=layers, n_draft_layers=2, batch=1, ctx=600, n_q_heads=8, n_kv_heads=2)
+    si, pools, step = _build(cfg)
+    step.run()
+    torch.cuda.synchronize()
+    ref_out, ref_lse = [o.cpu() for o in step.out], [l.cpu() for l in step.lse]
+    put = (lambda t: t.pin_memory()) if pinned else (lambda t: t)
+    dp_host = [None if x is None else put(torch.from_numpy(x)) for x in si.draft_probs]
+    q_host = [put(bf16.bits_to_torch(q)) for q in si.q]
+    out_host = [put(torch.zeros(o.shape, dtype=torch.float32)) for o in step.out]
+    lse_host = [put(torch.zeros(l.shape, dtype=torch.float32)) for l in step.lse]
+    for t in step.q + step.out:
+        t.zero_()
+    step.run_host(dp_host, q_host, out_host, lse_host)
+    torch.cuda.synchronize()
+    for j in range(layers):
+        assert torch.equal(out_host[j], ref_out[j]) and torch.equal(lse_host[j], ref_lse[j])
