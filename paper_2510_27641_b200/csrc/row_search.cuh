@@ -147,17 +147,18 @@ __device__ __forceinline__ void level_add(LevelHist& lv, bool take, unsigned int
 }
 
 // Exact mass of a level bin with c keys, s the sum of their low bits.
-__device__ __forceinline__ unsigned long long level_mass(unsigned int prefix, int bin, int sh, unsigned int c, unsigned int s) {
-  return static_cast<unsigned long long>(c) * mantissa_of(((prefix << 10) | static_cast<unsigned int>(bin)) << sh) + s;
+__device__ __forceinline__ unsigned long long level_mass(unsigned int prefix, int bin, int sh, unsigned int c, unsigned int s,
+                                                        int bits = 10) {
+  return static_cast<unsigned long long>(c) * mantissa_of(((prefix << bits) | static_cast<unsigned int>(bin)) << sh) + s;
 }
 
 // CTA of NT threads, between barriers: the masses of the 32 groups of bins.
 template <int NT>
-__device__ __forceinline__ void level_groups(LevelHist& lv, unsigned int prefix, int sh) {
+__device__ __forceinline__ void level_groups(LevelHist& lv, unsigned int prefix, int sh, int bits = 10) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int gi = warp; gi < 32; gi += NT / 32) {
     const int bin = gi * 32 + lane;
-    unsigned long long s = level_mass(prefix, bin, sh, lv.cnt[bin], lv.sum[bin]);
+    unsigned long long s = level_mass(prefix, bin, sh, lv.cnt[bin], lv.sum[bin], bits);
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(kFull, s, d);
     if (lane == 0) lv.grp[gi] = s;
@@ -199,14 +200,14 @@ __device__ __forceinline__ unsigned int threshold_among(const unsigned int* keys
                                                         LevelHist& lv, Found& fd, Picks& pk, double& above, double& upto) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   while (n > kDirectMax && shift > 0) {
-    const int sh = shift - 10;
+    const int bits = min(shift, 10), sh = shift - bits;
     for (int i = tid; i < ((n + 31) & ~31); i += NT) {
       const unsigned int k = (i < n) ? keys[i] : 0u;
-      level_add(lv, i < n && (k >> shift) == prefix, k, sh);
+      level_add(lv, i < n && (k >> shift) == prefix, k, sh, bits);
     }
     if (tid == 0) pk.n_few = 0u;
     __syncthreads();
-    level_groups<NT>(lv, prefix, sh);
+    level_groups<NT>(lv, prefix, sh, bits);
     __syncthreads();
     if (warp == 0) {
       double ab, up;
@@ -214,8 +215,8 @@ __device__ __forceinline__ unsigned int threshold_among(const unsigned int* keys
       const int bin = gi * 32 + lane;
       const unsigned int c = lv.cnt[bin];
       double ab1, up1;
-      const int b = find_from_top<5>(static_cast<double>(level_mass(prefix, bin, sh, c, lv.sum[bin])) * scale, ab, carry,
-                                     target, ab1, up1);
+      const int b = find_from_top<5>(static_cast<double>(level_mass(prefix, bin, sh, c, lv.sum[bin], bits)) * scale, ab,
+                                     carry, target, ab1, up1);
       const unsigned int cb = __shfl_sync(kFull, c, b);
       if (lane == 0) {
         fd.bin = gi * 32 + b;
@@ -225,7 +226,7 @@ __device__ __forceinline__ unsigned int threshold_among(const unsigned int* keys
       }
     }
     __syncthreads();
-    prefix = (prefix << 10) | static_cast<unsigned int>(fd.bin);
+    prefix = (prefix << bits) | static_cast<unsigned int>(fd.bin);
     inner = fd.above;
     shift = sh;
     if (shift == 0) {

@@ -1,13 +1,21 @@
 // One CTA per row, for calls with more rows than the GPU can keep on chip at once.  Included by
 // select_topp.cu.
 //
-// What bounds this regime is bandwidth as long as enough rows are in flight: held in shared memory, 148
-// SMs take some 37 rows of 131072 entries, and the latencies of a search (barriers, exchanges, scans) are
-// paid once per wave of them (256 rows: 240 us).  Here every row has its own CTA, two per SM, nothing of
-// a row stays on chip but its histogram, and a row is read twice -- for the level-1 histogram and to mark
-// what lies above the threshold bin and collect the keys inside it -- each time through a ring of
-// 16-byte copies, so that the reads of the next 48 KB per CTA are under way while the last are worked on.
-// The searches of different rows overlap one another's reads; there is no cluster and no exchange.
+// Held in shared memory, 148 SMs take some 37 rows of 131072 entries, and the latencies of a search (barriers,
+// exchanges, scans) are paid once per wave of them (256 rows: 240 us).  Here every row has its own CTA, two
+// per SM, nothing of a row stays on chip but a histogram and bits, and a row is read twice, each time through
+// a ring of 16-byte copies that keeps 48 KB per CTA under way.  The searches of different rows overlap one
+// another's reads; there is no cluster and no exchange.
+//
+// With that, the passes are bound by instruction issue and by the wavefronts of shared-memory atomics, so each does
+// as little per entry as it can:
+//   pass 1  adds the top 15 mantissa bits to one word per bin (exponent and five mantissa bits) -- one atomic, not
+//           two words for an exact sum -- and the value itself to the thread's binary64 total.  The histogram is
+//           good to 2^-14, which names the threshold's bin in all but a few of 10^4 rows;
+//   pass 2  notes two bits per entry, above the bin / in the bin, in per-thread words (no votes) and adds up
+//           in binary64 what lies above.  The keys of the bin are then fetched by their bits.
+// The masses tell exactly whether the bin was the right one; if not, the row is read again for its neighbour.
+// 256 rows of 131072, uniform, p = 0.9: 117 us with exact two-word bins, votes and 128-entry emission.
 #pragma once
 
 constexpr int kStreamThreads = 512;
@@ -16,20 +24,21 @@ constexpr int kStreamRound = 4 * kStreamThreads;   // entries per round of the C
 constexpr int kStreamBatch = 2;                    // rounds per commit group
 constexpr int kStreamGroups = 4;                   // groups in the ring
 constexpr int kStreamMax = 131072;                 // entries per row: 64 rounds
-// Level-1 bins of the exponent and four mantissa bits: half as many keys per bin as with three.  A bin
-// keeps the sum of the low 14 mantissa bits in one word and the sum of the upper ten (hidden bit included) in
-// another; neither overflows in kStreamMax entries.
-constexpr int kStreamBins = 4096;
-// After the level-1 search the histogram's bytes hold the bit mask of the row and the keys of the bin.
-constexpr int kStreamStoreWords = 2 * kStreamBins + 1024;
+constexpr int kStreamShift = 18;                   // level-1 bins: the key's bits above these
+constexpr int kStreamBins = 8192;
+constexpr int kStreamCand = 4096;                  // keys of the bin that are gathered
+constexpr int kStreamWords = kStreamMax / 32;      // words of a bit per entry: [8 rounds][thread], 4 bits a round
+constexpr int kStreamStore = kStreamBins + kOctaves;
+static_assert(2 * kStreamWords <= kStreamStore, "both bit masks take the histogram's bytes");
+static_assert(static_cast<long long>(kStreamMax) << 15 <= (1ll << 32), "a bin's word cannot wrap");
 
 struct StreamShared {
-  alignas(16) unsigned int store[kStreamStoreWords];
+  alignas(16) unsigned int store[kStreamStore];  // histogram, then the bits "above the bin" and "in the bin"
   alignas(16) float ring[kStreamGroups * kStreamBatch * kStreamRound];
-  unsigned int kmax;
-  int oct_min, overflow;
-  unsigned int cl_kmax;
+  int negative;                // a negative input was met
+  int oct_min, oct_max, n_cand;
   Found fd;
+  double sum[kStreamWarps];
   int warp_cnt[kStreamWarps];
 };
 // The ring is idle outside the passes and then holds the scratch of the search and the staging lines of
@@ -38,20 +47,37 @@ struct StreamScratch {
   unsigned long long oct[kOctaves];
   LevelHist lv;
   Picks pk;
-  unsigned int keys[2 * kDirectMax];
+  unsigned int keys[kStreamCand];
+  unsigned int place[kStreamCand];   // entry of the row
 };
-static_assert(sizeof(StreamScratch) <= sizeof(float) * kStreamGroups * kStreamBatch * kStreamRound, "scratch in the ring");
+constexpr int kStreamStage = 528;    // ints of a warp's staging line (512 entries, shifted by up to 3)
+static_assert(sizeof(StreamScratch) <= sizeof(StreamShared::ring), "scratch in the ring");
+static_assert(kStreamWarps * kStreamStage * sizeof(int) <= sizeof(StreamShared::ring), "staging in the ring");
 static_assert(2 * (sizeof(StreamShared) + 1024) <= 227 * 1024, "two CTAs per SM");
-static_assert(kStreamThreads == 512, "a key of a warp's list: 13 bits of place, 19 bits of mantissa");
 
-__device__ __forceinline__ void stream_bump(unsigned int* hist, unsigned int key) {
-  unsigned int* const p = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(hist) + ((key >> 17) & 0x3ffcu));
-  atomicAdd(p, key & 0x3fffu);
-  atomicAdd(p + kStreamBins, ((key >> 14) & 0x1ffu) | ((key >= 0x800000u) ? 0x200u : 0u));
+// Word of a bin: 33 words to an octave's 32 bins, or values with one mantissa in many octaves (quantised rows) would
+// share a bank.
+__device__ __forceinline__ int stream_word(int bin) { return bin + (bin >> 5); }
+
+// Adds one positive key to the histogram at shared-memory address `hist`.  The two shifts of the address are
+// multiplications by values the compiler cannot see through: the multiply-add pipe has room, the integer
+// pipe (half a warp instruction a clock) is what bounds the pass.
+struct StreamConst {
+  unsigned int by18, by23, four;
+};
+__device__ __forceinline__ StreamConst stream_const() {
+  StreamConst c;
+  asm volatile("mov.u32 %0, 16384;\n\tmov.u32 %1, 512;\n\tmov.u32 %2, 4;" : "=r"(c.by18), "=r"(c.by23), "=r"(c.four));
+  return c;
+}
+__device__ __forceinline__ void stream_bump(uint32_t hist, const StreamConst& c, unsigned int key) {
+  const unsigned int bin = __umulhi(key, c.by18), oct = __umulhi(key, c.by23);
+  const uint32_t at = bin * c.four + (oct * c.four + hist);
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(((key >> 9) & 0x3fffu) | 0x4000u) : "memory");
 }
 
-// Walks the row through the ring: f(round, keys) for every round's float4 of this thread, zeros beyond n,
-// in rounds of the whole CTA (all threads call f equally often).
+// Walks the row through the ring: f(round, bit patterns) for every batch of rounds, this thread's float4 of each,
+// zeros beyond n, in whole batches of the CTA (all threads call f equally often).
 template <class F>
 __device__ __forceinline__ void stream_pass(StreamShared& sh, const float* A, int n, F f) {
   const int tid = threadIdx.x;
@@ -77,11 +103,11 @@ __device__ __forceinline__ void stream_pass(StreamShared& sh, const float* A, in
     unsigned int k[4 * kStreamBatch];
 #pragma unroll
     for (int j = 0; j < kStreamBatch; ++j) {
-      const float4 v = *reinterpret_cast<const float4*>(sh.ring + ((gq % kStreamGroups) * kStreamBatch + j) * kStreamRound + 4 * tid);
-      k[4 * j] = __float_as_uint(v.x + 0.f);  // -0.0 reads as +0.0
-      k[4 * j + 1] = __float_as_uint(v.y + 0.f);
-      k[4 * j + 2] = __float_as_uint(v.z + 0.f);
-      k[4 * j + 3] = __float_as_uint(v.w + 0.f);
+      const uint4 v = *reinterpret_cast<const uint4*>(sh.ring + ((gq % kStreamGroups) * kStreamBatch + j) * kStreamRound + 4 * tid);
+      k[4 * j] = v.x;
+      k[4 * j + 1] = v.y;
+      k[4 * j + 2] = v.z;
+      k[4 * j + 3] = v.w;
     }
     f(gq * kStreamBatch, k);
   }
@@ -89,10 +115,24 @@ __device__ __forceinline__ void stream_pass(StreamShared& sh, const float* A, in
   __syncthreads();
 }
 
+// Sum over the CTA in a fixed order; every thread gets it.  Two barriers.
+__device__ __forceinline__ double stream_sum(StreamShared& sh, double s) {
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(kFull, s, d);
+  if ((threadIdx.x & 31) == 0) sh.sum[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = sh.sum[0];
+#pragma unroll
+  for (int w = 1; w < kStreamWarps; ++w) s += sh.sum[w];
+  __syncthreads();
+  return s;
+}
+
 __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __grid_constant__ SelectParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamShared& sh = *reinterpret_cast<StreamShared*>(smem_raw);
   StreamScratch& sc = *reinterpret_cast<StreamScratch*>(sh.ring);
+  constexpr int N = 4 * kStreamBatch;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int list = blockIdx.x;  // (used slot, sequence, group)
   const int g = list % P.G;
@@ -100,13 +140,18 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   const int slot = list / (P.G * P.B);
   const long long out_list = (static_cast<long long>(P.layer_of[slot]) * P.B + b) * P.G + g;
   unsigned int* const hist = sh.store;
-  for (int i = tid; i < 2 * kStreamBins / 4; i += kStreamThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (tid == 0) {
-    sh.kmax = 0u;
-    sh.oct_min = kOctaves;
-    sh.overflow = 0;
-  }
-  __syncthreads();
+  const uint32_t hist_at = smem_u32(hist);
+  const StreamConst consts = stream_const();
+  auto clear = [&]() {
+    for (int i = tid; i < kStreamStore / 4; i += kStreamThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+      sh.negative = 0;
+      sh.oct_min = kOctaves;
+      sh.oct_max = -1;
+    }
+    __syncthreads();
+  };
+  clear();
   pdl_wait();  // nothing is read or written before the previous kernel's end ...
   pdl_launch_dependents();  // ... and only then may the next one be scheduled
   long long Lll = P.kv_len[b];
@@ -116,332 +161,345 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   const float* A = (P.agg != nullptr) ? P.agg + static_cast<long long>(list) * P.L_stride
                                       : P.probs[slot] + static_cast<long long>(b) * P.H * P.gamma * P.L_stride;
 
-  // ---- first pass: level-1 histogram and validity ----------------------------------------------------
-  unsigned int kmax = 0u;
-  stream_pass(sh, A, L, [&](int, const unsigned int (&k)[4 * kStreamBatch]) {
-    constexpr int N = 4 * kStreamBatch;
-#pragma unroll
-    for (int j = 0; j < N; ++j) kmax = max(kmax, k[j]);
-    // every value of the warp in one bin (ties, constant rows): the warp reduces first
-    const unsigned int bin0 = __shfl_sync(kFull, k[0] >> 19, 0);
-    bool one = false;
-    if (__all_sync(kFull, (k[0] >> 19) == bin0)) {
-      unsigned int differ = 0u;
-#pragma unroll
-      for (int j = 1; j < N; ++j) differ |= k[j] ^ k[0];
-      one = __all_sync(kFull, (differ >> 19) == 0u);
-    }
-    if (one) {
-      unsigned int lo = 0u, hi = 0u;
-#pragma unroll
-      for (int j = 0; j < N; ++j) {
-        lo += k[j] & 0x3fffu;
-        hi += mantissa_of(k[j]) >> 14;
-      }
-      lo = __reduce_add_sync(kFull, lo);
-      hi = __reduce_add_sync(kFull, hi);
-      if (lane == 0 && (lo | hi) != 0u) {
-        atomicAdd(&hist[bin0 & (kStreamBins - 1)], lo);
-        atomicAdd(&hist[kStreamBins + (bin0 & (kStreamBins - 1))], hi);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < N; ++j)
-        if (k[j] != 0u) stream_bump(hist, k[j]);
-    }
-  });
-  kmax = __reduce_max_sync(kFull, kmax);
-  if (lane == 0 && kmax != 0u) atomicMax(&sh.kmax, kmax);
-
-  // ---- the octave and the bin of the threshold -------------------------------------------------------
-  if (tid < kOctaves) {
-    unsigned long long s = 0ull;
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const uint4 lo = *reinterpret_cast<const uint4*>(&hist[16 * tid + 4 * h]);
-      const uint4 hi = *reinterpret_cast<const uint4*>(&hist[kStreamBins + 16 * tid + 4 * h]);
-      s += ((static_cast<unsigned long long>(hi.x) + hi.y + hi.z + hi.w) << 14) + lo.x + lo.y + lo.z + lo.w;
-    }
-    sc.oct[tid] = s;
-    const int first = __reduce_min_sync(kFull, (s != 0ull) ? tid : kOctaves);
-    if (lane == 0 && first < kOctaves) atomicMin(&sh.oct_min, first);
-  }
-  __syncthreads();
-  if (warp == 0) {
-    Found fd;
-    fd.total = fd.target = fd.carry = fd.above = fd.upto = 0.0;
-    fd.bin = fd.oct = 0;
-    fd.count = 0u;
-    const unsigned int km = sh.kmax;
-    if (km <= 0x7f7fffffu && sh.oct_min < kOctaves) {
-      fd.oct = find_octave(
-          static_cast<int>(km >> 23), sh.oct_min, P.p, [&](int e) { return sc.oct[e]; }, fd.total, fd.target, fd.carry);
-      const int bin = 16 * fd.oct + (lane & 15);
-      const unsigned long long s = (lane < 16) ? (static_cast<unsigned long long>(hist[kStreamBins + bin]) << 14) + hist[bin] : 0ull;
-      const int b16 = find_from_top<4>(static_cast<double>(s) * pow2_double(max(fd.oct, 1) - 150), 0.0, fd.carry, fd.target,
-                                       fd.above, fd.upto);
-      fd.bin = 16 * fd.oct + b16;
-      // a bin's smallest mantissa bounds the number of its keys (not in the bin of zero)
-      const unsigned long long sb = __shfl_sync(kFull, s, b16);
-      const unsigned int base = mantissa_of(static_cast<unsigned int>(fd.bin) << 19);
-      fd.count = (base != 0u) ? static_cast<unsigned int>(min(sb / base, 0x7fffffffull)) : 0x7fffffffu;
-    }
-    if (lane == 0) sh.fd = fd;
-  }
-  __syncthreads();
-  const bool invalid = sh.kmax > 0x7f7fffffu;
-  const double total = sh.fd.total, target = sh.fd.target, carry = sh.fd.carry;
-  double m_gt = 0.0, m_ge = total;
-  const bool searching = !invalid && target > 0.0 && !P.keep_all;  // else p >= 1 or an all-zero row: keep all
-  const int groups = (L + 127) / 128;                              // groups of 128 entries: four mask words each
-  unsigned int* const mask = sh.store;
+  double total = 0.0, target = 0.0, m_gt = 0.0, m_ge = 0.0;
+  bool invalid = false, searching = false;
   unsigned int theta = 0u;
-  if (searching) {
-    const double scale = pow2_double(max(sh.fd.oct, 1) - 150);
-    unsigned int prefix = static_cast<unsigned int>(sh.fd.bin);
-    int shift = 19;
-    double inner = sh.fd.above;
-    unsigned int M = sh.fd.count;
-    // room for keys behind the mask, an equal part for every warp
-    const int mask_words = (4 * groups + 3) & ~3;
-    const int cap = (kStreamStoreWords - mask_words) / kStreamWarps;
-    unsigned int* const list_w = sh.store + mask_words + warp * cap;
-    int n_list = 0;
-    for (;;) {
-      __syncthreads();  // (the histogram's bytes, the level histogram and the flags of the last trip were read by all)
-      if (tid == 0) sh.overflow = 0;
-      // ---- a well filled bin: 10 (then the last 9) more bits, one pass over the row ------------------------
-      while (M > static_cast<unsigned int>(kStreamWarps * cap) && shift > 0) {
-        // (the pass uses the ring, whose bytes the level histogram shares: it lives in the store meanwhile)
-        LevelHist& lv = *reinterpret_cast<LevelHist*>(sh.store);
-        const int sh_l = max(shift - 10, 0);
-        const int up = shift - sh_l;
-        level_clear<kStreamThreads>(lv);
-        __syncthreads();
-        stream_pass(sh, A, L, [&](int, const unsigned int (&k)[4 * kStreamBatch]) {
+  unsigned int* const above_bits = sh.store;
+  unsigned int* const in_bits = sh.store + kStreamWords;
+  int go = 0;                  // 1 / -1: the bin above / below the last one tried is wanted
+  for (;;) {
+    // ---- pass 1: histogram, total and validity -------------------------------------------------------
+    bool negative = false;
+    double mine = 0.0;
+    stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
+      unsigned int any = 0u;
 #pragma unroll
-          for (int j = 0; j < 4 * kStreamBatch; ++j)
-            level_add(lv, (k[j] >> shift) == prefix && k[j] != 0u, k[j], sh_l, up);
-        });
-        for (int gi = warp; gi < 32; gi += kStreamWarps) {
-          const int bin = gi * 32 + lane;
-          unsigned long long s = 0ull;
-          if (bin < (1 << up))
-            s = static_cast<unsigned long long>(lv.cnt[bin]) * mantissa_of(((prefix << up) | static_cast<unsigned int>(bin)) << sh_l) + lv.sum[bin];
+      for (int j = 0; j < N; ++j) any |= k[j];
+      if (static_cast<int>(any) < 0) {  // a sign bit: negative -- or -0.0, which is a zero
 #pragma unroll
-          for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(kFull, s, d);
-          if (lane == 0) lv.grp[gi] = s;
-        }
-        __syncthreads();
-        if (warp == 0) {
-          double above, upto, above1, upto1;
-          const int gi = find_from_top<5>(static_cast<double>(lv.grp[lane]) * scale, inner, carry, target, above, upto);
-          const int bin = gi * 32 + lane;
-          const unsigned int c = (bin < (1 << up)) ? lv.cnt[bin] : 0u;
-          const unsigned long long m = static_cast<unsigned long long>(c) * mantissa_of(((prefix << up) | static_cast<unsigned int>(bin)) << sh_l) +
-                                       (c != 0u ? lv.sum[bin] : 0u);
-          const int b1 = find_from_top<5>(static_cast<double>(m) * scale, above, carry, target, above1, upto1);
-          const unsigned int cb = __shfl_sync(kFull, c, b1);
-          if (lane == 0) {
-            sh.fd.bin = gi * 32 + b1;
-            sh.fd.count = cb;
-            sh.fd.above = above1;
-            sh.fd.upto = upto1;
-          }
-        }
-        __syncthreads();
-        prefix = (prefix << up) | static_cast<unsigned int>(sh.fd.bin);
-        M = sh.fd.count;
-        inner = sh.fd.above;
-        shift = sh_l;
-        if (shift == 0) {  // one distinct key left: the threshold
-          theta = prefix;
-          m_gt = carry + inner;
-          m_ge = carry + sh.fd.upto;
-        }
-        __syncthreads();
-      }
-      // ---- second pass: mark what lies above the bin (above or at a known threshold), collect its keys -----
-      const unsigned int lo_key = (prefix != 0u) ? prefix << shift : 1u;
-      const unsigned int top_key = (prefix << shift) + ((1u << shift) - 1u), span = top_key - lo_key;
-      const unsigned int keep_key = (shift == 0) ? theta : top_key + 1u;  // kept whatever the threshold turns out to be
-      n_list = 0;
-      stream_pass(sh, A, L, [&](int round, const unsigned int (&k)[4 * kStreamBatch]) {
-#pragma unroll
-        for (int j = 0; j < kStreamBatch; ++j) {
-          unsigned int mine = 0u;
-          bool any = false;
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const unsigned int m = __ballot_sync(kFull, k[4 * j + e] >= keep_key);
-            if (lane == e) mine = m;
-            any |= k[4 * j + e] - lo_key <= span;
-          }
-          const int grp = (round + j) * kStreamWarps + warp;
-          if (lane < 4 && grp < groups) mask[4 * grp + lane] = mine;
-          if (shift > 0 && __any_sync(kFull, any)) {
-            // one word per key: its place among the warp's entries and its bits below the prefix
-            const unsigned int place = static_cast<unsigned int>(((round + j) * 32 + lane) * 4) << 19;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const unsigned int d = k[4 * j + e] - (prefix << shift);
-              const bool in = k[4 * j + e] - lo_key <= span;
-              const unsigned int m = __ballot_sync(kFull, in);
-              const int at = n_list + __popc(m & ((1u << lane) - 1u));
-              if (in && at < cap) list_w[at] = place + (static_cast<unsigned int>(e) << 19) + d;
-              n_list += __popc(m);
-            }
-          }
-        }
-      });
-      if (n_list > cap && lane == 0) sh.overflow = 1;
-      __syncthreads();
-      if (!sh.overflow) break;
-      M = 0x7fffffffu;  // one warp's part was too small: narrow the bin down first
-    }
-    if (shift > 0) {
-      // ---- the threshold among the collected keys: 10 bits over all lists, then what is left of them -------
-      unsigned int pre = prefix;
-      const int sh_l = (shift == 19) ? 9 : 0;
-      const int up = shift - sh_l;
-      level_clear<kStreamThreads>(sc.lv);
-      if (tid == 0) sh.fd.key = 0u;
-      __syncthreads();
-      const int n_mine = min(n_list, cap);
-      const unsigned int key0 = prefix << shift;
-      for (int i = lane; i < ((n_mine + 31) & ~31); i += 32) {
-        const unsigned int k = (i < n_mine) ? key0 + (list_w[i] & 0x7ffffu) : 0u;
-        level_add(sc.lv, i < n_mine, k, sh_l, up);
-      }
-      __syncthreads();
-      for (int gi = warp; gi < 32; gi += kStreamWarps) {
-        const int bin = gi * 32 + lane;
-        unsigned long long s = 0ull;
-        if (bin < (1 << up))
-          s = static_cast<unsigned long long>(sc.lv.cnt[bin]) * mantissa_of(((pre << up) | static_cast<unsigned int>(bin)) << sh_l) + sc.lv.sum[bin];
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(kFull, s, d);
-        if (lane == 0) sc.lv.grp[gi] = s;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        double above, upto, above1, upto1;
-        const int gi = find_from_top<5>(static_cast<double>(sc.lv.grp[lane]) * scale, inner, carry, target, above, upto);
-        const int bin = gi * 32 + lane;
-        const unsigned int c = (bin < (1 << up)) ? sc.lv.cnt[bin] : 0u;
-        const unsigned long long m = static_cast<unsigned long long>(c) * mantissa_of(((pre << up) | static_cast<unsigned int>(bin)) << sh_l) +
-                                     (c != 0u ? sc.lv.sum[bin] : 0u);
-        const int b1 = find_from_top<5>(static_cast<double>(m) * scale, above, carry, target, above1, upto1);
-        const unsigned int cb = __shfl_sync(kFull, c, b1);
-        if (lane == 0) {
-          sh.fd.bin = gi * 32 + b1;
-          sh.fd.count = cb;
-          sh.fd.above = above1;
-          sh.fd.upto = upto1;
-          sh.overflow = 0;  // (counts the keys of that bin below)
+        for (int j = 0; j < N; ++j) {
+          negative |= k[j] > 0x80000000u;
+          k[j] = (static_cast<int>(k[j]) < 0) ? 0u : k[j];
         }
       }
-      __syncthreads();
-      pre = (pre << up) | static_cast<unsigned int>(sh.fd.bin);
-      inner = sh.fd.above;
-      if (sh_l == 0) {
-        theta = pre;
-        m_gt = carry + inner;
-        m_ge = carry + sh.fd.upto;
+      // every value of the warp in one bin (ties, constant rows): the warp reduces first
+      const unsigned int bin0 = __shfl_sync(kFull, k[0] >> kStreamShift, 0);
+      bool one = false;
+      if (__all_sync(kFull, (k[0] >> kStreamShift) == bin0)) {
+        unsigned int differ = 0u;
+#pragma unroll
+        for (int j = 1; j < N; ++j) differ |= k[j] ^ k[0];
+        one = __all_sync(kFull, (differ >> kStreamShift) == 0u);
+      }
+      if (one) {
+        unsigned int s = 0u;
+#pragma unroll
+        for (int j = 0; j < N; ++j) s += (k[j] != 0u) ? ((k[j] >> 9) & 0x3fffu) | 0x4000u : 0u;
+        s = __reduce_add_sync(kFull, s);
+        if (lane == 0 && s != 0u) atomicAdd(&hist[stream_word(bin0 & (kStreamBins - 1))], s);
       } else {
-        const int left = static_cast<int>(sh.fd.count);
-        double above, upto;
-        if (left <= kDirectMax) {
-          for (int i = lane; i < n_mine; i += 32) {
-            const unsigned int k = key0 + (list_w[i] & 0x7ffffu);
-            if ((k >> sh_l) == pre) sc.keys[atomicAdd(&sh.overflow, 1)] = k;
-          }
-          __syncthreads();
-          theta = threshold_among<kStreamThreads>(sc.keys, left, pre, sh_l, inner, carry, target, scale, sc.lv, sh.fd, sc.pk,
-                                                  above, upto);
-        } else {  // many equal keys: the last nine bits the same way
-          level_clear<kStreamThreads>(sc.lv);
-          __syncthreads();
-          for (int i = lane; i < ((n_mine + 31) & ~31); i += 32) {
-            const unsigned int k = (i < n_mine) ? key0 + (list_w[i] & 0x7ffffu) : 0u;
-            level_add(sc.lv, i < n_mine && (k >> sh_l) == pre, k, 0, 9);
-          }
-          __syncthreads();
-          if (warp == 0) {
-            // 512 bins, 16 per lane
-            unsigned long long s = 0ull;
-            for (int j = 0; j < 16; ++j)
-              s += static_cast<unsigned long long>(sc.lv.cnt[16 * lane + j]) * mantissa_of((pre << 9) | static_cast<unsigned int>(16 * lane + j));
-            double ab, up2, ab1, up1;
-            const int l = find_from_top<5>(static_cast<double>(s) * scale, inner, carry, target, ab, up2);
-            const int bin = 16 * l + (lane & 15);
-            const unsigned long long m = (lane < 16) ? static_cast<unsigned long long>(sc.lv.cnt[bin]) * mantissa_of((pre << 9) | static_cast<unsigned int>(bin)) : 0ull;
-            const int b1 = find_from_top<4>(static_cast<double>(m) * scale, ab, carry, target, ab1, up1);
-            if (lane == 0) {
-              sh.fd.key = (pre << 9) | static_cast<unsigned int>(16 * l + b1);
-              sh.fd.above = ab1;
-              sh.fd.upto = up1;
-            }
-          }
-          __syncthreads();
-          theta = sh.fd.key;
-          above = sh.fd.above;
-          upto = sh.fd.upto;
-        }
-        m_gt = carry + above;
-        m_ge = carry + upto;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+          if (k[j] != 0u) stream_bump(hist_at, consts, k[j]);
       }
-      // keys of the bin that made it join the mask (a warp's keys lie in its own words)
-      for (int i = lane; i < n_mine; i += 32) {
-        const unsigned int w = list_w[i];
-        if (key0 + (w & 0x7ffffu) >= theta) {
-          const int place = static_cast<int>(w >> 19);  // (round * 32 + lane) * 4 + e
-          const int grp = (place >> 7) * kStreamWarps + warp;
-          atomicOr(&mask[4 * grp + (place & 3)], 1u << ((place >> 2) & 31));
+#pragma unroll
+      for (int j = 0; j < N; ++j) mine += static_cast<double>(__uint_as_float(k[j]));
+    });
+    if (__any_sync(kFull, negative) && lane == 0) sh.negative = 1;
+
+    // ---- the bin of the threshold ---------------------------------------------------------------------
+    if (tid < kOctaves) {
+      unsigned long long s = 0ull;
+#pragma unroll 8
+      for (int h = 0; h < 32; ++h) s += hist[33 * tid + h];
+      sc.oct[tid] = s;
+      const int first = __reduce_min_sync(kFull, (s != 0ull) ? tid : kOctaves);
+      const int final = __reduce_max_sync(kFull, (s != 0ull) ? tid : -1);
+      if (lane == 0 && first < kOctaves) {
+        atomicMin(&sh.oct_min, first);
+        atomicMax(&sh.oct_max, final);
+      }
+    }
+    total = stream_sum(sh, mine);
+    target = static_cast<double>(P.p) * total;
+    // NaN and infinities survive into the sum (finite ones cannot overflow it)
+    invalid = sh.negative != 0 || !(total <= DBL_MAX);
+    if (invalid) total = target = 0.0;
+    m_ge = total;
+    searching = !invalid && target > 0.0 && !P.keep_all;  // else p >= 1 or an all-zero row: keep all
+    if (!searching) break;
+    if (warp == 0) {
+      int bin;
+      if (go == 0) {
+        double t, tg, carry, ab, up;
+        const int oct = find_octave(sh.oct_max, sh.oct_min, P.p, [&](int e) { return sc.oct[e] << 9; }, t,
+                                    tg, carry);
+        const double m = static_cast<double>(static_cast<unsigned long long>(hist[stream_word(32 * oct + lane)]) << 9) * pow2_double(max(oct, 1) - 150);
+        bin = 32 * oct + find_from_top<5>(m, 0.0, carry, tg, ab, up);
+      } else {  // the next one with an entry, or -1
+        int at = sh.fd.bin;
+        bin = -1;
+        for (;;) {
+          at = (go > 0) ? at + 1 : at - 1;
+          const int mine_at = (go > 0) ? at + lane : at - lane;
+          const unsigned some = __ballot_sync(kFull, mine_at >= 0 && mine_at < kStreamBins && hist[stream_word(mine_at & (kStreamBins - 1))] != 0u);
+          if (some != 0u) {
+            bin = (go > 0) ? at + __ffs(some) - 1 : at - (__ffs(some) - 1);
+            break;
+          }
+          at = (go > 0) ? at + 31 : at - 31;
+          if (at < 0 || at >= kStreamBins) break;
+        }
+      }
+      if (lane == 0) {
+        sh.fd.key = (bin < 0) ? 0xffffffffu : 0u;  // (no such bin)
+        if (bin >= 0) {
+          sh.fd.bin = bin;
+          // the bin's smallest term bounds the number of its keys
+          sh.fd.count = hist[stream_word(bin)] / (0x4000u | (static_cast<unsigned int>(bin & 31) << 9));
         }
       }
     }
     __syncthreads();
+    const bool last_resort = sh.fd.key == 0xffffffffu;   // keep the bin tried before
+    unsigned int prefix = static_cast<unsigned int>(sh.fd.bin);
+    const double scale = pow2_double(max(sh.fd.bin >> 5, 1) - 150);
+    unsigned int M = last_resort ? 0x7fffffffu : sh.fd.count;
+    int shift = kStreamShift;
+    int want = 0;
+    __syncthreads();
+    // ---- a well filled bin: 10 (then the last 8) more bits, one pass over the row each -----------------------
+    while (M > static_cast<unsigned int>(kStreamCand) && shift > 0) {
+      // (the pass uses the ring, so the level histogram takes the store)
+      LevelHist& lv = *reinterpret_cast<LevelHist*>(sh.store);
+      const int bits = min(shift, 10), sl = shift - bits;
+      const int top = static_cast<int>((prefix << shift) + ((1u << shift) - 1u));
+      level_clear<kStreamThreads>(lv);
+      __syncthreads();
+      double s = 0.0;
+      stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+          level_add(lv, (k[j] >> shift) == prefix && k[j] != 0u, k[j], sl, bits);
+          if (static_cast<int>(k[j]) > top) s += static_cast<double>(__uint_as_float(k[j]));
+        }
+      });
+      level_groups<kStreamThreads>(lv, prefix, sl, bits);
+      s = stream_sum(sh, s);
+      if (warp == 0) {
+        double above, upto, above1, upto1;
+        const double all = static_cast<double>(lv.grp[lane]) * scale;
+        const int gi = find_from_top<5>(all, 0.0, s, target, above, upto);
+        const int bin = gi * 32 + lane;
+        const unsigned int c = lv.cnt[bin];
+        const int b1 = find_from_top<5>(static_cast<double>(level_mass(prefix, bin, sl, c, lv.sum[bin], bits)) * scale, above, s,
+                                        target, above1, upto1);
+        const unsigned int cb = __shfl_sync(kFull, c, b1);
+        if (lane == 0) {
+          sh.fd.oct = gi * 32 + b1;
+          sh.fd.count = cb;
+          sh.fd.upto = s + upto1;
+        }
+      }
+      __syncthreads();
+      // (only the first level can show that the bin was the wrong one)
+      if (shift == kStreamShift && !last_resort) want = (s >= target) ? 1 : (sh.fd.upto < target) ? -1 : 0;
+      prefix = (prefix << bits) | static_cast<unsigned int>(sh.fd.oct);
+      M = sh.fd.count;
+      shift = sl;
+      __syncthreads();
+      if (want != 0 && go != -want) break;
+      want = 0;
+    }
+    if (want != 0) {
+      go = want;
+      clear();
+      continue;
+    }
+    // ---- pass 2: what lies above the bin, and in it ---------------------------------------------------
+    // (a prefix of all bits is one value: it is the threshold, and counts as the bin)
+    const unsigned int lo_key = (prefix != 0u) ? prefix << shift : 1u;
+    const unsigned int top_key = (prefix << shift) + ((1u << shift) - 1u), span = top_key - lo_key;
+    double carry = 0.0;
+    {
+      unsigned int ab = 0u, in = 0u;
+      const int last = ((L + kStreamRound - 1) / kStreamRound + kStreamBatch - 1) / kStreamBatch * kStreamBatch - kStreamBatch;
+      stream_pass(sh, A, L, [&](int round, unsigned int (&k)[N]) {
+        unsigned int a8 = 0u, i8 = 0u;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+          if (static_cast<int>(k[j]) > static_cast<int>(top_key)) {
+            a8 |= 1u << j;
+            carry += static_cast<double>(__uint_as_float(k[j]));
+          }
+          if (k[j] - lo_key <= span) i8 |= 1u << j;
+        }
+        const int at = 4 * (round & 7);
+        ab |= a8 << at;
+        in |= i8 << at;
+        if ((round & 7) == 8 - kStreamBatch || round == last) {
+          above_bits[(round >> 3) * kStreamThreads + tid] = ab;
+          in_bits[(round >> 3) * kStreamThreads + tid] = in;
+          ab = in = 0u;
+        }
+      });
+    }
+    if (tid == 0) sh.n_cand = 0;
+    carry = stream_sum(sh, carry);
+    if (shift > 0) level_clear<kStreamThreads>(sc.lv);
+    // fetch the keys of the bin by their bits
+    const int word_rows = (L + 8 * kStreamRound - 1) / (8 * kStreamRound);
+    for (int r8 = 0; r8 < word_rows; ++r8) {
+      unsigned int w = in_bits[r8 * kStreamThreads + tid];
+      if (!__any_sync(kFull, w != 0u)) continue;
+      int n = __popc(w), end = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(kFull, end, d);
+        if (lane >= d) end += v;
+      }
+      int at = 0;
+      if (lane == 31) at = atomicAdd(&sh.n_cand, end);
+      at = __shfl_sync(kFull, at, 31) + end - n;
+      for (; w != 0u; w &= w - 1u, ++at) {
+        const int bit = __ffs(w) - 1;
+        const unsigned int entry = static_cast<unsigned int>((r8 * 8 + (bit >> 2)) * kStreamRound + 4 * tid + (bit & 3));
+        if (at < kStreamCand) sc.place[at] = entry;
+      }
+    }
+    __syncthreads();
+    const int n = min(sh.n_cand, kStreamCand);  // (one value's entries may be more: their bits are all kept)
+    if (shift > 0) {  // (all loads of a thread in flight at once: one by one, as the places are found, took 7 us)
+      unsigned int key[kStreamCand / kStreamThreads];
+#pragma unroll
+      for (int j = 0; j < kStreamCand / kStreamThreads; ++j) {
+        const int i = tid + j * kStreamThreads;
+        if (i < n) key[j] = __float_as_uint(__ldg(A + sc.place[i]));
+      }
+#pragma unroll
+      for (int j = 0; j < kStreamCand / kStreamThreads; ++j) {
+        const int i = tid + j * kStreamThreads;
+        if (i < n) sc.keys[i] = key[j];
+      }
+      __syncthreads();
+    }
+    m_gt = m_ge = carry;
+    if (shift > 0 && n == 0) {
+      theta = top_key + 1u;
+    } else if (shift > 0) {
+      double above, upto;
+      theta = threshold_among<kStreamThreads>(sc.keys, n, prefix, shift, 0.0, carry, target, scale, sc.lv, sh.fd, sc.pk, above, upto);
+      m_gt = carry + above;
+      m_ge = carry + upto;
+    } else {
+      theta = prefix;
+      m_ge = carry + static_cast<double>(sh.n_cand) * static_cast<double>(__uint_as_float(prefix));
+    }
+    // The right bin?  (Once the search has gone one way it does not turn: masses that touch the target are
+    // then equal up to the rounding of their sums.)
+    if (shift == kStreamShift && !last_resort) {
+      want = (carry >= target) ? 1 : (m_ge < target) ? -1 : 0;
+      if (want != 0 && go != -want) {
+        __syncthreads();
+        if (tid == 0) sh.fd.bin = static_cast<int>(prefix);  // (threshold_among used the field)
+        go = want;
+        clear();
+        continue;
+      }
+      if (want > 0) {  // went down from a bin that fell short: everything above this one
+        theta = top_key + 1u;
+        m_gt = m_ge = carry;
+      }
+    }
+    // the bin's entries that make it join the bits
+    if (shift > 0) {
+      for (int i = tid; i < n; i += kStreamThreads) {
+        if (sc.keys[i] >= theta) {
+          const unsigned int e = sc.place[i];
+          const unsigned int round = e / kStreamRound, t = (e % kStreamRound) >> 2;
+          atomicOr(&above_bits[(round >> 3) * kStreamThreads + t], 1u << (4 * (round & 7) + (e & 3)));
+        }
+      }
+    } else {
+      for (int r8 = 0; r8 < word_rows; ++r8) above_bits[r8 * kStreamThreads + tid] |= in_bits[r8 * kStreamThreads + tid];
+    }
+    break;
   }
+  __syncthreads();
 
   // ---- ordered emission ---------------------------------------------------------------------------------
   int* const out = P.idx + out_list * P.idx_stride;
   const int stride = static_cast<int>(min(P.idx_stride, static_cast<long long>(INT_MAX)));
   int count = 0;
   if (searching) {
-    const int per_warp = (groups + kStreamWarps - 1) / kStreamWarps;
-    const int g_lo = min(groups, warp * per_warp), g_hi = min(groups, g_lo + per_warp);
+    // A warp takes a power of two of consecutive rounds, so that they lie in one row of words.
+    const int rounds = (L + kStreamRound - 1) / kStreamRound;
+    const int per = (rounds <= kStreamWarps) ? 1 : (rounds <= 2 * kStreamWarps) ? 2 : 4;
+    static_assert(kStreamMax / kStreamRound <= 4 * kStreamWarps, "four rounds per warp cover a row");
+    const int r_lo = warp * per, r_hi = min(rounds, r_lo + per);
+    const unsigned int* const words = above_bits + (r_lo >> 3) * kStreamThreads;
     int wc = 0;
-    for (int w = 4 * g_lo + lane; w < 4 * g_hi; w += 32) wc += __popc(mask[w]);
+    if (r_lo < r_hi) {
+      const unsigned int mine = ((per == 4) ? 0xffffu : (per == 2) ? 0xffu : 0xfu) << (4 * (r_lo & 7));
+#pragma unroll
+      for (int c = 0; c < kStreamThreads / 32; ++c) wc += __popc(words[32 * c + lane] & mine);
+    }
     wc = __reduce_add_sync(kFull, wc);
     if (lane == 0) sh.warp_cnt[warp] = wc;
     __syncthreads();
     const int v = (lane < kStreamWarps) ? sh.warp_cnt[lane] : 0;
     count = __reduce_add_sync(kFull, v);
     int pos = __reduce_add_sync(kFull, lane < warp ? v : 0);
-    // The kept positions of 128 entries go through a per-warp staging line, so that the global stores
-    // are whole 128-byte runs (a lane storing its own up to four positions spreads every store
-    // instruction over the whole 512-byte range: four partial writes per sector).
-    int* const stage = reinterpret_cast<int*>(sh.ring) + warp * 128;
-    const unsigned int lt = (1u << lane) - 1u;
-    for (int gi = g_lo; gi < g_hi; ++gi) {
-      const uint4 m = *reinterpret_cast<const uint4*>(mask + 4 * gi);  // (the same words in every lane)
-      if ((m.x | m.y | m.z | m.w) == 0u) continue;
-      const int first = 128 * gi + 4 * lane;
-      int at = __popc(m.x & lt) + __popc(m.y & lt) + __popc(m.z & lt) + __popc(m.w & lt);
-      const int kept = __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
-      if ((m.x >> lane) & 1u) stage[at++] = first;
-      if ((m.y >> lane) & 1u) stage[at++] = first + 1;
-      if ((m.z >> lane) & 1u) stage[at++] = first + 2;
-      if ((m.w >> lane) & 1u) stage[at++] = first + 3;
-      __syncwarp();
+    // 512 entries at a time: the lanes' counts of four 128-entry chunks are scanned as four bytes of one word, the
+    // kept positions go through a per-warp staging line that lies like the output modulo 16 bytes, and leave
+    // in 16-byte stores.
+    int* const stage = reinterpret_cast<int*>(sh.ring) + warp * kStreamStage;
+    const bool wide = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    for (int r = r_lo; r < r_hi; ++r) {
+      const int nib_at = 4 * (r & 7);
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        unsigned int x = 0u;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int t = 32 * j + lane;
-        if (t < kept && pos + t < stride) out[pos + t] = stage[t];
+        for (int i = 0; i < 4; ++i) x |= ((words[32 * (4 * q + i) + lane] >> nib_at) & 15u) << (8 * i);
+        if (!__any_sync(kFull, x != 0u)) continue;
+        unsigned int c = x - ((x >> 1) & 0x05050505u);
+        c = (c & 0x03030303u) + ((c >> 2) & 0x03030303u);
+        unsigned int incl = c;  // (at most 128 per byte)
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const unsigned int u = __shfl_up_sync(kFull, incl, d);
+          if (lane >= d) incl += u;
+        }
+        const unsigned int t4 = __shfl_sync(kFull, incl, 31);
+        incl -= c;
+        const int off = pos & 3;
+        int base = off;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          int at = base + static_cast<int>((incl >> (8 * i)) & 255u);
+          const int first = r * kStreamRound + (4 * q + i) * 128 + 4 * lane;
+          const unsigned int nib = x >> (8 * i);
+          if (nib & 1u) stage[at++] = first;
+          if (nib & 2u) stage[at++] = first + 1;
+          if (nib & 4u) stage[at++] = first + 2;
+          if (nib & 8u) stage[at++] = first + 3;
+          base += static_cast<int>((t4 >> (8 * i)) & 255u);
+        }
+        __syncwarp();
+        const int from = pos - off;  // output position of stage[0]
+        for (int j = 4 * lane; j < base; j += 128) {
+          if (wide && j >= off && j + 4 <= base && from + j + 4 <= stride) {
+            *reinterpret_cast<int4*>(out + from + j) = *reinterpret_cast<const int4*>(stage + j);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (j + e >= off && j + e < base && from + j + e < stride) out[from + j + e] = stage[j + e];
+          }
+        }
+        __syncwarp();
+        pos += base - off;
       }
-      __syncwarp();
-      pos += kept;
     }
   } else if (!invalid) {
     count = L;
