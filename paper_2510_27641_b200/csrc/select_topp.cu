@@ -31,6 +31,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "ptx.cuh"
 #include "nvtx_range.h"

@@ -10,19 +10,21 @@
 // With that, the passes are bound by instruction issue and by the wavefronts of shared-memory atomics, so each does
 // as little per entry as it can:
 //   pass 1  adds the top 15 mantissa bits to one word per bin (exponent and five mantissa bits) -- one atomic, not
-//           two words for an exact sum -- and the value itself to the thread's binary64 total.  The histogram is
-//           good to 2^-14, which names the threshold's bin in all but a few of 10^4 rows;
+//           two words for an exact sum -- which names the threshold's bin in all but a few of 10^4 rows.  The
+//           other nine bits, times 2^e, are added up by the thread, sixteen in binary32 (exact as a rule) and
+//           their sums in binary64.  What bounds the pass is the atomic: 4.1 wavefronts of random banks, two cycles each;
 //   pass 2  notes two bits per entry, above the bin / in the bin, in per-thread words (no votes) and adds up
-//           in binary64 what lies above.  The keys of the bin are then fetched by their bits.
+//           the low bits of what lies above.  The keys of the bin are then fetched by their bits.
 // The masses tell exactly whether the bin was the right one; if not, the row is read again for its neighbour.
-// 256 rows of 131072, uniform, p = 0.9: 117 us with exact two-word bins, votes and 128-entry emission.
+// 256 rows of 131072, p = 0.9, uniform / Zipf / ties: 96 / 81 / 93 us; with exact two-word bins, votes and 128-entry
+// emission 117 / 102 / 142.
 #pragma once
 
 constexpr int kStreamThreads = 512;
 constexpr int kStreamWarps = kStreamThreads / 32;
 constexpr int kStreamRound = 4 * kStreamThreads;   // entries per round of the CTA: 8 KB
-constexpr int kStreamBatch = 2;                    // rounds per commit group
-constexpr int kStreamGroups = 4;                   // groups in the ring
+constexpr int kStreamBatch = 4;                    // rounds per commit group
+constexpr int kStreamGroups = 2;                   // groups in the ring
 constexpr int kStreamMax = 131072;                 // entries per row: 64 rounds
 constexpr int kStreamShift = 18;                   // level-1 bins: the key's bits above these
 constexpr int kStreamBins = 8192;
@@ -115,6 +117,9 @@ __device__ __forceinline__ void stream_pass(StreamShared& sh, const float* A, in
   __syncthreads();
 }
 
+// What a key's 15 bits in the histogram leave of its value: its low nine mantissa bits.
+__device__ __forceinline__ float stream_rest(unsigned int k) { return __uint_as_float(k) - __uint_as_float(k & ~0x1ffu); }
+
 // Sum over the CTA in a fixed order; every thread gets it.  Two barriers.
 __device__ __forceinline__ double stream_sum(StreamShared& sh, double s) {
 #pragma unroll
@@ -166,6 +171,10 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   unsigned int theta = 0u;
   unsigned int* const above_bits = sh.store;
   unsigned int* const in_bits = sh.store + kStreamWords;
+  bool exact_sums = false;     // a row so small that every value is added up in binary64
+  auto bin_mass9 = [&](int oct) {  // lane: bin of an octave
+    return static_cast<double>(static_cast<unsigned long long>(hist[stream_word(32 * oct + lane)]) << 9) * pow2_double(max(oct, 1) - 150);
+  };
   int go = 0;                  // 1 / -1: the bin above / below the last one tried is wanted
   for (;;) {
     // ---- pass 1: histogram, total and validity -------------------------------------------------------
@@ -202,12 +211,15 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
         for (int j = 0; j < N; ++j)
           if (k[j] != 0u) stream_bump(hist_at, consts, k[j]);
       }
+      float rest = 0.f;  // (sixteen 9-bit pieces: exact while their exponents lie within 2^12)
 #pragma unroll
-      for (int j = 0; j < N; ++j) mine += static_cast<double>(__uint_as_float(k[j]));
+      for (int j = 0; j < N; ++j) rest += stream_rest(k[j]);
+      mine += static_cast<double>(rest);
     });
     if (__any_sync(kFull, negative) && lane == 0) sh.negative = 1;
 
     // ---- the bin of the threshold ---------------------------------------------------------------------
+    const double rest = stream_sum(sh, mine);
     if (tid < kOctaves) {
       unsigned long long s = 0ull;
 #pragma unroll 8
@@ -220,52 +232,72 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
         atomicMax(&sh.oct_max, final);
       }
     }
-    total = stream_sum(sh, mine);
-    target = static_cast<double>(P.p) * total;
-    // NaN and infinities survive into the sum (finite ones cannot overflow it)
-    invalid = sh.negative != 0 || !(total <= DBL_MAX);
-    if (invalid) total = target = 0.0;
-    m_ge = total;
-    searching = !invalid && target > 0.0 && !P.keep_all;  // else p >= 1 or an all-zero row: keep all
-    if (!searching) break;
+    __syncthreads();
+    invalid = sh.negative != 0 || sh.oct_max == kOctaves - 1;  // (the last octave: infinities and NaN)
     if (warp == 0) {
-      int bin;
-      if (go == 0) {
-        double t, tg, carry, ab, up;
-        const int oct = find_octave(sh.oct_max, sh.oct_min, P.p, [&](int e) { return sc.oct[e] << 9; }, t,
-                                    tg, carry);
-        const double m = static_cast<double>(static_cast<unsigned long long>(hist[stream_word(32 * oct + lane)]) << 9) * pow2_double(max(oct, 1) - 150);
-        bin = 32 * oct + find_from_top<5>(m, 0.0, carry, tg, ab, up);
-      } else {  // the next one with an entry, or -1
-        int at = sh.fd.bin;
-        bin = -1;
-        for (;;) {
-          at = (go > 0) ? at + 1 : at - 1;
-          const int mine_at = (go > 0) ? at + lane : at - lane;
-          const unsigned some = __ballot_sync(kFull, mine_at >= 0 && mine_at < kStreamBins && hist[stream_word(mine_at & (kStreamBins - 1))] != 0u);
-          if (some != 0u) {
-            bin = (go > 0) ? at + __ffs(some) - 1 : at - (__ffs(some) - 1);
-            break;
+      double t = 0.0, tg = 0.0, carry = 0.0, ab = 0.0, up;
+      int bin = -1;
+      if (sh.oct_max >= 0 && !invalid) {
+        const int oct = find_octave(sh.oct_max, sh.oct_min, P.p, [&](int e) { return sc.oct[e] << 9; }, t, tg, carry);
+        bin = 32 * oct + find_from_top<5>(bin_mass9(oct), 0.0, carry, tg, ab, up);
+        if (go != 0) {  // the next one with an entry, or none
+          int at = sh.fd.bin;
+          bin = -1;
+          for (;;) {
+            at = (go > 0) ? at + 1 : at - 1;
+            const int mine_at = (go > 0) ? at + lane : at - lane;
+            const unsigned some = __ballot_sync(kFull, mine_at >= 0 && mine_at < kStreamBins && hist[stream_word(mine_at & (kStreamBins - 1))] != 0u);
+            if (some != 0u) {
+              bin = (go > 0) ? at + __ffs(some) - 1 : at - (__ffs(some) - 1);
+              break;
+            }
+            at = (go > 0) ? at + 31 : at - 31;
+            if (at < 0 || at >= kStreamBins) break;
           }
-          at = (go > 0) ? at + 31 : at - 31;
-          if (at < 0 || at >= kStreamBins) break;
+          // its mass above, octave by octave from the top
+          carry = ab = 0.0;
+          if (bin >= 0) {
+            for (int e = sh.oct_max; e > (bin >> 5); --e) carry += static_cast<double>(sc.oct[e] << 9) * pow2_double(max(e, 1) - 150);
+            ab = suffix_sum<5>((lane > (bin & 31)) ? bin_mass9(bin >> 5) : 0.0);
+            ab = __shfl_sync(kFull, ab, 0);
+          }
         }
       }
       if (lane == 0) {
+        sh.fd.total = t;
         sh.fd.key = (bin < 0) ? 0xffffffffu : 0u;  // (no such bin)
         if (bin >= 0) {
           sh.fd.bin = bin;
+          sh.fd.carry = carry + ab;
           // the bin's smallest term bounds the number of its keys
           sh.fd.count = hist[stream_word(bin)] / (0x4000u | (static_cast<unsigned int>(bin & 31) << 9));
         }
       }
     }
     __syncthreads();
+    total = sh.fd.total + rest;
+    if (!invalid && !(total >= 0x1p-40)) {
+      // (the histogram takes a denormal for a number of at least 2^-126, which only counts in a total as small
+      // as this: every value is added up)
+      double again = 0.0;
+      stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) again += static_cast<double>(__uint_as_float(k[j]));
+      });
+      total = stream_sum(sh, again);
+      exact_sums = true;
+    }
+    if (invalid) total = 0.0;
+    target = static_cast<double>(P.p) * total;
+    m_ge = total;
+    searching = !invalid && target > 0.0 && !P.keep_all;  // else p >= 1 or an all-zero row: keep all
+    if (!searching) break;
     const bool last_resort = sh.fd.key == 0xffffffffu;   // keep the bin tried before
     unsigned int prefix = static_cast<unsigned int>(sh.fd.bin);
     const double scale = pow2_double(max(sh.fd.bin >> 5, 1) - 150);
     unsigned int M = last_resort ? 0x7fffffffu : sh.fd.count;
     int shift = kStreamShift;
+    const double above_hist = sh.fd.carry;
     int want = 0;
     __syncthreads();
     // ---- a well filled bin: 10 (then the last 8) more bits, one pass over the row each -----------------------
@@ -321,19 +353,23 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     const unsigned int lo_key = (prefix != 0u) ? prefix << shift : 1u;
     const unsigned int top_key = (prefix << shift) + ((1u << shift) - 1u), span = top_key - lo_key;
     double carry = 0.0;
-    {
+    auto pass2 = [&](auto whole) {
+      double s = 0.0;
       unsigned int ab = 0u, in = 0u;
       const int last = ((L + kStreamRound - 1) / kStreamRound + kStreamBatch - 1) / kStreamBatch * kStreamBatch - kStreamBatch;
       stream_pass(sh, A, L, [&](int round, unsigned int (&k)[N]) {
         unsigned int a8 = 0u, i8 = 0u;
+        float rest = 0.f;
 #pragma unroll
         for (int j = 0; j < N; ++j) {
+          const float r = stream_rest(k[j]);
           if (static_cast<int>(k[j]) > static_cast<int>(top_key)) {
             a8 |= 1u << j;
-            carry += static_cast<double>(__uint_as_float(k[j]));
+            if (decltype(whole)::value) s += static_cast<double>(__uint_as_float(k[j])); else rest += r;
           }
           if (k[j] - lo_key <= span) i8 |= 1u << j;
         }
+        if (!decltype(whole)::value) s += static_cast<double>(rest);
         const int at = 4 * (round & 7);
         ab |= a8 << at;
         in |= i8 << at;
@@ -343,9 +379,14 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
           ab = in = 0u;
         }
       });
-    }
+      carry = s;
+    };
+    // above a whole bin the histogram has the upper part of the sum; above a part of one, or in a row of
+    // denormals, every value is added up
+    const bool by_hist = shift == kStreamShift && !exact_sums;
+    if (by_hist) pass2(std::false_type()); else pass2(std::true_type());
     if (tid == 0) sh.n_cand = 0;
-    carry = stream_sum(sh, carry);
+    carry = stream_sum(sh, carry) + (by_hist ? above_hist : 0.0);
     if (shift > 0) level_clear<kStreamThreads>(sc.lv);
     // fetch the keys of the bin by their bits
     const int word_rows = (L + 8 * kStreamRound - 1) / (8 * kStreamRound);

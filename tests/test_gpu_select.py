@@ -467,3 +467,51 @@ def test_few_lists_wide_clusters_thresholds_above_two():
             st = compare_lists(lambda i: oracle.aggregate(probs[i], L=int(kv[i]))[0], p, gi.cpu().numpy(),
                                gc.cpu().numpy(), gs.cpu().numpy(), oi, oc, os_, od)
             assert st["n"] == B
+
+
+@pytest.mark.parametrize("n", [16388, 65536, 70001, 131072])
+@pytest.mark.parametrize("family", ["uniform", "zipf", "quantised", "narrow", "denormal", "sparse", "huge"])
+def test_many_rows_stream_one_cta_each(family, n, form):
+    """More rows than the GPU holds on chip: one CTA per row reads it twice.  Values all in one level-1 bin (more
+    keys than are gathered), denormal rows, mostly zeros, values up to 2^100, -0.0, an invalid row; lengths that
+    leave a part of a round, of a batch and of a row of words.  The oracle checks a sample; every row obeys
+    M_> < target <= M_>=."""
+    if form == "cluster":
+        pytest.skip("single-row lists take the same path with and without a workspace")
+    import paper_2510_27641_b200 as sa
+    n_rows, Ls = 300, (n + 3) // 4 * 4
+    rng = np.random.default_rng(n)
+    if family in wl.TOPP_FAMILIES:
+        rows = wl.topp_rows(family, n_rows, n, seed=4)
+    else:
+        rows = rng.random((n_rows, n), dtype=np.float32)
+        if family == "narrow":
+            rows = (np.float32(1.0) + rows * np.float32(2.0 ** -7)).astype(np.float32)
+        elif family == "denormal":
+            rows = (rows * np.float32(1e-41)).astype(np.float32)
+        elif family == "sparse":
+            rows *= rng.random((n_rows, n), dtype=np.float32) < 0.02
+        else:
+            rows = np.exp2(rows * 100.0).astype(np.float32)
+        rows[1, ::5] = -0.0
+    rows[2, n - 1] = np.nan
+    rows[3, 0] = -1e-30
+    full = np.full((n_rows, Ls), np.float32(7.0))
+    full[:, :n] = rows
+    kv = np.full(n_rows, n, np.int32)
+    kv[4], kv[5] = 1, 0
+    sample = np.r_[0:6, rng.choice(n_rows, size=6, replace=False)]
+    d = to_dev(full.reshape(n_rows, 1, 1, Ls))
+    for p in (0.02, 0.9, 0.999):
+        gi, gc, gs, gd = sa.select_topp.func([d], to_dev(kv), [0], p, want_diag=True)
+        torch.cuda.synchronize()
+        gc_h, gs_h, gd_h = gc.cpu().numpy().ravel(), gs.cpu().numpy().ravel(), gd.cpu().numpy().reshape(n_rows, 4)
+        ok = gs_h == 0
+        assert np.flatnonzero(~ok).tolist() == [2, 3]
+        pos = ok & (gd_h[:, 0] > 0)
+        assert np.all(gd_h[pos, 3] >= gd_h[pos, 1] * (1 - 1e-12)) and np.all(gd_h[pos, 2] < gd_h[pos, 1] * (1 + 1e-12))
+        sub = full[sample]
+        oi, oc, os_, od = oracle.select_topp([sub.reshape(12, 1, 1, Ls)], np.zeros(1, np.int32), kv[sample], p)
+        st = compare_lists(lambda i: sub[i, :kv[sample][i]], p, gi.cpu().numpy()[0, sample][None], gc_h[sample].reshape(1, 12, 1),
+                           gs_h[sample].reshape(1, 12, 1), oi, oc, os_, od)
+        assert st["n"] == 12
