@@ -18,12 +18,13 @@
 #pragma once
 
 constexpr int kSliceMax = 16384;         // entries per CTA of a cluster
-constexpr int kCandCap = 2048;           // keys of the threshold bin that a cluster gathers
+constexpr int kCandCap = 4096;           // keys of the threshold bin that a cluster gathers
 constexpr int kDirectMax = 128;          // up to this many gathered keys the threshold is found by comparing all pairs
 constexpr int kL1Bins = 2048;            // sign(0) + 8 exponent bits + 3 mantissa bits
 constexpr int kLevelBins = 1024;         // 10 mantissa bits per further level
 constexpr int kOctaves = 256;
 constexpr int kMaxCluster = 16;
+constexpr int kMaxApart = 64;            // speculated queries of searches apart
 
 struct SearchResult {
   unsigned int theta;   // keep every entry whose key is >= theta
@@ -316,6 +317,10 @@ struct SearchFixed {
   Found fd;
   int warp_cnt[16];                // kept entries per warp
   int kept[kMaxCluster];           // kept entries of every CTA of the cluster
+  // searches apart (one CTA per query, see select_topp_kernel); read by peers
+  int bad;                         // an invalid input was met
+  unsigned int theta[kMaxApart];   // thresholds of the queries this CTA searched (0xffffffff: invalid)
+  double masses[4];                // of the last query
 };
 // ... and the part that may share its bytes with the staging ring of the aggregation.
 struct SearchScratch {
@@ -377,9 +382,10 @@ template <> struct HitWord<true> { using type = unsigned long long; };
 // slice), complete and histogrammed (fx.hist, fx.kmax; fx.oct_min = kOctaves), every thread past a barrier.
 // bisect: number of halvings of the literal Alg. 2 loop, 0 = exact threshold.  The caller keeps the
 // cluster together (a cluster barrier) before any of the shared memory is used again or a CTA leaves.
+// The row lies in the CTAs of ranks r0 ... r0 + cs - 1 (cs = 1: this one's alone).
 template <int NT>
 __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScratch& sc, const float* a, int n4_pad,
-                                                     float p, bool keep_all, int bisect, int cs) {
+                                                     float p, bool keep_all, int bisect, int cs, int r0 = 0) {
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kW = NT / 32;
@@ -410,8 +416,8 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
   csync();
   if (warp == 0) {
     // largest key and lowest octave over the cluster, then the octave and its eight bins
-    unsigned int km = (lane < cs) ? *cluster.map_shared_rank(&fx.kmax, lane) : 0u;
-    int om = (lane < cs) ? *cluster.map_shared_rank(&fx.oct_min, lane) : kOctaves;
+    unsigned int km = (lane < cs) ? *cluster.map_shared_rank(&fx.kmax, r0 + lane) : 0u;
+    int om = (lane < cs) ? *cluster.map_shared_rank(&fx.oct_min, r0 + lane) : kOctaves;
     km = __reduce_max_sync(kFull, km);
     om = __reduce_min_sync(kFull, om);
     Found fd;
@@ -425,7 +431,7 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
           [&](int e) -> unsigned long long {
             unsigned long long s = 0ull;
             if (cs == 1) return sc.oct[e];
-            for (int r = 0; r < cs; ++r) s += *cluster.map_shared_rank(&sc.oct[e], r);
+            for (int r = 0; r < cs; ++r) s += *cluster.map_shared_rank(&sc.oct[e], r0 + r);
             return s;
           },
           fd.total, fd.target, fd.carry);
@@ -433,7 +439,7 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
       unsigned int c = 0u;
       fd.bin = 8 * fd.oct + (lane & 7);  // lane = (bin, rank mod 4)
       for (int r = lane >> 3; r < cs; r += 4) {
-        const unsigned int* h = cluster.map_shared_rank(fx.hist, r);
+        const unsigned int* h = cluster.map_shared_rank(fx.hist, r0 + r);
         const unsigned int lo = h[fd.bin], hi = h[kL1Bins + fd.bin];
         s += bin_mass(fd.bin, lo, hi);
         c += hi >> 17;
@@ -491,14 +497,14 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
     csync();
     if (warp == 0) {
       unsigned long long s = 0ull;
-      for (int r = 0; r < cs; ++r) s += *cluster.map_shared_rank(&sc.lv.grp[lane], r);
+      for (int r = 0; r < cs; ++r) s += *cluster.map_shared_rank(&sc.lv.grp[lane], r0 + r);
       double above, upto;
       const int gi = find_from_top<5>(static_cast<double>(s) * scale, inner, carry, res.target, above, upto);
       const int bin = gi * 32 + lane;
       unsigned int c = 0u;
       s = 0ull;
       for (int r = 0; r < cs; ++r) {
-        const LevelHist* peer = cluster.map_shared_rank(&sc.lv, r);
+        const LevelHist* peer = cluster.map_shared_rank(&sc.lv, r0 + r);
         c += peer->cnt[bin];
         s += peer->sum[bin];
       }
@@ -569,8 +575,8 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
     }
     csync();
     // every warp: how many keys each CTA has in the bin and above it, and where its keys begin
-    const int c_r = (lane < cs) ? min(*cluster.map_shared_rank(&fx.n_cand, lane), kCandCap) : 0;
-    const int above_r = (lane < cs) ? *cluster.map_shared_rank(&fx.n_above, lane) : 0;
+    const int c_r = (lane < cs) ? min(*cluster.map_shared_rank(&fx.n_cand, r0 + lane), kCandCap) : 0;
+    const int above_r = (lane < cs) ? *cluster.map_shared_rank(&fx.n_above, r0 + lane) : 0;
     int end_r = c_r;
 #pragma unroll
     for (int d = 1; d < kMaxCluster; d <<= 1) {
@@ -584,7 +590,7 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
       const int share = max(kW / cs, 1);  // warps per rank
       for (int r = warp / share; r < cs; r += kW / share) {
         const int c = __shfl_sync(kFull, c_r, r), off = __shfl_sync(kFull, end_r, r) - c;
-        const unsigned int* src = cluster.map_shared_rank(sc.cand, r);
+        const unsigned int* src = cluster.map_shared_rank(sc.cand, r0 + r);
         for (int i = (warp % share) * 32 + lane; i < c && off + i < kCandCap; i += share * 32) all_keys[off + i] = src[i];
       }
       keys = all_keys;

@@ -67,6 +67,7 @@ struct SelectParams {
   int per_step;    // Alg. 2 as printed: one nucleus per speculated query, unioned
   int bisect_iters;  // > 0: the threshold is the last midpoint of that many bisection steps
   int chunk;         // > 1: selection over per-chunk sums (power of two, 4..64); kept chunks keep all positions
+  int apart;         // per_step at chunk granularity: the queries are searched by one CTA each, all at once
   const float* agg;  // two-launch form: the aggregated rows, [list][L_stride], written by aggregate_rows_kernel
 };
 
@@ -234,8 +235,19 @@ __global__ void __launch_bounds__(NT, NT >= 512 || kAgg ? 2 : 8) select_topp_ker
   const int w4 = n4_pad / kW;  // float4s per warp in the passes over the slice
   SearchResult res;
   bool invalid = false;
+  // Searches apart: chunk scores of all queries are few (a list of 32768 positions in chunks of 16: 2048 per
+  // query), so they are kept while the rows of all queries stream in one go; then every CTA of the
+  // cluster gathers the scores of one query and searches them alone, all queries at once, instead of the
+  // cluster searching one query after the other (9 us each, the streaming idle meanwhile: five queries of 32 such
+  // lists 88 us).
+  const bool apart = kAgg && kVariant && P.apart;
+  const int row_room = apart ? slice_of(static_cast<int>(P.L_stride), cs, chunk) / chunk : 0;  // entries per query and CTA
+  float* const scores = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(mask) +
+                                                 (apart ? slice_room(slice_of(static_cast<int>(P.L_stride), cs, chunk), NT) / 8 : 0));
+  bool bad = false;
+  int ic = 0, ih = 0, is = 0, istep = 0, islot = 0, slot_c = 0;  // column, head, query, step and ring slots of the next piece
   for (int step = 0; step < n_steps; ++step) {
-    if (kAgg && step > 0) {
+    if (kAgg && step > 0 && !apart) {
       clear();
       __syncthreads();
     }
@@ -290,37 +302,42 @@ __global__ void __launch_bounds__(NT, NT >= 512 || kAgg ? 2 : 8) select_topp_ker
       constexpr int kCols = kChunk / (4 * NT);
       const int n_pos4 = (n_loc + 3) & ~3;
       const int n_chunks = (n_pos4 + kChunk - 1) / kChunk;
-      const int s_lo = use_mask ? step : 0, s_hi = use_mask ? step + 1 : P.gamma;
-      const int R = *n_heads * (s_hi - s_lo);
+      const int n_q = use_mask ? 1 : P.gamma;  // rows per head
+      const int R = *n_heads * n_q;
       const uint32_t ring_addr = smem_u32(ring) + tid * 16;
       const float* src0 = A + 4 * tid;
-      int ic = 0, ih = 0, is = s_lo, islot = 0;  // piece column, head, query and ring slot of the next request
       auto issue = [&]() {
         if (ic < n_chunks && R > 0) {
           const int len4 = min(kChunk, n_pos4 - ic * kChunk) >> 2;
-          const float* src = src0 + static_cast<long long>(heads[ih] * P.gamma + is) * P.L_stride + ic * kChunk;
+          const float* src = src0 + static_cast<long long>(heads[ih] * P.gamma + (use_mask ? istep : is)) * P.L_stride + ic * kChunk;
           const uint32_t dst = ring_addr + islot * (kChunk * 4);
 #pragma unroll
           for (int k = 0; k < kCols; ++k)
             if (tid + k * NT < len4) cp_async16(dst + k * NT * 16, src + k * NT * 4);
-          if (++is == s_hi) {
-            is = s_lo;
+          if (++is == n_q) {
+            is = 0;
             if (++ih == *n_heads) {
               ih = 0;
-              ++ic;
+              if (++ic == n_chunks && apart && istep + 1 < n_steps) {  // on to the next query's rows without a break
+                ic = 0;
+                ++istep;
+              }
             }
           }
           islot = (islot + 1) & (kDepth - 1);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
       };
-      for (int q = 0; q < kDepth - 1; ++q) issue();
+      if (step == 0 || !apart) {
+        ic = ih = is = islot = slot_c = 0;
+        istep = step;
+        for (int q = 0; q < kDepth - 1; ++q) issue();
+      }
       // Validity of the inputs is tracked with a running minimum (a negative input, the only
       // invalid value a sum can hide) -- NaN and Inf survive into the aggregated value itself.
       float4 acc[kCols], mn[kCols];
 #pragma unroll
       for (int k = 0; k < kCols; ++k) acc[k] = mn[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      int slot_c = 0;
       for (int c = 0; c < n_chunks; ++c) {
         const int len4 = min(kChunk, n_pos4 - c * kChunk) >> 2;
         // positions of this thread's float4s that lie beyond the slice (last float4 only)
@@ -366,7 +383,29 @@ __global__ void __launch_bounds__(NT, NT >= 512 || kAgg ? 2 : 8) select_topp_ker
           if (!chunked || m > 0x7f7fffffu) kmax = max(kmax, m);
           if (!chunked) hist_add<4>(fx.hist, key);
           acc[k] = mn[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (apart) {  // the chunks of the warp's 128 positions, one per lane
+            __syncwarp();
+            const int p0 = c * kChunk + 4 * (32 * warp + k * NT) + lane * chunk;
+            if (lane * chunk < 128 && p0 < n_loc) {
+              float s = 0.f;
+              for (int e = 0; e < chunk; e += 4) {
+                const float4 u = *reinterpret_cast<const float4*>(a + p0 + e);
+                const int left = n_loc - (p0 + e);
+                if (left > 0) s = s + u.x;
+                if (left > 1) s = s + u.y;
+                if (left > 2) s = s + u.z;
+                if (left > 3) s = s + u.w;
+              }
+              scores[step * row_room + p0 / chunk] = s;
+              bad |= !(s <= FLT_MAX);
+            }
+            __syncwarp();  // (the next query's values overwrite these)
+          }
         }
+      }
+      if (apart) {
+        bad |= kmax > 0x7f7fffffu;
+        continue;
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       if (chunked) {
@@ -418,6 +457,68 @@ __global__ void __launch_bounds__(NT, NT >= 512 || kAgg ? 2 : 8) select_topp_ker
       // the next query's row overwrites the slice and the staging ring, which peers may still be reading
       csync();
     }
+  }
+
+  if (apart) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (tid == 0) fx.bad = 0;
+    __syncthreads();
+    if (bad) fx.bad = 1;
+    csync();  // every CTA's scores are complete
+    const int n_all = (L + chunk - 1) / chunk, per_e = per / chunk;
+    const int n4_all = slice_room(n_all, NT) / 4;
+    for (int s = rank; s < n_steps; s += cs) {
+      clear();
+      __syncthreads();
+      unsigned int kmax = 0u;
+      for (int i = tid; i < 4 * n4_all; i += NT) {
+        float v = 0.f;
+        if (i < n_all) {
+          const int r = i / per_e;
+          v = *cluster.map_shared_rank(scores + s * row_room + (i - r * per_e), r);
+        }
+        a[i] = v;
+        const unsigned int key[1] = {__float_as_uint(v)};
+        kmax = max(kmax, key[0]);
+        hist_add<1>(fx.hist, key);
+      }
+      kmax = __reduce_max_sync(kFull, kmax);
+      if (lane == 0 && kmax != 0u) atomicMax(&fx.kmax, kmax);
+      __syncthreads();
+      res = search_slice<NT>(fx, sc, a, n4_all, P.p, P.keep_all != 0, P.bisect_iters, 1, rank);
+      if (tid == 0) {
+        fx.theta[s] = res.invalid ? 0xffffffffu : res.theta;
+        if (s == n_steps - 1) {
+          fx.masses[0] = res.total;
+          fx.masses[1] = res.target;
+          fx.masses[2] = res.m_gt;
+          fx.masses[3] = res.m_ge;
+        }
+      }
+      __syncthreads();
+    }
+    csync();  // every query has its threshold
+    invalid = __any_sync(kFull, lane < cs && *cluster.map_shared_rank(&fx.bad, lane < cs ? lane : 0) != 0);
+    unsigned int* const thetas = reinterpret_cast<unsigned int*>(ring);  // (the search's scratch is idle)
+    if (tid < n_steps) thetas[tid] = *cluster.map_shared_rank(&fx.theta[tid], tid % cs);
+    if (tid == 0) {
+      const double* m = cluster.map_shared_rank(fx.masses, (n_steps - 1) % cs);
+      res.total = m[0];
+      res.target = m[1];
+      res.m_gt = m[2];
+      res.m_ge = m[3];
+    }
+    __syncthreads();
+    for (int s = 0; s < n_steps; ++s) invalid |= thetas[s] == 0xffffffffu;
+    for (int i0 = 4 * warp * w4; i0 < 4 * (warp + 1) * w4; i0 += 32) {
+      const int i = i0 + lane;
+      bool keep = false;
+      if (i < n_srch && !invalid)
+        for (int s = 0; s < n_steps; ++s) keep |= __float_as_uint(scores[s * row_room + i]) >= thetas[s];
+      const unsigned int m = __ballot_sync(kFull, keep);
+      if (lane == 0) mask[i0 >> 5] = m;
+    }
+    __syncthreads();
   }
 
   // ---- ordered compaction ------------------------------------------------------------------------
@@ -707,19 +808,30 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
   const bool variant = P.per_step || P.bisect_iters > 0 || P.chunk > 1;
   const bool one_row = static_cast<long long>(A.n_draft_heads) * A.gamma == 1 && P.chunk == 1;
   const bool agg = !two_launch && !one_row;  // the CTAs sum the rows (or the chunks) themselves
-  // (rows that are many: one CTA each)
+  // One CTA per row (stream_rows.cuh), where a cluster per row would need more than one wave of CTAs, or where
+  // there is about a row for every SM and a cluster's exchanges gain nothing (100 rows of 8192: 11.6 us against
+  // 13.5; of 32768: 18.9 against 22.8; of 131072: 55 against 95; 64 rows of 32768: 18.7 against 17.4).
+  const long long row_ctas = agg ? 0 : n_lists * specattn::pick_cluster_row(A.L_stride, n_lists);
   const bool stream = !agg && !variant && A.L_stride <= specattn::kStreamMax && A.L_stride > 4096 &&
-                      n_lists * specattn::pick_cluster_row(A.L_stride, n_lists) > 296;
+                      (row_ctas > 296 || (n_lists > 72 && n_lists <= 148));
   const bool small = !agg && !variant && A.L_stride <= 2048;
   const int cs = stream ? 1 : agg ? specattn::pick_cluster(A.L_stride, n_lists) : specattn::pick_cluster_row(A.L_stride, n_lists);
   const int slice = specattn::slice_of(static_cast<int>(A.L_stride), cs, (P.chunk > 4) ? P.chunk : 4);
   const int nt = small ? 128 : agg ? 256 : 512;
   if (slice > specattn::kSliceMax && !stream) return SPECATTN_ERR_UNSUPPORTED;
+  // searches apart: the scores of all queries are kept, and one query's scores fit a CTA's slice
+  const long long n_scores = (A.L_stride + P.chunk - 1) / P.chunk;
+  const size_t score_bytes = static_cast<size_t>(A.gamma) * (slice / P.chunk) * sizeof(float);
+  P.apart = (agg && P.per_step && P.chunk > 1 && A.gamma <= specattn::kMaxApart && n_scores <= specattn::kSliceMax &&
+             specattn::slice_room(static_cast<int>(n_scores), nt) <= specattn::slice_room(slice, nt) && score_bytes <= 48 * 1024)
+                ? 1
+                : 0;
+  const size_t apart_bytes = P.apart ? score_bytes : 0;
   const size_t smem = stream ? sizeof(specattn::StreamShared) : specattn::kFixedBytes + (agg ? specattn::kHeadBytes : 0) +
                       static_cast<size_t>(specattn::slice_room(slice, nt)) * sizeof(float) +
                       (agg ? specattn::kRingBytes : specattn::kScratchBytes) +
                       // the union's bit mask: one bit per entry of the slice
-                      (P.per_step ? static_cast<size_t>(specattn::slice_room(slice, nt) / 8) : 0);
+                      (P.per_step ? static_cast<size_t>(specattn::slice_room(slice, nt) / 8) : 0) + apart_bytes;
   const void* const kernels[6] = {
       (const void*)specattn::select_topp_kernel<false, false, 128>, (const void*)specattn::select_topp_kernel<false, false, 512>,
       (const void*)specattn::select_topp_kernel<false, true, 512>, (const void*)specattn::select_topp_kernel<true, false, 256>,

@@ -515,3 +515,22 @@ def test_many_rows_stream_one_cta_each(family, n, form):
         st = compare_lists(lambda i: sub[i, :kv[sample][i]], p, gi.cpu().numpy()[0, sample][None], gc_h[sample].reshape(1, 12, 1),
                            gs_h[sample].reshape(1, 12, 1), oi, oc, os_, od)
         assert st["n"] == 12
+
+
+@pytest.mark.parametrize("chunk,gamma,Ls,lens", [(16, 11, 3000, [3000, 17, 0]), (8, 3, 40000, [40000, 12345]),
+                                                 (64, 20, 8192, [8191, 64]), (4, 2, 2048, [2048, 2045])])
+def test_queries_searched_apart_at_chunk_granularity(chunk, gamma, Ls, lens):
+    """The union at chunk granularity searches the queries in one CTA each: more queries than CTAs in a
+    cluster, lists that leave CTAs empty, a last chunk that is cut, an invalid input that the sums hide."""
+    import paper_2510_27641_b200 as sa
+    kv = np.asarray(lens, np.int32)
+    probs = wl.draft_probs(21, 0, kv, 3, gamma, Ls, sink=6.0, slope=0.004)
+    bad = probs.copy()
+    bad[0, 1, gamma - 1, 5] = -1e-30
+    for a, iters in ((probs, 0), (probs, 10), (bad, 0)):
+        gi, gc, gs, gd = sa.select_topp([to_dev(a)], to_dev(kv), [0], 0.9, per_step=True, bisect_iters=iters, chunk=chunk,
+                                        want_diag=True)
+        torch.cuda.synchronize()
+        oi, oc, os_, od = oracle.select_variant([a], [0], kv, 0.9, per_step=True, n_iters=iters, chunk=chunk)
+        assert _compare_variant(gi, gc, gs, oi, oc, os_, od) == len(lens)
+        assert gs[0, 0, 0].item() == (sa.ROW_INVALID_PROB if a is bad else 0)
