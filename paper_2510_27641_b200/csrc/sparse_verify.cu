@@ -707,6 +707,13 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   const int lane = tid & 31;
   const int warp = tid >> 5;
   const int U = P.B * P.Hkv;
+  // In the CTA's first turn the four producer warps share the first four tiles (16 rows of each), so that the
+  // first tile lands ahead of the others instead of all four at the end of one burst.  The barrier of a tile
+  // then counts four arrivals per lane, its owner's come fourfold later on.  For query blocks of 33 - 64
+  // rows: 40 rows, 4 x 1100 positions 14.05 -> 13.7 us, 16 x 700 21.4 -> 20.9; with four consumer warps per slab the
+  // extra arrivals cost long lists more (16 x 2048: 35.5 -> 36.6) than short ones gain.
+  constexpr bool kShareFirst = (WPM == 2);
+  constexpr int kArrivals = kShareFirst ? kProdWarps : 1;
   constexpr bool kQReload = (WPM == 2);   // query fragments re-read from shared memory per block
   constexpr bool kDirectQ = true;         // consumers fetch the CTA's first query block themselves
 
@@ -723,7 +730,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   }
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sh.full[s], 32);   // one deferred arrival per producer lane
+      mbar_init(&sh.full[s], 32 * kArrivals);  // deferred arrivals per producer lane
       mbar_init(&sh.empty[s], NCS);
     }
     mbar_init(&sh.q_full, 1);
@@ -895,11 +902,12 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       // list -> position -> block table -> page, two dependent loads, in two steps so that a
       // warp can keep the chain one tile of its own ahead (positions of its tile after next,
       // offsets of its next tile): neither load is then waited for between two tiles
+      bool first = kShareFirst && seg == 0;
       auto load_pos = [&](int t0, int (&pos)[2]) {
-        const int ntok = min(kStageTok, tok_hi - t0);
 #pragma unroll
         for (int jj = 0; jj < 2; ++jj) {
-          const int k = t0 + min(lane + jj * 32, ntok - 1);  // token index inside the unit: the list first, then the tail
+          // token index inside the unit: the list first, then the tail
+          const int k = min(t0 + (first ? (2 * jj + (lane >> 4)) * kStageTok + 16 * pw + (lane & 15) : lane + jj * 32), tok_hi - 1);
           pos[jj] = (k >= c_list) ? (kvlen_b + (k - c_list)) : (P.dense ? k : __ldg(list + k));
         }
       };
@@ -932,7 +940,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       int pos_nn[2] = {0, 0};
       int t0_nn = -1;    // tile whose positions are already loaded
       for (int t0 = tok_lo; t0 < tok_hi; t0 += kStageTok, ++it) {
-        if ((it % kProdWarps) != pw) continue;
+        if (!first && (it % kProdWarps) != pw) continue;
         const int s = it % kStages;
         const unsigned ph = (it / kStages) & 1u;
         long long off[2];
@@ -945,30 +953,51 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
           bad = resolve(t0, off);
         }
         if (!mbar_wait(&sh.empty[s], ph ^ 1u, &sh.abort_flag)) { sh.abort_flag = 1; dead = true; break; }
-        const int ntok = min(kStageTok, tok_hi - t0);
         // The tail of a segment is padded to a whole 32-key block with copies of its last
         // token, so that every row a consumer multiplies by a zero weight holds finite data.
-        const int npad = (ntok + 31) & ~31;
         // 16 lanes move one 256-byte row with 16-byte cp.async copies: a warp instruction
         // fetches two rows (four full 128-byte lines)
         const char* kbase = reinterpret_cast<const char*>(kv_head) + (lane & 15) * 16;
         const long long v_delta = P.s_kv * 2;
-        const uint32_t k_dst = smem_u32(sh.kv[s][0]) + (lane >> 4) * kPitch + (lane & 15) * 16;
-        const uint32_t v_dst = smem_u32(sh.kv[s][1]) + (lane >> 4) * kPitch + (lane & 15) * 16;
-#pragma unroll
-        for (int jj = 0; jj < 2; ++jj) {
+        if (first) {
+#pragma unroll 1
+          for (int blk = 0; blk < kStages; ++blk) {
+            const int left = tok_hi - (t0 + blk * kStageTok);
+            if (left <= 0) break;
+            const int npad = (min(kStageTok, left) + 31) & ~31;
+            const uint32_t k_dst = smem_u32(sh.kv[blk][0]) + (16 * pw + (lane >> 4)) * kPitch + (lane & 15) * 16;
+            const long long off_b = (blk & 2) ? off[1] : off[0];
 #pragma unroll 4
-          for (int i = 0; i < 16; ++i) {
-            const int tok = jj * 32 + 2 * i + (lane >> 4);
-            const long long o = __shfl_sync(0xffffffffu, off[jj], 2 * i + (lane >> 4));
-            if (tok < npad) {
-              cp_async16(k_dst + (jj * 32 + 2 * i) * kPitch, kbase + o);
-              cp_async16(v_dst + (jj * 32 + 2 * i) * kPitch, kbase + o + v_delta);
+            for (int i = 0; i < 8; ++i) {
+              const long long o = __shfl_sync(0xffffffffu, off_b, (blk & 1) * 16 + 2 * i + (lane >> 4));
+              if (16 * pw < npad) {
+                cp_async16(k_dst + 2 * i * kPitch, kbase + o);
+                cp_async16(k_dst + (kStageTok + 2 * i) * kPitch, kbase + o + v_delta);
+              }
+            }
+            // (test hook: the first tile of CTA 0 never completes, so the bounded waits run out)
+            if (!(P.test_lose && blockIdx.x == 0 && pw == 0 && blk == 0)) cp_async_mbar_arrive_noinc(&sh.full[blk]);
+          }
+        } else {
+          const int npad = (min(kStageTok, tok_hi - t0) + 31) & ~31;
+          const uint32_t k_dst = smem_u32(sh.kv[s][0]) + (lane >> 4) * kPitch + (lane & 15) * 16;
+          const uint32_t v_dst = smem_u32(sh.kv[s][1]) + (lane >> 4) * kPitch + (lane & 15) * 16;
+#pragma unroll
+          for (int jj = 0; jj < 2; ++jj) {
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i) {
+              const int tok = jj * 32 + 2 * i + (lane >> 4);
+              const long long o = __shfl_sync(0xffffffffu, off[jj], 2 * i + (lane >> 4));
+              if (tok < npad) {
+                cp_async16(k_dst + (jj * 32 + 2 * i) * kPitch, kbase + o);
+                cp_async16(v_dst + (jj * 32 + 2 * i) * kPitch, kbase + o + v_delta);
+              }
             }
           }
+#pragma unroll
+          for (int w = 0; w < kArrivals; ++w)
+            if (!(P.test_lose && blockIdx.x == 0 && it == 0)) cp_async_mbar_arrive_noinc(&sh.full[s]);
         }
-        // (test hook: the first tile of CTA 0 never completes, so the bounded waits run out)
-        if (!(P.test_lose && blockIdx.x == 0 && it == 0)) cp_async_mbar_arrive_noinc(&sh.full[s]);
         if (q_pending) {
           q_pending = false;
           if (!load_q()) { sh.abort_flag = 1; dead = true; break; }
@@ -976,7 +1005,10 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
         // Resolve this warp's next tile of the segment right after the copies went out (not
         // before: while the ring still has free slots the two dependent loads would delay
         // them by ~1.3 us), so that a slot's turnaround holds only the copy itself.
-        t0_next = t0 + kProdWarps * kStageTok;
+        const int last_tile = first ? min(it + kStages, (tok_hi - tok_lo + kStageTok - 1) / kStageTok) - 1 : it;
+        t0_next = t0 + (kProdWarps + (first ? pw : 0)) * kStageTok;
+        const bool was_first = first;
+        first = false;
         if (t0_next < tok_hi) {
           if (t0_nn != t0_next) load_pos(t0_next, pos_nn);  // (first tile of the segment only)
           // positions of the tile after next first (independent), then the block-table loads
@@ -990,7 +1022,12 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
           t0_next = -1;
         }
         if (bad && P.status) atomicOr(P.status + b, SPECATTN_ROW_BAD_INDEX);
-        last_it = it;
+        last_it = last_tile;
+        if (was_first) {  // the loop goes on behind the tiles that the turn covered
+          const int extra = last_tile - it;
+          it += extra;
+          t0 += extra * kStageTok;
+        }
       }
       a = seg_hi;
       ++seg;
