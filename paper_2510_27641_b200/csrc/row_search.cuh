@@ -337,9 +337,11 @@ __device__ __forceinline__ void hist_bump(unsigned int* hist, unsigned int key) 
   atomicAdd(p + kL1Bins, ((key >> 17) & 7u) | 0x20000u);
 }
 
-// Adds N keys per lane (all 32 lanes call this together).  Zeros carry no mass and are left out.
-// When every key of the warp falls into one bin (ties, constant rows) the warp reduces first: 32
-// updates of one address would be serialised.
+// Adds N keys per lane (all 32 lanes call this together), except those of bin 0: zeros carry no mass, and the
+// denormals below 2^-129 -- twenty octaves in one bin, on attention rows thousands of neighbours -- would serialise
+// the updates of one address (a slice of them took 17 us instead of 3); hist_add_tiny enters them where
+// they can matter.  When every key of the warp falls into one bin (ties, constant rows) the warp reduces first.
+constexpr unsigned int kTinyKeys = 0x100000u;
 template <int N>
 __device__ __forceinline__ void hist_add(unsigned int* hist, const unsigned int (&k)[N]) {
   const unsigned int bin0 = __shfl_sync(kFull, k[0] >> 20, 0);
@@ -348,15 +350,16 @@ __device__ __forceinline__ void hist_add(unsigned int* hist, const unsigned int 
 #pragma unroll
     for (int j = 1; j < N; ++j) differ |= k[j] ^ k[0];
     if (__all_sync(kFull, (differ >> 20) == 0u)) {
+      if (bin0 == 0u) return;
       unsigned int lo = 0u, hi = 0u;
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         lo += k[j] & 0x1ffffu;
-        hi += (k[j] != 0u) ? (((k[j] >> 17) & 7u) | 0x20000u) : 0u;
+        hi += ((k[j] >> 17) & 7u) | 0x20000u;
       }
       lo = __reduce_add_sync(kFull, lo);
       hi = __reduce_add_sync(kFull, hi);
-      if ((threadIdx.x & 31) == 0 && hi != 0u) {
+      if ((threadIdx.x & 31) == 0) {
         atomicAdd(&hist[bin0 & (kL1Bins - 1)], lo);
         atomicAdd(&hist[kL1Bins + (bin0 & (kL1Bins - 1))], hi);
       }
@@ -365,7 +368,34 @@ __device__ __forceinline__ void hist_add(unsigned int* hist, const unsigned int 
   }
 #pragma unroll
   for (int j = 0; j < N; ++j)
-    if (k[j] != 0u) hist_bump(hist, k[j]);
+    if (k[j] >= kTinyKeys) hist_bump(hist, k[j]);
+}
+
+// Enters the keys of bin 0 of a slice (n4_pad float4s), if its largest key is below 2^-50: beside a larger one
+// their sum, at most 2^17 times 2^-129, is less than the last place of the total.  Called by all threads between
+// barriers.
+template <int NT>
+__device__ __forceinline__ void hist_add_tiny(unsigned int* hist, unsigned int kmax, const float* a, int n4_pad) {
+  if (kmax == 0u || kmax >= 0x26800000u) return;
+  unsigned int lo = 0u, hi = 0u;
+  for (int i4 = threadIdx.x; i4 < n4_pad; i4 += NT) {
+    const uint4 v = *reinterpret_cast<const uint4*>(a + 4 * i4);
+    const unsigned int k[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (k[e] != 0u && k[e] < kTinyKeys) {
+        lo += k[e] & 0x1ffffu;
+        hi += ((k[e] >> 17) & 7u) | 0x20000u;
+      }
+    }
+  }
+  lo = __reduce_add_sync(kFull, lo);
+  hi = __reduce_add_sync(kFull, hi);
+  if ((threadIdx.x & 31) == 0 && hi != 0u) {
+    atomicAdd(&hist[0], lo);
+    atomicAdd(&hist[kL1Bins], hi);
+  }
+  __syncthreads();
 }
 
 // Exact integer mass of a level-1 bin (units of its exponent's last place).

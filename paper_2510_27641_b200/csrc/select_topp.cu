@@ -444,6 +444,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 || kAgg ? 2 : 8) select_topp_ker
     kmax = __reduce_max_sync(kFull, kmax);
     if (lane == 0 && kmax != 0u) atomicMax(&fx.kmax, kmax);
     __syncthreads();
+    hist_add_tiny<NT>(fx.hist, fx.kmax, a, n4_pad);
 
     res = search_slice<NT>(fx, sc, a, n4_pad, P.p, P.keep_all != 0, kVariant ? P.bisect_iters : 0, cs);
     invalid |= res.invalid;  // one query's invalid input voids the list
@@ -485,6 +486,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 || kAgg ? 2 : 8) select_topp_ker
       kmax = __reduce_max_sync(kFull, kmax);
       if (lane == 0 && kmax != 0u) atomicMax(&fx.kmax, kmax);
       __syncthreads();
+      hist_add_tiny<NT>(fx.hist, fx.kmax, a, n4_all);
       res = search_slice<NT>(fx, sc, a, n4_all, P.p, P.keep_all != 0, P.bisect_iters, 1, rank);
       if (tid == 0) {
         fx.theta[s] = res.invalid ? 0xffffffffu : res.theta;

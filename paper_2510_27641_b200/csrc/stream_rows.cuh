@@ -178,6 +178,9 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   int go = 0;                  // 1 / -1: the bin above / below the last one tried is wanted
   for (;;) {
     // ---- pass 1: histogram, total and validity -------------------------------------------------------
+    // (bin 0, zeros apart: eighteen octaves of denormals whose updates of one word would be serialised; they
+    // only count in a row without larger values)
+    const unsigned int min_key = exact_sums ? 1u : 1u << kStreamShift;
     bool negative = false;
     double mine = 0.0;
     stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
@@ -203,18 +206,23 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       if (one) {
         unsigned int s = 0u;
 #pragma unroll
-        for (int j = 0; j < N; ++j) s += (k[j] != 0u) ? ((k[j] >> 9) & 0x3fffu) | 0x4000u : 0u;
+        for (int j = 0; j < N; ++j) s += (k[j] >= min_key) ? ((k[j] >> 9) & 0x3fffu) | 0x4000u : 0u;
         s = __reduce_add_sync(kFull, s);
         if (lane == 0 && s != 0u) atomicAdd(&hist[stream_word(bin0 & (kStreamBins - 1))], s);
       } else {
 #pragma unroll
         for (int j = 0; j < N; ++j)
-          if (k[j] != 0u) stream_bump(hist_at, consts, k[j]);
+          if (k[j] >= min_key) stream_bump(hist_at, consts, k[j]);
       }
       float rest = 0.f;  // (sixteen 9-bit pieces: exact while their exponents lie within 2^12)
 #pragma unroll
       for (int j = 0; j < N; ++j) rest += stream_rest(k[j]);
-      mine += static_cast<double>(rest);
+      if (!exact_sums) {
+        mine += static_cast<double>(rest);
+      } else {
+#pragma unroll
+        for (int j = 0; j < N; ++j) mine += static_cast<double>(__uint_as_float(k[j]));
+      }
     });
     if (__any_sync(kFull, negative) && lane == 0) sh.negative = 1;
 
@@ -275,17 +283,13 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       }
     }
     __syncthreads();
-    total = sh.fd.total + rest;
-    if (!invalid && !(total >= 0x1p-40)) {
+    total = exact_sums ? rest : sh.fd.total + rest;
+    if (!invalid && !exact_sums && !(total >= 0x1p-40)) {
       // (the histogram takes a denormal for a number of at least 2^-126, which only counts in a total as small
-      // as this: every value is added up)
-      double again = 0.0;
-      stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) again += static_cast<double>(__uint_as_float(k[j]));
-      });
-      total = stream_sum(sh, again);
+      // as this: once more, with every value added up)
       exact_sums = true;
+      clear();
+      continue;
     }
     if (invalid) total = 0.0;
     target = static_cast<double>(P.p) * total;
