@@ -200,6 +200,17 @@ __device__ __forceinline__ unsigned int threshold_among(const unsigned int* keys
                                                         double inner, double carry, double target, double scale,
                                                         LevelHist& lv, Found& fd, Picks& pk, double& above, double& upto) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  {  // One value (ties, as in a quantised row): it is the threshold.  (256 rows of 8191 such: 14.5 -> 12.0 us; a row
+     // without ties leaves after one look at its few keys.)
+    const unsigned int k0 = keys[0];
+    bool same = true;
+    for (int i = tid; i < n; i += NT) same &= keys[i] == k0;
+    if (__syncthreads_and(same)) {
+      above = inner;
+      upto = inner + static_cast<double>(static_cast<unsigned long long>(n) * mantissa_of(k0)) * scale;
+      return k0;
+    }
+  }
   while (n > kDirectMax && shift > 0) {
     const int bits = min(shift, 10), sh = shift - bits;
     for (int i = tid; i < ((n + 31) & ~31); i += NT) {
@@ -516,11 +527,38 @@ __device__ __forceinline__ SearchResult search_slice(SearchFixed& fx, SearchScra
     }
     deep = true;
     const int sh = shift - 10;
-    for (int i4 = tid; i4 < n4_pad; i4 += NT) {
+    // A warp whose keys of the bin are all one value (ties) adds them up by itself; the first lane that holds two
+    // values sends it to the general way, which pays two atomics for every round of 32 keys.
+    unsigned int first = 0xffffffffu, last = 0u, held = 0u;
+    bool ties = true;
+    for (int i4 = tid; ties && i4 < n4_pad; i4 += NT) {
       const uint4 k4 = *reinterpret_cast<const uint4*>(a + 4 * i4);
       const unsigned int k[4] = {k4.x, k4.y, k4.z, k4.w};
 #pragma unroll
-      for (int e = 0; e < 4; ++e) level_add(sc.lv, (k[e] >> shift) == prefix && k[e] != 0u, k[e], sh);
+      for (int e = 0; e < 4; ++e) {
+        if ((k[e] >> shift) != prefix || k[e] == 0u) continue;
+        first = min(first, k[e]);
+        last = max(last, k[e]);
+        ++held;
+      }
+      ties = __all_sync(kFull, held == 0u || first == last);
+    }
+    first = __reduce_min_sync(kFull, first);
+    last = __reduce_max_sync(kFull, last);
+    held = __reduce_add_sync(kFull, held);
+    if (ties && (held == 0u || first == last)) {
+      if (lane == 0 && held != 0u) {
+        const unsigned int bin = (first >> sh) & 1023u;
+        atomicAdd(&sc.lv.cnt[bin], held);
+        atomicAdd(&sc.lv.sum[bin], held * (first & ((1u << sh) - 1u)));
+      }
+    } else {
+      for (int i4 = tid; i4 < n4_pad; i4 += NT) {
+        const uint4 k4 = *reinterpret_cast<const uint4*>(a + 4 * i4);
+        const unsigned int k[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) level_add(sc.lv, (k[e] >> shift) == prefix && k[e] != 0u, k[e], sh);
+      }
     }
     __syncthreads();
     level_groups<NT>(sc.lv, prefix, sh);
