@@ -812,10 +812,12 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
   const bool agg = !two_launch && !one_row;  // the CTAs sum the rows (or the chunks) themselves
   // One CTA per row (stream_rows.cuh), where a cluster per row would need more than one wave of CTAs, or where
   // there is about a row for every SM and a cluster's exchanges gain nothing (100 rows of 8192: 11.6 us against
-  // 13.5; of 32768: 18.9 against 22.8; of 131072: 55 against 95; 64 rows of 32768: 18.7 against 17.4).
+  // 13.5; of 32768: 18.9 against 22.8; of 131072: 55 against 95; 64 rows of 32768: 18.7 against 17.4).  Up to 64
+  // rows too long for one wave of clusters leave most SMs without a row, and a second wave of clusters costs less
+  // (131072 entries, clusters / one CTA a row: 40 rows 34 / 47 us, 64 rows 41 / 47, 68 rows 51 / 47).
   const long long row_ctas = agg ? 0 : n_lists * specattn::pick_cluster_row(A.L_stride, n_lists);
   const bool stream = !agg && !variant && A.L_stride <= specattn::kStreamMax && A.L_stride > 4096 &&
-                      (row_ctas > 296 || (n_lists > 72 && n_lists <= 148));
+                      ((row_ctas > 296 && n_lists > 64) || (n_lists > 72 && n_lists <= 148));
   const bool small = !agg && !variant && A.L_stride <= 2048;
   const int cs = stream ? 1 : agg ? specattn::pick_cluster(A.L_stride, n_lists) : specattn::pick_cluster_row(A.L_stride, n_lists);
   const int slice = specattn::slice_of(static_cast<int>(A.L_stride), cs, (P.chunk > 4) ? P.chunk : 4);

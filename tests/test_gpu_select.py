@@ -534,3 +534,30 @@ def test_queries_searched_apart_at_chunk_granularity(chunk, gamma, Ls, lens):
         oi, oc, os_, od = oracle.select_variant([a], [0], kv, 0.9, per_step=True, n_iters=iters, chunk=chunk)
         assert _compare_variant(gi, gc, gs, oi, oc, os_, od) == len(lens)
         assert gs[0, 0, 0].item() == (sa.ROW_INVALID_PROB if a is bad else 0)
+
+
+@pytest.mark.parametrize("n_rows", [64, 65])
+@pytest.mark.parametrize("mixed", [0, 1, 40])
+def test_ties_fill_a_bin_of_long_rows(n_rows, mixed, form):
+    """Either side of the line between a second wave of clusters and one CTA per row.  One value fills a bin beyond
+    what is gathered, alone or with `mixed` neighbours one unit in the last place above it: warps that hold one
+    value of the bin beside warps that hold two, thresholds at the tie and at its neighbour."""
+    if form == "cluster":
+        pytest.skip("single-row lists take the same path with and without a workspace")
+    import paper_2510_27641_b200 as sa
+    n = 66004
+    rng = np.random.default_rng(mixed)
+    rows = np.full((n_rows, n), np.float32(0.0078125))
+    rows[:, rng.choice(n, size=n // 2, replace=False)] = np.float32(0.001953125)
+    rows[:, rng.choice(n, size=mixed, replace=False)] = np.nextafter(np.float32(0.0078125), np.float32(1))
+    rows[1, 7:] = 0.0
+    kv = np.full(n_rows, n, np.int32)
+    kv[2] = 4099
+    sample = [0, 1, 2, n_rows - 1]
+    for p in (1e-4, 0.5, 0.9):
+        gi, gc, gs, gd = sa.select_topp([to_dev(rows.reshape(n_rows, 1, 1, n))], to_dev(kv), [0], p, want_diag=True)
+        torch.cuda.synchronize()
+        oi, oc, os_, od = oracle.select_topp([rows[sample].reshape(4, 1, 1, n)], np.zeros(1, np.int32), kv[sample], p)
+        st = compare_lists(lambda i: rows[sample][i, :kv[sample][i]], p, gi.cpu().numpy()[:, sample], gc.cpu().numpy()[:, sample],
+                           gs.cpu().numpy()[:, sample], oi, oc, os_, od)
+        assert st["n"] == 4
