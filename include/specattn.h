@@ -58,7 +58,7 @@ extern "C" {
 #define SPECATTN_MAX_DRAFT_LAYERS 64
 #define SPECATTN_MAX_DRAFT_HEADS 256
 #define SPECATTN_MAX_ROWS_PER_LIST 1024  /* contributing (head, query) rows per list */
-#define SPECATTN_MAX_KV_LEN 196608       /* positions per sequence for select (8 x 24576) */
+#define SPECATTN_MAX_KV_LEN 196608       /* positions per sequence for select         */
 #define SPECATTN_MAX_VERIFY_UNITS 2048   /* batch * n_kv_heads for verify */
 #define SPECATTN_MAX_QUERY_ROWS 64       /* n_q * (n_q_heads / n_kv_heads) for verify */
 
@@ -111,7 +111,7 @@ extern "C" {
  *
  * workspace (optional, device, 16-byte aligned, specattn_select_workspace_bytes() bytes; no
  * counterpart in the paper): without it each list is aggregated and searched inside the shared
- * memory of one thread-block cluster (at most 8 CTAs per list, one launch).  With it, and for
+ * memory of one thread-block cluster (at most 16 CTAs per list, one launch).  With it, and for
  * the default selection (no variant) over rows of >= 2048 positions when the lists are so few
  * that one cluster each would leave SMs idle (lists x CTAs per cluster < 148), the call runs two
  * launches: every list's rows are summed by CTAs of 512 positions each -- in the same order,
