@@ -1399,10 +1399,30 @@ const void* verify_kernel_of(int m_tiles, size_t* smem, int* threads) {
   }
 }
 
+int m_tiles(const specattn_verify_args& A) {
+  const int grp = A.n_q_heads / A.n_kv_heads;
+  return (A.n_q * grp + 15) / 16;
+}
+
+// Whether the host can tell that lists may be too long for clusters of cs: by idx_stride, where that is a bound of
+// its own (well below the cache's room) and not the room itself.  (Dense calls count as lists of the room, with
+// which they share every bit of their results.)
+// Clusters of four and eight leave up to a tenth of the SMs without one.  Short lists gain more from the merge
+// inside a cluster; long ones, of the kernels that the consumers bound (33 to 64 query rows), lose (us, clusters /
+// pairs): clusters of eight, 1 x 8 units of 4000 tokens 16.6 / 22.0, of 8000 27.0 / 27.3, of 13000 40.3 / 32.9;
+// 2 x 8 units of 4000 22.2 / 22.9, of 8000 32.9 / 32.0; clusters of four, 4 x 8 units of 8000 49.9 / 52.8,
+// of 13000 78.2 / 76.3, of 30000 173 / 159.
+bool long_lists(const specattn_verify_args& A, int cs) {
+  const long long line = (cs > 4) ? 6144 : 12288;
+  const long long room = A.block_table_stride * A.page_size;  // (pages per sequence also without a block table)
+  return !A.dense && A.idx_stride > line && 2 * A.idx_stride <= room;
+}
+
 // Grid and cluster size of a launch: whole clusters, as many as run at once (GPCs do not hold a multiple of
 // every cluster size).  Opts the kernel in to its shared memory and asks the runtime once per device,
 // kernel and cluster size.  false: the runtime refused.
-bool verify_grid(int m_tiles, long long units, int n_sm, int* n_ctas, int* cluster) {
+bool verify_grid(const specattn_verify_args& A, int n_sm, int* n_ctas, int* cluster) {
+  const int mt = m_tiles(A);
   static std::atomic<int> known[64][4][kMaxCluster + 1];  // clusters that fit + 1, 0 = not asked yet
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
@@ -1411,10 +1431,12 @@ bool verify_grid(int m_tiles, long long units, int n_sm, int* n_ctas, int* clust
   }
   size_t smem;
   int threads;
-  const void* fn = verify_kernel_of(m_tiles, &smem, &threads);
+  const void* fn = verify_kernel_of(mt, &smem, &threads);
+  const long long units = static_cast<long long>(A.batch) * A.n_kv_heads;
   int cs = want_cluster(units, n_sm);
+  if (cs > 2 && mt > 2 && long_lists(A, cs)) cs = 2;
   for (;;) {
-    std::atomic<int>& slot = known[dev][m_tiles - 1][cs];
+    std::atomic<int>& slot = known[dev][mt - 1][cs];
     int n = slot.load(std::memory_order_acquire);
     if (n == 0) {
       if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) {
@@ -1484,11 +1506,6 @@ cudaError_t launch_verify(const VerifyParams& P, int m_tiles, int n_ctas, cudaSt
 }
 
 #include "sparse_verify_tc.cuh"
-
-int m_tiles(const specattn_verify_args& A) {
-  const int grp = A.n_q_heads / A.n_kv_heads;
-  return (A.n_q * grp + 15) / 16;
-}
 
 int validate(const specattn_verify_args* args) {
   if (args == nullptr) return SPECATTN_ERR_NULL;
@@ -1725,7 +1742,7 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
     }
   } else {
     int grid = 0;
-    if (!specattn::verify_grid(specattn::m_tiles(A), static_cast<long long>(A.batch) * A.n_kv_heads, n_ctas, &grid, &P.cluster))
+    if (!specattn::verify_grid(A, n_ctas, &grid, &P.cluster))
       return SPECATTN_ERR_CUDA;
     err = specattn::launch_verify(P, specattn::m_tiles(A), grid, stream);
   }
@@ -1756,7 +1773,7 @@ extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan
   if (A.batch == 0) return SPECATTN_OK;
   VerifyParams P = specattn::make_params(A);
   int grid = 0;
-  if (!specattn::verify_grid(specattn::m_tiles(A), static_cast<long long>(A.batch) * A.n_kv_heads, n_ctas, &grid, &P.cluster))
+  if (!specattn::verify_grid(A, n_ctas, &grid, &P.cluster))
     return SPECATTN_ERR_CUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
@@ -1801,8 +1818,7 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
       if (args[i]->batch == 0) continue;
       B.p[m] = specattn::make_params(*args[i]);
       B.plan[m] = static_cast<int*>(plans[i]);
-      if (!specattn::verify_grid(specattn::m_tiles(*args[i]), static_cast<long long>(args[i]->batch) * args[i]->n_kv_heads,
-                                 n_ctas, &B.grid[m], &B.p[m].cluster))
+      if (!specattn::verify_grid(*args[i], n_ctas, &B.grid[m], &B.p[m].cluster))
         return SPECATTN_ERR_CUDA;
       ++m;
     }

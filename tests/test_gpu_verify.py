@@ -526,3 +526,31 @@ def test_a_call_that_clears_its_own_workspace_and_status(kept):
         torch.cuda.synchronize()
         assert torch.equal(o, out) and torch.equal(l, lse)
         assert st.tolist() == ([0, 0, 0] if init_status else [1, 1, 1])
+
+
+@pytest.mark.parametrize("stride,lens,counts", [
+    (6145, 12300, [6145]),          # long by idx_stride: pairs
+    (6144, 12300, [6144]),          # the line
+    (6000, 8000, [6000, 300]),      # one unit far above the average: parts anywhere
+])
+def test_long_and_skewed_lists_of_33_and_more_query_rows(stride, lens, counts):
+    """Either side of the line between larger clusters and pairs, and a small batch whose longest list a cluster
+    cannot cut finely enough; with and without a precomputed partition."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    case = _make_case(97, len(counts), 5, 32, 4, 16, [lens] * len(counts), counts=[[c] for c in counts])
+    case["idx"] = case["idx"][:, :, :stride].copy()
+    out, lse, status = _run(case)
+    assert int(status.abs().sum()) == 0
+    check_attention(out, lse, *_oracle(case))
+    o, l, st = torch.empty_like(out), torch.empty_like(lse), torch.zeros_like(status)
+    keep = [bf16_to_dev(case["q"]), case["kv"].to(dev()), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]),
+            to_dev(case["cnt"])]
+    a = sa.make_verify_args(keep[0], keep[1], keep[2], block_table=keep[3], idx=keep[4], counts=keep[5], out=o, lse=l,
+                            status=st, flags=_ENGINE["flags"])
+    ws, plan = sa.verify_workspace(a), sa.verify_plan_buffer(a)
+    a.workspace, a.workspace_bytes, a.plan = ws.data_ptr(), ws.numel(), plan.data_ptr()
+    sa.verify_plan(a, plan)
+    assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(o, out) and torch.equal(l, lse)
