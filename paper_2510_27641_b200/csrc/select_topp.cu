@@ -808,7 +808,9 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
   P.bisect_iters = A.bisect_iters;
   P.chunk = (A.chunk > 1) ? A.chunk : 1;
   const bool variant = P.per_step || P.bisect_iters > 0 || P.chunk > 1;
-  const bool one_row = static_cast<long long>(A.n_draft_heads) * A.gamma == 1 && P.chunk == 1;
+  // the row is searched where it lies only if it is every group's: a group that the head does not feed has a row of
+  // zeros
+  const bool one_row = static_cast<long long>(A.n_draft_heads) * A.gamma == 1 && P.chunk == 1 && (!P.has_groups || A.n_groups == 1);
   const bool agg = !two_launch && !one_row;  // the CTAs sum the rows (or the chunks) themselves
   // One CTA per row (stream_rows.cuh), where a cluster per row would need more than one wave of CTAs, or where
   // there is about a row for every SM and a cluster's exchanges gain nothing (100 rows of 8192: 11.6 us against

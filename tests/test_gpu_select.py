@@ -561,3 +561,20 @@ def test_ties_fill_a_bin_of_long_rows(n_rows, mixed, form):
         st = compare_lists(lambda i: rows[sample][i, :kv[sample][i]], p, gi.cpu().numpy()[:, sample], gc.cpu().numpy()[:, sample],
                            gs.cpu().numpy()[:, sample], oi, oc, os_, od)
         assert st["n"] == 4
+
+
+@pytest.mark.parametrize("n", [1000, 4096, 20000])
+def test_a_single_head_that_feeds_one_of_two_groups(n):
+    """One head, one query: the group that the head does not feed has a row of zeros and keeps every position."""
+    import paper_2510_27641_b200 as sa
+    rows = wl.topp_rows("zipf", 2, n, seed=8).reshape(2, 1, 1, n)
+    kv = np.array([n, n - 7], np.int32)
+    for fed in (0, 1):
+        gi, gc, gs, gd = sa.select_topp([to_dev(rows)], to_dev(kv), [0], 0.9, n_groups=2, head_group=[fed])
+        oi, oc, os_, od = oracle.select_topp([rows], np.zeros(1, np.int32), kv, 0.9, n_groups=2,
+                                             head_group=np.array([fed], np.int32))
+        assert oc[0, :, 1 - fed].tolist() == kv.tolist()
+        zero = np.zeros(n, np.float32)
+        st = compare_lists(lambda i: rows[i // 2, 0, 0, :kv[i // 2]] if i % 2 == fed else zero[:kv[i // 2]], 0.9,
+                           gi.cpu().numpy(), gc.cpu().numpy(), gs.cpu().numpy(), oi, oc, os_, od)
+        assert st["n"] == st["exact"] == 4
