@@ -838,11 +838,12 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
                       (agg ? specattn::kRingBytes : specattn::kScratchBytes) +
                       // the union's bit mask: one bit per entry of the slice
                       (P.per_step ? static_cast<size_t>(specattn::slice_room(slice, nt) / 8) : 0) + apart_bytes;
-  const void* const kernels[6] = {
+  const void* const kernels[7] = {
       (const void*)specattn::select_topp_kernel<false, false, 128>, (const void*)specattn::select_topp_kernel<false, false, 512>,
       (const void*)specattn::select_topp_kernel<false, true, 512>, (const void*)specattn::select_topp_kernel<true, false, 256>,
-      (const void*)specattn::select_topp_kernel<true, true, 256>, (const void*)specattn::stream_rows_kernel};
-  const int kidx = stream ? 5 : agg ? (variant ? 4 : 3) : (variant ? 2 : (small ? 0 : 1));
+      (const void*)specattn::select_topp_kernel<true, true, 256>, (const void*)specattn::stream_rows_kernel<false>,
+      (const void*)specattn::stream_rows_kernel<true>};
+  const int kidx = stream ? (A.diag != nullptr ? 6 : 5) : agg ? (variant ? 4 : 3) : (variant ? 2 : (small ? 0 : 1));
   // Opt in to large dynamic shared memory and clusters of 16 once per device, so that later calls
   // issue nothing but the launch.
   int dev = 0;
@@ -894,7 +895,7 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
   // more).  The limits are asked of the runtime once per kernel and cluster size and cached.
   {
     static const size_t pads[3] = {120 * 1024, 100 * 1024, 70 * 1024};
-    static std::atomic<int> fit[64][6][5][3];  // [device][kernel][log2 cs][pad]: clusters + 1, 0 = unknown
+    static std::atomic<int> fit[64][7][5][3];  // [device][kernel][log2 cs][pad]: clusters + 1, 0 = unknown
     int lcs = 0;
     while ((1 << lcs) < cs) ++lcs;
     for (int k = 0; k < 3 && !stream; ++k) {

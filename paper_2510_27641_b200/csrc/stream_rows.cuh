@@ -11,11 +11,16 @@
 // as little per entry as it can:
 //   pass 1  adds the top 15 mantissa bits to one word per bin (exponent and five mantissa bits) -- one atomic, not
 //           two words for an exact sum -- which names the threshold's bin in all but a few of 10^4 rows.  The
-//           other nine bits, times 2^e, are added up by the thread, sixteen in binary32 (exact as a rule) and
-//           their sums in binary64.  What bounds the pass is the atomic: 4.1 wavefronts of random banks, two cycles each;
+//           other nine bits, times 2^e, are added up by the thread.  What bounds the pass is the atomic: 4.1
+//           wavefronts of random banks, two cycles each;
 //   pass 2  notes two bits per entry, above the bin / in the bin, in per-thread words (no votes) and adds up
 //           the low bits of what lies above.  The keys of the bin are then fetched by their bits.
-// The masses tell exactly whether the bin was the right one; if not, the row is read again for its neighbour.
+// The masses tell whether the bin was the right one; if not, the row is read again for its neighbour.  They are floating
+// point sums whose rounding depends on how the row was dealt to threads, so a threshold counts only if the target
+// is further from both of its masses than rounding can reach (kStreamDoubt); else -- rows whose masses meet the
+// target exactly, rows of tiny values -- the row is searched once more with the low bits added up
+// per octave too (a second atomic), in the same integers and with the same comparisons as the search in shared memory.
+// The lists are therefore the same in every form.
 // 256 rows of 131072, p = 0.9, uniform / Zipf / ties: 96 / 81 / 93 us; with exact two-word bins, votes and 128-entry
 // emission 117 / 102 / 142.
 #pragma once
@@ -30,7 +35,12 @@ constexpr int kStreamShift = 18;                   // level-1 bins: the key's bi
 constexpr int kStreamBins = 8192;
 constexpr int kStreamCand = 4096;                  // keys of the bin that are gathered
 constexpr int kStreamWords = kStreamMax / 32;      // words of a bit per entry: [8 rounds][thread], 4 bits a round
-constexpr int kStreamStore = kStreamBins + kOctaves;
+constexpr int kStreamLow = kStreamBins + kOctaves;  // (exact search) sums of the low nine bits per octave, behind the bins
+constexpr int kStreamStore = kStreamLow + kOctaves;
+// Two ways to add up the target, or a mass it is compared with, differ by less than this share of the total.  In
+// binary64 a thread adds up to 256 values and the CTA 512 such sums (2^-44 if every one rounded the same way); sixteen
+// low parts in binary32 are off by at most 15 x 2^-25 of their sum, which is at most 2^-14 of the values'.
+constexpr double kStreamDoubt = 0x1p-40, kStreamDoubt32 = 0x1p-34;
 static_assert(2 * kStreamWords <= kStreamStore, "both bit masks take the histogram's bytes");
 static_assert(static_cast<long long>(kStreamMax) << 15 <= (1ll << 32), "a bin's word cannot wrap");
 
@@ -38,6 +48,7 @@ struct StreamShared {
   alignas(16) unsigned int store[kStreamStore];  // histogram, then the bits "above the bin" and "in the bin"
   alignas(16) float ring[kStreamGroups * kStreamBatch * kStreamRound];
   int negative;                // a negative input was met
+  int tiny;                    // (exact search) a key below 512, of which the histogram's word of bin 0 holds nothing
   int oct_min, oct_max, n_cand;
   Found fd;
   double sum[kStreamWarps];
@@ -72,10 +83,15 @@ __device__ __forceinline__ StreamConst stream_const() {
   asm volatile("mov.u32 %0, 16384;\n\tmov.u32 %1, 512;\n\tmov.u32 %2, 4;" : "=r"(c.by18), "=r"(c.by23), "=r"(c.four));
   return c;
 }
-__device__ __forceinline__ void stream_bump(uint32_t hist, const StreamConst& c, unsigned int key) {
+__device__ __forceinline__ void stream_bump(uint32_t hist, const StreamConst& c, unsigned int key, unsigned int piece) {
   const unsigned int bin = __umulhi(key, c.by18), oct = __umulhi(key, c.by23);
   const uint32_t at = bin * c.four + (oct * c.four + hist);
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(((key >> 9) & 0x3fffu) | 0x4000u) : "memory");
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(piece) : "memory");
+}
+// The top 15 mantissa bits of a key.  (Unless the search is exact, a denormal counts as if it were normal.)
+template <bool kExact>
+__device__ __forceinline__ unsigned int stream_piece(unsigned int key) {
+  return ((key >> 9) & 0x3fffu) | ((!kExact || key >= 0x800000u) ? 0x4000u : 0u);
 }
 
 // Walks the row through the ring: f(round, bit patterns) for every batch of rounds, this thread's float4 of each,
@@ -133,6 +149,10 @@ __device__ __forceinline__ double stream_sum(StreamShared& sh, double s) {
   return s;
 }
 
+// kMasses: the caller wants the masses (diag), so they are added up in binary64.  Otherwise they only have to tell
+// which threshold is the right one, and the low parts of a batch are added up in binary32 first, the rare row in doubt
+// being searched again (256 rows of 131072, uniform / Zipf / ties: 107 / 96 / 102 us with masses, 103 / 90 / 97 without).
+template <bool kMasses>
 __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __grid_constant__ SelectParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamShared& sh = *reinterpret_cast<StreamShared*>(smem_raw);
@@ -151,6 +171,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     for (int i = tid; i < kStreamStore / 4; i += kStreamThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
       sh.negative = 0;
+      sh.tiny = 0;
       sh.oct_min = kOctaves;
       sh.oct_max = -1;
     }
@@ -171,67 +192,89 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   unsigned int theta = 0u;
   unsigned int* const above_bits = sh.store;
   unsigned int* const in_bits = sh.store + kStreamWords;
-  bool exact_sums = false;     // a row so small that every value is added up in binary64
+  bool exact = false, last_resort = false;
   auto bin_mass9 = [&](int oct) {  // lane: bin of an octave
     return static_cast<double>(static_cast<unsigned long long>(hist[stream_word(32 * oct + lane)]) << 9) * pow2_double(max(oct, 1) - 150);
   };
   int go = 0;                  // 1 / -1: the bin above / below the last one tried is wanted
+  auto turn = [&](int want) {  // on to the bin above or below -- or, after a turn back, to an exact search
+    if (go == -want) exact = true;
+    go = (go == -want) ? 0 : want;
+    clear();
+  };
   for (;;) {
     // ---- pass 1: histogram, total and validity -------------------------------------------------------
-    // (bin 0, zeros apart: eighteen octaves of denormals whose updates of one word would be serialised; they
-    // only count in a row without larger values)
-    const unsigned int min_key = exact_sums ? 1u : 1u << kStreamShift;
-    bool negative = false;
-    double mine = 0.0;
-    stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
-      unsigned int any = 0u;
+    // (unless the search is exact, bin 0 is left out, zeros apart eighteen octaves of denormals whose updates of one
+    // word would be serialised; they only count in a row without larger values)
+    bool negative = false, tiny = false;
+    double mine[4] = {0.0, 0.0, 0.0, 0.0};  // (one sum waits for its adds)
+    auto pass1 = [&](auto exactly) {
+      constexpr bool kExact = decltype(exactly)::value;
+      constexpr unsigned int min_key = kExact ? 1u : 1u << kStreamShift;
+      stream_pass(sh, A, L, [&](int, unsigned int (&k)[N]) {
+        unsigned int any = 0u;
 #pragma unroll
-      for (int j = 0; j < N; ++j) any |= k[j];
-      if (static_cast<int>(any) < 0) {  // a sign bit: negative -- or -0.0, which is a zero
+        for (int j = 0; j < N; ++j) any |= k[j];
+        if (static_cast<int>(any) < 0) {  // a sign bit: negative -- or -0.0, which is a zero
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-          negative |= k[j] > 0x80000000u;
-          k[j] = (static_cast<int>(k[j]) < 0) ? 0u : k[j];
+          for (int j = 0; j < N; ++j) {
+            negative |= k[j] > 0x80000000u;
+            k[j] = (static_cast<int>(k[j]) < 0) ? 0u : k[j];
+          }
         }
-      }
-      // every value of the warp in one bin (ties, constant rows): the warp reduces first
-      const unsigned int bin0 = __shfl_sync(kFull, k[0] >> kStreamShift, 0);
-      bool one = false;
-      if (__all_sync(kFull, (k[0] >> kStreamShift) == bin0)) {
-        unsigned int differ = 0u;
+        // every value of the warp in one bin (ties, constant rows): the warp reduces first
+        const unsigned int bin0 = __shfl_sync(kFull, k[0] >> kStreamShift, 0);
+        bool one = false;
+        if (__all_sync(kFull, (k[0] >> kStreamShift) == bin0)) {
+          unsigned int differ = 0u;
 #pragma unroll
-        for (int j = 1; j < N; ++j) differ |= k[j] ^ k[0];
-        one = __all_sync(kFull, (differ >> kStreamShift) == 0u);
-      }
-      if (one) {
-        unsigned int s = 0u;
+          for (int j = 1; j < N; ++j) differ |= k[j] ^ k[0];
+          one = __all_sync(kFull, (differ >> kStreamShift) == 0u);
+        }
+        if (one) {
+          unsigned int s = 0u, low = 0u;
 #pragma unroll
-        for (int j = 0; j < N; ++j) s += (k[j] >= min_key) ? ((k[j] >> 9) & 0x3fffu) | 0x4000u : 0u;
-        s = __reduce_add_sync(kFull, s);
-        if (lane == 0 && s != 0u) atomicAdd(&hist[stream_word(bin0 & (kStreamBins - 1))], s);
-      } else {
+          for (int j = 0; j < N; ++j) {
+            s += (k[j] >= min_key) ? stream_piece<kExact>(k[j]) : 0u;
+            tiny |= kExact && k[j] - 1u < 0x1ffu;
+            low += k[j] & 0x1ffu;
+          }
+          s = __reduce_add_sync(kFull, s);
+          if (lane == 0 && s != 0u) atomicAdd(&hist[stream_word(bin0 & (kStreamBins - 1))], s);
+          if (kExact) {
+            low = __reduce_add_sync(kFull, low);
+            if (lane == 0 && low != 0u) atomicAdd(&hist[kStreamLow + ((bin0 >> 5) & (kOctaves - 1))], low);
+          }
+        } else {
 #pragma unroll
-        for (int j = 0; j < N; ++j)
-          if (k[j] >= min_key) stream_bump(hist_at, consts, k[j]);
-      }
-      float rest = 0.f;  // (sixteen 9-bit pieces: exact while their exponents lie within 2^12)
+          for (int j = 0; j < N; ++j) {
+            if (k[j] >= min_key) stream_bump(hist_at, consts, k[j], stream_piece<kExact>(k[j]));
+            tiny |= kExact && k[j] - 1u < 0x1ffu;
+            if (kExact && (k[j] & 0x1ffu) != 0u) atomicAdd(&hist[kStreamLow + (k[j] >> 23)], k[j] & 0x1ffu);
+          }
+        }
+        if (!kExact && kMasses) {
 #pragma unroll
-      for (int j = 0; j < N; ++j) rest += stream_rest(k[j]);
-      if (!exact_sums) {
-        mine += static_cast<double>(rest);
-      } else {
+          for (int j = 0; j < N; ++j) mine[j & 3] += static_cast<double>(stream_rest(k[j]));
+        } else if (!kExact) {
+          float part = 0.f;
 #pragma unroll
-        for (int j = 0; j < N; ++j) mine += static_cast<double>(__uint_as_float(k[j]));
-      }
-    });
+          for (int j = 0; j < N; ++j) part += stream_rest(k[j]);
+          mine[0] += static_cast<double>(part);
+        }
+      });
+    };
+    if (exact) pass1(std::true_type()); else pass1(std::false_type());
     if (__any_sync(kFull, negative) && lane == 0) sh.negative = 1;
+    if (__any_sync(kFull, tiny) && lane == 0) sh.tiny = 1;
 
     // ---- the bin of the threshold ---------------------------------------------------------------------
-    const double rest = stream_sum(sh, mine);
+    const double rest = stream_sum(sh, (mine[0] + mine[1]) + (mine[2] + mine[3]));
     if (tid < kOctaves) {
       unsigned long long s = 0ull;
 #pragma unroll 8
       for (int h = 0; h < 32; ++h) s += hist[33 * tid + h];
+      s = (s << 9) + hist[kStreamLow + tid];  // (the low parts: zero unless the search is exact)
       sc.oct[tid] = s;
       const int first = __reduce_min_sync(kFull, (s != 0ull) ? tid : kOctaves);
       const int final = __reduce_max_sync(kFull, (s != 0ull) ? tid : -1);
@@ -245,8 +288,9 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     if (warp == 0) {
       double t = 0.0, tg = 0.0, carry = 0.0, ab = 0.0, up;
       int bin = -1;
+      last_resort = false;
       if (sh.oct_max >= 0 && !invalid) {
-        const int oct = find_octave(sh.oct_max, sh.oct_min, P.p, [&](int e) { return sc.oct[e] << 9; }, t, tg, carry);
+        const int oct = find_octave(sh.oct_max, sh.oct_min, P.p, [&](int e) { return sc.oct[e]; }, t, tg, carry);
         bin = 32 * oct + find_from_top<5>(bin_mass9(oct), 0.0, carry, tg, ab, up);
         if (go != 0) {  // the next one with an entry, or none
           int at = sh.fd.bin;
@@ -254,7 +298,8 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
           for (;;) {
             at = (go > 0) ? at + 1 : at - 1;
             const int mine_at = (go > 0) ? at + lane : at - lane;
-            const unsigned some = __ballot_sync(kFull, mine_at >= 0 && mine_at < kStreamBins && hist[stream_word(mine_at & (kStreamBins - 1))] != 0u);
+            const unsigned some = __ballot_sync(kFull, mine_at >= 0 && mine_at < kStreamBins &&
+                                                           (hist[stream_word(mine_at & (kStreamBins - 1))] != 0u || (mine_at == 0 && sh.tiny != 0)));
             if (some != 0u) {
               bin = (go > 0) ? at + __ffs(some) - 1 : at - (__ffs(some) - 1);
               break;
@@ -262,10 +307,15 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
             at = (go > 0) ? at + 31 : at - 31;
             if (at < 0 || at >= kStreamBins) break;
           }
-          // its mass above, octave by octave from the top
-          carry = ab = 0.0;
+          // (the octave of an exact search is the right one: no bin of it reaches the target only through rounding
+          // between two summation orders, and the last one tried, the lowest, is kept whole)
+          last_resort = exact && (bin < 0 || (bin >> 5) != oct);
+          if (last_resort) bin = sh.fd.bin;
           if (bin >= 0) {
-            for (int e = sh.oct_max; e > (bin >> 5); --e) carry += static_cast<double>(sc.oct[e] << 9) * pow2_double(max(e, 1) - 150);
+            if (!exact) {  // its mass above, octave by octave from the top
+              carry = 0.0;
+              for (int e = sh.oct_max; e > (bin >> 5); --e) carry += static_cast<double>(sc.oct[e]) * pow2_double(max(e, 1) - 150);
+            }
             ab = suffix_sum<5>((lane > (bin & 31)) ? bin_mass9(bin >> 5) : 0.0);
             ab = __shfl_sync(kFull, ab, 0);
           }
@@ -273,35 +323,42 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       }
       if (lane == 0) {
         sh.fd.total = t;
-        sh.fd.key = (bin < 0) ? 0xffffffffu : 0u;  // (no such bin)
+        sh.fd.key = last_resort ? 1u : 0u;
+        sh.fd.bin = bin;
         if (bin >= 0) {
-          sh.fd.bin = bin;
-          sh.fd.carry = carry + ab;
+          sh.fd.carry = exact ? carry : 0.0;
+          sh.fd.above = exact ? ab : carry + ab;
           // the bin's smallest term bounds the number of its keys
-          sh.fd.count = hist[stream_word(bin)] / (0x4000u | (static_cast<unsigned int>(bin & 31) << 9));
+          const unsigned int least = (static_cast<unsigned int>(bin & 31) << 9) | ((bin >= 32) ? 0x4000u : 0u);
+          sh.fd.count = (least == 0u) ? 0x7fffffffu : hist[stream_word(bin)] / least;
         }
       }
     }
     __syncthreads();
-    total = exact_sums ? rest : sh.fd.total + rest;
-    if (!invalid && !exact_sums && !(total >= 0x1p-40)) {
+    total = sh.fd.total + rest;
+    if (!invalid && !exact && (!(total >= 0x1p-40) || (go != 0 && sh.fd.bin < 0))) {
       // (the histogram takes a denormal for a number of at least 2^-126, which only counts in a total as small
-      // as this: once more, with every value added up)
-      exact_sums = true;
+      // as this; or there is no neighbour where the masses asked for one)
+      exact = true;
+      go = 0;
+      __syncthreads();
       clear();
       continue;
     }
     if (invalid) total = 0.0;
     target = static_cast<double>(P.p) * total;
+    m_gt = 0.0;
     m_ge = total;
     searching = !invalid && target > 0.0 && !P.keep_all;  // else p >= 1 or an all-zero row: keep all
     if (!searching) break;
-    const bool last_resort = sh.fd.key == 0xffffffffu;   // keep the bin tried before
+    last_resort = sh.fd.key != 0u;
     unsigned int prefix = static_cast<unsigned int>(sh.fd.bin);
     const double scale = pow2_double(max(sh.fd.bin >> 5, 1) - 150);
-    unsigned int M = last_resort ? 0x7fffffffu : sh.fd.count;
+    unsigned int M = sh.fd.count;
     int shift = kStreamShift;
-    const double above_hist = sh.fd.carry;
+    // An exact search has the mass of the octaves above apart (`carry`) and exact integer masses inside its octave.
+    const double carry = sh.fd.carry, above_hist = sh.fd.above;
+    const int hi_key = exact ? static_cast<int>((prefix >> 5 << 23) | 0x7fffffu) : INT_MAX;
     int want = 0;
     __syncthreads();
     // ---- a well filled bin: 10 (then the last 8) more bits, one pass over the row each -----------------------
@@ -317,7 +374,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
 #pragma unroll
         for (int j = 0; j < N; ++j) {
           level_add(lv, (k[j] >> shift) == prefix && k[j] != 0u, k[j], sl, bits);
-          if (static_cast<int>(k[j]) > top) s += static_cast<double>(__uint_as_float(k[j]));
+          if (static_cast<int>(k[j]) > top && static_cast<int>(k[j]) <= hi_key) s += static_cast<double>(__uint_as_float(k[j]));
         }
       });
       level_groups<kStreamThreads>(lv, prefix, sl, bits);
@@ -325,55 +382,72 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       if (warp == 0) {
         double above, upto, above1, upto1;
         const double all = static_cast<double>(lv.grp[lane]) * scale;
-        const int gi = find_from_top<5>(all, 0.0, s, target, above, upto);
+        const int gi = find_from_top<5>(all, s, carry, target, above, upto);
         const int bin = gi * 32 + lane;
         const unsigned int c = lv.cnt[bin];
-        const int b1 = find_from_top<5>(static_cast<double>(level_mass(prefix, bin, sl, c, lv.sum[bin], bits)) * scale, above, s,
+        const int b1 = find_from_top<5>(static_cast<double>(level_mass(prefix, bin, sl, c, lv.sum[bin], bits)) * scale, above, carry,
                                         target, above1, upto1);
         const unsigned int cb = __shfl_sync(kFull, c, b1);
         if (lane == 0) {
           sh.fd.oct = gi * 32 + b1;
           sh.fd.count = cb;
-          sh.fd.upto = s + upto1;
+          sh.fd.upto = upto1;
         }
       }
       __syncthreads();
       // (only the first level can show that the bin was the wrong one)
-      if (shift == kStreamShift && !last_resort) want = (s >= target) ? 1 : (sh.fd.upto < target) ? -1 : 0;
+      if (shift == kStreamShift && !last_resort) want = (carry + s >= target) ? 1 : (carry + sh.fd.upto < target) ? -1 : 0;
       prefix = (prefix << bits) | static_cast<unsigned int>(sh.fd.oct);
       M = sh.fd.count;
       shift = sl;
       __syncthreads();
-      if (want != 0 && go != -want) break;
-      want = 0;
+      if (want != 0) break;
     }
     if (want != 0) {
-      go = want;
-      clear();
+      turn(want);
       continue;
     }
     // ---- pass 2: what lies above the bin, and in it ---------------------------------------------------
     // (a prefix of all bits is one value: it is the threshold, and counts as the bin)
     const unsigned int lo_key = (prefix != 0u) ? prefix << shift : 1u;
     const unsigned int top_key = (prefix << shift) + ((1u << shift) - 1u), span = top_key - lo_key;
-    double carry = 0.0;
+    // above a whole bin the histogram has the upper part of the sum; above a part of one every value is added up
+    const bool by_hist = shift == kStreamShift;
+    // (masses) The low parts of a batch are added up in binary32, which is exact while their octaves lie within 2^11
+    // (16 x 2^9 x 2^11 units are 2^24); batches with a key further above the bin, few of them, go the long way.
+    const int far_key = exact || ((sh.fd.bin >> 5) + 12) >= kOctaves ? INT_MAX : (((sh.fd.bin >> 5) + 12) << 23) - 1;
+    double inner = 0.0;
     auto pass2 = [&](auto whole) {
       double s = 0.0;
       unsigned int ab = 0u, in = 0u;
       const int last = ((L + kStreamRound - 1) / kStreamRound + kStreamBatch - 1) / kStreamBatch * kStreamBatch - kStreamBatch;
       stream_pass(sh, A, L, [&](int round, unsigned int (&k)[N]) {
         unsigned int a8 = 0u, i8 = 0u;
-        float rest = 0.f;
+        float part = 0.f;
+        bool apart = decltype(whole)::value;
+        if (kMasses && !apart) {
+          int most = 0;
+#pragma unroll
+          for (int j = 0; j < N; ++j) most = max(most, static_cast<int>(k[j]));
+          apart = __any_sync(kFull, most > far_key);
+        }
 #pragma unroll
         for (int j = 0; j < N; ++j) {
           const float r = stream_rest(k[j]);
           if (static_cast<int>(k[j]) > static_cast<int>(top_key)) {
             a8 |= 1u << j;
-            if (decltype(whole)::value) s += static_cast<double>(__uint_as_float(k[j])); else rest += r;
+            if (static_cast<int>(k[j]) <= hi_key) part += r;
           }
           if (k[j] - lo_key <= span) i8 |= 1u << j;
         }
-        if (!decltype(whole)::value) s += static_cast<double>(rest);
+        if (!apart) {
+          s += static_cast<double>(part);
+        } else {
+#pragma unroll
+          for (int j = 0; j < N; ++j)
+            if (static_cast<int>(k[j]) > static_cast<int>(top_key) && static_cast<int>(k[j]) <= hi_key)
+              s += static_cast<double>(decltype(whole)::value ? __uint_as_float(k[j]) : stream_rest(k[j]));
+        }
         const int at = 4 * (round & 7);
         ab |= a8 << at;
         in |= i8 << at;
@@ -383,14 +457,11 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
           ab = in = 0u;
         }
       });
-      carry = s;
+      inner = s;
     };
-    // above a whole bin the histogram has the upper part of the sum; above a part of one, or in a row of
-    // denormals, every value is added up
-    const bool by_hist = shift == kStreamShift && !exact_sums;
     if (by_hist) pass2(std::false_type()); else pass2(std::true_type());
     if (tid == 0) sh.n_cand = 0;
-    carry = stream_sum(sh, carry) + (by_hist ? above_hist : 0.0);
+    inner = stream_sum(sh, inner) + (by_hist ? above_hist : 0.0);
     if (shift > 0) level_clear<kStreamThreads>(sc.lv);
     // fetch the keys of the bin by their bits
     const int word_rows = (L + 8 * kStreamRound - 1) / (8 * kStreamRound);
@@ -428,33 +499,36 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       }
       __syncthreads();
     }
-    m_gt = m_ge = carry;
     if (shift > 0 && n == 0) {
       theta = top_key + 1u;
+      m_gt = m_ge = carry + inner;
     } else if (shift > 0) {
       double above, upto;
-      theta = threshold_among<kStreamThreads>(sc.keys, n, prefix, shift, 0.0, carry, target, scale, sc.lv, sh.fd, sc.pk, above, upto);
+      theta = threshold_among<kStreamThreads>(sc.keys, n, prefix, shift, inner, carry, target, scale, sc.lv, sh.fd, sc.pk, above, upto);
       m_gt = carry + above;
       m_ge = carry + upto;
     } else {
       theta = prefix;
-      m_ge = carry + static_cast<double>(sh.n_cand) * static_cast<double>(__uint_as_float(prefix));
+      m_gt = carry + inner;
+      m_ge = carry + (inner + static_cast<double>(sh.n_cand) * static_cast<double>(__uint_as_float(prefix)));
     }
-    // The right bin?  (Once the search has gone one way it does not turn: masses that touch the target are
-    // then equal up to the rounding of their sums.)
+    // the right bin?
     if (shift == kStreamShift && !last_resort) {
-      want = (carry >= target) ? 1 : (m_ge < target) ? -1 : 0;
-      if (want != 0 && go != -want) {
+      want = (carry + inner >= target) ? 1 : (m_ge < target) ? -1 : 0;
+      if (want != 0) {
         __syncthreads();
         if (tid == 0) sh.fd.bin = static_cast<int>(prefix);  // (threshold_among used the field)
-        go = want;
-        clear();
+        turn(want);
         continue;
       }
-      if (want > 0) {  // went down from a bin that fell short: everything above this one
-        theta = top_key + 1u;
-        m_gt = m_ge = carry;
-      }
+    }
+    const double doubt = (kMasses ? kStreamDoubt : kStreamDoubt32) * total;
+    if (!exact && !(m_gt < target - doubt && m_ge > target + doubt)) {
+      __syncthreads();
+      exact = true;
+      go = 0;
+      clear();
+      continue;
     }
     // the bin's entries that make it join the bits
     if (shift > 0) {

@@ -578,3 +578,56 @@ def test_a_single_head_that_feeds_one_of_two_groups(n):
         st = compare_lists(lambda i: rows[i // 2, 0, 0, :kv[i // 2]] if i % 2 == fed else zero[:kv[i // 2]], 0.9,
                            gi.cpu().numpy(), gc.cpu().numpy(), gs.cpu().numpy(), oi, oc, os_, od)
         assert st["n"] == st["exact"] == 4
+
+
+def _rows_that_meet_the_target(n_rows, seed, tiny=False):
+    """Rows of 65535 values: 2^k of the value v 2^-k, k = 0 ... 15, shuffled, so that each of the sixteen levels has
+    the mass v and the target of p = j / 16 is met exactly by the j largest levels.  v has all 24 mantissa
+    bits; tiny: v = 5 2^-134, so that the smallest values are single units of the last denormal place."""
+    rng = np.random.default_rng(seed)
+    level = np.concatenate([np.full(1 << k, k) for k in range(16)])
+    rows = np.zeros((n_rows, 65536), np.float32)
+    for i in range(n_rows):
+        v = 5 * 2.0 ** -134 if tiny else float(np.uint32(1 << 23 | rng.integers(1 << 23) | 1)) * 2.0 ** -24
+        rows[i, :65535] = (v * np.exp2(-rng.permutation(level).astype(np.float64))).astype(np.float32)
+    return rows
+
+
+@pytest.mark.parametrize("n_rows", [64, 100, 300])
+@pytest.mark.parametrize("tiny", [False, True])
+def test_targets_met_exactly_in_every_form(n_rows, tiny, form):
+    """M_>= equal to the target is enough, one unit less is not: no summation order may decide otherwise, whether
+    a row is searched in shared memory or streamed.  (All the sums of these rows are exact in binary64, so the
+    oracle's lists admit no exception.)"""
+    if form == "cluster":
+        pytest.skip("single-row lists take the same path with and without a workspace")
+    rows = _rows_that_meet_the_target(n_rows, n_rows, tiny)
+    rows[1, 7:] = 0.0
+    for j in (1, 5, 8, 15):
+        st, gd, od = _run_rows(rows, 65535, j / 16)
+        assert st["n"] == st["exact"] == n_rows
+        for i in (0, 2, n_rows - 1):
+            assert gd[0, i, 0, 3] == gd[0, i, 0, 1] == od[0, i, 0, 1]
+
+
+def test_many_aggregated_lists_are_the_same_bits_in_every_form():
+    """80 lists in the two-launch form, whose search then streams one CTA a list: the lists of the one-launch form,
+    on draft rows and on rows whose masses meet the target exactly."""
+    import paper_2510_27641_b200 as sa
+    B, Ls = 80, 65536
+    kv = np.full(B, 65535, np.int32)
+    kv[3], kv[4] = 1, 5000
+    exact = np.zeros((B, 2, 1, Ls), np.float32)
+    exact[:, 1, 0] = _rows_that_meet_the_target(B, 7)
+    draft = np.concatenate([wl.draft_probs(31, 0, kv[:8], 2, 1, Ls, sink=6.0, slope=0.0005)] * 10)
+    draft[:, 0, 0] *= np.linspace(0.1, 3.0, B, dtype=np.float32)[:, None]
+    for probs, p in ((exact, 0.5), (exact, 0.9375), (draft, 0.9)):
+        d, res = to_dev(probs), []
+        for ws, f in ((True, sa.SELECT_FORM_TWO_LAUNCH), (False, sa.SELECT_FORM_CLUSTER)):
+            res.append(sa.select_topp.func([d], to_dev(kv), [0], p, want_diag=True, workspace=ws, form=f))
+        torch.cuda.synchronize()
+        (i1, c1, s1, d1), (i0, c0, s0, d0) = res
+        assert torch.equal(c1, c0) and torch.equal(s1, s0) and int(s0.abs().sum()) == 0
+        for b in range(B):
+            assert torch.equal(i1[0, b, 0, :int(c0[0, b, 0])], i0[0, b, 0, :int(c0[0, b, 0])])
+        assert torch.allclose(d1, d0, rtol=1e-14, atol=0)   # a few roundings of binary64 apart
