@@ -307,13 +307,14 @@ int specattn_sparse_verify(const specattn_verify_args* args, void* cuda_stream);
  *
  * Not an operation of the paper: an engineering shortcut of this implementation.  How the kernel
  * deals its (sequence, kv head) lists to the SMs depends only on the list lengths (counts, or
- * kv_len for dense calls), tail_len, the shapes and the GPU -- not on q, the K/V pool or the
- * outputs.  Target layers that share a draft layer's lists therefore share the partition, and a
+ * kv_len for dense calls), tail_len, the shapes (n_q, idx_stride and the room of the block table among
+ * them) and the GPU -- not on q, the K/V pool or the outputs.  Target layers that share a draft layer's lists therefore share the partition, and a
  * verify kernel that finds a matching plan in args->plan skips computing it (a few microseconds
  * of start-up per launch).  `plan` is a device buffer of specattn_verify_plan_bytes(args) bytes,
  * 16-byte aligned, written by a small kernel on the stream (after whatever produces counts /
  * kv_len, e.g. specattn_select_topp) and valid until those change.  A kernel given a plan that
- * does not fit its launch (other batch, heads, tail_len, dense flag or GPU) ignores it.  Only
+ * does not fit its launch (other batch, heads, tail_len, dense flag, GPU, or a shape that is launched
+ * in clusters of another size) ignores it.  Only
  * the mma.sync engine reads plans.
  * Ordering: a plan must be at least as new as the lists it describes -- call this after every
  * specattn_select_topp that rewrites counts -- and a verify call flagged

@@ -323,9 +323,11 @@ __device__ __forceinline__ void merge_scales(float m, float im, float& mn, float
 // ---- precomputed work partition ("plan") ------------------------------------------------------
 // The partition of a launch depends only on the list lengths, the shapes and the grid: target
 // layers that share a draft layer's lists share it.  A plan holds, as int32:
-//   [0] magic  [1] U  [2] grid  [3] 0: ranges, else the partition's cluster size  [4] NP  [5] N (atoms)  [6] tail  [7] dense
+//   [0] magic  [1] U  [2] grid  [3] 0: ranges, else the partition's cluster size, | the launch's cluster size << 8
+//   [4] NP  [5] N (atoms)  [6] tail  [7] dense
 //   unit_start[U + 1], unit_cnt[U], a pad, then (a0, a1, u_first, part | parts << 8) per CTA
-// A kernel whose launch does not match the header ignores the plan and partitions itself.
+// A kernel whose launch does not match the header ignores the plan and partitions itself.  (The cluster size is part
+// of the match: the parts of a unit find one another by their ranks in the cluster.)
 constexpr int kPlanMagic = 0x5a17a9e1;
 constexpr int kPlanHeader = 8;
 __host__ __device__ inline size_t plan_ints(int U, int grid) {
@@ -393,7 +395,7 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   if (tid == 0) {
     plan[1] = U;
     plan[2] = G;
-    plan[3] = aligned ? cluster : 0;
+    plan[3] = (aligned ? cluster : 0) | (P.cluster << 8);
     plan[4] = static_cast<int>(NP);
     plan[5] = static_cast<int>(N);
     plan[6] = P.tail;
@@ -758,7 +760,8 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   // partition below by one coalesced copy.
   const int* const plan = P.plan;
   const bool planned = plan != nullptr && plan[0] == kPlanMagic && plan[1] == U &&
-                       plan[2] == static_cast<int>(gridDim.x) && plan[6] == P.tail && plan[7] == P.dense;
+                       plan[2] == static_cast<int>(gridDim.x) && (plan[3] >> 8) == P.cluster && plan[6] == P.tail &&
+                       plan[7] == P.dense;
   if (planned) {
     const int* const p_us = plan + kPlanHeader;
     const int* const p_cnt = p_us + (U + 1);
@@ -784,8 +787,8 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   const int G = static_cast<int>(gridDim.x);
   if (planned) {
     N = plan[5];
-    aligned = plan[3] != 0;
-    cluster = plan[3];
+    cluster = plan[3] & 0xff;
+    aligned = cluster != 0;
     NP = plan[4];
     const int* const p_cta = plan + kPlanHeader + 2 * (U + 1) + 4 * blockIdx.x;
     a0 = p_cta[0];

@@ -554,3 +554,54 @@ def test_long_and_skewed_lists_of_33_and_more_query_rows(stride, lens, counts):
     assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
     torch.cuda.synchronize()
     assert torch.equal(o, out) and torch.equal(l, lse)
+
+
+def test_a_plan_for_clusters_of_another_size_is_ignored():
+    """A plan names the cluster size of the launch it was made for, which depends on the query rows and on idx_stride
+    too.  A plan of calls with 16 query rows serves one with 40 where both are launched alike and is ignored
+    elsewhere; and a plan whose header names another size, and which deals no work at all, changes nothing."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC:
+        pytest.skip("only the mma.sync engine reads plans")
+
+    def prepare(T, stride):
+        case = _make_case(98, 2, T, 64, 8, 16, [12300] * 2, counts=[[700], [1500]])
+        case["idx"] = case["idx"][:, :, :stride].copy()
+        keep = [bf16_to_dev(case["q"]), case["kv"].to(dev()), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]),
+                to_dev(case["cnt"])]
+        out = torch.full((2, T, 64, 128), float("nan"), device=dev())
+        lse = torch.full((2, T, 64), float("nan"), device=dev())
+        a = sa.make_verify_args(keep[0], keep[1], keep[2], block_table=keep[3], idx=keep[4], counts=keep[5], out=out, lse=lse,
+                                flags=_ENGINE["flags"])
+        ws = sa.verify_workspace(a)
+        a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+        return case, a, out, lse, keep + [ws]
+
+    def call(a, out, lse, plan=None):
+        out.fill_(float("nan"))
+        lse.fill_(float("nan"))
+        a.plan = None if plan is None else plan.data_ptr()
+        assert sa.lib().specattn_sparse_verify(C.byref(a), None) == 0
+        torch.cuda.synchronize()
+        return out.clone(), lse.clone()
+
+    few = prepare(2, 6144)               # 16 query rows
+    plan = sa.verify_plan_buffer(few[1])
+    sa.verify_plan(few[1], plan)
+    for stride in (6144, 6145):         # larger clusters, pairs
+        case, a, out, lse, keep = prepare(5, stride)   # 40 query rows
+        ref = call(a, out, lse)
+        check_attention(*ref, *_oracle(case))
+        got = call(a, out, lse, plan)
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+        own = sa.verify_plan_buffer(a)
+        sa.verify_plan(a, own)
+        words = own.cpu()
+        size = int(words[3]) >> 8
+        assert size in (1, 2, 4, 8)
+        other = words.clone()
+        other[3] = (1 if size > 1 else 2) << 8             # ranges, in a launch of another cluster size
+        other[8 + 2 * (2 * 8 + 1):] = 0                    # no CTA has work
+        got = call(a, out, lse, other.to(dev()))
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
