@@ -2,6 +2,7 @@
 // whole-step entry point that moves a step's inputs and results across PCIe around the two
 // kernels (Alg. 1, blocks "Sparse Attention Mask Creation" and "Verification with Sparse
 // Attention").
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -102,17 +103,36 @@ __global__ void __launch_bounds__(256) copy_host_blocks(const __grid_constant__ 
   }
 }
 
-// The address at which the current device sees host memory `p`, or nullptr if it does not (pageable
-// memory) or if 16-byte accesses to the block, or its size, do not suit the kernel above.
+// The address at which the current device sees host memory `p`, or nullptr if it does not see the whole block
+// (pageable memory, a block that reaches beyond its pinned allocation or registered range) or if 16-byte accesses to
+// the block, or its size, do not suit the kernel above.  The driver's query is looked up through the runtime (no
+// link-time dependency on the driver library).
 uint4* device_view(const void* p, const void* device_side, size_t bytes) {
   if (bytes % 16 != 0 || bytes > kGatherMost || reinterpret_cast<uintptr_t>(device_side) % 16 != 0) return nullptr;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
+  typedef CUresult (*query_fn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static std::atomic<query_fn> cached{nullptr};
+  query_fn fn = cached.load(std::memory_order_acquire);
+  if (fn == nullptr) {
+    void* sym = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &sym, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess || sym == nullptr) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    fn = reinterpret_cast<query_fn>(sym);
+    cached.store(fn, std::memory_order_release);
   }
-  if (at.type != cudaMemoryTypeHost || reinterpret_cast<uintptr_t>(at.devicePointer) % 16 != 0) return nullptr;
-  return static_cast<uint4*>(at.devicePointer);
+  unsigned int type = 0, managed = 0;
+  CUdeviceptr seen = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* into[5] = {&type, &managed, &seen, &start, &size};
+  if (fn(5, what, into, static_cast<CUdeviceptr>(reinterpret_cast<uintptr_t>(p))) != CUDA_SUCCESS) return nullptr;
+  if (type != CU_MEMORYTYPE_HOST || managed != 0 || seen == 0 || seen % 16 != 0) return nullptr;
+  if (seen < start || seen - start > size || size - (seen - start) < bytes) return nullptr;
+  return reinterpret_cast<uint4*>(static_cast<uintptr_t>(seen));
 }
 
 bool make_event(cudaEvent_t* e) {

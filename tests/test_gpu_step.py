@@ -369,3 +369,80 @@ def test_host_buffer_step_from_pageable_memory_and_with_many_layers(pinned, laye
     torch.cuda.synchronize()
     for j in range(layers):
         assert torch.equal(out_host[j], ref_out[j]) and torch.equal(lse_host[j], ref_lse[j])
+
+
+def _capture_host_step(step, *host):
+    """Records a step from host buffers into a graph that is never launched.  Returns the launches of the
+    library's kernels, and per kernel node the number of copy nodes that it waits for."""
+    from cuda.bindings import runtime as rt
+    import paper_2510_27641_b200 as sa
+
+    def ok(r):
+        assert r[0] == rt.cudaError_t.cudaSuccess, r[0]
+        return r[1] if len(r) == 2 else r[1:]
+
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    n0 = sa.kernel_launch_count()
+    ok(rt.cudaStreamBeginCapture(stream.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed))
+    try:
+        step.run_host(*host, stream=stream)
+    finally:
+        graph = rt.cudaStreamEndCapture(stream.cuda_stream)
+    graph = ok(graph)
+    launches = sa.kernel_launch_count() - n0
+    nodes = ok(rt.cudaGraphGetNodes(graph, ok(rt.cudaGraphGetNodes(graph))[1]))[0]
+    before = {}
+    for node in nodes:
+        n = ok(rt.cudaGraphNodeGetDependencies_v2(node))[-1]
+        before[int(node)] = [int(d) for d in ok(rt.cudaGraphNodeGetDependencies_v2(node, n))[0][:n]] if n else []
+    kind = {int(node): ok(rt.cudaGraphNodeGetType(node)) for node in nodes}
+
+    def copies(node):
+        seen, todo = set(), list(before[node])
+        while todo:
+            d = todo.pop()
+            if d not in seen:
+                seen.add(d)
+                todo += before[d]
+        return sum(kind[d] == rt.cudaGraphNodeType.cudaGraphNodeTypeMemcpy for d in seen)
+
+    waits = [copies(n) for n, k in kind.items() if k == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel]
+    ok(rt.cudaGraphDestroy(graph) + (None,))
+    return launches, waits
+
+
+def _host_step(layers, ctx=600):
+    cfg = wl.config1().scaled(n_target_layers=layers, n_draft_layers=2, batch=1, ctx=ctx, n_q_heads=8, n_kv_heads=2)
+    si, pools, step = _build(cfg, layer_map=[j * 2 // layers for j in range(layers)])
+    dp_host = [torch.from_numpy(x).pin_memory() for x in si.draft_probs]
+    q_host = [bf16.bits_to_torch(q).pin_memory() for q in si.q]
+    out_host = [torch.zeros(o.shape, dtype=torch.float32).pin_memory() for o in step.out]
+    lse_host = [torch.zeros(l.shape, dtype=torch.float32).pin_memory() for l in step.lse]
+    step.run_host(dp_host, q_host, out_host, lse_host)   # makes the lanes and their events
+    torch.cuda.synchronize()
+    return step, dp_host, q_host, out_host, lse_host
+
+
+def test_host_blocks_beyond_a_registered_range_are_left_to_the_copy_engine():
+    """A host block of which only the first page is registered must not be read by the kernel that moves small
+    blocks.  (The step is recorded, not run.)"""
+    import mmap
+    from cuda.bindings import runtime as rt
+    import paper_2510_27641_b200 as sa
+    step, dp_host, q_host, out_host, lse_host = _host_step(2)
+    size = q_host[1].numel() * 2
+    assert size > 4096
+    memory = mmap.mmap(-1, 4 * 4096)
+    block = torch.frombuffer(memory, dtype=torch.bfloat16, count=q_host[1].numel()).view(q_host[1].shape)
+    registered = []
+    for pages, by_kernel in ((4, True), (1, False)):
+        assert rt.cudaHostRegister(block.data_ptr(), pages * 4096, 0)[0] == rt.cudaError_t.cudaSuccess
+        try:
+            n, _ = _capture_host_step(step, dp_host, [block, block], out_host, lse_host)
+            registered.append(n)
+        except sa.SpecAttnError as e:   # the runtime may refuse such a copy, as it may any other
+            assert not by_kernel and e.code == -7
+        finally:
+            assert rt.cudaHostUnregister(block.data_ptr())[0] == rt.cudaError_t.cudaSuccess
+    assert len(registered) == 1 or registered[1] == registered[0] - 1   # both query blocks are one launch
