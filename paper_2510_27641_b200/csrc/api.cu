@@ -231,6 +231,38 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
       !ok(cudaStreamWaitEvent(pipe.d2h, pipe.start, 0)))
     return SPECATTN_ERR_CUDA;
 
+  // The query blocks: one kernel on the caller's stream, which has nothing else to do until the first
+  // draft layer is in, reads those that the GPU can read.  The others (pageable, unaligned, large) go by the copy
+  // engine ahead of the draft rows: behind them they would hold up the first layer until the last one's rows are in.
+  bool q_copied = false;  // by the copy engine: the first verify call waits for it
+  specattn::HostBlocks blocks;
+  int n_blocks = 0;
+  auto fetch_blocks = [&]() {
+    if (n_blocks == 0) return true;
+    specattn::copy_host_blocks<<<dim3(8, static_cast<unsigned>(n_blocks)), 256, 0, stream>>>(blocks);
+    n_blocks = 0;
+    specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
+    return ok(cudaGetLastError());
+  };
+  for (int j = 0; j < S.n_target_layers; ++j) {
+    const specattn_verify_args& v = S.verify[j];
+    const size_t bytes = static_cast<size_t>(v.batch) * v.n_q * v.n_q_heads * v.head_dim * 2;
+    if (bytes == 0) continue;
+    const uint4* src = specattn::device_view(S.q_host[j], v.q, bytes);
+    if (src != nullptr) {
+      if (n_blocks == specattn::kGatherBlocks && !fetch_blocks()) return SPECATTN_ERR_CUDA;
+      blocks.src[n_blocks] = src;
+      blocks.dst[n_blocks] = static_cast<uint4*>(const_cast<void*>(v.q));
+      blocks.n16[n_blocks] = static_cast<unsigned int>(bytes / 16);
+      ++n_blocks;
+    } else {
+      q_copied = true;
+      if (!ok(cudaMemcpyAsync(const_cast<void*>(v.q), S.q_host[j], bytes, cudaMemcpyHostToDevice, pipe.h2d)))
+        return SPECATTN_ERR_CUDA;
+    }
+  }
+  if (q_copied && !ok(cudaEventRecord(pipe.q_in, pipe.h2d))) return SPECATTN_ERR_CUDA;
+
   // lane "in": the draft rows in the order the layers need them.  They bound the step (a PCIe link's ~53 GB/s).
   const size_t layer_bytes = static_cast<size_t>(sel.batch) * sel.n_draft_heads * sel.gamma *
                              static_cast<size_t>(sel.L_stride) * sizeof(float);
@@ -244,39 +276,7 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
   };
   for (int j = 0; j < S.n_target_layers; ++j)
     if (sel.layer_map[j] >= 0 && !upload(sel.layer_map[j])) return SPECATTN_ERR_CUDA;
-  // The query blocks: one kernel on the caller's stream, which has nothing else to do until the first
-  // draft layer is in, reads those that the GPU can read; the others follow the draft rows.
-  {
-    bool copied = false;
-    specattn::HostBlocks blocks;
-    int n_blocks = 0;
-    auto launch = [&]() {
-      if (n_blocks == 0) return true;
-      specattn::copy_host_blocks<<<dim3(8, static_cast<unsigned>(n_blocks)), 256, 0, stream>>>(blocks);
-      n_blocks = 0;
-      specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
-      return ok(cudaGetLastError());
-    };
-    for (int j = 0; j < S.n_target_layers; ++j) {
-      const specattn_verify_args& v = S.verify[j];
-      const size_t bytes = static_cast<size_t>(v.batch) * v.n_q * v.n_q_heads * v.head_dim * 2;
-      if (bytes == 0) continue;
-      const uint4* src = specattn::device_view(S.q_host[j], v.q, bytes);
-      if (src != nullptr) {
-        blocks.src[n_blocks] = src;
-        blocks.dst[n_blocks] = static_cast<uint4*>(const_cast<void*>(v.q));
-        blocks.n16[n_blocks] = static_cast<unsigned int>(bytes / 16);
-        if (++n_blocks == specattn::kGatherBlocks && !launch()) return SPECATTN_ERR_CUDA;
-      } else {
-        copied = true;
-        if (!ok(cudaMemcpyAsync(const_cast<void*>(v.q), S.q_host[j], bytes, cudaMemcpyHostToDevice, pipe.h2d)))
-          return SPECATTN_ERR_CUDA;
-      }
-    }
-    if (!launch()) return SPECATTN_ERR_CUDA;
-    if (copied && (!ok(cudaEventRecord(pipe.q_in, pipe.h2d)) || !ok(cudaStreamWaitEvent(stream, pipe.q_in, 0))))
-      return SPECATTN_ERR_CUDA;
-  }
+  if (!fetch_blocks()) return SPECATTN_ERR_CUDA;
 
   // the caller's stream: selection per draft layer when first needed, then the verify launches
   bool selected[SPECATTN_MAX_DRAFT_LAYERS] = {false};
@@ -314,6 +314,10 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
         fresh = true;
       }
     }
+    if (q_copied) {
+      q_copied = false;
+      if (!ok(cudaStreamWaitEvent(stream, pipe.q_in, 0))) return SPECATTN_ERR_CUDA;
+    }
     specattn_verify_args call = v;
     if (fresh) call.flags &= ~SPECATTN_VERIFY_LISTS_STABLE;
     fresh = false;
@@ -330,7 +334,6 @@ extern "C" int specattn_verify_step_host(const specattn_step_host_args* args, vo
     uint4* const out_view = (to_select == 0) ? specattn::device_view(S.out_host[j], v.out, out_bytes) : nullptr;
     uint4* const lse_view = (to_select == 0) ? specattn::device_view(S.lse_host[j], v.lse, lse_bytes) : nullptr;
     if (out_view != nullptr && lse_view != nullptr) {
-      specattn::HostBlocks blocks;
       blocks.src[0] = reinterpret_cast<const uint4*>(v.out);
       blocks.dst[0] = out_view;
       blocks.n16[0] = static_cast<unsigned int>(out_bytes / 16);

@@ -446,3 +446,24 @@ def test_host_blocks_beyond_a_registered_range_are_left_to_the_copy_engine():
         finally:
             assert rt.cudaHostUnregister(block.data_ptr())[0] == rt.cudaError_t.cudaSuccess
     assert len(registered) == 1 or registered[1] == registered[0] - 1   # both query blocks are one launch
+
+
+def test_query_blocks_for_the_copy_engine_do_not_wait_behind_the_draft_rows():
+    """Query blocks that the kernel does not take (here: unaligned) reach the GPU ahead of the draft rows: the
+    first selection waits for its own layer's rows, not for every layer's."""
+    layers = 4
+    step, dp_host, q_host, out_host, lse_host = _host_step(layers)
+    ref_out, ref_lse = [o.clone() for o in out_host], [l.clone() for l in lse_host]
+    odd = []
+    for q in q_host:
+        flat = torch.empty(q.numel() + 1, dtype=q.dtype).pin_memory()
+        odd.append(flat[1:].view(q.shape))
+        odd[-1].copy_(q)
+    _, waits = _capture_host_step(step, dp_host, odd, out_host, lse_host)
+    assert min(w for w in waits if w > 0) <= layers + 1   # the queries and one draft layer of two
+    for t in step.q + step.out + out_host:
+        t.zero_()
+    step.run_host(dp_host, odd, out_host, lse_host)
+    torch.cuda.synchronize()
+    for j in range(layers):
+        assert torch.equal(out_host[j], ref_out[j]) and torch.equal(lse_host[j], ref_lse[j])
