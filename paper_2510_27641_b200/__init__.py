@@ -123,18 +123,29 @@ def kernel_launch_count() -> int:
     return int(lib().specattn_kernel_launch_count())
 
 
+# torch's C layer, where this build of torch has it: torch.cuda.current_stream() builds a Python object, ~4 us a call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
+
+
 def _stream_ptr(stream) -> int:
-    """The cudaStream_t of a torch stream; None = the current stream of the current device (asked of
-    torch's C layer: torch.cuda.current_stream() builds a Python object, ~4 us a call)."""
-    if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    return stream.cuda_stream
+    """The cudaStream_t of a torch stream; None = the current stream of the current device."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch.cuda.current_stream().cuda_stream if _raw_stream is None else _raw_stream(_raw_device())
+
+
+def _plain(x):
+    """A key's element by value: a 0-d tensor or array may change in place, and an array has no hash."""
+    if isinstance(x, tuple):
+        return tuple(_plain(e) for e in x)
+    return x.item() if hasattr(x, "item") else x
 
 
 class _Calls(threading.local):
     """Argument structs of the one-call entry points, kept per thread and per shape: filling the ~20
     fields of a struct that a call shares with the previous one of its shape took most of the call's host time.  A
-    call overwrites every pointer before the library sees the struct."""
+    call overwrites every pointer before the library sees the struct.  Keys hold plain values only."""
 
     LIMIT = 64
 
@@ -142,11 +153,18 @@ class _Calls(threading.local):
         self.made = {}
 
     def get(self, key, make):
-        call = self.made.get(key)
+        try:
+            call = self.made.get(key)
+        except TypeError:
+            call = None
         if call is None:
+            key = _plain(key)
+            call = self.made.get(key)
+        if call is None:
+            call = make()
             if len(self.made) >= self.LIMIT:
                 self.made.clear()
-            call = self.made[key] = make()
+            self.made[key] = call
         return call
 
 
@@ -350,7 +368,8 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
     if made:
         own |= VERIFY_INIT_WORKSPACE
     key = (shape, kv_pages.shape, kv_pages.stride(), None if block_table is None else block_table.stride(),
-           pages_per_seq, None if dense else (idx.shape, idx.stride()), n_groups, dense, sm_scale, flags, tail_len)
+           pages_per_seq, None if dense else (idx.shape, idx.stride()), n_groups, dense, sm_scale, flags, tail_len,
+           _raw_device())   # (whose number of SMs decides the workspace's size)
 
     def make():
         a = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq, idx=idx,
