@@ -42,6 +42,7 @@ namespace cg = cooperative_groups;
 namespace specattn {
 
 extern std::atomic<long long> g_launch_count;
+int device_sm_count();
 
 namespace {
 
@@ -704,6 +705,45 @@ int pick_cluster_row(long long L_stride, long long n_lists) {
   return cs;
 }
 
+// CTAs per streamed list: as many as leave every CTA an SM to itself (two on one share its atomics), in slices that
+// pay for the exchanges.  131072 entries, uniform / Zipf, us, in one / two / four CTAs: 32 rows 64/57, 43/40, 35/32;
+// 72 rows 64/57, 45/41, 65/59; 100 rows 65/57, 66/59, 66/59.  196608 entries in two / four: 32 rows 57/51, 39/37;
+// 64 rows 59/53, 59/55; 128 rows 90/82, 102/93.
+int pick_cluster_stream(long long L_stride, long long n_lists, int n_sm) {
+  int cs = (L_stride > kStreamMax) ? 2 : 1;
+  while (cs < 4 && n_lists * cs * 2 <= n_sm && L_stride / (2 * cs) >= kSliceMax) cs *= 2;
+  return cs;
+}
+
+// Clusters of cs CTAs with a whole slice each that hold their rows on this device at once (GPCs do not hold a
+// multiple of every cluster size: of 148 SMs, 66 clusters of four and 30 of eight).  Asked once per device and size.
+int rows_at_once(const void* kernel, int dev, int cs) {
+  static std::atomic<int> known[64][kMaxCluster + 1];  // + 1; 0 = not asked yet
+  int n = known[dev][cs].load(std::memory_order_relaxed);
+  if (n == 0) {
+    cudaLaunchConfig_t q;
+    memset(&q, 0, sizeof(q));
+    q.gridDim = dim3(static_cast<unsigned>(cs), 1024, 1);
+    q.blockDim = dim3(512, 1, 1);
+    q.dynamicSmemBytes = kFixedBytes + kSliceMax * sizeof(float) + kScratchBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(cs);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    q.attrs = attr;
+    q.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, kernel, &q) != cudaSuccess) {
+      cudaGetLastError();
+      fit = 0;
+    }
+    n = fit + 1;
+    known[dev][cs].store(n, std::memory_order_relaxed);
+  }
+  return n - 1;
+}
+
 // The two-launch form applies to the default selection over multi-row lists of >= 2048
 // positions, and pays when one cluster per list would leave SMs without a CTA: a CTA streams
 // ~35 GB/s, so the cluster kernel is bound by (bytes per list) / (8 x 35 GB/s) however few the
@@ -812,42 +852,17 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
   // zeros
   const bool one_row = static_cast<long long>(A.n_draft_heads) * A.gamma == 1 && P.chunk == 1 && (!P.has_groups || A.n_groups == 1);
   const bool agg = !two_launch && !one_row;  // the CTAs sum the rows (or the chunks) themselves
-  // One CTA per row (stream_rows.cuh), where a cluster per row would need more than one wave of CTAs, or where
-  // there is about a row for every SM and a cluster's exchanges gain nothing (100 rows of 8192: 11.6 us against
-  // 13.5; of 32768: 18.9 against 22.8; of 131072: 55 against 95; 64 rows of 32768: 18.7 against 17.4).  Up to 64
-  // rows too long for one wave of clusters leave most SMs without a row, and a second wave of clusters costs less
-  // (131072 entries, clusters / one CTA a row: 40 rows 34 / 47 us, 64 rows 41 / 47, 68 rows 51 / 47).
-  const long long row_ctas = agg ? 0 : n_lists * specattn::pick_cluster_row(A.L_stride, n_lists);
-  const bool stream = !agg && !variant && A.L_stride <= specattn::kStreamMax && A.L_stride > 4096 &&
-                      ((row_ctas > 296 && n_lists > 64) || (n_lists > 72 && n_lists <= 148));
-  const bool small = !agg && !variant && A.L_stride <= 2048;
-  const int cs = stream ? 1 : agg ? specattn::pick_cluster(A.L_stride, n_lists) : specattn::pick_cluster_row(A.L_stride, n_lists);
-  const int slice = specattn::slice_of(static_cast<int>(A.L_stride), cs, (P.chunk > 4) ? P.chunk : 4);
-  const int nt = small ? 128 : agg ? 256 : 512;
-  if (slice > specattn::kSliceMax && !stream) return SPECATTN_ERR_UNSUPPORTED;
-  // searches apart: the scores of all queries are kept, and one query's scores fit a CTA's slice
-  const long long n_scores = (A.L_stride + P.chunk - 1) / P.chunk;
-  const size_t score_bytes = static_cast<size_t>(A.gamma) * (slice / P.chunk) * sizeof(float);
-  P.apart = (agg && P.per_step && P.chunk > 1 && A.gamma <= specattn::kMaxApart && n_scores <= specattn::kSliceMax &&
-             specattn::slice_room(static_cast<int>(n_scores), nt) <= specattn::slice_room(slice, nt) && score_bytes <= 48 * 1024)
-                ? 1
-                : 0;
-  const size_t apart_bytes = P.apart ? score_bytes : 0;
-  const size_t smem = stream ? sizeof(specattn::StreamShared) : specattn::kFixedBytes + (agg ? specattn::kHeadBytes : 0) +
-                      static_cast<size_t>(specattn::slice_room(slice, nt)) * sizeof(float) +
-                      (agg ? specattn::kRingBytes : specattn::kScratchBytes) +
-                      // the union's bit mask: one bit per entry of the slice
-                      (P.per_step ? static_cast<size_t>(specattn::slice_room(slice, nt) / 8) : 0) + apart_bytes;
-  const void* const kernels[7] = {
+  const void* const kernels[9] = {
       (const void*)specattn::select_topp_kernel<false, false, 128>, (const void*)specattn::select_topp_kernel<false, false, 512>,
       (const void*)specattn::select_topp_kernel<false, true, 512>, (const void*)specattn::select_topp_kernel<true, false, 256>,
-      (const void*)specattn::select_topp_kernel<true, true, 256>, (const void*)specattn::stream_rows_kernel<false>,
-      (const void*)specattn::stream_rows_kernel<true>};
-  const int kidx = stream ? (A.diag != nullptr ? 6 : 5) : agg ? (variant ? 4 : 3) : (variant ? 2 : (small ? 0 : 1));
+      (const void*)specattn::select_topp_kernel<true, true, 256>, (const void*)specattn::stream_rows_kernel<false, false>,
+      (const void*)specattn::stream_rows_kernel<true, false>, (const void*)specattn::stream_rows_kernel<false, true>,
+      (const void*)specattn::stream_rows_kernel<true, true>};
   // Opt in to large dynamic shared memory and clusters of 16 once per device, so that later calls
   // issue nothing but the launch.
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+  const int n_sm = specattn::device_sm_count();
+  if (n_sm <= 0 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
     cudaGetLastError();
     return SPECATTN_ERR_CUDA;
   }
@@ -864,10 +879,35 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
       done_mask.fetch_or(1ull << dev, std::memory_order_release);
     }
   }
-
+  // Rows are streamed (stream_rows.cuh) where clusters that hold them would need more than one wave (uniform / Zipf,
+  // us, held / streamed: 40 rows of 98304 entries 45/39, 39/35; 72 of 65536 45/39, 31/30; 64 of 131072 62/47, 45/41;
+  // 16 of 196608 51/39, 39/37 -- but 12 of them 33/27, 39/36), or where there is about a row for every SM and a
+  // cluster's exchanges gain nothing (100 rows of 8192: 18/18, 18/18; of 32768 29/29, 28/25; of 65536 45/41, 41/37).
+  const int row_cs = specattn::pick_cluster_row(A.L_stride, n_lists);
+  const bool stream = !agg && !variant && A.L_stride > 4096 &&
+                      (n_lists > specattn::rows_at_once(kernels[1], dev, row_cs) || (2 * n_lists > n_sm && n_lists <= n_sm));
+  const bool small = !agg && !variant && A.L_stride <= 2048;
+  const int cs = stream ? specattn::pick_cluster_stream(A.L_stride, n_lists, n_sm) : agg ? specattn::pick_cluster(A.L_stride, n_lists) : row_cs;
+  const int slice = specattn::slice_of(static_cast<int>(A.L_stride), cs, (P.chunk > 4) ? P.chunk : 4);
+  const int nt = small ? 128 : agg ? 256 : 512;
+  if (slice > specattn::kSliceMax && !stream) return SPECATTN_ERR_UNSUPPORTED;
+  // searches apart: the scores of all queries are kept, and one query's scores fit a CTA's slice
+  const long long n_scores = (A.L_stride + P.chunk - 1) / P.chunk;
+  const size_t score_bytes = static_cast<size_t>(A.gamma) * (slice / P.chunk) * sizeof(float);
+  P.apart = (agg && P.per_step && P.chunk > 1 && A.gamma <= specattn::kMaxApart && n_scores <= specattn::kSliceMax &&
+             specattn::slice_room(static_cast<int>(n_scores), nt) <= specattn::slice_room(slice, nt) && score_bytes <= 48 * 1024)
+                ? 1
+                : 0;
+  const size_t apart_bytes = P.apart ? score_bytes : 0;
+  const size_t smem = stream ? sizeof(specattn::StreamShared) : specattn::kFixedBytes + (agg ? specattn::kHeadBytes : 0) +
+                      static_cast<size_t>(specattn::slice_room(slice, nt)) * sizeof(float) +
+                      (agg ? specattn::kRingBytes : specattn::kScratchBytes) +
+                      // the union's bit mask: one bit per entry of the slice
+                      (P.per_step ? static_cast<size_t>(specattn::slice_room(slice, nt) / 8) : 0) + apart_bytes;
+  const int kidx = stream ? 5 + (A.diag != nullptr ? 1 : 0) + (cs > 1 ? 2 : 0) : agg ? (variant ? 4 : 3) : (variant ? 2 : (small ? 0 : 1));
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = stream ? dim3(static_cast<unsigned>(n_lists), 1, 1) : dim3(static_cast<unsigned>(cs), static_cast<unsigned>(n_lists), 1);
+  cfg.gridDim = (stream && cs == 1) ? dim3(static_cast<unsigned>(n_lists), 1, 1) : dim3(static_cast<unsigned>(cs), static_cast<unsigned>(n_lists), 1);
   cfg.blockDim = dim3(static_cast<unsigned>(nt), 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = static_cast<cudaStream_t>(cuda_stream);
@@ -895,7 +935,7 @@ extern "C" int specattn_select_topp(const specattn_select_args* args, void* cuda
   // more).  The limits are asked of the runtime once per kernel and cluster size and cached.
   {
     static const size_t pads[3] = {120 * 1024, 100 * 1024, 70 * 1024};
-    static std::atomic<int> fit[64][7][5][3];  // [device][kernel][log2 cs][pad]: clusters + 1, 0 = unknown
+    static std::atomic<int> fit[64][5][5][3];  // [device][kernel, none of the streaming ones][log2 cs][pad]: clusters + 1, 0 = unknown
     int lcs = 0;
     while ((1 << lcs) < cs) ++lcs;
     for (int k = 0; k < 3 && !stream; ++k) {

@@ -1,11 +1,13 @@
-// One CTA per row, for calls with more rows than the GPU can keep on chip at once.  Included by
+// Rows that are streamed: for calls with more rows than the GPU can keep on chip at once.  Included by
 // select_topp.cu.
 //
 // Held in shared memory, 148 SMs take some 37 rows of 131072 entries, and the latencies of a search (barriers,
-// exchanges, scans) are paid once per wave of them (256 rows: 240 us).  Here every row has its own CTA, two
-// per SM, nothing of a row stays on chip but a histogram and bits, and a row is read twice, each time through
-// a ring of 16-byte copies that keeps 48 KB per CTA under way.  The searches of different rows overlap one
-// another's reads; there is no cluster and no exchange.
+// exchanges, scans) are paid once per wave of them (256 rows: 240 us).  Here nothing of a row stays on chip but a
+// histogram and bits, and a row is read twice, each time through a ring of 16-byte copies that keeps 32 to 64 KB
+// per CTA under way.  A row is dealt to a cluster of one, two or four CTAs (pick_cluster_stream; at least two where it is
+// longer than a CTA's words allow); the searches of different rows overlap one another's reads.
+// The CTAs of a row exchange their octaves and one octave's bins after the first pass, the keys of the bin after the
+// second, and their kept counts, and each decides for itself.
 //
 // With that, the passes are bound by instruction issue and by the wavefronts of shared-memory atomics, so each does
 // as little per entry as it can:
@@ -30,7 +32,8 @@ constexpr int kStreamWarps = kStreamThreads / 32;
 constexpr int kStreamRound = 4 * kStreamThreads;   // entries per round of the CTA: 8 KB
 constexpr int kStreamBatch = 4;                    // rounds per commit group
 constexpr int kStreamGroups = 2;                   // groups in the ring
-constexpr int kStreamMax = 131072;                 // entries per row: 64 rounds
+constexpr int kStreamMax = 131072;                 // entries per CTA: 64 rounds
+constexpr int kStreamAlign = 32;                   // slices of a cluster start on whole 128-byte lines
 constexpr int kStreamShift = 18;                   // level-1 bins: the key's bits above these
 constexpr int kStreamBins = 8192;
 constexpr int kStreamCand = 4096;                  // keys of the bin that are gathered
@@ -50,6 +53,11 @@ struct StreamShared {
   int negative;                // a negative input was met
   int tiny;                    // (exact search) a key below 512, of which the histogram's word of bin 0 holds nothing
   int oct_min, oct_max, n_cand;
+  double part;                 // this CTA's share of a sum over the row
+  int kept;                    // kept entries of this CTA (these seven are read by peers, like the store and the scratch's
+                               // octaves and keys)
+  int row_max;                 // highest octave of the row; the last one if an input is invalid
+  double row_part;             // (a level of a well filled bin) the row's sum
   Found fd;
   double sum[kStreamWarps];
   int warp_cnt[kStreamWarps];
@@ -61,7 +69,8 @@ struct StreamScratch {
   LevelHist lv;
   Picks pk;
   unsigned int keys[kStreamCand];
-  unsigned int place[kStreamCand];   // entry of the row
+  unsigned int place[kStreamCand];   // entry of the slice
+  unsigned int all_keys[kStreamCand];  // (clusters) the keys of the whole row's bin
 };
 constexpr int kStreamStage = 528;    // ints of a warp's staging line (512 entries, shifted by up to 3)
 static_assert(sizeof(StreamScratch) <= sizeof(StreamShared::ring), "scratch in the ring");
@@ -152,14 +161,27 @@ __device__ __forceinline__ double stream_sum(StreamShared& sh, double s) {
 // kMasses: the caller wants the masses (diag), so they are added up in binary64.  Otherwise they only have to tell
 // which threshold is the right one, and the low parts of a batch are added up in binary32 first, the rare row in doubt
 // being searched again (256 rows of 131072, uniform / Zipf / ties: 107 / 96 / 102 us with masses, 103 / 90 / 97 without).
-template <bool kMasses>
+// kShared: a row has several CTAs (known to the compiler, since the exchanges cost one CTA a row 3 us of 104).
+template <bool kMasses, bool kShared>
 __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __grid_constant__ SelectParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamShared& sh = *reinterpret_cast<StreamShared*>(smem_raw);
   StreamScratch& sc = *reinterpret_cast<StreamScratch*>(sh.ring);
   constexpr int N = 4 * kStreamBatch;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int list = blockIdx.x;  // (used slot, sequence, group)
+  cg::cluster_group cluster = cg::this_cluster();
+  const int cs = kShared ? static_cast<int>(cluster.num_blocks()) : 1, rank = kShared ? static_cast<int>(cluster.block_rank()) : 0;
+  auto csync = [&]() {
+    if (kShared) cluster.sync(); else __syncthreads();
+  };
+  // sum of a number of every CTA of the row, in their order (all lanes of a warp)
+  auto row_sum = [&](double* at) {
+    const double mine = (lane < cs) ? *cluster.map_shared_rank(at, lane < cs ? lane : 0) : 0.0;
+    double s = __shfl_sync(kFull, mine, 0);
+    for (int r = 1; r < cs; ++r) s += __shfl_sync(kFull, mine, r);
+    return s;
+  };
+  const int list = kShared ? blockIdx.y : blockIdx.x;  // (used slot, sequence, group)
   const int g = list % P.G;
   const int b = (list / P.G) % P.B;
   const int slot = list / (P.G * P.B);
@@ -183,9 +205,11 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   long long Lll = P.kv_len[b];
   if (Lll < 0) Lll = 0;
   if (Lll > P.L_stride) Lll = P.L_stride;
-  const int L = static_cast<int>(Lll);
-  const float* A = (P.agg != nullptr) ? P.agg + static_cast<long long>(list) * P.L_stride
-                                      : P.probs[slot] + static_cast<long long>(b) * P.H * P.gamma * P.L_stride;
+  const int L_row = static_cast<int>(Lll);
+  const int per_cta = kShared ? slice_of(L_row, cs, kStreamAlign) : L_row;
+  const int lo = kShared ? min(L_row, rank * per_cta) : 0, L = kShared ? min(L_row, lo + per_cta) - lo : L_row;  // this CTA's entries
+  const float* A = ((P.agg != nullptr) ? P.agg + static_cast<long long>(list) * P.L_stride
+                                       : P.probs[slot] + static_cast<long long>(b) * P.H * P.gamma * P.L_stride) + lo;
 
   double total = 0.0, target = 0.0, m_gt = 0.0, m_ge = 0.0;
   bool invalid = false, searching = false;
@@ -193,13 +217,20 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
   unsigned int* const above_bits = sh.store;
   unsigned int* const in_bits = sh.store + kStreamWords;
   bool exact = false, last_resort = false;
+  auto row_word = [&](int bin) {  // a bin's word, over the row
+    unsigned long long w = 0ull;
+    if constexpr (!kShared) w = hist[stream_word(bin)];
+    else for (int r = 0; r < cs; ++r) w += *cluster.map_shared_rank(&hist[stream_word(bin)], r);
+    return w;
+  };
   auto bin_mass9 = [&](int oct) {  // lane: bin of an octave
-    return static_cast<double>(static_cast<unsigned long long>(hist[stream_word(32 * oct + lane)]) << 9) * pow2_double(max(oct, 1) - 150);
+    return static_cast<double>(row_word(32 * oct + lane) << 9) * pow2_double(max(oct, 1) - 150);
   };
   int go = 0;                  // 1 / -1: the bin above / below the last one tried is wanted
   auto turn = [&](int want) {  // on to the bin above or below -- or, after a turn back, to an exact search
     if (go == -want) exact = true;
     go = (go == -want) ? 0 : want;
+    csync();
     clear();
   };
   for (;;) {
@@ -270,6 +301,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
 
     // ---- the bin of the threshold ---------------------------------------------------------------------
     const double rest = stream_sum(sh, (mine[0] + mine[1]) + (mine[2] + mine[3]));
+    if (kShared && tid == 0) sh.part = rest;
     if (tid < kOctaves) {
       unsigned long long s = 0ull;
 #pragma unroll 8
@@ -283,14 +315,25 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
         atomicMax(&sh.oct_max, final);
       }
     }
-    __syncthreads();
-    invalid = sh.negative != 0 || sh.oct_max == kOctaves - 1;  // (the last octave: infinities and NaN)
+    csync();
     if (warp == 0) {
       double t = 0.0, tg = 0.0, carry = 0.0, ab = 0.0, up;
       int bin = -1;
       last_resort = false;
-      if (sh.oct_max >= 0 && !invalid) {
-        const int oct = find_octave(sh.oct_max, sh.oct_min, P.p, [&](int e) { return sc.oct[e]; }, t, tg, carry);
+      // of the row: octaves with an entry, and whether an input is invalid (the last octave: infinities and NaN)
+      const StreamShared* const peer = (kShared && lane < cs) ? cluster.map_shared_rank(&sh, lane) : &sh;
+      const int top = __reduce_max_sync(kFull, (peer->negative != 0) ? kOctaves - 1 : peer->oct_max);
+      const int bottom = __reduce_min_sync(kFull, peer->oct_min);
+      const bool some_tiny = __any_sync(kFull, peer->tiny != 0);
+      auto mass = [&](int e) {
+        unsigned long long s = 0ull;
+        if constexpr (!kShared) s = sc.oct[e];
+        else for (int r = 0; r < cs; ++r) s += *cluster.map_shared_rank(&sc.oct[e], r);
+        return s;
+      };
+      const double row_rest = kShared ? row_sum(&sh.part) : rest;
+      if (top >= 0 && top < kOctaves - 1) {
+        const int oct = find_octave(top, bottom, P.p, mass, t, tg, carry);
         bin = 32 * oct + find_from_top<5>(bin_mass9(oct), 0.0, carry, tg, ab, up);
         if (go != 0) {  // the next one with an entry, or none
           int at = sh.fd.bin;
@@ -299,7 +342,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
             at = (go > 0) ? at + 1 : at - 1;
             const int mine_at = (go > 0) ? at + lane : at - lane;
             const unsigned some = __ballot_sync(kFull, mine_at >= 0 && mine_at < kStreamBins &&
-                                                           (hist[stream_word(mine_at & (kStreamBins - 1))] != 0u || (mine_at == 0 && sh.tiny != 0)));
+                                                           (row_word(mine_at & (kStreamBins - 1)) != 0ull || (mine_at == 0 && some_tiny)));
             if (some != 0u) {
               bin = (go > 0) ? at + __ffs(some) - 1 : at - (__ffs(some) - 1);
               break;
@@ -314,15 +357,17 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
           if (bin >= 0) {
             if (!exact) {  // its mass above, octave by octave from the top
               carry = 0.0;
-              for (int e = sh.oct_max; e > (bin >> 5); --e) carry += static_cast<double>(sc.oct[e]) * pow2_double(max(e, 1) - 150);
+              for (int e = top; e > (bin >> 5); --e) carry += static_cast<double>(mass(e)) * pow2_double(max(e, 1) - 150);
             }
             ab = suffix_sum<5>((lane > (bin & 31)) ? bin_mass9(bin >> 5) : 0.0);
             ab = __shfl_sync(kFull, ab, 0);
           }
         }
       }
+      const unsigned long long word = (bin >= 0) ? row_word(bin) : 0ull;
       if (lane == 0) {
-        sh.fd.total = t;
+        sh.row_max = top;
+        sh.fd.total = t + row_rest;
         sh.fd.key = last_resort ? 1u : 0u;
         sh.fd.bin = bin;
         if (bin >= 0) {
@@ -330,18 +375,19 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
           sh.fd.above = exact ? ab : carry + ab;
           // the bin's smallest term bounds the number of its keys
           const unsigned int least = (static_cast<unsigned int>(bin & 31) << 9) | ((bin >= 32) ? 0x4000u : 0u);
-          sh.fd.count = (least == 0u) ? 0x7fffffffu : hist[stream_word(bin)] / least;
+          sh.fd.count = (least == 0u) ? 0x7fffffffu : static_cast<unsigned int>(word / least);  // (at most 2^32 / 2^9 a CTA)
         }
       }
     }
     __syncthreads();
-    total = sh.fd.total + rest;
+    invalid = sh.row_max == kOctaves - 1;
+    total = sh.fd.total;
     if (!invalid && !exact && (!(total >= 0x1p-40) || (go != 0 && sh.fd.bin < 0))) {
       // (the histogram takes a denormal for a number of at least 2^-126, which only counts in a total as small
       // as this; or there is no neighbour where the masses asked for one)
       exact = true;
       go = 0;
-      __syncthreads();
+      csync();
       clear();
       continue;
     }
@@ -360,7 +406,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     const double carry = sh.fd.carry, above_hist = sh.fd.above;
     const int hi_key = exact ? static_cast<int>((prefix >> 5 << 23) | 0x7fffffu) : INT_MAX;
     int want = 0;
-    __syncthreads();
+    csync();  // the histograms and octaves have been read: the store and the ring are free
     // ---- a well filled bin: 10 (then the last 8) more bits, one pass over the row each -----------------------
     while (M > static_cast<unsigned int>(kStreamCand) && shift > 0) {
       // (the pass uses the ring, so the level histogram takes the store)
@@ -379,28 +425,41 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       });
       level_groups<kStreamThreads>(lv, prefix, sl, bits);
       s = stream_sum(sh, s);
+      if (kShared && tid == 0) sh.part = s;
+      csync();
       if (warp == 0) {
         double above, upto, above1, upto1;
-        const double all = static_cast<double>(lv.grp[lane]) * scale;
+        if (kShared) s = row_sum(&sh.part);
+        unsigned long long m = lv.grp[lane];
+        for (int r = 1; r < cs; ++r) m += *cluster.map_shared_rank(&lv.grp[lane], (rank + r) % cs);
+        const double all = static_cast<double>(m) * scale;
         const int gi = find_from_top<5>(all, s, carry, target, above, upto);
         const int bin = gi * 32 + lane;
-        const unsigned int c = lv.cnt[bin];
-        const int b1 = find_from_top<5>(static_cast<double>(level_mass(prefix, bin, sl, c, lv.sum[bin], bits)) * scale, above, carry,
-                                        target, above1, upto1);
+        unsigned int c = lv.cnt[bin];
+        m = level_mass(prefix, bin, sl, c, lv.sum[bin], bits);
+        for (int r = 1; r < cs; ++r) {
+          const LevelHist* const peer = cluster.map_shared_rank(&lv, (rank + r) % cs);
+          const unsigned int c_r = peer->cnt[bin];
+          m += level_mass(prefix, bin, sl, c_r, peer->sum[bin], bits);
+          c += c_r;
+        }
+        const int b1 = find_from_top<5>(static_cast<double>(m) * scale, above, carry, target, above1, upto1);
         const unsigned int cb = __shfl_sync(kFull, c, b1);
         if (lane == 0) {
           sh.fd.oct = gi * 32 + b1;
           sh.fd.count = cb;
           sh.fd.upto = upto1;
+          sh.row_part = s;
         }
       }
       __syncthreads();
       // (only the first level can show that the bin was the wrong one)
-      if (shift == kStreamShift && !last_resort) want = (carry + s >= target) ? 1 : (carry + sh.fd.upto < target) ? -1 : 0;
+      if (shift == kStreamShift && !last_resort) want = (carry + sh.row_part >= target) ? 1 : (carry + sh.fd.upto < target) ? -1 : 0;
       prefix = (prefix << bits) | static_cast<unsigned int>(sh.fd.oct);
       M = sh.fd.count;
       shift = sl;
-      __syncthreads();
+      csync();
+      if (exact && want == -go) want = 0;  // (never: in whole numbers the bins agree with one another)
       if (want != 0) break;
     }
     if (want != 0) {
@@ -461,7 +520,8 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     };
     if (by_hist) pass2(std::false_type()); else pass2(std::true_type());
     if (tid == 0) sh.n_cand = 0;
-    inner = stream_sum(sh, inner) + (by_hist ? above_hist : 0.0);
+    inner = stream_sum(sh, inner);
+    if (kShared && tid == 0) sh.part = inner;
     if (shift > 0) level_clear<kStreamThreads>(sc.lv);
     // fetch the keys of the bin by their bits
     const int word_rows = (L + 8 * kStreamRound - 1) / (8 * kStreamRound);
@@ -484,38 +544,58 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       }
     }
     __syncthreads();
-    const int n = min(sh.n_cand, kStreamCand);  // (one value's entries may be more: their bits are all kept)
+    const int own = min(sh.n_cand, kStreamCand);  // (one value's entries may be more: their bits are all kept)
     if (shift > 0) {  // (all loads of a thread in flight at once: one by one, as the places are found, took 7 us)
       unsigned int key[kStreamCand / kStreamThreads];
 #pragma unroll
       for (int j = 0; j < kStreamCand / kStreamThreads; ++j) {
         const int i = tid + j * kStreamThreads;
-        if (i < n) key[j] = __float_as_uint(__ldg(A + sc.place[i]));
+        if (i < own) key[j] = __float_as_uint(__ldg(A + sc.place[i]));
       }
 #pragma unroll
       for (int j = 0; j < kStreamCand / kStreamThreads; ++j) {
         const int i = tid + j * kStreamThreads;
-        if (i < n) sc.keys[i] = key[j];
+        if (i < own) sc.keys[i] = key[j];
       }
-      __syncthreads();
+    }
+    csync();
+    if (kShared) inner = row_sum(&sh.part);
+    inner += by_hist ? above_hist : 0.0;
+    int n = own, n_in = sh.n_cand;  // keys of the row's bin, and its entries
+    const unsigned int* keys = sc.keys;
+    if (kShared) {
+      const int c_r = (lane < cs) ? *cluster.map_shared_rank(&sh.n_cand, lane < cs ? lane : 0) : 0;
+      n_in = __reduce_add_sync(kFull, c_r);
+      n = min(n_in, kStreamCand);
+      keys = sc.all_keys;
+      if (shift > 0) {
+        int off = 0;
+        for (int r = 0; r < cs; ++r) {
+          const int c = min(__shfl_sync(kFull, c_r, r), kStreamCand - off);
+          const unsigned int* const src = cluster.map_shared_rank(sc.keys, r);
+          for (int i = tid; i < c; i += kStreamThreads) sc.all_keys[off + i] = src[i];
+          off += c;
+        }
+        __syncthreads();
+      }
     }
     if (shift > 0 && n == 0) {
       theta = top_key + 1u;
       m_gt = m_ge = carry + inner;
     } else if (shift > 0) {
       double above, upto;
-      theta = threshold_among<kStreamThreads>(sc.keys, n, prefix, shift, inner, carry, target, scale, sc.lv, sh.fd, sc.pk, above, upto);
+      theta = threshold_among<kStreamThreads>(keys, n, prefix, shift, inner, carry, target, scale, sc.lv, sh.fd, sc.pk, above, upto);
       m_gt = carry + above;
       m_ge = carry + upto;
     } else {
       theta = prefix;
       m_gt = carry + inner;
-      m_ge = carry + (inner + static_cast<double>(sh.n_cand) * static_cast<double>(__uint_as_float(prefix)));
+      m_ge = carry + (inner + static_cast<double>(n_in) * static_cast<double>(__uint_as_float(prefix)));
     }
     // the right bin?
     if (shift == kStreamShift && !last_resort) {
       want = (carry + inner >= target) ? 1 : (m_ge < target) ? -1 : 0;
-      if (want != 0) {
+      if (want != 0 && !(exact && want == -go)) {
         __syncthreads();
         if (tid == 0) sh.fd.bin = static_cast<int>(prefix);  // (threshold_among used the field)
         turn(want);
@@ -524,15 +604,15 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     }
     const double doubt = (kMasses ? kStreamDoubt : kStreamDoubt32) * total;
     if (!exact && !(m_gt < target - doubt && m_ge > target + doubt)) {
-      __syncthreads();
       exact = true;
       go = 0;
+      csync();
       clear();
       continue;
     }
     // the bin's entries that make it join the bits
     if (shift > 0) {
-      for (int i = tid; i < n; i += kStreamThreads) {
+      for (int i = tid; i < own; i += kStreamThreads) {
         if (sc.keys[i] >= theta) {
           const unsigned int e = sc.place[i];
           const unsigned int round = e / kStreamRound, t = (e % kStreamRound) >> 2;
@@ -569,6 +649,15 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
     const int v = (lane < kStreamWarps) ? sh.warp_cnt[lane] : 0;
     count = __reduce_add_sync(kFull, v);
     int pos = __reduce_add_sync(kFull, lane < warp ? v : 0);
+    if (kShared) {
+      if (tid == 0) sh.kept = count;
+      csync();  // (every CTA is also done with its peers' keys: the ring may be written)
+      const int c_r = (lane < cs) ? *cluster.map_shared_rank(&sh.kept, lane < cs ? lane : 0) : 0;
+      count = __reduce_add_sync(kFull, c_r);
+      pos += __reduce_add_sync(kFull, lane < rank ? c_r : 0);
+      __syncwarp();
+      cluster_arrive_release();  // this CTA reads no peer's shared memory from here on
+    }
     // 512 entries at a time: the lanes' counts of four 128-entry chunks are scanned as four bytes of one word, the
     // kept positions go through a per-warp staging line that lies like the output modulo 16 bytes, and leave
     // in 16-byte stores.
@@ -597,7 +686,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           int at = base + static_cast<int>((incl >> (8 * i)) & 255u);
-          const int first = r * kStreamRound + (4 * q + i) * 128 + 4 * lane;
+          const int first = lo + r * kStreamRound + (4 * q + i) * 128 + 4 * lane;
           const unsigned int nib = x >> (8 * i);
           if (nib & 1u) stage[at++] = first;
           if (nib & 2u) stage[at++] = first + 1;
@@ -620,11 +709,14 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
         pos += base - off;
       }
     }
-  } else if (!invalid) {
-    count = L;
-    for (int i = tid; i < min(L, stride); i += kStreamThreads) out[i] = i;
+  } else {
+    if (kShared) cluster_arrive_release();
+    if (!invalid) {
+      count = L_row;
+      for (int i = lo + tid; i < min(lo + L, stride); i += kStreamThreads) out[i] = i;
+    }
   }
-  if (tid == 0) {
+  if (tid == 0 && rank == 0) {
     P.counts[out_list] = count;
     P.status[out_list] = invalid ? SPECATTN_ROW_INVALID_PROB : (count > P.idx_stride ? SPECATTN_ROW_OVERFLOW : SPECATTN_ROW_OK);
     if (P.diag != nullptr) {
@@ -635,4 +727,6 @@ __global__ void __launch_bounds__(kStreamThreads, 2) stream_rows_kernel(const __
       d[3] = m_ge;
     }
   }
+  __syncwarp();
+  if (kShared) cluster_wait();  // nobody leaves while its shared memory may still be read remotely
 }

@@ -631,3 +631,94 @@ def test_many_aggregated_lists_are_the_same_bits_in_every_form():
         for b in range(B):
             assert torch.equal(i1[0, b, 0, :int(c0[0, b, 0])], i0[0, b, 0, :int(c0[0, b, 0])])
         assert torch.allclose(d1, d0, rtol=1e-14, atol=0)   # a few roundings of binary64 apart
+
+
+@pytest.mark.parametrize("n", [131076, 196607])
+@pytest.mark.parametrize("n_rows", [3, 20, 40, 70, 150, 300])
+def test_rows_beyond_131072_entries(n, n_rows, form):
+    """Single rows longer than one CTA's words: clusters of sixteen CTAs that hold the row, clusters that stream it, for few
+    and for many rows; flat, peaked and tied values, a row whose masses meet the target, an invalid and a short row."""
+    if form == "cluster":
+        pytest.skip("single-row lists take the same path with and without a workspace")
+    Ls = (n + 3) // 4 * 4
+    rows = np.full((n_rows, Ls), np.float32(7.0))
+    rows[:, :n] = np.random.default_rng(n_rows).random((n_rows, n), dtype=np.float32) ** 2
+    sample = [0, 1, 2] if n_rows == 3 else [0, 1, 2, 3, 4, 5, n_rows - 1]
+    rows[0, :n] = wl.topp_rows("zipf", 1, n, seed=3)[0]
+    rows[1, :n] = np.float32(0.0078125)
+    rows[1, ::3] = np.nextafter(np.float32(0.0078125), np.float32(1))
+    rows[2, :n] = 0.0
+    rows[2, n - 65536:n] = _rows_that_meet_the_target(1, n)[0]
+    kv = np.full(n_rows, n, np.int32)
+    if n_rows > 3:
+        rows[3, n - 1] = np.inf
+        kv[4], kv[5] = 5, 0
+    for p in (0.5, 0.9375):
+        import paper_2510_27641_b200 as sa
+        gi, gc, gs, gd = sa.select_topp.func([to_dev(rows.reshape(n_rows, 1, 1, Ls))], to_dev(kv), [0], p, want_diag=n_rows != 70)
+        torch.cuda.synchronize()
+        oi, oc, os_, od = oracle.select_topp([rows[sample].reshape(len(sample), 1, 1, Ls)], np.zeros(1, np.int32), kv[sample], p)
+        st = compare_lists(lambda i: rows[sample][i, :kv[sample][i]], p, gi.cpu().numpy()[:, sample], gc.cpu().numpy()[:, sample],
+                           gs.cpu().numpy()[:, sample], oi, oc, os_, od)
+        assert st["n"] == len(sample)
+        assert gc[0, 2, 0].item() == oc[0, 2, 0] == (1 << int(16 * p)) - 1
+        gc_h = gc.cpu().numpy().ravel()
+        others = [i for i in range(n_rows) if i not in sample]
+        assert np.all(gc_h[others] > 0.2 * n) and np.all(gc_h[others] < 0.9 * n)
+
+
+@pytest.mark.parametrize("variant", [{}, {"chunk": 16}, {"bisect_iters": 10}, {"per_step": True}, {"per_step": True, "chunk": 32}])
+def test_aggregated_lists_beyond_131072_positions(variant):
+    """The one-launch form in clusters of sixteen CTAs and the two-launch form, with the variants of the search."""
+    import paper_2510_27641_b200 as sa
+    Ls, kv = 196608, np.array([196608, 131077], np.int32)
+    probs = wl.draft_probs(41, 0, kv, 2, 2, Ls, sink=6.0, slope=0.0002)
+    gi, gc, gs, _ = sa.select_topp([to_dev(probs)], to_dev(kv), [0], 0.9, **variant)
+    torch.cuda.synchronize()
+    if variant:
+        oi, oc, os_, od = oracle.select_variant([probs], [0], kv, 0.9, **{"n_iters" if k == "bisect_iters" else k: v for k, v in variant.items()})
+        assert _compare_variant(gi, gc, gs, oi, oc, os_, od) == 2
+    else:
+        oi, oc, os_, od = oracle.select_topp([probs], np.zeros(1, np.int32), kv, 0.9)
+        st = compare_lists(lambda i: oracle.aggregate(probs[i], L=int(kv[i]))[0], 0.9, gi.cpu().numpy(), gc.cpu().numpy(),
+                           gs.cpu().numpy(), oi, oc, os_, od)
+        assert st["n"] == 2
+    # a single row, searched in place with the literal bisection
+    row = wl.topp_rows("zipf", 2, Ls, 3).reshape(2, 1, 1, Ls)
+    gi, gc, gs, _ = sa.select_topp([to_dev(row)], to_dev(kv), [0], 0.9, **variant)
+    oi, oc, os_, od = oracle.select_variant([row], [0], kv, 0.9, **{"n_iters" if k == "bisect_iters" else k: v for k, v in variant.items()})
+    _compare_variant(gi, gc, gs, oi, oc, os_, od)
+
+
+@pytest.mark.parametrize("n_rows,n", [(32, 131069), (70, 65541)])
+@pytest.mark.parametrize("family", ["narrow", "denormal", "sparse", "huge", "quantised"])
+def test_rows_streamed_by_clusters(family, n_rows, n, form):
+    """A streamed row dealt to four or two CTAs: more keys in the bin than are gathered, denormals, a row whose values
+    all lie in one CTA's slice, values up to 2^100, -0.0, an invalid input in one slice, short and empty rows."""
+    if form == "cluster":
+        pytest.skip("single-row lists take the same path with and without a workspace")
+    import paper_2510_27641_b200 as sa
+    Ls = (n + 3) // 4 * 4
+    a = np.random.default_rng(n_rows).random((n_rows, n), dtype=np.float32)
+    a = {"narrow": lambda: np.float32(1.0) + a * np.float32(2.0 ** -7), "denormal": lambda: a * np.float32(1e-41),
+         "sparse": lambda: a * (a > 0.98), "huge": lambda: np.exp2(a * 100.0),
+         "quantised": lambda: wl.topp_rows("quantised", n_rows, n, seed=4)}[family]().astype(np.float32)
+    rows = np.full((n_rows, Ls), np.float32(7.0))
+    rows[:, :n] = a
+    rows[0, ::5] = -0.0
+    rows[1, : n - 3000] = 0.0
+    rows[2, n - 1] = np.nan
+    rows[3, 0] = -1e-30
+    kv = np.full(n_rows, n, np.int32)
+    kv[4], kv[5], kv[6] = 1, 0, 40000
+    sample = [0, 1, 2, 3, 4, 5, 6, n_rows - 1]
+    for p in (0.02, 0.9, 0.999):
+        gi, gc, gs, gd = sa.select_topp.func([to_dev(rows.reshape(n_rows, 1, 1, Ls))], to_dev(kv), [0], p, want_diag=True)
+        torch.cuda.synchronize()
+        assert torch.nonzero(gs.flatten()).flatten().tolist() == [2, 3]
+        oi, oc, os_, od = oracle.select_topp([rows[sample].reshape(8, 1, 1, Ls)], np.zeros(1, np.int32), kv[sample], p)
+        st = compare_lists(lambda i: rows[sample][i, :kv[sample][i]], p, gi.cpu().numpy()[:, sample], gc.cpu().numpy()[:, sample],
+                           gs.cpu().numpy()[:, sample], oi, oc, os_, od)
+        assert st["n"] == 8
+        ok = gs.cpu().numpy()[0, sample, 0] == 0
+        assert np.allclose(gd.cpu().numpy()[0, sample, 0][ok], od[0, :, 0, :4][ok], rtol=1e-9, atol=0)
