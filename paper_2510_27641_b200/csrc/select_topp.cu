@@ -30,6 +30,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <type_traits>
 
@@ -747,9 +748,10 @@ int rows_at_once(const void* kernel, int dev, int cs) {
 // The two-launch form applies to the default selection over multi-row lists of >= 2048
 // positions, and pays when one cluster per list would leave SMs without a CTA: a CTA streams
 // ~35 GB/s, so the cluster kernel is bound by (bytes per list) / (8 x 35 GB/s) however few the
-// lists, while the search launch adds ~25 us of its own.  Measured (us, cluster / two-launch):
-// 4 lists x 64 rows x 131072: 121 / 94; 16 such lists: 237 / 152; 32 lists x 60 rows x 32768
-// (256 CTAs): 71 / 94.
+// lists, while the search launch adds ~13 us of its own.  Measured (us, cluster / two launches, lists of 48 rows):
+// 4 x 4096 positions 23 / 20; 18 x 16384 27 / 30; 8 x 32768 36 / 28; 18 x 32768 42 / 42; 32 x 32768 59 / 58;
+// 4 x 131072 97 / 42; 18 x 131072 188 / 101; 18 x 196608 218 / 144.  (Lists longer than 131072 take clusters of
+// sixteen, since only those hold them; their SMs stream no faster, so they count like clusters of eight.)
 bool two_launch_shape(const specattn_select_args& A) {
   const bool variant = (A.per_step && A.gamma > 1) || A.bisect_iters > 0 || A.chunk > 1;
   if (variant || static_cast<long long>(A.n_draft_heads) * A.gamma <= 1 || A.L_stride < 2048 || A.L_stride % 4 != 0)
@@ -757,7 +759,7 @@ bool two_launch_shape(const specattn_select_args& A) {
   const long long n_lists = count_lists(A);
   if (n_lists <= 0 || A.form == SPECATTN_SELECT_FORM_CLUSTER) return false;
   if (A.form == SPECATTN_SELECT_FORM_TWO_LAUNCH) return true;  // the caller knows its batch (ragged lengths)
-  return n_lists * pick_cluster(A.L_stride, n_lists) < 148;
+  return n_lists * std::min(pick_cluster(A.L_stride, n_lists), 8) < 148;
 }
 
 }  // namespace

@@ -121,3 +121,16 @@ def test_select_workspace_query_follows_the_documented_rule(sa):
     assert L.specattn_select_workspace_bytes(None) == 0
     bad = sa.SelectArgs()
     assert L.specattn_select_workspace_bytes(C.byref(bad)) == 0   # struct_size not set
+
+
+def test_lists_beyond_131072_positions_ask_for_a_workspace_like_shorter_ones(sa):
+    """Clusters of sixteen, which only hold such lists, do not stream faster than clusters of eight."""
+    a = sa.SelectArgs()
+    a.struct_size = C.sizeof(sa.SelectArgs)
+    a.n_draft_layers = a.n_target_layers = 1
+    a.layer_map = (C.c_int32 * 1)(0)
+    a.n_draft_heads, a.gamma, a.n_groups = 12, 4, 1
+    for Ls in (131072, 131076, 196608):
+        for batch in (1, 9, 10, 18, 19):
+            a.batch, a.L_stride = batch, Ls
+            assert sa.lib().specattn_select_workspace_bytes(C.byref(a)) == (batch * Ls * 4 if batch <= 18 else 0)
