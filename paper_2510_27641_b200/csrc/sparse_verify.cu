@@ -112,13 +112,25 @@ struct Partition {
   int cluster;               // of the partition: 1 where parts merge through global memory
 };
 
+// What the partition weighs depends on the kernel (an atom takes about 0.23 us with up to 32 query rows, 0.33 with
+// more).  A merge of r records through global memory costs, in atoms' time: 20 rows, 8 units in 4 / 8 / 15 parts
+// 5 / 17 / 49, 16 units in eight 26, 32 in four 11; 40 rows 3 / 11 / 29, 17, 8, 40 units in three 11.
+__device__ __forceinline__ int merge_cost(int rows, int r) { return (rows <= 32) ? 6 + 3 * r : 8 + (3 * r) / 2; }
+
 // Parts of a unit for a target share of `share` atoms, out of U units on G CTAs.  Inside clusters a part has at
 // least kMinPartAtoms atoms, half as many again where all the parts would take more than half of the GPU (32
-// units of 19 atoms: 8.5 us in four parts, 7.6 us in two; 8 such units: 6.3 us in four, 7.3 us in two).
-__device__ __forceinline__ int unit_parts(int atoms, int share, int cluster, int U, int G) {
+// units of 19 atoms: 8.5 us in four parts, 7.6 us in two; 8 such units: 6.3 us in four, 7.3 us in two), and three times
+// as many where up to 32 query rows would take most of it in more than two parts a unit (20 rows, 32 units of 32 atoms,
+// four / two parts: 10.75 / 9.5 us, 24 units 9.7 / 9.2; of 69 atoms 14.1 / 15.9; 8 units of 69, eight / four: 10.0 / 10.5).
+__device__ __forceinline__ int unit_parts(int atoms, int share, int cluster, int U, int G, int rows) {
   if (cluster == 1) return max(1, min((atoms + share / 2) / share, atoms / kMinGlobalAtoms));
   int k = cluster;
-  while (k > 1 && (2 * k * kMinPartAtoms > ((2 * U * k > G) ? atoms + atoms / 3 : 2 * atoms) || (k >> 1) * share >= atoms)) k >>= 1;
+  for (; k > 1; k >>= 1) {
+    const int least = (rows <= 32 && k > 2 && 3 * U * k > 2 * G) ? 3 * kMinPartAtoms
+                      : (2 * U * k > G)                          ? kMinPartAtoms + kMinPartAtoms / 2
+                                                                 : kMinPartAtoms;
+    if (k * least <= atoms && (k >> 1) * share < atoms) break;
+  }
   return k;
 }
 
@@ -137,7 +149,7 @@ __device__ __forceinline__ int class_of(int k, int cluster) { return __ffs(clust
 // place(unit, first CTA, number of parts) for every unit of an aligned partition, each from one thread.  Two
 // barriers (three where both kinds of aligned partition are compared one after the other), none after the last place().
 template <int NT, class Place>
-__device__ __forceinline__ int partition_units(Partition& pt, const int* unit_start, int U, int G, int& cluster, Place place) {
+__device__ __forceinline__ int partition_units(Partition& pt, const int* unit_start, int U, int G, int rows, int& cluster, Place place) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int N = unit_start[U];
   const bool try_aligned = U <= kAlignedMaxUnits && N > 0;
@@ -155,7 +167,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
       for (int u = lane; u < U; u += 32) {
         const int atoms = unit_start[u + 1] - unit_start[u];
         if (atoms == 0) continue;
-        const int k = unit_parts(atoms, share, cl, U, G);
+        const int k = unit_parts(atoms, share, cl, U, G, rows);
         sum += k;
         big = max(big, (atoms + k - 1) / k);
         most = max(most, atoms);
@@ -174,19 +186,19 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   __syncthreads();
   if (try_aligned && cluster > 2) {
     // Larger clusters: where the cluster's size leaves the longest unit in parts far above the average (8 units
-    // of 2900 and 8 of 480 atoms on 148 SMs, 64 rows each: 41.4 us in clusters, 37.9 anywhere).
+    // of 2900 and 8 of 480 atoms on 148 SMs, 64 rows each: 41.4 us in clusters, 37.9 anywhere; 8 units of 813, 40
+    // rows: 41.2 and 35.1).
     int part = 0;
     for (int c = 0; c < kCandidates && part == 0; ++c)
       if (pt.parts[0][c] <= G) part = pt.largest[0][c];
     const int fair = N / G + 1;
-    if (part + 3 > fair + 6 + 3 * (pt.unit_max / fair + 1)) {
+    if (part + 3 > fair + merge_cost(rows, pt.unit_max / fair + 1)) {
       consider(kCandidates, 2 * kCandidates);
       way_hi = 2;
       __syncthreads();
     }
   }
-  // Costs in atoms' time (~0.23 us): a straddling CTA ~24; a unit's merge through global memory ~6 and ~3 a record;
-  // inside a cluster ~3.
+  // Costs in atoms' time: a straddling CTA ~24; a unit's merge through global memory as above; inside a cluster ~3.
   int cand = -1, way = 1;
   if (try_aligned) {
     int best = (N + kSegAtoms * U) / G + 24 + 3 * (pt.unit_max / (N / G + 1) + 1);
@@ -194,7 +206,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
       for (int c = 0; c < kCandidates; ++c) {
         if (pt.parts[w][c] > G) continue;
         const int part = pt.largest[w][c];
-        const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : 6 + 3 * ((pt.unit_max + part - 1) / part));
+        const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : merge_cost(rows, (pt.unit_max + part - 1) / part));
         if (cost <= best) {
           best = cost;
           cand = c;
@@ -212,7 +224,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   for (int base = (tid >> 5) * 32; base < U; base += NT) {
     const int u = base + lane;
     const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G, rows) : 0;
     const int at = (cluster == 1) ? 0 : 16 * class_of(k, cluster);
     const unsigned one = (k == 0) ? 0u : (cluster == 1) ? static_cast<unsigned>(k) : 1u << (at & 31);
     const unsigned long long hi = __reduce_add_sync(0xffffffffu, at < 32 ? 0u : one);
@@ -223,7 +235,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   for (int base = (tid >> 5) * 32; base < U; base += NT) {
     const int u = base + lane;
     const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G) : 0;
+    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G, rows) : 0;
     unsigned long long before = 0ull, all = 0ull;
     for (int i = 0; i < (U + 31) / 32; ++i) {
       if (32 * i < base) before += pt.units[i];
@@ -375,7 +387,7 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
     *reinterpret_cast<int2*>(p_cta + 4 * i) = make_int2(a0, a1);
     *reinterpret_cast<int2*>(p_cta + 4 * i + 2) = make_int2(u_first, what);
   };
-  const int cand = partition_units<256>(pt, unit_start, U, G, cluster, [&](int u, int first, int k) {
+  const int cand = partition_units<256>(pt, unit_start, U, G, P.M, cluster, [&](int u, int first, int k) {
     const int us = unit_start[u], atoms = unit_start[u + 1] - us;
     for (int j = 0; j < k; ++j) entry(first + j, us + j * atoms / k, us + (j + 1) * atoms / k, u, j | (k << 8));
   });
@@ -815,7 +827,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
 
   N = sh.unit_start[U];
   cluster = P.cluster;
-  const int cand = partition_units<NT>(sh.part, sh.unit_start, U, G, cluster, [&](int u, int first, int k) {
+  const int cand = partition_units<NT>(sh.part, sh.unit_start, U, G, 16 * MT, cluster, [&](int u, int first, int k) {
     const int j = static_cast<int>(blockIdx.x) - first;
     if (j >= 0 && j < k) {
       sh.part.mine[0] = u;

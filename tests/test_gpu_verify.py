@@ -605,3 +605,32 @@ def test_a_plan_for_clusters_of_another_size_is_ignored():
         other[8 + 2 * (2 * 8 + 1):] = 0                    # no CTA has work
         got = call(a, out, lse, other.to(dev()))
         assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("batch,n_q,n_q_heads,tokens,parts,cluster", [
+    (1, 5, 64, 13000, 15, 1),    # 40 rows: more parts than a cluster has CTAs, wherever there is room
+    (1, 5, 64, 1100, 8, 8),
+    (1, 5, 32, 1100, 8, 8),      # 20 rows
+    (4, 5, 32, 500, 2, 4),       # four parts of eight atoms each would take most of the GPU
+    (4, 5, 32, 1100, 4, 4),
+    (4, 5, 64, 500, 4, 4),
+    (6, 5, 32, 300, 2, 2),
+    (6, 5, 64, 800, 2, 2),
+])
+def test_how_units_are_cut(batch, n_q, n_q_heads, tokens, parts, cluster):
+    """Parts per unit where the two ways of merging them, or two numbers of parts, come close (8 KV heads, equal lists)."""
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC or torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the plan of the mma.sync engine on 148 SMs")
+    d = dev()
+    keep = [torch.zeros(batch, n_q, n_q_heads, 128, dtype=torch.bfloat16, device=d),
+            torch.zeros(1, 2, 16, 8, 128, dtype=torch.bfloat16, device=d),
+            torch.full((batch,), 65536, dtype=torch.int32, device=d), torch.zeros(batch, 4096, dtype=torch.int32, device=d),
+            torch.zeros(batch, 1, 65536, dtype=torch.int32, device=d),
+            torch.full((batch, 1), tokens, dtype=torch.int32, device=d), torch.zeros(4, device=d), torch.zeros(4, device=d)]
+    a = sa.make_verify_args(keep[0], keep[1], keep[2], block_table=keep[3], idx=keep[4], counts=keep[5], out=keep[6],
+                            lse=keep[7], flags=_ENGINE["flags"])
+    plan = sa.verify_plan_buffer(a)
+    sa.verify_plan(a, plan)
+    words = plan[:8].cpu().tolist()
+    assert words[3] & 0xff == cluster and words[4] == 8 * batch * parts
