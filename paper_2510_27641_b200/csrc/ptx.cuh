@@ -97,9 +97,9 @@ __device__ __forceinline__ float4 ld_cluster_v4(uint32_t cluster_addr) {
   return v;
 }
 // The two halves of a cluster barrier: arrive early, wait only where the peer's state is needed.
-// (relaxed: what the peer must see -- the mbarrier initialisation -- has its own
-// fence.mbarrier_init.release.cluster; a releasing arrive would also wait for every earlier
-// shared-memory store of the thread, ~0.7 us at kernel start)
+// (relaxed: for an arrival that only tells the peers that their shared memory has been read.  The values read
+// were consumed by instructions before it, so the reads are done; a releasing arrival would also wait for the
+// thread's earlier stores, ~0.7 us where outputs have just been written)
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }

@@ -21,9 +21,11 @@
 //     runs long independent chains: S = Q K^T and O += P V on the tensor cores (bf16 mma.sync,
 //     fp32 accumulate; P is split into two bf16 terms so that it carries 16 mantissa bits),
 //     online softmax in fp32 registers in the log2 domain;
-//   - at the end of a unit the warps of a slab combine through shared memory; a unit that was
-//     cut between CTAs is finished by whichever CTA arrives last at the unit's counter, which
-//     merges all partial (O, m, l) records in a fixed order -- nobody ever waits on a peer.
+//   - at the end of a unit the warps of a slab combine through shared memory.  A unit whose parts all
+//     lie in one thread-block cluster is merged there: after one cluster barrier every CTA reads its
+//     share of the output columns from all parts' records (merge_cluster).  A unit that was cut
+//     otherwise is finished by whichever CTA arrives last at the unit's counter, which merges all
+//     partial (O, m, l) records from global memory in a fixed order, without anybody waiting.
 // Every mbarrier wait is bounded; on expiry the CTA flags SPECATTN_ROW_TIMEOUT and leaves.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -1422,11 +1424,11 @@ int m_tiles(const specattn_verify_args& A) {
 // Whether the host can tell that lists may be too long for clusters of cs: by idx_stride, where that is a bound of
 // its own (well below the cache's room) and not the room itself.  (Dense calls count as lists of the room, with
 // which they share every bit of their results.)
-// Clusters of four and eight leave up to a tenth of the SMs without one.  Short lists gain more from the merge
-// inside a cluster; long ones, of the kernels that the consumers bound (33 to 64 query rows), lose (us, clusters /
-// pairs): clusters of eight, 1 x 8 units of 4000 tokens 16.6 / 22.0, of 8000 27.0 / 27.3, of 13000 40.3 / 32.9;
-// 2 x 8 units of 4000 22.2 / 22.9, of 8000 32.9 / 32.0; clusters of four, 4 x 8 units of 8000 49.9 / 52.8,
-// of 13000 78.2 / 76.3, of 30000 173 / 159.
+// A launch in clusters of four has 132 CTAs on 148 SMs, one in clusters of eight 120.  Short lists gain more from the
+// merge inside a cluster; long ones, of the kernels that the consumers bound (33 to 64 query rows), lose (40 rows, us,
+// clusters / pairs): clusters of eight, 8 units of 4000 tokens 18.2 / 23.6, of 8000 28.4 / 28.7, of 13000 35.1 / 34.3,
+// of 30000 59.7 / 54.5; clusters of four, 16 units of 2000 17.4 / 19.5, of 8000 34.8 / 33.5, of 30000 94 / 88; 32 units
+// of 8000 51.7 / 53.8, of 13000 78.1 / 77.8, of 30000 172 / 159.
 bool long_lists(const specattn_verify_args& A, int cs) {
   const long long line = (cs > 4) ? 6144 : 12288;
   const long long room = A.block_table_stride * A.page_size;  // (pages per sequence also without a block table)

@@ -250,7 +250,7 @@ def test_selection_variants_special_cases():
     oi, oc, os_, od = oracle.select_variant([bad], [0], kv, 0.9, per_step=True, n_iters=10)
     assert gs.cpu().numpy().reshape(-1).tolist() == os_.reshape(-1).tolist() == [sa.ROW_INVALID_PROB, 0]
     assert gc.cpu().numpy().reshape(-1).tolist() == oc.reshape(-1).tolist()
-    # a single long row (read in place) with the literal bisection
+    # a single long row (held by a cluster) with the literal bisection
     row = wl.topp_rows("zipf", 2, 65536, 3).reshape(2, 1, 1, 65536)
     kv1 = np.array([65536, 50001], np.int32)
     gi, gc, gs, _ = sa.select_topp([to_dev(row)], to_dev(kv1), [0], 0.9, bisect_iters=10)
@@ -351,13 +351,10 @@ def test_both_forms_give_the_same_bits_and_flag_hidden_negative_inputs(form):
 @pytest.mark.parametrize("n", [1024, 4096, 40000])
 @pytest.mark.parametrize("n_bin", [1, 37, 128, 129, 512, 513])
 def test_threshold_bin_population_around_the_short_cut_capacity(n, n_bin):
-    """The search takes a short cut when the level-1 threshold bin can hold at most 512 values
-    (it gathers them instead of refining with two more histogram levels over the row; up to 128
-    gathered values are searched directly, more through two histogram levels over the gathered
-    values).  Rows whose threshold
-    bin holds exactly n_bin distinct values just above 2^-10 (so the bin's mantissa sum >> 23
-    equals n_bin), for populations on both sides of that capacity, in a shared-memory slice
-    (n = 1024), a row read in place by one CTA and one read by a cluster."""
+    """The keys of the level-1 threshold bin are gathered; up to 128 of them (32 after a histogram level over the
+    gathered ones) are compared in pairs, more go through a histogram level first.  Rows whose threshold bin holds
+    exactly n_bin distinct values just above 2^-10, for populations on both sides of those numbers, in one
+    small CTA (n = 1024), one large one and a cluster."""
     rng = np.random.default_rng(n + n_bin)
     rows = np.full((3, n), 1e-9, np.float32)
     for r in range(3):
@@ -435,7 +432,7 @@ def test_sum_overflow_voids_the_list_like_the_oracle(variant):
 
 
 def test_single_rows_at_the_edge_of_binary32():
-    """R = 1 (a row read in place from 2048 positions on, and the shared-memory path below that):
+    """R = 1 (a large CTA, and the small one of rows up to 2048 positions):
     FLT_MAX is a valid value, +inf is not."""
     for n in (1024, 4096):
         rows = np.full((3, n), 1e-3, np.float32)
@@ -683,7 +680,7 @@ def test_aggregated_lists_beyond_131072_positions(variant):
         st = compare_lists(lambda i: oracle.aggregate(probs[i], L=int(kv[i]))[0], 0.9, gi.cpu().numpy(), gc.cpu().numpy(),
                            gs.cpu().numpy(), oi, oc, os_, od)
         assert st["n"] == 2
-    # a single row, searched in place with the literal bisection
+    # a single row with the variants
     row = wl.topp_rows("zipf", 2, Ls, 3).reshape(2, 1, 1, Ls)
     gi, gc, gs, _ = sa.select_topp([to_dev(row)], to_dev(kv), [0], 0.9, **variant)
     oi, oc, os_, od = oracle.select_variant([row], [0], kv, 0.9, **{"n_iters" if k == "bisect_iters" else k: v for k, v in variant.items()})
