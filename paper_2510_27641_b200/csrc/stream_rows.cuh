@@ -23,8 +23,8 @@
 // target exactly, rows of tiny values -- the row is searched once more with the low bits added up
 // per octave too (a second atomic), in the same integers and with the same comparisons as the search in shared memory.
 // The lists are therefore the same in every form.
-// 256 rows of 131072, p = 0.9, uniform / Zipf / ties: 96 / 81 / 93 us; with exact two-word bins, votes and 128-entry
-// emission 117 / 102 / 142.
+// 256 rows of 131072, p = 0.9, uniform / Zipf / ties: 96 / 81 / 93 us against 117 / 102 / 142 with exact two-word bins,
+// votes and 128-entry emission; the test against rounding then added 1 % (cold cache 102 / 90 / 96 -> 104 / 90 / 97).
 #pragma once
 
 constexpr int kStreamThreads = 512;
