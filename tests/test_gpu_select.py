@@ -719,3 +719,27 @@ def test_rows_streamed_by_clusters(family, n_rows, n, form):
         assert st["n"] == 8
         ok = gs.cpu().numpy()[0, sample, 0] == 0
         assert np.allclose(gd.cpu().numpy()[0, sample, 0][ok], od[0, :, 0, :4][ok], rtol=1e-9, atol=0)
+
+
+@pytest.mark.parametrize("idx_stride", [777, 98301, None])
+def test_rows_streamed_by_clusters_into_short_and_unaligned_lists(idx_stride, form):
+    """Lists of several draft layers (one of them unmapped) whose rows two CTAs stream: list buffers shorter than the
+    lists, and of a length that puts every second list off a 16-byte boundary."""
+    if form == "cluster":
+        pytest.skip("single-row lists take the same path with and without a workspace")
+    import paper_2510_27641_b200 as sa
+    B, n = 30, 98301
+    lens = np.linspace(n // 3, n, B).astype(np.int32)
+    probs = [np.random.default_rng(u).random((B, 1, 1, n + 3), dtype=np.float32) ** 4 for u in range(3)]
+    idx = torch.full((3, B, 1, idx_stride or n + 3), -7, dtype=torch.int32, device=dev())
+    gi, gc, gs, gd = sa.select_topp([to_dev(x) for x in probs], to_dev(lens), [0, 2, 2, -1], 0.8, idx=idx, want_diag=True)
+    torch.cuda.synchronize()
+    assert torch.all(gi[1] == -7) and torch.all(gc[1] == -1)
+    oi, oc, os_, od = oracle.select_topp([probs[0], None, probs[2]], np.array([0, 2, 2, -1], np.int32), lens, 0.8,
+                                         idx_stride=idx.shape[3])
+    st = compare_lists(lambda i: probs[i // B][i % B, 0, 0, :lens[i % B]], 0.8, gi.cpu().numpy(), gc.cpu().numpy(),
+                       gs.cpu().numpy(), oi, oc, os_, od)
+    assert st["n"] == 2 * B
+    for u in (0, 2):
+        for b in range(B):
+            assert torch.all(gi[u, b, 0, min(int(gc[u, b, 0]), idx.shape[3]):] == -7)   # nothing behind the list
