@@ -152,7 +152,7 @@ class _Calls(threading.local):
     def __init__(self):
         self.made = {}
 
-    def get(self, key, make):
+    def get(self, key, make, *given):
         try:
             call = self.made.get(key)
         except TypeError:
@@ -161,7 +161,7 @@ class _Calls(threading.local):
             key = _plain(key)
             call = self.made.get(key)
         if call is None:
-            call = make()
+            call = make(*given)
             if len(self.made) >= self.LIMIT:
                 self.made.clear()
             self.made[key] = call
@@ -232,34 +232,30 @@ def select_topp(draft_probs: Sequence[torch.Tensor | None], kv_len: torch.Tensor
     [B, H_d, gamma, L_stride] (None for layers no target layer maps to).  Returns
     (idx [n_d,B,G,idx_stride] int32, counts [n_d,B,G], row_status [n_d,B,G], diag or None)."""
     n_d = len(draft_probs)
-    ref = next(t for t in draft_probs if t is not None)
+    ref = draft_probs[0]
+    if ref is None:
+        ref = next(t for t in draft_probs if t is not None)
     shape, layer_map = ref.shape, tuple(layer_map)
-    B, Ls = shape[0], shape[3]
-    dev = ref.device
     if idx is None:
-        idx = torch.empty((n_d, B, n_groups, int(Ls if idx_stride is None else idx_stride)), dtype=torch.int32, device=dev)
-    # the library leaves the entries of unmapped draft layers alone
-    new = torch.empty if set(layer_map).issuperset(range(n_d)) else _minus_one
-    if counts is None:
-        counts = new((n_d, B, n_groups), dtype=torch.int32, device=dev)
-    if row_status is None:
-        row_status = new((n_d, B, n_groups), dtype=torch.int32, device=dev)
+        idx = torch.empty((n_d, shape[0], n_groups, int(shape[3] if idx_stride is None else idx_stride)), dtype=torch.int32,
+                          device=ref.device)
+    if counts is None or row_status is None:
+        # the library leaves the entries of unmapped draft layers alone
+        new = torch.empty if set(layer_map).issuperset(range(n_d)) else _minus_one
+        if counts is None:
+            counts = new((n_d, shape[0], n_groups), dtype=torch.int32, device=ref.device)
+        if row_status is None:
+            row_status = new((n_d, shape[0], n_groups), dtype=torch.int32, device=ref.device)
     if diag is None and want_diag:
-        diag = torch.zeros((n_d, B, n_groups, 4), dtype=torch.float64, device=dev)
-    held = tuple([t is not None for t in draft_probs])
-    groups = None if head_group is None else tuple(head_group)
-    key = (held, shape, layer_map, p, n_groups, groups, idx.shape, per_step, bisect_iters, chunk, form)
-
-    def make():
-        args, keep = make_select_args(draft_probs, kv_len, layer_map, p, n_groups=n_groups, head_group=head_group,
-                                      idx=idx, counts=counts, row_status=row_status, diag=diag, per_step=per_step,
-                                      bisect_iters=bisect_iters, chunk=chunk, workspace=None, form=form)
-        return args, C.byref(args), keep[:3], int(lib().specattn_select_workspace_bytes(C.byref(args)))
-
-    args, ref_args, (ptrs, _, _), need = _calls.get(key, make)
+        diag = torch.zeros((n_d, shape[0], n_groups, 4), dtype=torch.float64, device=ref.device)
+    held = None if n_d == 1 else tuple([t is not None for t in draft_probs])
+    key = (held, shape, layer_map, p, n_groups, None if head_group is None else tuple(head_group), idx.shape, per_step,
+           bisect_iters, chunk, form)
+    args, ref_args, (ptrs, _, _), need = _calls.get(key, _make_select, draft_probs, kv_len, layer_map, p, n_groups, head_group, idx,
+                                            counts, row_status, diag, per_step, bisect_iters, chunk, form)
     for u, t in enumerate(draft_probs):
         if t is not None:
-            assert t.dtype is torch.float32 and t.is_contiguous() and t.shape == shape
+            assert t.dtype is torch.float32 and t.is_contiguous() and (t is ref or t.shape == shape)
             ptrs[u] = t.data_ptr()
     assert kv_len.dtype is torch.int32 and idx.dtype is torch.int32 and counts.dtype is torch.int32
     assert idx.is_contiguous()
@@ -268,7 +264,7 @@ def select_topp(draft_probs: Sequence[torch.Tensor | None], kv_len: torch.Tensor
     args.diag = None if diag is None else diag.data_ptr()
     given = workspace
     if workspace is True:
-        workspace = torch.empty((need,), dtype=torch.uint8, device=dev) if need > 0 else None
+        workspace = torch.empty((need,), dtype=torch.uint8, device=ref.device) if need > 0 else None
     elif workspace is False:
         workspace = None
     if workspace is None:
@@ -282,6 +278,15 @@ def select_topp(draft_probs: Sequence[torch.Tensor | None], kv_len: torch.Tensor
     if workspace is not None and stream is not None and given is True:
         workspace.record_stream(stream)   # allocated here, used on the caller's stream
     return idx, counts, row_status, diag
+
+
+def _make_select(draft_probs, kv_len, layer_map, p, n_groups, head_group, idx, counts, row_status, diag, per_step,
+                 bisect_iters, chunk, form):
+    args, keep = make_select_args(draft_probs, kv_len, layer_map, p, n_groups=n_groups, head_group=head_group,
+                                  idx=idx, counts=counts, row_status=row_status, diag=diag, per_step=per_step,
+                                  bisect_iters=bisect_iters, chunk=chunk, workspace=None, form=form)
+    # (the struct points at three arrays)
+    return args, C.byref(args), keep[:3], int(lib().specattn_select_workspace_bytes(C.byref(args)))
 
 
 def _minus_one(shape, dtype, device):
@@ -354,15 +359,14 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
                   flags: int = 0, tail_len: int = 0, stream=None):
     """specattn_sparse_verify for one target layer.  Returns (out f32 [B,T,H_q,d], lse f32
     [B,T,H_q], status int32 [B])."""
-    B, T, Hq, d = shape = q.shape
-    dev = q.device
+    shape, dev = q.shape, q.device
     own = 0   # what the call has to clear: buffers that were made here
     if out is None:
         out = torch.empty(shape, dtype=torch.float32, device=dev)
     if lse is None:
-        lse = torch.empty((B, T, Hq), dtype=torch.float32, device=dev)
+        lse = torch.empty(shape[:3], dtype=torch.float32, device=dev)
     if status is None:
-        status = torch.empty((B,), dtype=torch.int32, device=dev)
+        status = torch.empty(shape[:1], dtype=torch.int32, device=dev)
         own |= VERIFY_INIT_STATUS
     made = workspace is None
     if made:
@@ -370,14 +374,8 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
     key = (shape, kv_pages.shape, kv_pages.stride(), None if block_table is None else block_table.stride(),
            pages_per_seq, None if dense else (idx.shape, idx.stride()), n_groups, dense, sm_scale, flags, tail_len,
            _raw_device())   # (whose number of SMs decides the workspace's size)
-
-    def make():
-        a = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq, idx=idx,
-                             counts=counts, n_groups=n_groups, dense=dense, sm_scale=sm_scale, out=out, lse=lse,
-                             flags=flags, tail_len=tail_len)
-        return a, C.byref(a), verify_workspace_bytes(a)
-
-    args, ref_args, need = _calls.get(key, make)
+    args, ref_args, need = _calls.get(key, _make_verify, q, kv_pages, kv_len, block_table, pages_per_seq, idx, counts,
+                                      n_groups, dense, sm_scale, out, lse, flags, tail_len)
     assert q.is_contiguous() and q.dtype is torch.bfloat16 and kv_pages.dtype is torch.bfloat16
     if made:
         if need == 0:
@@ -399,6 +397,14 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
     if made and stream is not None:
         workspace.record_stream(stream)   # allocated here, used on the caller's stream
     return out, lse, status
+
+
+def _make_verify(q, kv_pages, kv_len, block_table, pages_per_seq, idx, counts, n_groups, dense, sm_scale, out, lse, flags,
+                 tail_len):
+    a = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq, idx=idx,
+                         counts=counts, n_groups=n_groups, dense=dense, sm_scale=sm_scale, out=out, lse=lse,
+                         flags=flags, tail_len=tail_len)
+    return a, C.byref(a), verify_workspace_bytes(a)
 
 
 def verify_plan_buffer(args: VerifyArgs, device=None) -> torch.Tensor:
