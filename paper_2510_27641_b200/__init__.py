@@ -359,14 +359,15 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
                   flags: int = 0, tail_len: int = 0, stream=None):
     """specattn_sparse_verify for one target layer.  Returns (out f32 [B,T,H_q,d], lse f32
     [B,T,H_q], status int32 [B])."""
-    shape, dev = q.shape, q.device
+    B, T, Hq, d = shape = q.shape
+    dev = q.device
     own = 0   # what the call has to clear: buffers that were made here
     if out is None:
         out = torch.empty(shape, dtype=torch.float32, device=dev)
     if lse is None:
-        lse = torch.empty(shape[:3], dtype=torch.float32, device=dev)
+        lse = torch.empty((B, T, Hq), dtype=torch.float32, device=dev)
     if status is None:
-        status = torch.empty(shape[:1], dtype=torch.int32, device=dev)
+        status = torch.empty((B,), dtype=torch.int32, device=dev)
         own |= VERIFY_INIT_STATUS
     made = workspace is None
     if made:
@@ -374,8 +375,14 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
     key = (shape, kv_pages.shape, kv_pages.stride(), None if block_table is None else block_table.stride(),
            pages_per_seq, None if dense else (idx.shape, idx.stride()), n_groups, dense, sm_scale, flags, tail_len,
            _raw_device())   # (whose number of SMs decides the workspace's size)
-    args, ref_args, need = _calls.get(key, _make_verify, q, kv_pages, kv_len, block_table, pages_per_seq, idx, counts,
-                                      n_groups, dense, sm_scale, out, lse, flags, tail_len)
+
+    def make():
+        a = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq, idx=idx,
+                             counts=counts, n_groups=n_groups, dense=dense, sm_scale=sm_scale, out=out, lse=lse,
+                             flags=flags, tail_len=tail_len)
+        return a, C.byref(a), verify_workspace_bytes(a)
+
+    args, ref_args, need = _calls.get(key, make)
     assert q.is_contiguous() and q.dtype is torch.bfloat16 and kv_pages.dtype is torch.bfloat16
     if made:
         if need == 0:
@@ -397,14 +404,6 @@ def sparse_verify(q: torch.Tensor, kv_pages: torch.Tensor, kv_len: torch.Tensor,
     if made and stream is not None:
         workspace.record_stream(stream)   # allocated here, used on the caller's stream
     return out, lse, status
-
-
-def _make_verify(q, kv_pages, kv_len, block_table, pages_per_seq, idx, counts, n_groups, dense, sm_scale, out, lse, flags,
-                 tail_len):
-    a = make_verify_args(q, kv_pages, kv_len, block_table=block_table, pages_per_seq=pages_per_seq, idx=idx,
-                         counts=counts, n_groups=n_groups, dense=dense, sm_scale=sm_scale, out=out, lse=lse,
-                         flags=flags, tail_len=tail_len)
-    return a, C.byref(a), verify_workspace_bytes(a)
 
 
 def verify_plan_buffer(args: VerifyArgs, device=None) -> torch.Tensor:
