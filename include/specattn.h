@@ -346,10 +346,11 @@ int specattn_verify_plan_many(const specattn_verify_args* const* args, void* con
  *
  * Same arguments, results and status codes as specattn_sparse_verify, except:
  *   - args->workspace and args->workspace_bytes are ignored;
- *   - a shape whose scratch need (specattn_verify_workspace_bytes) exceeds
- *     SPECATTN_STATIC_SCRATCH_BYTES is rejected with SPECATTN_ERR_STATIC_SCRATCH and nothing
- *     is launched.  The buffer covers up to 32 query rows per KV head (n_q * group <= 32) on
- *     GPUs with up to 160 SMs;
+ *   - a shape that needs more scratch than SPECATTN_STATIC_SCRATCH_BYTES is rejected with
+ *     SPECATTN_ERR_STATIC_SCRATCH and nothing is launched.  The buffer covers up to 32 query rows per
+ *     KV head (n_q * group <= 32) on GPUs with up to 160 SMs.  (Batches of many sequences, for which
+ *     specattn_verify_workspace_bytes asks for more because two CTAs share an SM, run with one CTA per SM
+ *     where the buffer does not hold that much; so does specattn_sparse_verify with such a workspace.);
  *   - the first call on each device looks up the device address of the array (with that
  *     device current); make that first call outside any stream capture;
  *   - all calls on a device share the one array, which still holds what the previous call left

@@ -139,7 +139,7 @@ __device__ __forceinline__ int unit_parts(int atoms, int share, int cluster, int
 // Candidate share c: (N / G) (1 + c / 7), rounded up -- rounding part counts up to the chain can ask for
 // twice the CTAs.
 __device__ __forceinline__ int cand_share(long long N, int G, int c) {
-  // 32-bit: N <= 2048 * 12288
+  // 32-bit: N <= 2048 * 12288, times 21
   return static_cast<int>((static_cast<unsigned>(N) * (7u + c) + 7u * G - 1u) / (7u * G));
 }
 
@@ -155,6 +155,8 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   const int tid = threadIdx.x, lane = tid & 31;
   const int N = unit_start[U];
   const bool try_aligned = U <= kAlignedMaxUnits && N > 0;
+  // (CTAs of half an SM, more units than half of them: their sizes decide, so the shares go up to three times the average)
+  const int wide = (rows <= 24 && 2 * U > G) ? 1 : 0;
   // Parts anywhere are worth a look where the cluster holds only two and the GPU has room for three.
   const int way_lo = (cluster > 1) ? 0 : 1;
   int way_hi = (cluster > 2 || (cluster == 2 && 3 * U > G)) ? 1 : 2;
@@ -163,7 +165,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
 #pragma unroll 1
     for (int slot = slot_lo + (tid >> 5); slot < slot_hi; slot += NT / 32) {
       const int way = slot / kCandidates, c = slot % kCandidates;
-      const int share = cand_share(N, G, c), cl = way ? 1 : cluster;
+      const int share = cand_share(N, G, c << wide), cl = way ? 1 : cluster;
       int sum = 0, big = 0, most = 0;
 #pragma unroll 1
       for (int u = lane; u < U; u += 32) {
@@ -222,7 +224,7 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   if (cand < 0) return cand;
   // A warp takes 32 units.  Inside clusters units are placed by class, so a unit's place is the CTAs of the
   // classes before its own plus its rank in its class; otherwise units lie in their order.
-  const int share = cand_share(N, G, cand);
+  const int share = cand_share(N, G, cand << wide);
   for (int base = (tid >> 5) * 32; base < U; base += NT) {
     const int u = base + lane;
     const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
@@ -332,6 +334,23 @@ __device__ __forceinline__ void merge_scales(float m, float im, float& mn, float
   const float base = (mn == -INFINITY) ? 0.f : mn;
   a_old = ex2(m - base);   // ex2(-inf) = 0
   a_in = ex2(im - base);
+}
+
+// Inclusive prefix sums of the atom counts in unit_start[1 .. U] (one warp, 32 units at a time).
+__device__ __forceinline__ void scan_units(int* unit_start, int U) {
+  const int lane = threadIdx.x & 31;
+  int carry = 0;
+  for (int base = 0; base < U; base += 32) {
+    const int u = base + lane;
+    int v = (u < U) ? unit_start[u + 1] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += n;
+    }
+    if (u < U) unit_start[u + 1] = v + carry;
+    carry += __shfl_sync(0xffffffffu, v, 31);
+  }
 }
 
 // ---- precomputed work partition ("plan") ------------------------------------------------------
@@ -1391,6 +1410,8 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   if (!ok && P.status && lane == 0) atomicOr(P.status, SPECATTN_ROW_TIMEOUT);
 }
 
+#include "sparse_verify_rows.cuh"
+
 // CTAs per cluster for U units on n_sm SMs: as many parts per unit as there are SMs for, as a power of
 // two (clusters of three do not fill the GPCs: 48 of them do not run at once).  Pairs also serve calls with one
 // CTA per unit: they let a long list among short ones be cut.
@@ -1407,13 +1428,30 @@ constexpr size_t verify_smem() {
   return sizeof(VShared<MT, WPM>) + 128;
 }
 
-const void* verify_kernel_of(int m_tiles, size_t* smem, int* threads) {
-  switch (m_tiles) {
-    case 1: *smem = verify_smem<1, 4>(); *threads = (4 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<1, 4>;
-    case 2: *smem = verify_smem<2, 4>(); *threads = (8 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<2, 4>;
-    case 3: *smem = verify_smem<3, 2>(); *threads = (6 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<3, 2>;
-    default: *smem = verify_smem<4, 2>(); *threads = (8 + kProdWarps) * 32; return (const void*)sparse_verify_kernel<4, 2>;
-  }
+int query_rows(const specattn_verify_args& A) { return A.n_q * (A.n_q_heads / A.n_kv_heads); }
+
+// CTAs of half an SM (sparse_verify_rows.cuh, with the figures): up to 24 query rows and more units than half of the SMs.
+bool many_units(const specattn_verify_args& A, int n_sm) {
+  return query_rows(A) <= 24 && 2ll * A.batch * A.n_kv_heads > n_sm;
+}
+
+// The kernel for M query rows, its shared memory and its threads.
+struct VerifyKernel {
+  const void* fn;
+  size_t smem;
+  int threads, record_floats;   // ... of one CTA's record of a unit
+};
+template <int NT8>
+VerifyKernel rows_kernel() {
+  return {(const void*)rows::sparse_verify_rows_kernel<NT8>, rows::verify_smem<NT8>(), rows::kThreads, rows::record_floats<NT8>()};
+}
+template <int MT, int WPM>
+VerifyKernel slab_kernel() {
+  return {(const void*)sparse_verify_kernel<MT, WPM>, verify_smem<MT, WPM>(), (MT * WPM + kProdWarps) * 32, MT * kRec};
+}
+VerifyKernel verify_kernel_of(int M, bool half) {
+  if (!half) return (M <= 16) ? slab_kernel<1, 4>() : (M <= 32) ? slab_kernel<2, 4>() : (M <= 48) ? slab_kernel<3, 2>() : slab_kernel<4, 2>();
+  return (M <= 16) ? rows_kernel<2>() : rows_kernel<3>();
 }
 
 int m_tiles(const specattn_verify_args& A) {
@@ -1438,35 +1476,35 @@ bool long_lists(const specattn_verify_args& A, int cs) {
 // Grid and cluster size of a launch: whole clusters, as many as run at once (GPCs do not hold a multiple of
 // every cluster size).  Opts the kernel in to its shared memory and asks the runtime once per device,
 // kernel and cluster size.  false: the runtime refused.
-bool verify_grid(const specattn_verify_args& A, int n_sm, int* n_ctas, int* cluster) {
-  const int mt = m_tiles(A);
-  static std::atomic<int> known[64][4][kMaxCluster + 1];  // clusters that fit + 1, 0 = not asked yet
+bool verify_grid(const specattn_verify_args& A, int n_sm, bool half, int* n_ctas, int* cluster) {
+  const int M = query_rows(A);
+  const long long units = static_cast<long long>(A.batch) * A.n_kv_heads;
+  const int kind = half ? 4 + (M - 1) / 16 : (M - 1) / 16;   // one per kernel
+  static std::atomic<int> known[64][6][kMaxCluster + 1];  // clusters that fit + 1, 0 = not asked yet
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
     cudaGetLastError();
     return false;
   }
-  size_t smem;
-  int threads;
-  const void* fn = verify_kernel_of(mt, &smem, &threads);
-  const long long units = static_cast<long long>(A.batch) * A.n_kv_heads;
-  int cs = want_cluster(units, n_sm);
-  if (cs > 2 && mt > 2 && long_lists(A, cs)) cs = 2;
+  const VerifyKernel k = verify_kernel_of(M, half);
+  const int slots = half ? 2 * n_sm : n_sm;
+  int cs = want_cluster(units, slots);
+  if (cs > 2 && M > 32 && long_lists(A, cs)) cs = 2;
   for (;;) {
-    std::atomic<int>& slot = known[dev][mt - 1][cs];
+    std::atomic<int>& slot = known[dev][kind][cs];
     int n = slot.load(std::memory_order_acquire);
     if (n == 0) {
-      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) {
+      if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(k.smem)) != cudaSuccess) {
         cudaGetLastError();
         return false;
       }
-      int fit = n_sm;
+      int fit = slots;
       if (cs > 1) {
         cudaLaunchConfig_t q;
         memset(&q, 0, sizeof(q));
-        q.gridDim = dim3(static_cast<unsigned>(n_sm / cs * cs), 1, 1);
-        q.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-        q.dynamicSmemBytes = smem;
+        q.gridDim = dim3(static_cast<unsigned>(slots / cs * cs), 1, 1);
+        q.blockDim = dim3(static_cast<unsigned>(k.threads), 1, 1);
+        q.dynamicSmemBytes = k.smem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = static_cast<unsigned>(cs);
@@ -1475,7 +1513,7 @@ bool verify_grid(const specattn_verify_args& A, int n_sm, int* n_ctas, int* clus
         q.attrs = attr;
         q.numAttrs = 1;
         fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, fn, &q) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&fit, k.fn, &q) != cudaSuccess) {
           cudaGetLastError();
           fit = 0;
         }
@@ -1483,9 +1521,9 @@ bool verify_grid(const specattn_verify_args& A, int n_sm, int* n_ctas, int* clus
       n = fit + 1;
       slot.store(n, std::memory_order_release);
     }
-    const int ctas = (n - 1 < n_sm / cs ? n - 1 : n_sm / cs) * cs;
+    const int ctas = (n - 1 < slots / cs ? n - 1 : slots / cs) * cs;
     // a size that leaves too much of the GPU idle is not worth its merges
-    if (cs == 1 || ctas * 8 >= n_sm * 7 || (ctas > 0 && ctas >= units * cs)) {
+    if (cs == 1 || ctas * 8 >= slots * 7 || (ctas > 0 && ctas >= units * cs)) {
       *n_ctas = ctas;
       *cluster = cs;
       return ctas > 0;
@@ -1494,15 +1532,13 @@ bool verify_grid(const specattn_verify_args& A, int n_sm, int* n_ctas, int* clus
   }
 }
 
-cudaError_t launch_verify(const VerifyParams& P, int m_tiles, int n_ctas, cudaStream_t stream) {
-  size_t smem;
-  int threads;
-  const void* fn = verify_kernel_of(m_tiles, &smem, &threads);
+cudaError_t launch_verify(const VerifyParams& P, bool half, int n_ctas, cudaStream_t stream) {
+  const VerifyKernel k = verify_kernel_of(P.M, half);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(static_cast<unsigned>(n_ctas), 1, 1);
-  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-  cfg.dynamicSmemBytes = smem;
+  cfg.blockDim = dim3(static_cast<unsigned>(k.threads), 1, 1);
+  cfg.dynamicSmemBytes = k.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1517,7 +1553,7 @@ cudaError_t launch_verify(const VerifyParams& P, int m_tiles, int n_ctas, cudaSt
     cfg.numAttrs = 2;
   }
   void* params[1] = {const_cast<VerifyParams*>(&P)};
-  const cudaError_t err = cudaLaunchKernelExC(&cfg, fn, params);
+  const cudaError_t err = cudaLaunchKernelExC(&cfg, k.fn, params);
   if (err != cudaSuccess) cudaGetLastError();
   return err;
 }
@@ -1604,10 +1640,16 @@ bool make_kv_map(const specattn_verify_args& A, CUtensorMap* map) {
 }
 
 // Sized for either engine, so that the choice never depends on the workspace at hand.
-size_t workspace_bytes_for(const specattn_verify_args& A, int n_ctas) {
-  const size_t a = static_cast<size_t>(m_tiles(A)) * kRec;
+// (half: for CTAs of half an SM, where the shape has them; a call with less, as much as the others need, does without)
+size_t workspace_bytes_for(const specattn_verify_args& A, int n_sm, bool half) {
+  const size_t a = static_cast<size_t>(half ? 2 : 1) * verify_kernel_of(query_rows(A), half).record_floats;
   const size_t b = static_cast<size_t>(row_blocks(A)) * kTcRec;
-  return kCounterBytes + static_cast<size_t>(2) * n_ctas * (a > b ? a : b) * sizeof(float);
+  return kCounterBytes + static_cast<size_t>(2) * n_sm * (a > b ? a : b) * sizeof(float);
+}
+
+// Plans have an entry per CTA.
+size_t plan_bytes_for(const specattn_verify_args& A, int n_sm) {
+  return plan_ints(A.batch * A.n_kv_heads, many_units(A, n_sm) ? 2 * n_sm : n_sm) * sizeof(int);
 }
 
 }  // namespace
@@ -1684,7 +1726,7 @@ extern "C" size_t specattn_verify_workspace_bytes(const specattn_verify_args* ar
   if (specattn::validate(args) != SPECATTN_OK) return 0;
   const int n = specattn::device_sm_count();
   if (n <= 0) return 0;
-  return specattn::workspace_bytes_for(*args, n);
+  return specattn::workspace_bytes_for(*args, n, specattn::many_units(*args, n));
 }
 
 extern "C" int specattn_verify_workspace_init(void* workspace, size_t workspace_bytes, void* cuda_stream) {
@@ -1710,7 +1752,7 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
   if (reinterpret_cast<uintptr_t>(A.workspace) % 256 != 0) return SPECATTN_ERR_ALIGN;
   const int n_ctas = specattn::device_sm_count();
   if (n_ctas <= 0) return SPECATTN_ERR_CUDA;
-  if (A.workspace_bytes < specattn::workspace_bytes_for(A, n_ctas)) return SPECATTN_ERR_WORKSPACE;
+  if (A.workspace_bytes < specattn::workspace_bytes_for(A, n_ctas, false)) return SPECATTN_ERR_WORKSPACE;
 
   VerifyParams P = specattn::make_params(A);
   P.counters = static_cast<unsigned int*>(A.workspace);
@@ -1758,10 +1800,11 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
       }
     }
   } else {
+    const bool half = specattn::many_units(A, n_ctas) && A.workspace_bytes >= specattn::workspace_bytes_for(A, n_ctas, true);
     int grid = 0;
-    if (!specattn::verify_grid(A, n_ctas, &grid, &P.cluster))
+    if (!specattn::verify_grid(A, n_ctas, half, &grid, &P.cluster))
       return SPECATTN_ERR_CUDA;
-    err = specattn::launch_verify(P, specattn::m_tiles(A), grid, stream);
+    err = specattn::launch_verify(P, half, grid, stream);
   }
   if (err != cudaSuccess) return SPECATTN_ERR_CUDA;
   specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
@@ -1772,7 +1815,7 @@ extern "C" size_t specattn_verify_plan_bytes(const specattn_verify_args* args) {
   if (specattn::validate(args) != SPECATTN_OK) return 0;
   const int n = specattn::device_sm_count();
   if (n <= 0) return 0;
-  return specattn::plan_ints(args->batch * args->n_kv_heads, n) * sizeof(int);
+  return specattn::plan_bytes_for(*args, n);
 }
 
 extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan, size_t plan_bytes,
@@ -1786,11 +1829,11 @@ extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan
   if (reinterpret_cast<uintptr_t>(plan) % 16 != 0) return SPECATTN_ERR_ALIGN;
   const int n_ctas = specattn::device_sm_count();
   if (n_ctas <= 0) return SPECATTN_ERR_CUDA;
-  if (plan_bytes < specattn::plan_ints(A.batch * A.n_kv_heads, n_ctas) * sizeof(int)) return SPECATTN_ERR_WORKSPACE;
+  if (plan_bytes < specattn::plan_bytes_for(A, n_ctas)) return SPECATTN_ERR_WORKSPACE;
   if (A.batch == 0) return SPECATTN_OK;
   VerifyParams P = specattn::make_params(A);
   int grid = 0;
-  if (!specattn::verify_grid(A, n_ctas, &grid, &P.cluster))
+  if (!specattn::verify_grid(A, n_ctas, specattn::many_units(A, n_ctas), &grid, &P.cluster))
     return SPECATTN_ERR_CUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
@@ -1825,7 +1868,7 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
     if (plans[i] == nullptr || !A.kv_len) return SPECATTN_ERR_NULL;
     if (!A.dense && !A.counts) return SPECATTN_ERR_NULL;
     if (reinterpret_cast<uintptr_t>(plans[i]) % 16 != 0) return SPECATTN_ERR_ALIGN;
-    if (plan_bytes[i] < specattn::plan_ints(A.batch * A.n_kv_heads, n_ctas) * sizeof(int)) return SPECATTN_ERR_WORKSPACE;
+    if (plan_bytes[i] < specattn::plan_bytes_for(A, n_ctas)) return SPECATTN_ERR_WORKSPACE;
   }
   for (int i0 = 0; i0 < n; i0 += specattn::kPlanBatch) {
     specattn::PlanBatch B;
@@ -1835,7 +1878,7 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
       if (args[i]->batch == 0) continue;
       B.p[m] = specattn::make_params(*args[i]);
       B.plan[m] = static_cast<int*>(plans[i]);
-      if (!specattn::verify_grid(*args[i], n_ctas, &B.grid[m], &B.p[m].cluster))
+      if (!specattn::verify_grid(*args[i], n_ctas, specattn::many_units(*args[i], n_ctas), &B.grid[m], &B.p[m].cluster))
         return SPECATTN_ERR_CUDA;
       ++m;
     }
@@ -1882,7 +1925,7 @@ extern "C" int specattn_sparse_verify_static(const specattn_verify_args* args, v
   }
   const int n_ctas = specattn::device_sm_count();
   if (n_ctas <= 0) return SPECATTN_ERR_CUDA;
-  if (specattn::workspace_bytes_for(*args, n_ctas) > SPECATTN_STATIC_SCRATCH_BYTES)
+  if (specattn::workspace_bytes_for(*args, n_ctas, false) > SPECATTN_STATIC_SCRATCH_BYTES)
     return SPECATTN_ERR_STATIC_SCRATCH;
   // In host code the array's name is only a handle; the kernel needs its device address,
   // looked up once per device with that device current (racing first callers store the same

@@ -126,18 +126,6 @@ __device__ __forceinline__ void tc_st8(uint32_t addr, const uint32_t (&r)[8]) {
                "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                : "memory");
 }
-// named barrier that also ORs a predicate over its participants: everyone gets the same answer,
-// so a group that must leave together can decide to leave on it
-__device__ __forceinline__ bool named_bar_or(int id, int nthreads, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %3, 0;\n\t"
-      "barrier.red.or.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"(id), "r"(nthreads), "r"(static_cast<uint32_t>(pred))
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   // (no memory clobber: the target bytes are only ever touched through such stores and by the
   // tensor core, and ordinary loads may move across them; the proxy fence that follows orders them)

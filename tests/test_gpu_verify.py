@@ -634,3 +634,45 @@ def test_how_units_are_cut(batch, n_q, n_q_heads, tokens, parts, cluster):
     sa.verify_plan(a, plan)
     words = plan[:8].cpu().tolist()
     assert words[3] & 0xff == cluster and words[4] == 8 * batch * parts
+
+
+@pytest.mark.parametrize("counts,tail", [
+    ([0, 1, 15, 16, 17, 33, 64, 65, 127, 128, 129, 300], 3),   # edges of a 16-token tile and of four of them, in-flight tokens
+    ([5, 2100, 40, 900, 17, 0, 64, 1300, 3, 700], 0),          # long lists among short ones: cut into parts, several a CTA
+    ([4100] + [260] * 9, 0),                                   # one unit far above the average
+])
+@pytest.mark.parametrize("T,Hq", [(1, 32), (3, 32), (5, 32), (6, 32), (7, 32), (5, 64), (6, 64), (7, 64), (8, 64)])
+def test_many_units_by_all_their_query_rows(T, Hq, counts, tail):
+    """More units than half of the SMs, 4 to 64 query rows (every number of eight-row blocks a warp or a row group may have):
+    the oracle's results, the same bits with a precomputed partition and again on the same workspace, and a call
+    with the smaller workspace that other shapes need agrees."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC:
+        pytest.skip("the mma.sync engine's rule")
+    case = _make_case(99, len(counts), T, Hq, 8, 16, [max(2 * c, 50) for c in counts], counts=[[c] for c in counts], tail=tail)
+    out, lse, status = _run(case)
+    assert int(status.abs().sum()) == 0
+    ref = _oracle(case)
+    check_attention(out, lse, *ref)
+    kv_d = case["kv"].to(dev())
+    o, l, st = torch.empty_like(out), torch.empty_like(lse), torch.zeros_like(status)
+    keep = [bf16_to_dev(case["q"]), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]), to_dev(case["cnt"])]
+    a = sa.make_verify_args(keep[0], kv_d, keep[1], block_table=keep[2], idx=keep[3], counts=keep[4], out=o, lse=l,
+                            status=st, flags=_ENGINE["flags"], tail_len=tail)
+    ws, plan = sa.verify_workspace(a), sa.verify_plan_buffer(a)
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    sa.verify_plan(a, plan)
+    for p in (plan.data_ptr(), None, plan.data_ptr()):
+        a.plan = p
+        o.fill_(float("nan"))
+        assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(o, out) and torch.equal(l, lse)
+    few = sa.make_verify_args(keep[0][:1], kv_d, keep[1][:1], block_table=keep[2][:1], idx=keep[3][:1], counts=keep[4][:1], out=o, lse=l)
+    a.workspace_bytes = sa.verify_workspace_bytes(few)   # (8 units: one CTA per SM)
+    assert a.workspace_bytes <= ws.numel()
+    assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    torch.cuda.synchronize()
+    assert int(st.abs().sum()) == 0
+    check_attention(o, l, *ref)
