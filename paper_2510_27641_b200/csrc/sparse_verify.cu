@@ -26,6 +26,7 @@
 //     share of the output columns from all parts' records (merge_cluster).  A unit that was cut
 //     otherwise is finished by whichever CTA arrives last at the unit's counter, which merges all
 //     partial (O, m, l) records from global memory in a fixed order, without anybody waiting.
+// (Calls of many units with up to 24 query rows run in CTAs of half an SM: sparse_verify_rows.cuh.)
 // Every mbarrier wait is bounded; on expiry the CTA flags SPECATTN_ROW_TIMEOUT and leaves.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -273,11 +274,17 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
 template <int MT, int WPM>
 struct VShared {
   alignas(128) unsigned char kv[kStages][2][kStageTok * kPitch];
-  alignas(16) unsigned char q[MT * 16 * kPitch];
+  // With two warps per slab the queries are read from shared memory until a unit's last tile.  Two buffers let the
+  // next unit's come under this one's tiles, and producer warp 0 go on to its own tiles of it (56 rows, us: 192 units x 400
+  // tokens 33.3 -> 28.3, 256 x 400 41.6 -> 33.7, x 2000 103.6 -> 96.5, 512 x 60 26.7 -> 22.6).  Not with three
+  // slabs: the second address takes a register that the tile loop has not left (40 rows, 256 x 400 40.0 -> 33.4, but
+  // 32 x 890 12.0 -> 12.3).
+  static constexpr int kQBuf = (MT == 4) ? 2 : 1;
+  alignas(16) unsigned char q[kQBuf][MT * 16 * kPitch];
   alignas(16) float scratch[MT][WPM / 2][kRec];
   alignas(8) unsigned long long full[kStages];
   unsigned long long empty[kStages];
-  unsigned long long q_full, q_empty;
+  unsigned long long q_full[kQBuf], q_empty[kQBuf];
   int unit_start[kMaxUnits + 1];
   int unit_cnt[kMaxUnits];
   Partition part;
@@ -783,8 +790,10 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       mbar_init(&sh.full[s], 32 * kArrivals);  // deferred arrivals per producer lane
       mbar_init(&sh.empty[s], NCS);
     }
-    mbar_init(&sh.q_full, 1);
-    mbar_init(&sh.q_empty, NC);
+    for (int i = 0; i < Sh::kQBuf; ++i) {
+      mbar_init(&sh.q_full[i], 1);
+      mbar_init(&sh.q_empty[i], NC);
+    }
     mbar_fence_init();
     sh.abort_flag = 0;
     sh.unit_start[0] = 0;
@@ -931,16 +940,17 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
           // phase is completed here, so that later segments find the parity they expect.  (No wait
           // on q_empty: nobody reads an older block, and the consumers may already have released
           // this one -- the "previous phase" a fresh barrier grants would then be one they hold.)
-          if (lane == 0) mbar_arrive(&sh.q_full);
+          if (lane == 0) mbar_arrive(&sh.q_full[0]);
           return true;
         }
-        if (!mbar_wait(&sh.q_empty, (seg & 1u) ^ 1u, &sh.abort_flag)) return false;
-        if (lane == 0) mbar_arrive_expect_tx(&sh.q_full, static_cast<uint32_t>(P.M) * kRowBytes);
+        const int qb = seg % Sh::kQBuf;
+        if (!mbar_wait(&sh.q_empty[qb], ((seg / Sh::kQBuf) & 1u) ^ 1u, &sh.abort_flag)) return false;
+        if (lane == 0) mbar_arrive_expect_tx(&sh.q_full[qb], static_cast<uint32_t>(P.M) * kRowBytes);
         __syncwarp();
         for (int r = lane; r < P.M; r += 32) {
           const int t = r / P.grp, h = kvh * P.grp + r % P.grp;
-          bulk_g2s(sh.q + r * kPitch, P.q + ((static_cast<long long>(b) * P.T + t) * P.Hq + h) * kD,
-                   kRowBytes, &sh.q_full);
+          bulk_g2s(sh.q[qb] + r * kPitch, P.q + ((static_cast<long long>(b) * P.T + t) * P.Hq + h) * kD,
+                   kRowBytes, &sh.q_full[qb]);
         }
         return true;
       };
@@ -1104,7 +1114,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   const int parity = ((WPM == 4) ? (wr >> 1) : wr) ^ ((warp >> 2) & 1);
   const int g = lane >> 2, tq = lane & 3;
   const int lm = lane >> 3, lr = lane & 7;  // ldmatrix: matrix id, row within it
-  const uint32_t q_addr = smem_u32(sh.q) + (mt * 16 + (lm & 1) * 8 + lr) * kPitch + (lm >> 1) * 16;
+  const uint32_t q_addr0 = smem_u32(sh.q) + (mt * 16 + (lm & 1) * 8 + lr) * kPitch + (lm >> 1) * 16;
   // per-lane byte offsets inside a tile for the K (non-transposed) and V (transposed) fragments
   const uint32_t k_off = ((lm >> 1) * 8 + lr) * kPitch + (lm & 1) * 16;
   const uint32_t v_off = ((lm & 1) * 8 + lr) * kPitch + (lm >> 1) * 16;
@@ -1134,6 +1144,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     // re-read from shared memory for every block instead of being held in 32 registers: the
     // compiler spends those on fragment prefetch (dense, 40 rows: 3.11 -> 3.37 TB/s); with
     // four warps per slab the same change loses 3 %.
+    const uint32_t q_addr = q_addr0 + (seg % Sh::kQBuf) * static_cast<uint32_t>(sizeof(sh.q[0]));
     uint32_t qf[8][4];
     if (kDirectQ && seg == 0) {
       // First query block of the CTA: every consumer warp copies the 16 rows of its own slab
@@ -1145,7 +1156,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
         const int r = mt * 16 + (i >> 4), c = i & 15;
         if (r < P.M) {
           const int t = r / P.grp, h = kvh * P.grp + r % P.grp;
-          cp_async16(smem_u32(sh.q) + r * kPitch + c * 16,
+          cp_async16(smem_u32(sh.q[0]) + r * kPitch + c * 16,
                      P.q + ((static_cast<long long>(b) * P.T + t) * P.Hq + h) * kD + c * 8);
         }
       }
@@ -1153,14 +1164,14 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       __syncwarp();
       ok = true;
     } else {
-      ok = mbar_wait(&sh.q_full, seg & 1u, &sh.abort_flag);
+      ok = mbar_wait(&sh.q_full[seg % Sh::kQBuf], (seg / Sh::kQBuf) & 1u, &sh.abort_flag);
     }
     if (!ok) sh.abort_flag = 1;
     if (!kQReload) {
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) ldmatrix_x4(qf[kk], q_addr + kk * 32);
       __syncwarp();
-      if (ok && lane == 0) mbar_arrive(&sh.q_empty);
+      if (ok && lane == 0) mbar_arrive(&sh.q_empty[seg % Sh::kQBuf]);
     }
 
     WarpState st;
@@ -1197,7 +1208,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
 
     if (kQReload) {
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.q_empty);   // the query tile was read for the last time
+      if (lane == 0) mbar_arrive(&sh.q_empty[seg % Sh::kQBuf]);   // the query tile was read for the last time
     }
     // ---- end of the segment: row sums across the quad, then combine the slab's warps ---------
     float m0 = st.m0, m1 = st.m1, l0 = st.l0, l1 = st.l1;
