@@ -1442,8 +1442,16 @@ constexpr size_t verify_smem() {
 int query_rows(const specattn_verify_args& A) { return A.n_q * (A.n_q_heads / A.n_kv_heads); }
 
 // CTAs of half an SM (sparse_verify_rows.cuh, with the figures): up to 24 query rows and more units than half of the SMs.
-bool many_units(const specattn_verify_args& A, int n_sm) {
+bool half_sm(const specattn_verify_args& A, int n_sm) {
   return query_rows(A) <= 24 && 2ll * A.batch * A.n_kv_heads > n_sm;
+}
+// Many units have a kernel of their own: those, and 33 to 48 rows with more units than SMs the one of four slabs.  It
+// has two more consumer warps and fetches the next unit's queries early, which counts for more there than
+// the padding (40 rows, us, three slabs / four: 192 units x 400 tokens 32.5 / 27.7, 256 x 60 15.1 / 14.0, x 400 40.0 / 33.0, x 2000 106.9 / 95.3, 512 x 400
+// 76.0 / 63.4; not with a unit per CTA or less: 128 x 400 14.6 / 15.4).
+bool many_units(const specattn_verify_args& A, int n_sm) {
+  const int rows = query_rows(A);
+  return half_sm(A, n_sm) || (rows > 32 && rows <= 48 && static_cast<long long>(A.batch) * A.n_kv_heads > n_sm);
 }
 
 // The kernel for M query rows, its shared memory and its threads.
@@ -1460,9 +1468,9 @@ template <int MT, int WPM>
 VerifyKernel slab_kernel() {
   return {(const void*)sparse_verify_kernel<MT, WPM>, verify_smem<MT, WPM>(), (MT * WPM + kProdWarps) * 32, MT * kRec};
 }
-VerifyKernel verify_kernel_of(int M, bool half) {
-  if (!half) return (M <= 16) ? slab_kernel<1, 4>() : (M <= 32) ? slab_kernel<2, 4>() : (M <= 48) ? slab_kernel<3, 2>() : slab_kernel<4, 2>();
-  return (M <= 16) ? rows_kernel<2>() : rows_kernel<3>();
+VerifyKernel verify_kernel_of(int M, bool many) {
+  if (!many) return (M <= 16) ? slab_kernel<1, 4>() : (M <= 32) ? slab_kernel<2, 4>() : (M <= 48) ? slab_kernel<3, 2>() : slab_kernel<4, 2>();
+  return (M <= 16) ? rows_kernel<2>() : (M <= 24) ? rows_kernel<3>() : slab_kernel<4, 2>();
 }
 
 int m_tiles(const specattn_verify_args& A) {
@@ -1487,17 +1495,18 @@ bool long_lists(const specattn_verify_args& A, int cs) {
 // Grid and cluster size of a launch: whole clusters, as many as run at once (GPCs do not hold a multiple of
 // every cluster size).  Opts the kernel in to its shared memory and asks the runtime once per device,
 // kernel and cluster size.  false: the runtime refused.
-bool verify_grid(const specattn_verify_args& A, int n_sm, bool half, int* n_ctas, int* cluster) {
+bool verify_grid(const specattn_verify_args& A, int n_sm, bool many, int* n_ctas, int* cluster) {
   const int M = query_rows(A);
   const long long units = static_cast<long long>(A.batch) * A.n_kv_heads;
-  const int kind = half ? 4 + (M - 1) / 16 : (M - 1) / 16;   // one per kernel
+  const bool half = many && half_sm(A, n_sm);
+  const int kind = half ? 4 + (M - 1) / 16 : many ? 3 : (M - 1) / 16;   // one per kernel
   static std::atomic<int> known[64][6][kMaxCluster + 1];  // clusters that fit + 1, 0 = not asked yet
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
     cudaGetLastError();
     return false;
   }
-  const VerifyKernel k = verify_kernel_of(M, half);
+  const VerifyKernel k = verify_kernel_of(M, many);
   const int slots = half ? 2 * n_sm : n_sm;
   int cs = want_cluster(units, slots);
   if (cs > 2 && M > 32 && long_lists(A, cs)) cs = 2;
@@ -1543,8 +1552,8 @@ bool verify_grid(const specattn_verify_args& A, int n_sm, bool half, int* n_ctas
   }
 }
 
-cudaError_t launch_verify(const VerifyParams& P, bool half, int n_ctas, cudaStream_t stream) {
-  const VerifyKernel k = verify_kernel_of(P.M, half);
+cudaError_t launch_verify(const VerifyParams& P, bool many, int n_ctas, cudaStream_t stream) {
+  const VerifyKernel k = verify_kernel_of(P.M, many);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(static_cast<unsigned>(n_ctas), 1, 1);
@@ -1651,16 +1660,16 @@ bool make_kv_map(const specattn_verify_args& A, CUtensorMap* map) {
 }
 
 // Sized for either engine, so that the choice never depends on the workspace at hand.
-// (half: for CTAs of half an SM, where the shape has them; a call with less, as much as the others need, does without)
-size_t workspace_bytes_for(const specattn_verify_args& A, int n_sm, bool half) {
-  const size_t a = static_cast<size_t>(half ? 2 : 1) * verify_kernel_of(query_rows(A), half).record_floats;
+// (many: for the kernel of many units, where the shape has it; a call with less, as much as the others need, does without)
+size_t workspace_bytes_for(const specattn_verify_args& A, int n_sm, bool many) {
+  const size_t a = static_cast<size_t>(many && half_sm(A, n_sm) ? 2 : 1) * verify_kernel_of(query_rows(A), many).record_floats;
   const size_t b = static_cast<size_t>(row_blocks(A)) * kTcRec;
   return kCounterBytes + static_cast<size_t>(2) * n_sm * (a > b ? a : b) * sizeof(float);
 }
 
 // Plans have an entry per CTA.
 size_t plan_bytes_for(const specattn_verify_args& A, int n_sm) {
-  return plan_ints(A.batch * A.n_kv_heads, many_units(A, n_sm) ? 2 * n_sm : n_sm) * sizeof(int);
+  return plan_ints(A.batch * A.n_kv_heads, half_sm(A, n_sm) ? 2 * n_sm : n_sm) * sizeof(int);
 }
 
 }  // namespace
@@ -1811,11 +1820,11 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
       }
     }
   } else {
-    const bool half = specattn::many_units(A, n_ctas) && A.workspace_bytes >= specattn::workspace_bytes_for(A, n_ctas, true);
+    const bool many = specattn::many_units(A, n_ctas) && A.workspace_bytes >= specattn::workspace_bytes_for(A, n_ctas, true);
     int grid = 0;
-    if (!specattn::verify_grid(A, n_ctas, half, &grid, &P.cluster))
+    if (!specattn::verify_grid(A, n_ctas, many, &grid, &P.cluster))
       return SPECATTN_ERR_CUDA;
-    err = specattn::launch_verify(P, half, grid, stream);
+    err = specattn::launch_verify(P, many, grid, stream);
   }
   if (err != cudaSuccess) return SPECATTN_ERR_CUDA;
   specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);

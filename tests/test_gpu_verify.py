@@ -640,6 +640,7 @@ def test_how_units_are_cut(batch, n_q, n_q_heads, tokens, parts, cluster):
     ([0, 1, 15, 16, 17, 33, 64, 65, 127, 128, 129, 300], 3),   # edges of a 16-token tile and of four of them, in-flight tokens
     ([5, 2100, 40, 900, 17, 0, 64, 1300, 3, 700], 0),          # long lists among short ones: cut into parts, several a CTA
     ([4100] + [260] * 9, 0),                                   # one unit far above the average
+    ([17 * i for i in range(20)], 2),                          # more units than SMs
 ])
 @pytest.mark.parametrize("T,Hq", [(1, 32), (3, 32), (5, 32), (6, 32), (7, 32), (5, 64), (6, 64), (7, 64), (8, 64)])
 def test_many_units_by_all_their_query_rows(T, Hq, counts, tail):
