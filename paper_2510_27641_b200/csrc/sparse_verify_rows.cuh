@@ -547,6 +547,9 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
         if (seg == 0) {
           if (lane == 0) mbar_arrive(&sh.q_full[0]);
         } else {
+          // (The second buffer is free from the start: nothing but this wait puts its first block behind the previous
+          // launch, which may have written the queries.  The first segment's K/V copies are out by now.)
+          if (seg == 1 && P.lists_stable) pdl_wait();
           if (!mbar_wait(&sh.q_empty[seg & 1], ((seg >> 1) & 1u) ^ 1u, &sh.abort_flag)) { sh.abort_flag = 1; dead = true; break; }
           if (lane == 0) mbar_arrive_expect_tx(&sh.q_full[seg & 1], static_cast<uint32_t>(P.M) * kRowBytes);
           __syncwarp();

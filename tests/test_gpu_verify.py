@@ -677,3 +677,74 @@ def test_many_units_by_all_their_query_rows(T, Hq, counts, tail):
     torch.cuda.synchronize()
     assert int(st.abs().sum()) == 0
     check_attention(o, l, *ref)
+
+
+@pytest.mark.parametrize("B,kept", [(64, 60), (40, 400), (10, 500)])   # several units a CTA, one or two, less than one
+@pytest.mark.parametrize("T,Hq", [(2, 32), (4, 32), (5, 32), (5, 64), (7, 64)])
+def test_queries_that_the_launch_right_before_wrote(T, Hq, B, kept):
+    """SPECATTN_VERIFY_LISTS_STABLE vouches for lists and K/V rows, not for the queries: they may be the previous launch's
+    output, whatever segment of a CTA reads them.  Other queries at every turn, written by a copy kernel or by
+    another attention launch (which lets this one begin early); every turn gives the bits of an unflagged call."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    case = _make_case(100 + T, B, T, Hq, 8, 16, [500] * B, counts=[[kept]] * B)
+    d = dev()
+    kv, lens, bt, idx, cnt = case["kv"].to(d), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]), to_dev(case["cnt"])
+    shape, n = (B, T, Hq, 128), 6
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    keep = []
+
+    def call(q, kv, lens, bt, idx, cnt, out, flags):
+        lse = torch.empty(shape[:3], device=d)
+        a = sa.make_verify_args(q, kv, lens, block_table=bt, idx=idx, counts=cnt, out=out, lse=lse, flags=_ENGINE["flags"] | flags)
+        ws = sa.verify_workspace(a)
+        a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+        keep.append((a, ws, lse, q, idx))
+        return lambda: sa.lib().specattn_sparse_verify(C.byref(a), stream)
+
+    # The writing launch attends one key a sequence, so that its binary32 output is that V row: finite queries when read
+    # as bf16.  Sequences 1 and 2 have long lists, whose first key takes all the weight: they are written late.
+    long, few = 3000, 8 * 16
+    wkv = wl.kv_pool(7, 0, 8 * B, 16, 8, 128).to(d)
+    wbt = torch.arange(8 * B, device=d).view(B, 8).repeat(1, 1 + long // few).to(torch.int32)
+    wbt[1:3, 8:] = torch.arange(8 * B, device=d)[torch.arange(wbt.shape[1] - 8, device=d) % (5 * B) + 3 * B].to(torch.int32)
+    wq = torch.zeros(shape, dtype=torch.bfloat16, device=d)
+    wq[..., 0] = 16
+    wkv[:, 0, :, :, 0] = -100
+    wkv[:, 0, :n, :, 0] = 100          # (slots that a list holds at most one of)
+    wlens = torch.full((B,), few, dtype=torch.int32, device=d)
+    wcnt = torch.ones(B, 1, dtype=torch.int32, device=d)
+    wout = torch.empty(shape, device=d)
+    read = wout.view(torch.bfloat16).view(-1)[:wq.numel()].view(shape)
+    rest = torch.arange(16, long, device=d)
+    rest = rest[rest % 16 >= n].to(torch.int32)
+    wlens[1:3], wcnt[1:3] = long, 1 + len(rest)
+    writers, queries = [], []
+    for i in range(n):
+        widx = torch.zeros(B, 1, long, dtype=torch.int32, device=d)
+        widx[:, 0, 0] = i
+        widx[1:3, 0, 1:1 + len(rest)] = rest
+        writers.append(call(wq, wkv, wlens, wbt, widx, wcnt, wout, 0))
+        assert writers[i]() == 0
+        torch.cuda.synchronize()
+        queries.append(read.clone())
+        assert torch.all(torch.isfinite(queries[i])) and (i == 0 or not torch.equal(queries[i], queries[i - 1]))
+    case["q"] = bf16.torch_to_bits(queries[0].cpu()).reshape(shape)
+    want, got = torch.empty(n, *shape, device=d), torch.empty(n, *shape, device=d)
+    for i in range(n):
+        assert call(queries[i], kv, lens, bt, idx, cnt, want[i], 0)() == 0
+    torch.cuda.synchronize()
+    check_attention(want[0], keep[-n][2], *_oracle(case))
+    q = torch.empty(shape, dtype=torch.bfloat16, device=d)
+    for source in (q, read):
+        flagged = [call(source, kv, lens, bt, idx, cnt, got[i], sa.VERIFY_LISTS_STABLE) for i in range(n)]
+        torch.cuda.synchronize()
+        got.fill_(float("nan"))
+        for i in list(range(n)) * 3:
+            if source is q:
+                q.copy_(queries[i])
+            else:
+                assert writers[i]() == 0
+            assert flagged[i]() == 0
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
