@@ -365,11 +365,15 @@ __device__ __forceinline__ void scan_units(int* unit_start, int U) {
 // layers that share a draft layer's lists share it.  A plan holds, as int32:
 //   [0] magic  [1] U  [2] grid  [3] 0: ranges, else the partition's cluster size, | the launch's cluster size << 8
 //   [4] NP  [5] N (atoms)  [6] tail  [7] dense
-//   unit_start[U + 1], unit_cnt[U], a pad, then (a0, a1, u_first, part | parts << 8) per CTA
+//   unit_start[U + 1], unit_cnt[U], a pad, then (a0, a1, u_first, part | parts << 16) per CTA (there may be
+//   two CTAs per SM, and one long list among empty ones may be dealt to nearly all of them)
 // A kernel whose launch does not match the header ignores the plan and partitions itself.  (The cluster size is part
 // of the match: the parts of a unit find one another by their ranks in the cluster.)
-constexpr int kPlanMagic = 0x5a17a9e1;
+constexpr int kPlanMagic = 0x5a17a9e2;
 constexpr int kPlanHeader = 8;
+__host__ __device__ constexpr int pack_part(int part, int parts) { return part | (parts << 16); }
+__host__ __device__ constexpr int part_of(int w) { return w & 0xffff; }
+__host__ __device__ constexpr int parts_of(int w) { return w >> 16; }
 __host__ __device__ inline size_t plan_ints(int U, int grid) {
   return static_cast<size_t>(kPlanHeader) + 2 * (U + 1) + 4 * static_cast<size_t>(grid);
 }
@@ -417,7 +421,7 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
   };
   const int cand = partition_units<256>(pt, unit_start, U, G, P.M, cluster, [&](int u, int first, int k) {
     const int us = unit_start[u], atoms = unit_start[u + 1] - us;
-    for (int j = 0; j < k; ++j) entry(first + j, us + j * atoms / k, us + (j + 1) * atoms / k, u, j | (k << 8));
+    for (int j = 0; j < k; ++j) entry(first + j, us + j * atoms / k, us + (j + 1) * atoms / k, u, pack_part(j, k));
   });
   const bool aligned = cand >= 0;
   const long long NP = aligned ? pt.parts[cluster > 1 ? 0 : 1][cand] : ((N < G) ? N : static_cast<long long>(G));
@@ -836,8 +840,8 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     a0 = p_cta[0];
     a1 = p_cta[1];
     u_first = p_cta[2];
-    part = p_cta[3] & 0xff;
-    parts = p_cta[3] >> 8;
+    part = part_of(p_cta[3]);
+    parts = parts_of(p_cta[3]);
   } else {
   if (warp == 0) {  // inclusive scan of the atom counts, 32 at a time
     int carry = 0;

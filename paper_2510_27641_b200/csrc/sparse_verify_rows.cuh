@@ -465,8 +465,8 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
     a0 = range.x;
     a1 = range.y;
     u_first = what.x;
-    part = what.y & 0xff;
-    parts = what.y >> 8;
+    part = part_of(what.y);
+    parts = parts_of(what.y);
   } else {
     if (warp == 0) scan_units(unit_start, U);
     __syncthreads();

@@ -748,3 +748,39 @@ def test_queries_that_the_launch_right_before_wrote(T, Hq, B, kept):
             assert flagged[i]() == 0
         torch.cuda.synchronize()
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("tokens", [19000, 38400, 65536])   # up to 148 parts, 255 or more of them, and as many as there are CTAs
+@pytest.mark.parametrize("T", [2, 4, 5, 6])
+def test_one_long_list_among_empty_ones_is_dealt_alike_with_and_without_a_plan(T, tokens):
+    """80 units, one of them with a list: its parts, more than 255 of them where two CTAs share an SM, find one another by
+    what a plan says as they do without one.  Bits, and attention over the whole list."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC:
+        pytest.skip("only the mma.sync engine reads plans")
+    d, B, pps = dev(), 80, tokens // 16 + 1
+    kv = wl.kv_pool(5, 0, pps, 16, 1, 128).to(d)
+    q = bf16_to_dev(wl.queries(5, 0, B, T, 4, 128))
+    bt = torch.zeros(B, pps, dtype=torch.int32, device=d)
+    bt[33] = torch.randperm(pps, generator=torch.Generator().manual_seed(5)).to(torch.int32).to(d)
+    lens, cnt = (torch.zeros(B, dtype=torch.int32, device=d) for _ in range(2))
+    lens[33] = cnt[33] = tokens
+    idx = torch.arange(tokens, dtype=torch.int32, device=d).repeat(B, 1, 1)
+    out = [torch.full((B, T, 4, 128), float("nan"), device=d) for _ in range(2)]
+    lse = [torch.full((B, T, 4), float("nan"), device=d) for _ in range(2)]
+    a = sa.make_verify_args(q, kv, lens, block_table=bt, idx=idx, counts=cnt.view(B, 1), out=out[0], lse=lse[0], flags=_ENGINE["flags"])
+    ws, plan = sa.verify_workspace(a), sa.verify_plan_buffer(a)
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    sa.verify_plan(a, plan)
+    for i in range(2):
+        a.out, a.lse, a.plan = out[i].data_ptr(), lse[i].data_ptr(), plan.data_ptr() if i else None
+        assert sa.lib().specattn_sparse_verify(C.byref(a), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], out[1]) and torch.equal(lse[0], lse[1])
+    rows = kv[bt[33].long()].transpose(1, 2).reshape(-1, 2, 128)[:tokens].double()      # [token, K / V, dim]
+    s = q[33].double().reshape(-1, 128) @ rows[:, 0].T / 128 ** 0.5
+    check_attention(out[1][33].reshape(-1, 128), lse[1][33].reshape(-1), (s.softmax(-1) @ rows[:, 1]).cpu().numpy(),
+                    s.logsumexp(-1).cpu().numpy())
+    others = torch.arange(B, device=d) != 33
+    assert torch.all(out[1][others] == 0) and torch.all(torch.isneginf(lse[1][others]))
