@@ -919,7 +919,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     // =========================== producer warps ===========================================
     const int pw = warp - NC;
     int it = 0, seg = 0;
-    int last_it = -1;
+    int last_it = -1, q_seg = 0;   // the last tile, the last segment whose queries this warp sent for
     int a = a0, u = u_first;
     bool dead = false;
     while (a < a1 && !dead) {
@@ -956,6 +956,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
           bulk_g2s(sh.q[qb] + r * kPitch, P.q + ((static_cast<long long>(b) * P.T + t) * P.Hq + h) * kD,
                    kRowBytes, &sh.q_full[qb]);
         }
+        q_seg = seg;
         return true;
       };
       bool q_pending = (pw == 0);
@@ -1101,9 +1102,11 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
         while (u < U && sh.unit_start[u + 1] == sh.unit_start[u]) ++u;
       }
     }
-    if (sh.abort_flag && last_it >= 0) {
-      // give this warp's last copies a bounded chance to land before the CTA retires
-      mbar_wait(&sh.full[last_it % kStages], (last_it / kStages) & 1u, nullptr);
+    if (sh.abort_flag) {
+      // give this warp's last copies a bounded chance to land before the CTA retires (the queries of a unit that the
+      // consumers will not get to among them)
+      if (last_it >= 0) mbar_wait(&sh.full[last_it % kStages], (last_it / kStages) & 1u, nullptr);
+      if (q_seg > 0) mbar_wait(&sh.q_full[q_seg % Sh::kQBuf], (q_seg / Sh::kQBuf) & 1u, nullptr);
     }
     return;
   }

@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
     const int pw = warp - kConsWarps;
     const long long v_delta = P.s_kv * 2;
     int it0 = 0, seg = 0;
-    int last_it = -1;
+    int last_it = -1, q_seg = 0;   // the last tile, the last segment whose queries this warp sent for
     int a = a0, u = u_first;
     bool dead = false;
     while (a < a1 && !dead) {
@@ -556,6 +556,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
           for (int r = lane; r < P.M; r += 32)
             bulk_g2s(sh.q[seg & 1] + r * kPitch,
                      P.q + (static_cast<long long>(b) * P.T * P.Hq + kvh * P.grp + sh.row_off[r]) * kD, kRowBytes, &sh.q_full[seg & 1]);
+          q_seg = seg;
         }
       }
       // Lanes 0 - 15 resolve the tokens of this warp's tile, lanes 16 - 31 those of its next one (four tiles on), to
@@ -630,9 +631,11 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
         while (u < U && unit_start[u + 1] == unit_start[u]) ++u;
       }
     }
-    if (sh.abort_flag && last_it >= 0) {
-      // give this warp's last copies a bounded chance to land before the CTA retires
-      mbar_wait(&sh.full[last_it % kSlots], (last_it / kSlots) & 1u, nullptr);
+    if (sh.abort_flag) {
+      // give this warp's last copies a bounded chance to land before the CTA retires (the queries of a unit that the
+      // consumers will not get to among them)
+      if (last_it >= 0) mbar_wait(&sh.full[last_it % kSlots], (last_it / kSlots) & 1u, nullptr);
+      if (q_seg > 0) mbar_wait(&sh.q_full[q_seg & 1], (q_seg >> 1) & 1u, nullptr);
     }
     return;
   }

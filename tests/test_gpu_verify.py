@@ -784,3 +784,35 @@ def test_one_long_list_among_empty_ones_is_dealt_alike_with_and_without_a_plan(T
                     s.logsumexp(-1).cpu().numpy())
     others = torch.arange(B, device=d) != 33
     assert torch.all(out[1][others] == 0) and torch.all(torch.isneginf(lse[1][others]))
+
+
+@pytest.mark.parametrize("counts", [
+    [700] * 10,         # units cut in clusters: the CTA that gives up leaves with its peers
+    [2000] + [0] * 11,  # parts that merge through global memory
+    [20] * 40,          # several units a CTA, the queries of the second on their way when the first is given up
+])
+@pytest.mark.parametrize("T,Hq", [(4, 32), (5, 32), (5, 64), (7, 64)])
+def test_a_bounded_wait_that_runs_out_with_many_units(T, Hq, counts):
+    """As above where two CTAs share an SM and where two units' queries are held at a time: flagged, no hang, and the next
+    call on a fresh workspace is correct."""
+    import ctypes as C
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC:
+        pytest.skip("the mma.sync engine's kernels")
+    case = _make_case(35, len(counts), T, Hq, 8, 16, [max(2 * c, 50) for c in counts], counts=[[c] for c in counts])
+    keep = [bf16_to_dev(case["q"]), case["kv"].to(dev()), to_dev(case["lens"]), to_dev(case["bt"]), to_dev(case["idx"]),
+            to_dev(case["cnt"])]
+    o = torch.zeros((len(counts), T, Hq, 128), dtype=torch.float32, device=dev())
+    l, st = torch.zeros((len(counts), T, Hq), device=dev()), torch.zeros(len(counts), dtype=torch.int32, device=dev())
+    a = sa.make_verify_args(keep[0], keep[1], keep[2], block_table=keep[3], idx=keep[4], counts=keep[5], out=o, lse=l, status=st)
+    ws = sa.verify_workspace(a)
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    for flags, lost in ((sa.VERIFY_TEST_LOSE_ARRIVAL, sa.ROW_TIMEOUT), (0, 0)):
+        assert sa.lib().specattn_verify_workspace_init(ws.data_ptr(), ws.numel(), None) == 0
+        st.zero_()
+        a.flags = _ENGINE["flags"] | flags
+        assert sa.lib().specattn_sparse_verify(C.byref(a), None) == 0
+        torch.cuda.synchronize()
+        assert int(st[0]) & sa.ROW_TIMEOUT == lost
+    assert int(st.abs().sum()) == 0
+    check_attention(o, l, *_oracle(case))
