@@ -207,7 +207,10 @@ size_t specattn_select_workspace_bytes(const specattn_select_args* args);
  *
  * workspace: at least specattn_verify_workspace_bytes() bytes, 256-byte aligned, prepared
  * once with specattn_verify_workspace_init() and then reusable by consecutive calls on the
- * same stream; two calls that may overlap on the GPU need separate workspaces.
+ * same stream; two calls that may overlap on the GPU need separate workspaces.  (Up to 24 query rows per KV head
+ * and more (sequence, KV head) pairs than half of the SMs: two CTAs share an SM and need more workspace than
+ * one would.  A call with less, down to what one CTA per SM needs, runs with one; its results are the same within the
+ * tolerance of the operation, not bit for bit.)
  * ======================================================================================== */
 /* flags for specattn_verify_args.flags
  *
@@ -314,8 +317,11 @@ int specattn_sparse_verify(const specattn_verify_args* args, void* cuda_stream);
  * 16-byte aligned, written by a small kernel on the stream (after whatever produces counts /
  * kv_len, e.g. specattn_select_topp) and valid until those change.  A kernel given a plan that
  * does not fit its launch (other batch, heads, tail_len, dense flag, GPU, or a shape that is launched
- * in clusters of another size) ignores it.  Only
+ * in clusters of another size or with another number of CTAs) ignores it.  Only
  * the mma.sync engine reads plans.
+ * A plan is for the workspace in its arguments: with args->workspace set and workspace_bytes below
+ * specattn_verify_workspace_bytes(args) it fits calls with such a smaller workspace, otherwise those with
+ * the full one and specattn_sparse_verify_static.
  * Ordering: a plan must be at least as new as the lists it describes -- call this after every
  * specattn_select_topp that rewrites counts -- and a verify call flagged
  * SPECATTN_VERIFY_LISTS_STABLE must not be the first launch after the plan kernel (that flag's
@@ -340,17 +346,16 @@ int specattn_verify_plan_many(const specattn_verify_args* const* args, void* con
  * its own pool, so that a cudaMalloc from a plug-in fails or stalls the whole device; and
  * an allocation in the middle of a latency-critical decode loop synchronises the GPU.
  * For them this variant keeps the scratch inside the library: a file-scope
- * `static __device__` array of SPECATTN_STATIC_SCRATCH_BYTES bytes that every GPU loading the
- * library holds from load until the process exits.  The call allocates and frees nothing
+ * `static __device__` array (8 MiB) that every GPU loading the library holds from load until the
+ * process exits.  The call allocates and frees nothing
  * (no cudaMalloc, cudaFree or allocating library routine).
  *
  * Same arguments, results and status codes as specattn_sparse_verify, except:
  *   - args->workspace and args->workspace_bytes are ignored;
- *   - a shape that needs more scratch than SPECATTN_STATIC_SCRATCH_BYTES is rejected with
+ *   - a shape that needs more scratch than SPECATTN_STATIC_SCRATCH_BYTES with one CTA per SM is rejected with
  *     SPECATTN_ERR_STATIC_SCRATCH and nothing is launched.  The buffer covers up to 32 query rows per
- *     KV head (n_q * group <= 32) on GPUs with up to 160 SMs.  (Batches of many sequences, for which
- *     specattn_verify_workspace_bytes asks for more because two CTAs share an SM, run with one CTA per SM
- *     where the buffer does not hold that much; so does specattn_sparse_verify with such a workspace.);
+ *     KV head (n_q * group <= 32) on GPUs with up to 160 SMs (there it also holds what two CTAs per SM
+ *     need in batches of many sequences);
  *   - the first call on each device looks up the device address of the array (with that
  *     device current); make that first call outside any stream capture;
  *   - all calls on a device share the one array, which still holds what the previous call left

@@ -1449,9 +1449,8 @@ constexpr size_t verify_smem() {
 int query_rows(const specattn_verify_args& A) { return A.n_q * (A.n_q_heads / A.n_kv_heads); }
 
 // CTAs of half an SM (sparse_verify_rows.cuh, with the figures): up to 24 query rows and more units than half of the SMs.
-bool half_sm(const specattn_verify_args& A, int n_sm) {
-  return query_rows(A) <= 24 && 2ll * A.batch * A.n_kv_heads > n_sm;
-}
+bool beyond_half(const specattn_verify_args& A, int n_sm) { return 2ll * A.batch * A.n_kv_heads > n_sm; }
+bool half_sm(const specattn_verify_args& A, int n_sm) { return query_rows(A) <= 24 && beyond_half(A, n_sm); }
 // Many units have a kernel of their own: those, and 33 to 48 rows with more units than SMs the one of four slabs.  It
 // has two more consumer warps and fetches the next unit's queries early, which counts for more there than
 // the padding (40 rows, us, three slabs / four: 192 units x 400 tokens 32.5 / 27.7, 256 x 60 15.1 / 14.0, x 400 40.0 / 33.0, x 2000 106.9 / 95.3, 512 x 400
@@ -1666,17 +1665,27 @@ bool make_kv_map(const specattn_verify_args& A, CUtensorMap* map) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Sized for either engine, so that the choice never depends on the workspace at hand.
-// (many: for the kernel of many units, where the shape has it; a call with less, as much as the others need, does without)
+// Sized for either engine: which of them serves a call never depends on the workspace at hand.  The kernel of many units
+// does: it needs more, and a call with as much as the other kernels need does without it (many = false).
 size_t workspace_bytes_for(const specattn_verify_args& A, int n_sm, bool many) {
   const size_t a = static_cast<size_t>(many && half_sm(A, n_sm) ? 2 : 1) * verify_kernel_of(query_rows(A), many).record_floats;
   const size_t b = static_cast<size_t>(row_blocks(A)) * kTcRec;
   return kCounterBytes + static_cast<size_t>(2) * n_sm * (a > b ? a : b) * sizeof(float);
 }
 
-// Plans have an entry per CTA.
+// Whether a launch with these arguments runs the kernel of many units.  (A plan may be made before there is a workspace:
+// it is for a launch with all that specattn_verify_workspace_bytes asks for, as the call with the library's own
+// scratch has it.)
+bool runs_many(const specattn_verify_args& A, int n_sm) {
+  return many_units(A, n_sm) && (!A.workspace || A.workspace_bytes >= workspace_bytes_for(A, n_sm, true));
+}
+
+// Plans have an entry per CTA.  Buffers are sized by the units alone, so that one serves all numbers of query rows.
+size_t plan_bytes_for(const specattn_verify_args& A, int n_sm, bool half) {
+  return plan_ints(A.batch * A.n_kv_heads, half ? 2 * n_sm : n_sm) * sizeof(int);
+}
 size_t plan_bytes_for(const specattn_verify_args& A, int n_sm) {
-  return plan_ints(A.batch * A.n_kv_heads, half_sm(A, n_sm) ? 2 * n_sm : n_sm) * sizeof(int);
+  return plan_bytes_for(A, n_sm, runs_many(A, n_sm) && half_sm(A, n_sm));
 }
 
 }  // namespace
@@ -1827,7 +1836,7 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
       }
     }
   } else {
-    const bool many = specattn::many_units(A, n_ctas) && A.workspace_bytes >= specattn::workspace_bytes_for(A, n_ctas, true);
+    const bool many = specattn::runs_many(A, n_ctas);
     int grid = 0;
     if (!specattn::verify_grid(A, n_ctas, many, &grid, &P.cluster))
       return SPECATTN_ERR_CUDA;
@@ -1842,7 +1851,7 @@ extern "C" size_t specattn_verify_plan_bytes(const specattn_verify_args* args) {
   if (specattn::validate(args) != SPECATTN_OK) return 0;
   const int n = specattn::device_sm_count();
   if (n <= 0) return 0;
-  return specattn::plan_bytes_for(*args, n);
+  return specattn::plan_bytes_for(*args, n, specattn::beyond_half(*args, n));
 }
 
 extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan, size_t plan_bytes,
@@ -1860,7 +1869,7 @@ extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan
   if (A.batch == 0) return SPECATTN_OK;
   VerifyParams P = specattn::make_params(A);
   int grid = 0;
-  if (!specattn::verify_grid(A, n_ctas, specattn::many_units(A, n_ctas), &grid, &P.cluster))
+  if (!specattn::verify_grid(A, n_ctas, specattn::runs_many(A, n_ctas), &grid, &P.cluster))
     return SPECATTN_ERR_CUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
@@ -1905,7 +1914,7 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
       if (args[i]->batch == 0) continue;
       B.p[m] = specattn::make_params(*args[i]);
       B.plan[m] = static_cast<int*>(plans[i]);
-      if (!specattn::verify_grid(*args[i], n_ctas, specattn::many_units(*args[i], n_ctas), &B.grid[m], &B.p[m].cluster))
+      if (!specattn::verify_grid(*args[i], n_ctas, specattn::runs_many(*args[i], n_ctas), &B.grid[m], &B.p[m].cluster))
         return SPECATTN_ERR_CUDA;
       ++m;
     }
@@ -1933,8 +1942,11 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
 // The variant for callers that cannot allocate: scratch lives in this library image.
 namespace specattn {
 namespace {
-// One copy per GPU that loads the library, held until the process exits.
-static __device__ __align__(256) unsigned char g_static_scratch[SPECATTN_STATIC_SCRATCH_BYTES];
+// One copy per GPU that loads the library, held until the process exits.  Large enough for the kernel of two CTAs per
+// SM at 17 to 24 query rows on up to 160 SMs, so that a shape within SPECATTN_STATIC_SCRATCH_BYTES otherwise runs
+// the same kernel over the same partition as specattn_sparse_verify.
+constexpr size_t kStaticScratch = 8u << 20;
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratch];
 }  // namespace
 }  // namespace specattn
 
@@ -1977,6 +1989,6 @@ extern "C" int specattn_sparse_verify_static(const specattn_verify_args* args, v
   }
   specattn_verify_args a = *args;
   a.workspace = scratch;
-  a.workspace_bytes = SPECATTN_STATIC_SCRATCH_BYTES;
+  a.workspace_bytes = specattn::kStaticScratch;
   return specattn_sparse_verify(&a, cuda_stream);
 }

@@ -32,7 +32,11 @@ def _case(seed, B, T, Hq, Hkv, lens, counts):
 def test_static_scratch_entry_point_matches_the_regular_one_twice_in_a_row():
     import paper_2510_27641_b200 as sa
     cases = [_case(41, 3, 6, 32, 8, [5000, 300, 40], [3100, 300, 0]),      # units split across CTAs
-             _case(42, 2, 5, 32, 8, [900, 2000], [17, 1999])]
+             _case(42, 2, 5, 32, 8, [900, 2000], [17, 1999]),
+             # two CTAs per SM: cut units, several units a CTA
+             _case(45, 12, 5, 32, 8, [900] * 12, [70 * i for i in range(12)]),
+             _case(46, 12, 4, 32, 8, [900] * 12, [70 * i for i in range(12)]),
+             _case(47, 40, 6, 32, 8, [300] * 40, [7 * i for i in range(40)])]
     for q, kv, bt, kv_len, idx, cnt in cases:
         ref_out, ref_lse, ref_status = sa.sparse_verify(q, kv, kv_len, block_table=bt, idx=idx, counts=cnt)
         torch.cuda.synchronize()
@@ -84,3 +88,48 @@ def test_static_scratch_entry_point_rejects_shapes_beyond_its_buffer():
     args.out = None
     assert sa.lib().specattn_sparse_verify_static(C.byref(args), None) == -1
     assert sa.kernel_launch_count() == n0
+
+
+@pytest.mark.parametrize("T,rows_of", [(5, "all"), (6, "all"), (4, "all"), (5, "few"), (4, "few")])
+def test_a_plan_serves_the_workspace_that_it_was_made_for(T, rows_of):
+    """12 sequences (two CTAs per SM with the full workspace, one with the former smaller one), planned: the call with the
+    library's own scratch and the one with a workspace of either size read their plan -- one that deals no work leaves
+    the outputs alone -- and give the bits that they give without one."""
+    import paper_2510_27641_b200 as sa
+    q, kv, bt, kv_len, idx, cnt = _case(48, 12, T, 32, 8, [900] * 12, [75 * i + 1 for i in range(12)])
+    out, lse = torch.empty((12, T, 32, 128), device=dev()), torch.empty((12, T, 32), device=dev())
+    flags = sa.VERIFY_ENGINE_MMA_SYNC
+    a = sa.make_verify_args(q, kv, kv_len, block_table=bt, idx=idx, counts=cnt, out=out, lse=lse, flags=flags)
+    # (a buffer sized for another number of query rows serves this one too)
+    wide = sa.make_verify_args(q.repeat(1, 1, 2, 1)[:, :4].contiguous(), kv, kv_len, block_table=bt, idx=idx, counts=cnt, out=out, lse=lse)
+    plan = sa.verify_plan_buffer(wide)
+    assert plan.numel() == sa.verify_plan_buffer(a).numel()
+    ws = sa.verify_workspace(a)
+    if rows_of == "few":
+        one = sa.make_verify_args(q[:1], kv, kv_len[:1], block_table=bt[:1], idx=idx[:1], counts=cnt[:1], out=out, lse=lse)
+        ws = ws[:sa.verify_workspace_bytes(one)]
+        assert ws.numel() < sa.verify_workspace_bytes(a)
+
+    def call():
+        out.fill_(float("nan"))
+        lse.fill_(float("nan"))
+        if static:
+            sa.sparse_verify_static(a)
+        else:
+            assert sa.lib().specattn_sparse_verify(C.byref(a), None) == 0
+        torch.cuda.synchronize()
+        return out.clone(), lse.clone()
+
+    for static in ((False, True) if rows_of == "all" else (False,)):
+        a.workspace, a.workspace_bytes = (None, 0) if static else (ws.data_ptr(), ws.numel())
+        a.plan = None
+        ref = call()
+        sa.verify_plan(a, plan)
+        a.plan = plan.data_ptr()
+        got = call()
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+        assert not torch.any(torch.isnan(ref[0]))
+        idle = plan.clone()
+        idle[4] = 0                 # no CTA has work
+        a.plan = idle.data_ptr()
+        assert torch.all(torch.isnan(call()[0]))
