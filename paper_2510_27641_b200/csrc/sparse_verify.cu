@@ -94,6 +94,7 @@ struct VerifyParams {
   const int* plan;   // precomputed work partition (specattn_verify_plan) or nullptr
   int test_lose;     // SPECATTN_VERIFY_TEST_LOSE_ARRIVAL: CTA 0 withholds one barrier arrival
   int cluster;       // CTAs per cluster of the launch (the parts of a unit merge inside one cluster)
+  int half;          // two CTAs share an SM (sparse_verify_rows.cuh)
 };
 
 // ---- work partition -----------------------------------------------------------------------------
@@ -152,12 +153,12 @@ __device__ __forceinline__ int class_of(int k, int cluster) { return __ffs(clust
 // place(unit, first CTA, number of parts) for every unit of an aligned partition, each from one thread.  Two
 // barriers (three where both kinds of aligned partition are compared one after the other), none after the last place().
 template <int NT, class Place>
-__device__ __forceinline__ int partition_units(Partition& pt, const int* unit_start, int U, int G, int rows, int& cluster, Place place) {
+__device__ __forceinline__ int partition_units(Partition& pt, const int* unit_start, int U, int G, int rows, bool half, int& cluster, Place place) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int N = unit_start[U];
   const bool try_aligned = U <= kAlignedMaxUnits && N > 0;
   // (CTAs of half an SM, more units than half of them: their sizes decide, so the shares go up to three times the average)
-  const int wide = (rows <= 24 && 2 * U > G) ? 1 : 0;
+  const int wide = (half && 2 * U > G) ? 1 : 0;
   // Parts anywhere are worth a look where the cluster holds only two and the GPU has room for three.
   const int way_lo = (cluster > 1) ? 0 : 1;
   int way_hi = (cluster > 2 || (cluster == 2 && 3 * U > G)) ? 1 : 2;
@@ -419,7 +420,7 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
     *reinterpret_cast<int2*>(p_cta + 4 * i) = make_int2(a0, a1);
     *reinterpret_cast<int2*>(p_cta + 4 * i + 2) = make_int2(u_first, what);
   };
-  const int cand = partition_units<256>(pt, unit_start, U, G, P.M, cluster, [&](int u, int first, int k) {
+  const int cand = partition_units<256>(pt, unit_start, U, G, P.M, P.half != 0, cluster, [&](int u, int first, int k) {
     const int us = unit_start[u], atoms = unit_start[u + 1] - us;
     for (int j = 0; j < k; ++j) entry(first + j, us + j * atoms / k, us + (j + 1) * atoms / k, u, pack_part(j, k));
   });
@@ -861,7 +862,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
 
   N = sh.unit_start[U];
   cluster = P.cluster;
-  const int cand = partition_units<NT>(sh.part, sh.unit_start, U, G, 16 * MT, cluster, [&](int u, int first, int k) {
+  const int cand = partition_units<NT>(sh.part, sh.unit_start, U, G, 16 * MT, false, cluster, [&](int u, int first, int k) {
     const int j = static_cast<int>(blockIdx.x) - first;
     if (j >= 0 && j < k) {
       sh.part.mine[0] = u;
@@ -1680,6 +1681,13 @@ bool runs_many(const specattn_verify_args& A, int n_sm) {
   return many_units(A, n_sm) && (!A.workspace || A.workspace_bytes >= workspace_bytes_for(A, n_sm, true));
 }
 
+// The grid of the launch and what the partition depends on with it.
+bool launch_grid(const specattn_verify_args& A, int n_sm, VerifyParams* P, int* grid) {
+  const bool many = runs_many(A, n_sm);
+  P->half = many && half_sm(A, n_sm) ? 1 : 0;
+  return verify_grid(A, n_sm, many, grid, &P->cluster);
+}
+
 // Plans have an entry per CTA.  Buffers are sized by the units alone, so that one serves all numbers of query rows.
 size_t plan_bytes_for(const specattn_verify_args& A, int n_sm, bool half) {
   return plan_ints(A.batch * A.n_kv_heads, half ? 2 * n_sm : n_sm) * sizeof(int);
@@ -1836,11 +1844,10 @@ extern "C" int specattn_sparse_verify(const specattn_verify_args* args, void* cu
       }
     }
   } else {
-    const bool many = specattn::runs_many(A, n_ctas);
     int grid = 0;
-    if (!specattn::verify_grid(A, n_ctas, many, &grid, &P.cluster))
+    if (!specattn::launch_grid(A, n_ctas, &P, &grid))
       return SPECATTN_ERR_CUDA;
-    err = specattn::launch_verify(P, many, grid, stream);
+    err = specattn::launch_verify(P, specattn::runs_many(A, n_ctas), grid, stream);
   }
   if (err != cudaSuccess) return SPECATTN_ERR_CUDA;
   specattn::g_launch_count.fetch_add(1, std::memory_order_relaxed);
@@ -1869,7 +1876,7 @@ extern "C" int specattn_verify_plan(const specattn_verify_args* args, void* plan
   if (A.batch == 0) return SPECATTN_OK;
   VerifyParams P = specattn::make_params(A);
   int grid = 0;
-  if (!specattn::verify_grid(A, n_ctas, specattn::runs_many(A, n_ctas), &grid, &P.cluster))
+  if (!specattn::launch_grid(A, n_ctas, &P, &grid))
     return SPECATTN_ERR_CUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
@@ -1914,7 +1921,7 @@ extern "C" int specattn_verify_plan_many(const specattn_verify_args* const* args
       if (args[i]->batch == 0) continue;
       B.p[m] = specattn::make_params(*args[i]);
       B.plan[m] = static_cast<int*>(plans[i]);
-      if (!specattn::verify_grid(*args[i], n_ctas, specattn::runs_many(*args[i], n_ctas), &B.grid[m], &B.p[m].cluster))
+      if (!specattn::launch_grid(*args[i], n_ctas, &B.p[m], &B.grid[m]))
         return SPECATTN_ERR_CUDA;
       ++m;
     }

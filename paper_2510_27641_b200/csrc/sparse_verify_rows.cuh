@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
     N = unit_start[U];
     cluster = P.cluster;
     const int G = static_cast<int>(gridDim.x);
-    const int cand = partition_units<kThreads>(sh.part, unit_start, U, G, P.M, cluster, [&](int u, int first, int k) {
+    const int cand = partition_units<kThreads>(sh.part, unit_start, U, G, P.M, true, cluster, [&](int u, int first, int k) {
       const int j = static_cast<int>(blockIdx.x) - first;
       if (j >= 0 && j < k) {
         sh.part.mine[0] = u;

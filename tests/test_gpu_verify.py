@@ -816,3 +816,28 @@ def test_a_bounded_wait_that_runs_out_with_many_units(T, Hq, counts):
         assert int(st[0]) & sa.ROW_TIMEOUT == lost
     assert int(st.abs().sum()) == 0
     check_attention(o, l, *_oracle(case))
+
+
+def test_how_units_are_cut_with_one_cta_per_sm_and_few_query_rows():
+    """144 units of unequal lengths, 16 query rows, the workspace of one CTA per SM: ranges, as with 32 rows (the wider
+    choice of shares is for two CTAs per SM)."""
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC or torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the plan of the mma.sync engine on 148 SMs")
+    d, B = dev(), 18
+    counts = torch.tensor([[int(300 * 0.1 ** (b / 17))] for b in range(B)], dtype=torch.int32, device=d)
+    words = []
+    for T in (4, 8):
+        q = torch.zeros(B, T, 32, 128, dtype=torch.bfloat16, device=d)
+        keep = [torch.zeros(1, 2, 16, 8, 128, dtype=torch.bfloat16, device=d), torch.full((B,), 512, dtype=torch.int32, device=d),
+                torch.zeros(B, 32, dtype=torch.int32, device=d), torch.zeros(B, 1, 512, dtype=torch.int32, device=d), torch.zeros(4, device=d)]
+
+        def args(n, ws=None):
+            return sa.make_verify_args(q[:n], keep[0], keep[1][:n], block_table=keep[2][:n], idx=keep[3][:n], counts=counts[:n],
+                                       out=keep[4], lse=keep[4], flags=_ENGINE["flags"], workspace=ws)
+
+        a = args(B, torch.empty(sa.verify_workspace_bytes(args(1)), dtype=torch.uint8, device=d))
+        plan = sa.verify_plan_buffer(a)
+        sa.verify_plan(a, plan)
+        words.append(plan[:8].cpu().tolist())
+    assert words[0] == words[1] and words[0][3] & 0xff == 0
