@@ -378,8 +378,8 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
   using Sh = VShared<NT8>;
   constexpr int kItems = Sh::kItems;
   // Registers: a CTA is launched with 128 a thread; the producer warps hand theirs to the consumers (two warpgroups of
-  // 128 threads: 168 + 88 = 2 x 128).
-  constexpr int kConsRegs = 168, kProdRegs = 88;
+  // 128 threads: 168 + 88 = 152 + 104 = 2 x 128).  With 88 the producers spill, which up to 16 rows need not be.
+  constexpr int kConsRegs = (NT8 == 2) ? 152 : 168, kProdRegs = 256 - kConsRegs;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Sh& sh = *reinterpret_cast<Sh*>(smem_raw);
   int* const unit_start = sh.unit_start;
