@@ -31,6 +31,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -108,10 +109,12 @@ struct VerifyParams {
 struct Partition {
   int parts[2][kCandidates];    // inside clusters / anywhere, per candidate share: CTAs needed, largest part
   int largest[2][kCandidates];
+  int share[2][kCandidates];
   int unit_max;              // atoms of the largest unit
   unsigned long long units[kAlignedMaxUnits / 32];  // units per class (16 bits each) of each group of 32 units
   // this CTA's share, for the end of the kernel (kept out of registers meanwhile)
   int mine[3];               // unit (-1: none), part and number of parts
+  int range[2];              // (sparse_verify_rows.cuh) its atoms
   int atoms, ctas, aligned;  // N, the number of CTAs with work, whether units are dealt in equal parts
   int cluster;               // of the partition: 1 where parts merge through global memory
 };
@@ -121,21 +124,31 @@ struct Partition {
 // 5 / 17 / 49, 16 units in eight 26, 32 in four 11; 40 rows 3 / 11 / 29, 17, 8, 40 units in three 11.
 __device__ __forceinline__ int merge_cost(int rows, int r) { return (rows <= 32) ? 6 + 3 * r : 8 + (3 * r) / 2; }
 
-// Parts of a unit for a target share of `share` atoms, out of U units on G CTAs.  Inside clusters a part has at
+// Parts of a unit for a target share of `share` atoms, out of U units on G CTAs: inside clusters the largest power of
+// two up to the cluster size of which half would leave parts above the share, where a part has at
 // least kMinPartAtoms atoms, half as many again where all the parts would take more than half of the GPU (32
 // units of 19 atoms: 8.5 us in four parts, 7.6 us in two; 8 such units: 6.3 us in four, 7.3 us in two), and three times
 // as many where up to 32 query rows would take most of it in more than two parts a unit (20 rows, 32 units of 32 atoms,
 // four / two parts: 10.75 / 9.5 us, 24 units 9.7 / 9.2; of 69 atoms 14.1 / 15.9; 8 units of 69, eight / four: 10.0 / 10.5).
-__device__ __forceinline__ int unit_parts(int atoms, int share, int cluster, int U, int G, int rows) {
-  if (cluster == 1) return max(1, min((atoms + share / 2) / share, atoms / kMinGlobalAtoms));
-  int k = cluster;
-  for (; k > 1; k >>= 1) {
-    const int least = (rows <= 32 && k > 2 && 3 * U * k > 2 * G) ? 3 * kMinPartAtoms
-                      : (2 * U * k > G)                          ? kMinPartAtoms + kMinPartAtoms / 2
-                                                                 : kMinPartAtoms;
-    if (k * least <= atoms && (k >> 1) * share < atoms) break;
+struct ClusterCut {
+  int need[3];   // atoms from which a unit has 2, 4, 8 parts
+  __device__ __forceinline__ ClusterCut(int share, int cluster, int U, int G, int rows) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int k = 2 << i;
+      const int least = (rows <= 32 && k > 2 && 3 * U * k > 2 * G) ? 3 * kMinPartAtoms
+                        : (2 * U * k > G)                          ? kMinPartAtoms + kMinPartAtoms / 2
+                                                                   : kMinPartAtoms;
+      need[i] = (k <= cluster) ? max(k * least, (k >> 1) * share + 1) : INT_MAX;
+    }
   }
-  return k;
+  __device__ __forceinline__ int log2_parts(int atoms) const {
+    return atoms >= need[2] ? 3 : atoms >= need[1] ? 2 : atoms >= need[0] ? 1 : 0;
+  }
+};
+// ... merged anywhere.
+__device__ __forceinline__ int parts_anywhere(int atoms, int share) {
+  return max(1, min((atoms + share / 2) / share, atoms / kMinGlobalAtoms));
 }
 
 // Candidate share c: (N / G) (1 + c / 7), rounded up -- rounding part counts up to the chain can ask for
@@ -145,38 +158,55 @@ __device__ __forceinline__ int cand_share(long long N, int G, int c) {
   return static_cast<int>((static_cast<unsigned>(N) * (7u + c) + 7u * G - 1u) / (7u * G));
 }
 
-// Class of k parts: 0 for the cluster size, 1 for half of it, ...
-__device__ __forceinline__ int class_of(int k, int cluster) { return __ffs(cluster) - __ffs(k); }
-
 // Decides the partition (all NT threads of the CTA, after a barrier that follows unit_start[]): the candidate
 // share, or -1 for ranges; `cluster` becomes 1 where parts are to merge through global memory.  Then calls
 // place(unit, first CTA, number of parts) for every unit of an aligned partition, each from one thread.  Two
 // barriers (three where both kinds of aligned partition are compared one after the other), none after the last place().
+// It runs in every CTA before the first tile, once, and waits for its own instructions: few of them, no
+// division per unit inside clusters, no loop over candidates or groups.  (With those, two CTAs on an SM, 80 / 136 units: 3.2 /
+// 3.9 us; calls without a plan, 4 query rows, us, with / without them: 136 units of 100 to 40 tokens 10.4 / 8.9, 256
+// of 300 to 120 15.3 / 13.8.)
 template <int NT, class Place>
 __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_start, int U, int G, int rows, bool half, int& cluster, Place place) {
-  const int tid = threadIdx.x, lane = tid & 31;
+  static_assert(NT >= kAlignedMaxUnits && kAlignedMaxUnits == 32 * 8 && kCandidates == 8, "a thread per unit, a lane per candidate");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = unit_start[U];
-  const bool try_aligned = U <= kAlignedMaxUnits && N > 0;
+  if (U > kAlignedMaxUnits || N <= 0) {
+    cluster = 1;
+    return -1;
+  }
   // (CTAs of half an SM, more units than half of them: their sizes decide, so the shares go up to three times the average)
   const int wide = (half && 2 * U > G) ? 1 : 0;
   // Parts anywhere are worth a look where the cluster holds only two and the GPU has room for three.
   const int way_lo = (cluster > 1) ? 0 : 1;
   int way_hi = (cluster > 2 || (cluster == 2 && 3 * U > G)) ? 1 : 2;
   const auto consider = [&](int slot_lo, int slot_hi) {
-    // one warp per candidate: two divisions a lane, two reductions, no atomics
+    // one warp per candidate: two reductions, no atomics
 #pragma unroll 1
-    for (int slot = slot_lo + (tid >> 5); slot < slot_hi; slot += NT / 32) {
+    for (int slot = slot_lo + warp; slot < slot_hi; slot += NT / 32) {
       const int way = slot / kCandidates, c = slot % kCandidates;
-      const int share = cand_share(N, G, c << wide), cl = way ? 1 : cluster;
+      const int share = cand_share(N, G, c << wide);
       int sum = 0, big = 0, most = 0;
+      if (way == 0) {
+        const ClusterCut cut(share, cluster, U, G, rows);
 #pragma unroll 1
-      for (int u = lane; u < U; u += 32) {
-        const int atoms = unit_start[u + 1] - unit_start[u];
-        if (atoms == 0) continue;
-        const int k = unit_parts(atoms, share, cl, U, G, rows);
-        sum += k;
-        big = max(big, (atoms + k - 1) / k);
-        most = max(most, atoms);
+        for (int u = lane; u < U; u += 32) {
+          const int atoms = unit_start[u + 1] - unit_start[u];
+          const int s = cut.log2_parts(atoms);
+          sum += (atoms > 0) ? 1 << s : 0;
+          big = max(big, (atoms + (1 << s) - 1) >> s);
+          most = max(most, atoms);
+        }
+      } else {
+#pragma unroll 1
+        for (int u = lane; u < U; u += 32) {
+          const int atoms = unit_start[u + 1] - unit_start[u];
+          if (atoms == 0) continue;
+          const int k = parts_anywhere(atoms, share);
+          sum += k;
+          big = max(big, (atoms + k - 1) / k);
+          most = max(most, atoms);
+        }
       }
       sum = __reduce_add_sync(0xffffffffu, sum);
       big = __reduce_max_sync(0xffffffffu, big);
@@ -184,20 +214,28 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
       if (lane == 0) {
         pt.parts[way][c] = sum;
         pt.largest[way][c] = big;
+        pt.share[way][c] = share;
         pt.unit_max = most;  // (the same from every warp)
       }
     }
   };
-  if (try_aligned) consider(way_lo * kCandidates, way_hi * kCandidates);
+  // The first candidate whose parts have a CTA each, and its largest part (-1, 0: none has).
+  const auto first_fit = [&](int way, int& part) {
+    const int fits = pt.parts[way][lane & 7], most = pt.largest[way][lane & 7];
+    const unsigned m = __ballot_sync(0xffffffffu, fits <= G);
+    part = __shfl_sync(0xffffffffu, most, m ? __ffs(m) - 1 : 0);
+    if (m == 0) part = 0;
+    return __ffs(m) - 1;
+  };
+  consider(way_lo * kCandidates, way_hi * kCandidates);
   __syncthreads();
-  if (try_aligned && cluster > 2) {
+  const int fair = N / G + 1;
+  int part = 0;
+  if (cluster > 2) {
     // Larger clusters: where the cluster's size leaves the longest unit in parts far above the average (8 units
     // of 2900 and 8 of 480 atoms on 148 SMs, 64 rows each: 41.4 us in clusters, 37.9 anywhere; 8 units of 813, 40
     // rows: 41.2 and 35.1).
-    int part = 0;
-    for (int c = 0; c < kCandidates && part == 0; ++c)
-      if (pt.parts[0][c] <= G) part = pt.largest[0][c];
-    const int fair = N / G + 1;
+    first_fit(0, part);
     if (part + 3 > fair + merge_cost(rows, pt.unit_max / fair + 1)) {
       consider(kCandidates, 2 * kCandidates);
       way_hi = 2;
@@ -206,68 +244,66 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   }
   // Costs in atoms' time: a straddling CTA ~24; a unit's merge through global memory as above; inside a cluster ~3.
   int cand = -1, way = 1;
-  if (try_aligned) {
-    int best = (N + kSegAtoms * U) / G + 24 + 3 * (pt.unit_max / (N / G + 1) + 1);
-    for (int w = way_lo; w < way_hi; ++w) {
-      for (int c = 0; c < kCandidates; ++c) {
-        if (pt.parts[w][c] > G) continue;
-        const int part = pt.largest[w][c];
-        const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : merge_cost(rows, (pt.unit_max + part - 1) / part));
-        if (cost <= best) {
-          best = cost;
-          cand = c;
-          way = w;
-        }
-        break;
-      }
+  int best = (N + kSegAtoms * U) / G + 24 + 3 * (pt.unit_max / fair + 1);
+#pragma unroll 1
+  for (int w = way_lo; w < way_hi; ++w) {
+    const int c = first_fit(w, part);
+    if (c < 0) continue;
+    const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : merge_cost(rows, (pt.unit_max + part - 1) / part));
+    if (cost <= best) {
+      best = cost;
+      cand = c;
+      way = w;
     }
   }
   if (way == 1) cluster = 1;
   if (cand < 0) return cand;
-  // A warp takes 32 units.  Inside clusters units are placed by class, so a unit's place is the CTAs of the
-  // classes before its own plus its rank in its class; otherwise units lie in their order.
-  const int share = cand_share(N, G, cand << wide);
-  for (int base = (tid >> 5) * 32; base < U; base += NT) {
-    const int u = base + lane;
-    const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G, rows) : 0;
-    const int at = (cluster == 1) ? 0 : 16 * class_of(k, cluster);
-    const unsigned one = (k == 0) ? 0u : (cluster == 1) ? static_cast<unsigned>(k) : 1u << (at & 31);
-    const unsigned long long hi = __reduce_add_sync(0xffffffffu, at < 32 ? 0u : one);
-    const unsigned lo = __reduce_add_sync(0xffffffffu, at < 32 ? one : 0u);
-    if (lane == 0) pt.units[base >> 5] = (hi << 32) + lo;
+  // A thread per unit.  Inside clusters units are placed by class (0: as many parts as the cluster has CTAs, 1: half as
+  // many, ...), so a unit's place is the CTAs of the classes before its own plus its rank in its class; otherwise units lie in their order.
+  const int share = pt.share[way][cand];
+  const int atoms = (tid < U) ? unit_start[tid + 1] - unit_start[tid] : 0;
+  int k = 0;
+  if (atoms > 0) k = (cluster == 1) ? parts_anywhere(atoms, share) : 1 << ClusterCut(share, cluster, U, G, rows).log2_parts(atoms);
+  if (warp < kAlignedMaxUnits / 32) {
+    unsigned long long sums = 0ull;
+    if (cluster == 1) {
+      sums = static_cast<unsigned>(__reduce_add_sync(0xffffffffu, k));
+    } else {
+#pragma unroll 1
+      for (int at = 0, c = cluster; c > 0; at += 16, c >>= 1)
+        sums |= static_cast<unsigned long long>(__popc(__ballot_sync(0xffffffffu, k == c))) << at;
+    }
+    if (lane == 0) pt.units[warp] = sums;
   }
   __syncthreads();
-  for (int base = (tid >> 5) * 32; base < U; base += NT) {
-    const int u = base + lane;
-    const int atoms = (u < U) ? unit_start[u + 1] - unit_start[u] : 0;
-    const int k = (atoms > 0) ? unit_parts(atoms, share, cluster, U, G, rows) : 0;
-    unsigned long long before = 0ull, all = 0ull;
-    for (int i = 0; i < (U + 31) / 32; ++i) {
-      if (32 * i < base) before += pt.units[i];
-      all += pt.units[i];
-    }
-    int first;
-    if (cluster == 1) {
-      int end = k;
+  if (warp >= kAlignedMaxUnits / 32) return cand;
+  unsigned long long before = 0ull, all = 0ull;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, end, o);
-        if (lane >= o) end += v;
-      }
-      first = static_cast<int>(before) + end - k;
-    } else {
-      int cta = 0;
-      first = 0;
-      for (int cls = 0, c = cluster; c > 0; ++cls, c >>= 1) {
-        const unsigned m = __ballot_sync(0xffffffffu, k == c);
-        const int rank = static_cast<int>((before >> (16 * cls)) & 0xffffull) + __popc(m & ((1u << lane) - 1u));
-        if (k == c) first = cta + rank * c;
-        cta += static_cast<int>((all >> (16 * cls)) & 0xffffull) * c;
-      }
-    }
-    if (k > 0) place(u, first, k);
+  for (int i = 0; i < kAlignedMaxUnits / 32; ++i) {
+    const unsigned long long v = pt.units[i];
+    if (i < warp) before += v;
+    all += v;
   }
+  int first = 0;
+  if (cluster == 1) {
+    int end = k;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += v;
+    }
+    first = static_cast<int>(before) + end - k;
+  } else {
+    int cta = 0;
+#pragma unroll 1
+    for (int at = 0, c = cluster; c > 0; at += 16, c >>= 1) {
+      const unsigned m = __ballot_sync(0xffffffffu, k == c);
+      const int rank = static_cast<int>((before >> at) & 0xffffull) + __popc(m & ((1u << lane) - 1u));
+      if (k == c) first = cta + rank * c;
+      cta += static_cast<int>((all >> at) & 0xffffull) * c;
+    }
+  }
+  if (k > 0) place(tid, first, k);
   return cand;
 }
 

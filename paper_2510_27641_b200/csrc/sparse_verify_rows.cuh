@@ -373,6 +373,52 @@ __device__ __forceinline__ void merge_global(const Items<NT8>& items, int i_lo, 
   }
 }
 
+// The partition of a launch without a plan, and this CTA's share of it, into sh.part (all threads; the atom counts lie in
+// unit_start[1 .. U]).  Out of line: inline it left the tile loop of 17 to 24 rows too few registers (512 units of
+// 2000 tokens 103 -> 112 us).
+template <int NT8>
+__device__ __noinline__ void cut_units(int U, int rows, int cluster) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  VShared<NT8>& sh = *reinterpret_cast<VShared<NT8>*>(smem_raw);
+  int* const unit_start = sh.unit_start;
+  const int G = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
+  if (threadIdx.x < 32) scan_units(unit_start, U);
+  __syncthreads();
+  const int N = unit_start[U];
+  const int cand = partition_units<kThreads>(sh.part, unit_start, U, G, rows, true, cluster, [&](int u, int first, int k) {
+    const int j = cta - first;
+    if (j >= 0 && j < k) {
+      const int us = unit_start[u], atoms = unit_start[u + 1] - us;  // part < parts: the products fit 32 bits
+      sh.part.mine[0] = u;
+      sh.part.mine[1] = j;
+      sh.part.mine[2] = k;
+      sh.part.range[0] = us + j * atoms / k;
+      sh.part.range[1] = us + (j + 1) * atoms / k;
+    }
+  });
+  const bool aligned = cand >= 0;
+  const int NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : min(N, G);
+  if (aligned) {
+    __syncthreads();
+  } else if (cta < NP) {
+    int a0, a1, u, next;
+    range_start(unit_start, U, N, cta, NP, a0, u);
+    range_start(unit_start, U, N, cta + 1, NP, a1, next);
+    if ((threadIdx.x & 31) == 0) {
+      sh.part.mine[0] = u;
+      sh.part.mine[1] = sh.part.mine[2] = 0;
+      sh.part.range[0] = a0;
+      sh.part.range[1] = (cta + 1 == NP) ? N : a1;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sh.part.atoms = N;
+    sh.part.ctas = NP;
+    sh.part.aligned = aligned ? 1 : 0;
+    sh.part.cluster = cluster;
+  }
+}
+
 template <int NT8>
 __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const __grid_constant__ VerifyParams P) {
   using Sh = VShared<NT8>;
@@ -451,76 +497,33 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
   }
   fence_proxy_async();
   __syncthreads();
-  int N;              // atoms of all units
-  bool aligned;       // which of the two partitions
-  int NP;             // CTAs that get work
-  int a0 = 0, a1 = 0, u_first = 0;  // this CTA's atom range and the unit holding its first atom
-  int part = 0, parts = 0;          // (aligned) which part of how many of the unit
-  int cluster;                      // 1: parts merge through global memory
-  if (planned) {
-    cluster = plan[3] & 0xff;
-    aligned = cluster != 0;
-    NP = sizes.x;
-    N = sizes.y;
-    a0 = range.x;
-    a1 = range.y;
-    u_first = what.x;
-    part = part_of(what.y);
-    parts = parts_of(what.y);
-  } else {
-    if (warp == 0) scan_units(unit_start, U);
-    __syncthreads();
-    N = unit_start[U];
-    cluster = P.cluster;
-    const int G = static_cast<int>(gridDim.x);
-    const int cand = partition_units<kThreads>(sh.part, unit_start, U, G, P.M, true, cluster, [&](int u, int first, int k) {
-      const int j = static_cast<int>(blockIdx.x) - first;
-      if (j >= 0 && j < k) {
-        sh.part.mine[0] = u;
-        sh.part.mine[1] = j;
-        sh.part.mine[2] = k;
-      }
-    });
-    aligned = cand >= 0;
-    NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : min(N, G);
-    if (aligned) {
-      __syncthreads();
-      if (static_cast<int>(blockIdx.x) < NP) {
-        u_first = sh.part.mine[0];
-        part = sh.part.mine[1];
-        parts = sh.part.mine[2];
-        const int atoms = unit_start[u_first + 1] - unit_start[u_first];  // part < parts: the products fit 32 bits
-        a0 = unit_start[u_first] + part * atoms / parts;
-        a1 = unit_start[u_first] + (part + 1) * atoms / parts;
-      }
-    } else if (static_cast<int>(blockIdx.x) < NP) {
-      int next;
-      range_start(unit_start, U, N, blockIdx.x, NP, a0, u_first);
-      range_start(unit_start, U, N, blockIdx.x + 1, NP, a1, next);
-      if (static_cast<int>(blockIdx.x) + 1 == NP) a1 = N;
-    }
+  // (every warp leaves itself the same values)
+  if (!planned) {
+    cut_units<NT8>(U, P.M, P.cluster);
+  } else if (lane == 0) {
+    sh.part.mine[0] = what.x;
+    sh.part.mine[1] = part_of(what.y);
+    sh.part.mine[2] = parts_of(what.y);
+    sh.part.range[0] = range.x;
+    sh.part.range[1] = range.y;
+    sh.part.atoms = sizes.y;
+    sh.part.ctas = sizes.x;
+    sh.part.cluster = plan[3] & 0xff;
+    sh.part.aligned = sh.part.cluster != 0;
   }
-  if (static_cast<int>(blockIdx.x) >= NP) {
+  __syncwarp();
+  if (static_cast<int>(blockIdx.x) >= sh.part.ctas) {
     if (P.lists_stable) pdl_wait();
     for (int u = blockIdx.x; u < U; u += gridDim.x)
       if (unit_cnt[u] == 0) empty_unit(u, tid, kThreads);
     return;
   }
-  if (lane == 0) {  // (every warp leaves itself the same values)
-    sh.part.mine[0] = u_first;
-    sh.part.mine[1] = part;
-    sh.part.mine[2] = parts;
-    sh.part.atoms = N;
-    sh.part.ctas = NP;
-    sh.part.aligned = aligned ? 1 : 0;
-    sh.part.cluster = cluster;
-  }
-  __syncwarp();
 
   if (warp >= kConsWarps) {
     // =========================== producer warps ===========================================
     set_max_registers_dec<kProdRegs>();
     const int pw = warp - kConsWarps;
+    const int a0 = sh.part.range[0], a1 = sh.part.range[1], u_first = sh.part.mine[0];  // this CTA's atoms and the unit of the first
     const long long v_delta = P.s_kv * 2;
     int it0 = 0, seg = 0;
     int last_it = -1, q_seg = 0;   // the last tile, the last segment whose queries this warp sent for
@@ -642,6 +645,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
 
   // =============================== consumer warps ===========================================
   set_max_registers_inc<kConsRegs>();
+  const int a0 = sh.part.range[0], a1 = sh.part.range[1], u_first = sh.part.mine[0];
   if (P.lists_stable) {
     // the first query block on its way to L2 meanwhile (only there: the previous kernel may still be writing it)
     const int b = u_first / P.Hkv, kvh = u_first % P.Hkv;
