@@ -121,8 +121,9 @@ struct Partition {
 
 // What the partition weighs depends on the kernel (an atom takes about 0.23 us with up to 32 query rows, 0.33 with
 // more).  A merge of r records through global memory costs, in atoms' time: 20 rows, 8 units in 4 / 8 / 15 parts
-// 5 / 17 / 49, 16 units in eight 26, 32 in four 11; 40 rows 3 / 11 / 29, 17, 8, 40 units in three 11.
-__device__ __forceinline__ int merge_cost(int rows, int r) { return (rows <= 32) ? 6 + 3 * r : 8 + (3 * r) / 2; }
+// 5 / 17 / 49, 16 units in eight 26, 32 in four 11; 40 rows 3 / 11 / 29, 17, 8, 40 units in three 11.  Two CTAs per SM: 20 rows, 80
+// units of 1000 to 100 tokens, the longest in five, 38.
+__device__ __forceinline__ int merge_cost(int rows, bool half, int r) { return half ? 6 + 6 * r : (rows <= 32) ? 6 + 3 * r : 8 + (3 * r) / 2; }
 
 // Parts of a unit for a target share of `share` atoms, out of U units on G CTAs: inside clusters the largest power of
 // two up to the cluster size of which half would leave parts above the share, where a part has at
@@ -236,20 +237,21 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
     // of 2900 and 8 of 480 atoms on 148 SMs, 64 rows each: 41.4 us in clusters, 37.9 anywhere; 8 units of 813, 40
     // rows: 41.2 and 35.1).
     first_fit(0, part);
-    if (part + 3 > fair + merge_cost(rows, pt.unit_max / fair + 1)) {
+    if (part + 3 > fair + merge_cost(rows, half, pt.unit_max / fair + 1)) {
       consider(kCandidates, 2 * kCandidates);
       way_hi = 2;
       __syncthreads();
     }
   }
-  // Costs in atoms' time: a straddling CTA ~24; a unit's merge through global memory as above; inside a cluster ~3.
+  // Costs in atoms' time: a straddling CTA ~24, ~44 with half of an SM (20 rows, 104 units of 3000 to 150 tokens, us: ranges
+  // 35, in pairs 33, clusters of four 22); a unit's merge through global memory as above; inside a cluster ~3.
   int cand = -1, way = 1;
-  int best = (N + kSegAtoms * U) / G + 24 + 3 * (pt.unit_max / fair + 1);
+  int best = (N + kSegAtoms * U) / G + 24 + (half ? 20 : 0) + 3 * (pt.unit_max / fair + 1);
 #pragma unroll 1
   for (int w = way_lo; w < way_hi; ++w) {
     const int c = first_fit(w, part);
     if (c < 0) continue;
-    const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : merge_cost(rows, (pt.unit_max + part - 1) / part));
+    const int cost = part + ((w == 0) ? 3 : (part >= pt.unit_max) ? 0 : merge_cost(rows, half, (pt.unit_max + part - 1) / part));
     if (cost <= best) {
       best = cost;
       cand = c;
@@ -1551,7 +1553,12 @@ bool verify_grid(const specattn_verify_args& A, int n_sm, bool many, int* n_ctas
   }
   const VerifyKernel k = verify_kernel_of(M, many);
   const int slots = half ? 2 * n_sm : n_sm;
-  int cs = want_cluster(units, slots);
+  // Two CTAs per SM: clusters of four where they have two CTAs for every unit (71 of them run at once on 148 SMs), pairs up
+  // to a unit per CTA.  A long list among short ones is then cut in four; in pairs it set the time (20 rows, us, one CTA
+  // per SM / pairs / clusters of four: 96 units of 1000 to 50 tokens 11.8 / 17.4 / 11.9, of 3000 to 150 22.9 / 25.4 / 21.4; 128
+  // units of 3000 to 150 26.5 / 35.2 / 22.1, of 2053 each, without a plan, 43.3 / 37.7 / 37.2).  Equal short lists that
+  // leave no cluster free lose (16 rows, 136 units of 300 tokens 9.4 / 9.4 / 10.5).
+  int cs = !half ? want_cluster(units, n_sm) : (units <= n_sm) ? 4 : (units <= slots) ? 2 : 1;
   if (cs > 2 && M > 32 && long_lists(A, cs)) cs = 2;
   for (;;) {
     std::atomic<int>& slot = known[dev][kind][cs];
@@ -1586,7 +1593,8 @@ bool verify_grid(const specattn_verify_args& A, int n_sm, bool many, int* n_ctas
     }
     const int ctas = (n - 1 < slots / cs ? n - 1 : slots / cs) * cs;
     // a size that leaves too much of the GPU idle is not worth its merges
-    if (cs == 1 || ctas * 8 >= slots * 7 || (ctas > 0 && ctas >= units * cs)) {
+    const bool too_few = half && cs == 4 && ctas < 2 * units;
+    if (cs == 1 || (!too_few && (ctas * 8 >= slots * 7 || (ctas > 0 && ctas >= units * cs)))) {
       *n_ctas = ctas;
       *cluster = cs;
       return ctas > 0;

@@ -857,8 +857,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
     const uint32_t rec = smem_u32(sh.kv), sum = smem_u32(sh.sum);
     const int mu = sh.part.mine[0], me = sh.part.mine[1], k = sh.part.mine[2];
     if (k == 2) merge_cluster<NT8, 2>(P, sh.row_off, rec, sum, me, mu);
-    else if (k == 4) merge_cluster<NT8, 4>(P, sh.row_off, rec, sum, me, mu);
-    else merge_cluster<NT8, 8>(P, sh.row_off, rec, sum, me, mu);
+    else merge_cluster<NT8, 4>(P, sh.row_off, rec, sum, me, mu);   // (no larger clusters: verify_grid)
   }
   if (!ok && P.status && lane == 0) atomicOr(P.status, SPECATTN_ROW_TIMEOUT);
 }

@@ -841,3 +841,29 @@ def test_how_units_are_cut_with_one_cta_per_sm_and_few_query_rows():
         sa.verify_plan(a, plan)
         words.append(plan[:8].cpu().tolist())
     assert words[0] == words[1] and words[0][3] & 0xff == 0
+
+
+@pytest.mark.parametrize("n_q,counts,ctas,cluster", [
+    (5, [2000] + [100] * 9, 104, 4),   # the long list in four parts
+    (4, [2000] * 16, 256, 4),
+    (5, [2000] * 18, 288, 2),          # more units than clusters of four have pairs of CTAs for
+    (6, [3000] * 10, 240, 1),          # three parts a unit, anywhere
+    (2, [100] * 20, 160, 2),           # a unit per CTA at most
+    (5, [3000] * 38, 296, 0),          # ranges
+])
+def test_how_units_are_cut_with_two_ctas_per_sm(n_q, counts, ctas, cluster):
+    """CTAs with work and the clusters they merge in, 8 KV heads, up to 24 query rows, more units than half of the SMs."""
+    import paper_2510_27641_b200 as sa
+    if _ENGINE["flags"] != sa.VERIFY_ENGINE_MMA_SYNC or torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the plan of the mma.sync engine on 148 SMs")
+    d, B = dev(), len(counts)
+    keep = [torch.zeros(B, n_q, 32, 128, dtype=torch.bfloat16, device=d), torch.zeros(1, 2, 16, 8, 128, dtype=torch.bfloat16, device=d),
+            torch.full((B,), 4096, dtype=torch.int32, device=d), torch.zeros(B, 256, dtype=torch.int32, device=d),
+            torch.zeros(B, 1, 4096, dtype=torch.int32, device=d), torch.tensor([[c] for c in counts], dtype=torch.int32, device=d),
+            torch.zeros(4, device=d)]
+    a = sa.make_verify_args(keep[0], keep[1], keep[2], block_table=keep[3], idx=keep[4], counts=keep[5], out=keep[6],
+                            lse=keep[6], flags=_ENGINE["flags"])
+    plan = sa.verify_plan_buffer(a)
+    sa.verify_plan(a, plan)
+    words = plan[:8].cpu().tolist()
+    assert words[3] & 0xff == cluster and words[4] == ctas
