@@ -159,6 +159,12 @@ __device__ __forceinline__ int cand_share(long long N, int G, int c) {
   return static_cast<int>((static_cast<unsigned>(N) * (7u + c) + 7u * G - 1u) / (7u * G));
 }
 
+// Ranges, in atoms' time: a straddling CTA ~24, ~44 with half of an SM (20 rows, 104 units of 3000 to 150 tokens, us: ranges
+// 35, in pairs 33, clusters of four 22).
+__device__ __forceinline__ int ranges_cost(int N, int U, int G, bool half, int unit_max) {
+  return (N + kSegAtoms * U) / G + 24 + (half ? 20 : 0) + 3 * (unit_max / (N / G + 1) + 1);
+}
+
 // Decides the partition (all NT threads of the CTA, after a barrier that follows unit_start[]): the candidate
 // share, or -1 for ranges; `cluster` becomes 1 where parts are to merge through global memory.  Then calls
 // place(unit, first CTA, number of parts) for every unit of an aligned partition, each from one thread.  Two
@@ -174,7 +180,16 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   const int N = unit_start[U];
   if (U > kAlignedMaxUnits || N <= 0) {
     cluster = 1;
-    return -1;
+    if (U > G || N <= 0) return -1;
+    // (two CTAs per SM) Up to a CTA per unit: whole units, where none is longer than ranges would take (20 rows, 296 units of
+    // 60 to 12 tokens, us: ranges 21.9, whole 7.3; one CTA per SM 16.0).
+    int most = 0;
+    for (int u = lane; u < U; u += 32) most = max(most, unit_start[u + 1] - unit_start[u]);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (most > ranges_cost(N, U, G, half, most)) return -1;
+    pt.parts[1][0] = U;  // (the same from every thread)
+    for (int u = tid; u < U; u += NT) place(u, u, 1);
+    return 0;
   }
   // (CTAs of half an SM, more units than half of them: their sizes decide, so the shares go up to three times the average)
   const int wide = (half && 2 * U > G) ? 1 : 0;
@@ -243,10 +258,9 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
       __syncthreads();
     }
   }
-  // Costs in atoms' time: a straddling CTA ~24, ~44 with half of an SM (20 rows, 104 units of 3000 to 150 tokens, us: ranges
-  // 35, in pairs 33, clusters of four 22); a unit's merge through global memory as above; inside a cluster ~3.
+  // Costs in atoms' time: a unit's merge through global memory as above; inside a cluster ~3.
   int cand = -1, way = 1;
-  int best = (N + kSegAtoms * U) / G + 24 + (half ? 20 : 0) + 3 * (pt.unit_max / fair + 1);
+  int best = ranges_cost(N, U, G, half, pt.unit_max);
 #pragma unroll 1
   for (int w = way_lo; w < way_hi; ++w) {
     const int c = first_fit(w, part);

@@ -641,6 +641,7 @@ def test_how_units_are_cut(batch, n_q, n_q_heads, tokens, parts, cluster):
     ([5, 2100, 40, 900, 17, 0, 64, 1300, 3, 700], 0),          # long lists among short ones: cut into parts, several a CTA
     ([4100] + [260] * 9, 0),                                   # one unit far above the average
     ([17 * i for i in range(20)], 2),                          # more units than SMs
+    ([60, 3, 0, 17] * 9 + [33], 0),                            # as many units as CTAs
 ])
 @pytest.mark.parametrize("T,Hq", [(1, 32), (3, 32), (5, 32), (6, 32), (7, 32), (5, 64), (6, 64), (7, 64), (8, 64)])
 def test_many_units_by_all_their_query_rows(T, Hq, counts, tail):
@@ -850,6 +851,8 @@ def test_how_units_are_cut_with_one_cta_per_sm_and_few_query_rows():
     (6, [3000] * 10, 240, 1),          # three parts a unit, anywhere
     (2, [100] * 20, 160, 2),           # a unit per CTA at most
     (5, [3000] * 38, 296, 0),          # ranges
+    (5, [60, 3] * 18 + [0], 296, 1),   # a CTA per unit, the empty ones' idle
+    (5, [3000] + [60] * 36, 296, 0),
 ])
 def test_how_units_are_cut_with_two_ctas_per_sm(n_q, counts, ctas, cluster):
     """CTAs with work and the clusters they merge in, 8 KV heads, up to 24 query rows, more units than half of the SMs."""
