@@ -180,8 +180,8 @@ __device__ __forceinline__ int partition_units(Partition& pt, const int* unit_st
   const int N = unit_start[U];
   if (U > kAlignedMaxUnits || N <= 0) {
     cluster = 1;
-    if (U > G || N <= 0) return -1;
-    // (two CTAs per SM) Up to a CTA per unit: whole units, where none is longer than ranges would take (20 rows, 296 units of
+    if (!half || U > G || N <= 0) return -1;
+    // Two CTAs per SM, up to a CTA per unit: whole units, where none is longer than ranges would take (20 rows, 296 units of
     // 60 to 12 tokens, us: ranges 21.9, whole 7.3; one CTA per SM 16.0).
     int most = 0;
     for (int u = lane; u < U; u += 32) most = max(most, unit_start[u + 1] - unit_start[u]);
@@ -807,6 +807,14 @@ __device__ __noinline__ void merge_cluster(const VerifyParams& P, uint32_t rec_a
   cluster_wait();    // nobody leaves while its records may still be read
 }
 
+// After a failed wait: a bounded chance for a producer warp's last copies to land before the CTA retires, the queries of
+// segment `seg` or the one before, which the consumers will not get to, among them.  Out of line: it is never in a hurry.
+template <class Sh>
+__device__ __noinline__ void drain(Sh& sh, int last_it, int seg) {
+  if (last_it >= 0) mbar_wait(&sh.full[last_it % kStages], (last_it / kStages) & 1u, nullptr);
+  for (int i = max(seg - 1, 1); i <= seg; ++i) mbar_wait(&sh.q_full[i % Sh::kQBuf], (i / Sh::kQBuf) & 1u, nullptr);
+}
+
 template <int MT, int WPM>
 __global__ void __launch_bounds__((MT * WPM + kProdWarps) * 32, 1)
 sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
@@ -972,7 +980,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
     // =========================== producer warps ===========================================
     const int pw = warp - NC;
     int it = 0, seg = 0;
-    int last_it = -1, q_seg = 0;   // the last tile, the last segment whose queries this warp sent for
+    int last_it = -1;
     int a = a0, u = u_first;
     bool dead = false;
     while (a < a1 && !dead) {
@@ -1009,7 +1017,6 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
           bulk_g2s(sh.q[qb] + r * kPitch, P.q + ((static_cast<long long>(b) * P.T + t) * P.Hq + h) * kD,
                    kRowBytes, &sh.q_full[qb]);
         }
-        q_seg = seg;
         return true;
       };
       bool q_pending = (pw == 0);
@@ -1155,12 +1162,7 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
         while (u < U && sh.unit_start[u + 1] == sh.unit_start[u]) ++u;
       }
     }
-    if (sh.abort_flag) {
-      // give this warp's last copies a bounded chance to land before the CTA retires (the queries of a unit that the
-      // consumers will not get to among them)
-      if (last_it >= 0) mbar_wait(&sh.full[last_it % kStages], (last_it / kStages) & 1u, nullptr);
-      if (q_seg > 0) mbar_wait(&sh.q_full[q_seg % Sh::kQBuf], (q_seg / Sh::kQBuf) & 1u, nullptr);
-    }
+    if (sh.abort_flag) drain(sh, last_it, (pw == 0) ? seg : 0);
     return;
   }
 
