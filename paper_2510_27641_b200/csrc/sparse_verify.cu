@@ -435,7 +435,7 @@ __host__ __device__ inline size_t plan_ints(int U, int grid) {
 __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int G) {
   __shared__ int unit_start[kMaxUnits + 1];
   __shared__ Partition pt;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5;
   const int U = P.B * P.Hkv;
   // The lists are the previous kernel's output.  No early trigger for the next kernel either:
   // a verify launch flagged SPECATTN_VERIFY_LISTS_STABLE reads the plan without waiting, so it
@@ -451,20 +451,7 @@ __device__ __forceinline__ void plan_body(const VerifyParams& P, int* plan, int 
     unit_start[u + 1] = (c + kAtom - 1) / kAtom;
   }
   __syncthreads();
-  if (warp == 0) {
-    int carry = 0;
-    for (int base = 0; base < U; base += 32) {
-      const int u = base + lane;
-      int v = (u < U) ? unit_start[u + 1] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-      }
-      if (u < U) unit_start[u + 1] = v + carry;
-      carry += __shfl_sync(0xffffffffu, v, 31);
-    }
-  }
+  if (warp == 0) scan_units(unit_start, U);
   __syncthreads();
   const long long N = unit_start[U];
   int cluster = P.cluster;
@@ -807,6 +794,53 @@ __device__ __noinline__ void merge_cluster(const VerifyParams& P, uint32_t rec_a
   cluster_wait();    // nobody leaves while its records may still be read
 }
 
+// The partition of a launch without a plan, and this CTA's share of it, into sh.part (all threads; the atom counts lie in
+// unit_start[1 .. U]).  Out of line: inline it left the tile loop of 17 to 24 rows with two CTAs per SM too few registers (512
+// units of 2000 tokens 103 -> 112 us), and launches with a plan ran past it (48 rows, 64 units of 60 tokens 6.2 -> 6.05 us, 4 x 8 units
+// of 16000 at 40 rows 94.5 -> 92.5).
+template <class Sh, int NT, bool kHalf>
+__device__ __noinline__ void cut_units(int U, int rows, int cluster) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  Sh& sh = *reinterpret_cast<Sh*>(smem_raw);
+  int* const unit_start = sh.unit_start;
+  const int G = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
+  if (threadIdx.x < 32) scan_units(unit_start, U);
+  __syncthreads();
+  const int N = unit_start[U];
+  const int cand = partition_units<NT>(sh.part, unit_start, U, G, rows, kHalf, cluster, [&](int u, int first, int k) {
+    const int j = cta - first;
+    if (j >= 0 && j < k) {
+      const int us = unit_start[u], atoms = unit_start[u + 1] - us;  // part < parts: the products fit 32 bits
+      sh.part.mine[0] = u;
+      sh.part.mine[1] = j;
+      sh.part.mine[2] = k;
+      sh.part.range[0] = us + j * atoms / k;
+      sh.part.range[1] = us + (j + 1) * atoms / k;
+    }
+  });
+  const bool aligned = cand >= 0;
+  const int NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : min(N, G);
+  if (aligned) {
+    __syncthreads();
+  } else if (cta < NP) {
+    int a0, a1, u, next;
+    range_start(unit_start, U, N, cta, NP, a0, u);
+    range_start(unit_start, U, N, cta + 1, NP, a1, next);
+    if ((threadIdx.x & 31) == 0) {
+      sh.part.mine[0] = u;
+      sh.part.mine[1] = sh.part.mine[2] = 0;
+      sh.part.range[0] = a0;
+      sh.part.range[1] = (cta + 1 == NP) ? N : a1;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sh.part.atoms = N;
+    sh.part.ctas = NP;
+    sh.part.aligned = aligned ? 1 : 0;
+    sh.part.cluster = cluster;
+  }
+}
+
 // After a failed wait: a bounded chance for a producer warp's last copies to land before the CTA retires, the queries of
 // segment `seg` or the one before, which the consumers will not get to, among them.  Out of line: it is never in a hurry.
 template <class Sh>
@@ -885,70 +919,22 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
   }
   fence_proxy_async();
   __syncthreads();
-  long long N;        // atoms of all units
-  bool aligned;       // which of the two partitions
-  long long NP;       // CTAs that get work
-  int a0 = 0, a1 = 0, u_first = 0;  // this CTA's atom range and the unit holding its first atom
-  int part = 0, parts = 0;          // (aligned) which part of how many of the unit
-  int cluster;                      // 1: parts merge through global memory
-  const int G = static_cast<int>(gridDim.x);
-  if (planned) {
-    N = plan[5];
-    cluster = plan[3] & 0xff;
-    aligned = cluster != 0;
-    NP = plan[4];
+  // (every warp leaves itself the same values)
+  if (!planned) {
+    cut_units<Sh, NT, false>(U, 16 * MT, P.cluster);
+  } else if (lane == 0) {
     const int* const p_cta = plan + kPlanHeader + 2 * (U + 1) + 4 * blockIdx.x;
-    a0 = p_cta[0];
-    a1 = p_cta[1];
-    u_first = p_cta[2];
-    part = part_of(p_cta[3]);
-    parts = parts_of(p_cta[3]);
-  } else {
-  if (warp == 0) {  // inclusive scan of the atom counts, 32 at a time
-    int carry = 0;
-    for (int base = 0; base < U; base += 32) {
-      const int u = base + lane;
-      int v = (u < U) ? sh.unit_start[u + 1] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-      }
-      if (u < U) sh.unit_start[u + 1] = v + carry;
-      carry += __shfl_sync(0xffffffffu, v, 31);
-    }
+    sh.part.range[0] = p_cta[0];
+    sh.part.range[1] = p_cta[1];
+    sh.part.mine[0] = p_cta[2];
+    sh.part.mine[1] = part_of(p_cta[3]);
+    sh.part.mine[2] = parts_of(p_cta[3]);
+    sh.part.ctas = plan[4];
+    sh.part.atoms = plan[5];
+    sh.part.cluster = plan[3] & 0xff;
+    sh.part.aligned = sh.part.cluster != 0;
   }
-  __syncthreads();
-
-  N = sh.unit_start[U];
-  cluster = P.cluster;
-  const int cand = partition_units<NT>(sh.part, sh.unit_start, U, G, 16 * MT, false, cluster, [&](int u, int first, int k) {
-    const int j = static_cast<int>(blockIdx.x) - first;
-    if (j >= 0 && j < k) {
-      sh.part.mine[0] = u;
-      sh.part.mine[1] = j;
-      sh.part.mine[2] = k;
-    }
-  });
-  aligned = cand >= 0;
-  NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : ((N < G) ? N : static_cast<long long>(G));
-  if (aligned) {
-    __syncthreads();
-    if (static_cast<long long>(blockIdx.x) < NP) {
-      u_first = sh.part.mine[0];
-      part = sh.part.mine[1];
-      parts = sh.part.mine[2];
-      const int atoms = sh.unit_start[u_first + 1] - sh.unit_start[u_first];  // part < parts: the products fit 32 bits
-      a0 = sh.unit_start[u_first] + part * atoms / parts;
-      a1 = sh.unit_start[u_first] + (part + 1) * atoms / parts;
-    }
-  } else if (static_cast<long long>(blockIdx.x) < NP) {
-    int next;
-    range_start(sh.unit_start, U, static_cast<int>(N), blockIdx.x, NP, a0, u_first);
-    range_start(sh.unit_start, U, static_cast<int>(N), blockIdx.x + 1, NP, a1, next);
-    if (static_cast<long long>(blockIdx.x) + 1 == NP) a1 = static_cast<int>(N);
-  }
-  }  // !planned
+  __syncwarp();
   if (warp < NC) {
     // consumers are the only writers of global memory: from here on the previous kernel's
     // results (and its use of the shared workspace) are complete
@@ -964,17 +950,8 @@ sparse_verify_kernel(const __grid_constant__ VerifyParams P) {
       }
     }
   }
-  if (static_cast<long long>(blockIdx.x) >= NP) return;
-  if (lane == 0) {  // (every warp leaves itself the same values)
-    sh.part.mine[0] = u_first;
-    sh.part.mine[1] = part;
-    sh.part.mine[2] = parts;
-    sh.part.atoms = static_cast<int>(N);
-    sh.part.ctas = static_cast<int>(NP);
-    sh.part.aligned = aligned ? 1 : 0;
-    sh.part.cluster = cluster;
-  }
-  __syncwarp();
+  if (static_cast<int>(blockIdx.x) >= sh.part.ctas) return;
+  const int a0 = sh.part.range[0], a1 = sh.part.range[1], u_first = sh.part.mine[0];  // this CTA's atoms and the unit of the first
 
   if (warp >= NC) {
     // =========================== producer warps ===========================================

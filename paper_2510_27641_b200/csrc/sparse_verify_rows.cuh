@@ -68,8 +68,6 @@ __device__ __forceinline__ float2 row_to_col(float v, int tq) {
   return make_float2(__shfl_sync(0xffffffffu, v, 8 * tq), __shfl_sync(0xffffffffu, v, 8 * tq + 4));
 }
 
-// One tile of 16 keys.  `valid`: existing keys (rows beyond hold finite padding); `tail_begin`: index in the tile
-// of the first in-flight token (>= 16: none), of which row r may see the first row_lim(r) + 1 only.
 // Fragments of 16 query dims: the slabs of a warp's rows.  (Half a slab: rows 8 - 15 of the fragment are zero.)
 template <int NT8>
 __device__ __forceinline__ void load_q(uint32_t (*f)[4], uint32_t q_addr, uint32_t q_half, int kk) {
@@ -373,52 +371,6 @@ __device__ __forceinline__ void merge_global(const Items<NT8>& items, int i_lo, 
   }
 }
 
-// The partition of a launch without a plan, and this CTA's share of it, into sh.part (all threads; the atom counts lie in
-// unit_start[1 .. U]).  Out of line: inline it left the tile loop of 17 to 24 rows too few registers (512 units of
-// 2000 tokens 103 -> 112 us).
-template <int NT8>
-__device__ __noinline__ void cut_units(int U, int rows, int cluster) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  VShared<NT8>& sh = *reinterpret_cast<VShared<NT8>*>(smem_raw);
-  int* const unit_start = sh.unit_start;
-  const int G = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-  if (threadIdx.x < 32) scan_units(unit_start, U);
-  __syncthreads();
-  const int N = unit_start[U];
-  const int cand = partition_units<kThreads>(sh.part, unit_start, U, G, rows, true, cluster, [&](int u, int first, int k) {
-    const int j = cta - first;
-    if (j >= 0 && j < k) {
-      const int us = unit_start[u], atoms = unit_start[u + 1] - us;  // part < parts: the products fit 32 bits
-      sh.part.mine[0] = u;
-      sh.part.mine[1] = j;
-      sh.part.mine[2] = k;
-      sh.part.range[0] = us + j * atoms / k;
-      sh.part.range[1] = us + (j + 1) * atoms / k;
-    }
-  });
-  const bool aligned = cand >= 0;
-  const int NP = aligned ? sh.part.parts[cluster > 1 ? 0 : 1][cand] : min(N, G);
-  if (aligned) {
-    __syncthreads();
-  } else if (cta < NP) {
-    int a0, a1, u, next;
-    range_start(unit_start, U, N, cta, NP, a0, u);
-    range_start(unit_start, U, N, cta + 1, NP, a1, next);
-    if ((threadIdx.x & 31) == 0) {
-      sh.part.mine[0] = u;
-      sh.part.mine[1] = sh.part.mine[2] = 0;
-      sh.part.range[0] = a0;
-      sh.part.range[1] = (cta + 1 == NP) ? N : a1;
-    }
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sh.part.atoms = N;
-    sh.part.ctas = NP;
-    sh.part.aligned = aligned ? 1 : 0;
-    sh.part.cluster = cluster;
-  }
-}
-
 template <int NT8>
 __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const __grid_constant__ VerifyParams P) {
   using Sh = VShared<NT8>;
@@ -499,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
   __syncthreads();
   // (every warp leaves itself the same values)
   if (!planned) {
-    cut_units<NT8>(U, P.M, P.cluster);
+    cut_units<Sh, kThreads, true>(U, P.M, P.cluster);
   } else if (lane == 0) {
     sh.part.mine[0] = what.x;
     sh.part.mine[1] = part_of(what.y);
