@@ -795,11 +795,9 @@ __device__ __noinline__ void merge_cluster(const VerifyParams& P, uint32_t rec_a
 }
 
 // The partition of a launch without a plan, and this CTA's share of it, into sh.part (all threads; the atom counts lie in
-// unit_start[1 .. U]).  Out of line: inline it left the tile loop of 17 to 24 rows with two CTAs per SM too few registers (512
-// units of 2000 tokens 103 -> 112 us), and launches with a plan ran past it (48 rows, 64 units of 60 tokens 6.2 -> 6.05 us, 4 x 8 units
-// of 16000 at 40 rows 94.5 -> 92.5).
+// unit_start[1 .. U]).
 template <class Sh, int NT, bool kHalf>
-__device__ __noinline__ void cut_units(int U, int rows, int cluster) {
+__device__ __forceinline__ void cut_units_inline(int U, int rows, int cluster) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Sh& sh = *reinterpret_cast<Sh*>(smem_raw);
   int* const unit_start = sh.unit_start;
@@ -840,6 +838,13 @@ __device__ __noinline__ void cut_units(int U, int rows, int cluster) {
     sh.part.cluster = cluster;
   }
 }
+
+// ... out of line, which launches with a plan gain from, having less to run past (planned, us, inline / out of line: 48 rows, 64 units
+// of 60 tokens 6.2 / 6.05; 40 rows, 32 of 16000 94.5 / 92.5; two CTAs per SM and 16 rows, 192 of 300 10.5 / 9.8).  Not
+// with two CTAs per SM and 17 to 24 rows: a call, us, 128 units of 2053 tokens 36.3 / 37.7, 256 of 6000 to 600 75.0 / 76.7, planned
+// 80 of 300 10.3 / 10.15.
+template <class Sh, int NT, bool kHalf>
+__device__ __noinline__ void cut_units(int U, int rows, int cluster) { cut_units_inline<Sh, NT, kHalf>(U, rows, cluster); }
 
 // After a failed wait: a bounded chance for a producer warp's last copies to land before the CTA retires, the queries of
 // segment `seg` or the one before, which the consumers will not get to, among them.  Out of line: it is never in a hurry.

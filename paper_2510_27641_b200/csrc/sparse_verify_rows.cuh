@@ -451,7 +451,8 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_verify_rows_kernel(const _
   __syncthreads();
   // (every warp leaves itself the same values)
   if (!planned) {
-    cut_units<Sh, kThreads, true>(U, P.M, P.cluster);
+    if (NT8 == 3) cut_units_inline<Sh, kThreads, true>(U, P.M, P.cluster);
+    else cut_units<Sh, kThreads, true>(U, P.M, P.cluster);
   } else if (lane == 0) {
     sh.part.mine[0] = what.x;
     sh.part.mine[1] = part_of(what.y);
