@@ -95,3 +95,28 @@ def test_random_attention_cases(seed):
             assert int(status.abs().sum()) == 0
     finally:
         tv._ENGINE["flags"] = 0
+
+
+@pytest.mark.parametrize("seed", [0, 1])
+def test_random_attention_cases_of_many_units(seed):
+    """As above with 75 to 330 units, where up to 24 query rows run with two CTAs per SM."""
+    import paper_2510_27641_b200 as sa
+    import test_gpu_verify as tv
+    rng = np.random.default_rng(100 + seed)
+    try:
+        tv._ENGINE["flags"] = sa.VERIFY_ENGINE_MMA_SYNC
+        for _ in range(8):
+            T, Hq = [(1, 32), (2, 32), (4, 32), (5, 32), (6, 32), (2, 64), (3, 64), (6, 64)][rng.integers(0, 8)]
+            B = int(rng.integers(10, 42))
+            lens = rng.integers(1, int(rng.choice([40, 300, 900])) + 1, size=B).tolist()
+            if rng.random() < 0.4:
+                lens[rng.integers(0, B)] = int(rng.integers(1000, 4000))
+            G = 1 if rng.random() < 0.6 else 8
+            use_bt = bool(rng.random() < 0.85)
+            case = tv._make_case(int(rng.integers(1 << 30)), B, T, Hq, 8, int(rng.choice([16, 32, 24])), lens, G=G,
+                                 shuffle=use_bt, tail=int(rng.choice([0, 0, 1, T])))
+            out, lse, status = tv._run(case, use_bt=use_bt)
+            check_attention(out, lse, *tv._oracle(case, use_bt=use_bt)[:2])
+            assert int(status.abs().sum()) == 0
+    finally:
+        tv._ENGINE["flags"] = 0

@@ -480,7 +480,7 @@ def test_page_granular_per_head_lists_tails_and_contiguous_cache():
     (8, [65, 127, 513]),                               # up to four
     (8, [900, 17, 260, 0, 1024, 700]),                 # pairs, or more parts through global memory
     (8, [300] * 9 + [2048]),                           # one long list among short ones
-    (8, [40 + 16 * i for i in range(20)]),             # more units than CTAs
+    (8, [40 + 16 * i for i in range(20)]),             # more units than SMs
 ])
 def test_mixed_list_lengths_cut_into_parts_of_one_cluster(hkv, counts):
     """Units of one call cut into different numbers of parts (a power of two up to the cluster size),
@@ -638,10 +638,11 @@ def test_how_units_are_cut(batch, n_q, n_q_heads, tokens, parts, cluster):
 
 @pytest.mark.parametrize("counts,tail", [
     ([0, 1, 15, 16, 17, 33, 64, 65, 127, 128, 129, 300], 3),   # edges of a 16-token tile and of four of them, in-flight tokens
-    ([5, 2100, 40, 900, 17, 0, 64, 1300, 3, 700], 0),          # long lists among short ones: cut into parts, several a CTA
+    ([5, 2100, 40, 900, 17, 0, 64, 1300, 3, 700], 0),          # long lists among short ones, cut in up to four parts
     ([4100] + [260] * 9, 0),                                   # one unit far above the average
     ([17 * i for i in range(20)], 2),                          # more units than SMs
-    ([60, 3, 0, 17] * 9 + [33], 0),                            # as many units as CTAs
+    ([60, 3, 0, 17] * 9 + [33], 0),                            # as many units as CTAs where two share an SM
+    ([40 + 13 * (i % 7) for i in range(50)], 1),               # more: several units and parts of units a CTA, both query buffers in turn
 ])
 @pytest.mark.parametrize("T,Hq", [(1, 32), (3, 32), (5, 32), (6, 32), (7, 32), (5, 64), (6, 64), (7, 64), (8, 64)])
 def test_many_units_by_all_their_query_rows(T, Hq, counts, tail):
@@ -680,8 +681,8 @@ def test_many_units_by_all_their_query_rows(T, Hq, counts, tail):
     check_attention(o, l, *ref)
 
 
-@pytest.mark.parametrize("B,kept", [(64, 60), (40, 400), (10, 500)])   # several units a CTA, one or two, less than one
-@pytest.mark.parametrize("T,Hq", [(2, 32), (4, 32), (5, 32), (5, 64), (7, 64)])
+@pytest.mark.parametrize("B,kept", [(64, 60), (40, 400)])   # two CTAs per SM: several units each, one or two
+@pytest.mark.parametrize("T,Hq", [(4, 32), (5, 32), (7, 64)])
 def test_queries_that_the_launch_right_before_wrote(T, Hq, B, kept):
     """SPECATTN_VERIFY_LISTS_STABLE vouches for lists and K/V rows, not for the queries: they may be the previous launch's
     output, whatever segment of a CTA reads them.  Other queries at every turn, written by a copy kernel or by
@@ -870,3 +871,51 @@ def test_how_units_are_cut_with_two_ctas_per_sm(n_q, counts, ctas, cluster):
     sa.verify_plan(a, plan)
     words = plan[:8].cpu().tolist()
     assert words[3] & 0xff == cluster and words[4] == ctas
+
+
+@pytest.mark.parametrize("T", [2, 5, 6])
+@pytest.mark.parametrize("page,bt", [(16, True), (24, True), (1, True), (16, False)])
+def test_many_units_with_a_list_per_kv_head(T, page, bt):
+    """8, 20 and 24 query rows of 96 units (two CTAs per SM): lists per KV head, pages that are no power of two, a
+    contiguous cache, in-flight tokens, a scale of the caller's."""
+    rng = np.random.default_rng(page)
+    lens = rng.integers(1, 700, size=12).tolist()
+    case = _make_case(110 + page, 12, T, 32, 8, page, lens, G=8, shuffle=bt, tail=2)
+    out, lse, status = _run(case, use_bt=bt, sm_scale=0.11)
+    assert int(status.abs().sum()) == 0
+    check_attention(out, lse, *_oracle(case, use_bt=bt, scale=0.11))
+
+
+@pytest.mark.parametrize("T", [3, 5])
+def test_many_units_with_bad_positions_and_pages(T):
+    """Flagged, not followed, where two CTAs share an SM; the other sequences keep their results."""
+    import paper_2510_27641_b200 as sa
+    case = _make_case(111, 12, T, 32, 8, 16, [500] * 12, counts=[[100 + 7 * b] for b in range(12)])
+    case["idx"][3, 0, 5] = 500
+    case["idx"][3, 0, 101] = -3
+    case["bt"][7, 0:32] = 10 ** 6
+    out, lse, status = _run(case)
+    bad = [sa.ROW_BAD_INDEX if b in (3, 7) else 0 for b in range(12)]
+    assert status.cpu().tolist() == bad and torch.all(torch.isfinite(out))
+    good = [b for b in range(12) if not bad[b]]
+    part = dict(case, idx=case["idx"][good], cnt=case["cnt"][good], lens=case["lens"][good], bt=case["bt"][good], q=case["q"][good])
+    check_attention(out[good], lse[good], *_oracle(part))
+
+
+@pytest.mark.parametrize("counts", [[900] * 10, [300] * 40])   # units in parts; whole
+@pytest.mark.parametrize("T,step", [(3, 0.02), (5, 0.02), (6, 0.3), (5, -0.02)])
+def test_scores_that_grow_along_a_list(T, step, counts):
+    """The reference maximum of a row is raised (and all that was summed up rescaled) tile after tile, by less than 2^8 a
+    tile and by more, in every warp and part; or never, where scores fall."""
+    case = _make_case(112, len(counts), T, 32, 8, 16, [c + 50 for c in counts], counts=[[c] for c in counts])
+    vals = bf16.to_f32(bf16.torch_to_bits(case["kv"]))
+    for b, c in enumerate(counts):
+        for i, pos in enumerate(case["idx"][b, 0, :c]):
+            vals[case["bt"][b, pos // 16], 0, pos % 16, :, 0] = step * i * 128 ** 0.5 / 16     # (log2 of a weight: 1.44 step a key)
+    q = bf16.to_f32(case["q"])
+    q[..., 0] = 16
+    case["q"] = bf16.from_f32(q)
+    case["kv"] = bf16.bits_to_torch(bf16.from_f32(vals)).reshape(case["kv"].shape)
+    out, lse, status = _run(case)
+    assert int(status.abs().sum()) == 0
+    check_attention(out, lse, *_oracle(case))
