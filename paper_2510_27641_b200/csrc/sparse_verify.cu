@@ -1485,13 +1485,18 @@ constexpr size_t verify_smem() {
 
 int query_rows(const specattn_verify_args& A) { return A.n_q * (A.n_q_heads / A.n_kv_heads); }
 
-// CTAs of half an SM (sparse_verify_rows.cuh, with the figures): up to 24 query rows and more units than half of the SMs.
+// CTAs of half an SM (sparse_verify_rows.cuh): up to 24 query rows and more units than half of the SMs.  Planned, us, one / two CTAs
+// per SM, lists of equal length: 4 rows 80 units of 60 tokens 5.0 / 4.05, of 2000 26.6 / 23.2; 136 of 60 6.1 / 4.2, of 400 11.3 / 11.4,
+// of 2000 31.4 / 29.3; 256 of 400 22.8 / 13.4; 512 of 2000 103 / 97.  16 rows 80 of 400 10.1 / 9.4, 136 of 60 6.5 / 4.3, 256 of 400 23.5 / 13.9, 512 of
+// 2000 107 / 97.  20 rows 80 of 400 11.5 / 11.0, 136 of 400 13.0 / 13.1, of 2000 35.8 / 31.0; 256 of 400 26.1 / 15.4.  Not won: 75 to 148 units of 150 to 600
+// tokens with 17 to 24 rows (80 of 300 to 90: 8.0 / 9.2, 128 of 300: 11.0 / 12.0), where one CTA per SM has twice the warps
+// for a list that is not worth cutting; the host does not see how long lists are.
 bool beyond_half(const specattn_verify_args& A, int n_sm) { return 2ll * A.batch * A.n_kv_heads > n_sm; }
 bool half_sm(const specattn_verify_args& A, int n_sm) { return query_rows(A) <= 24 && beyond_half(A, n_sm); }
-// Many units have a kernel of their own: those, and 33 to 48 rows with more units than SMs the one of four slabs.  It
-// has two more consumer warps and fetches the next unit's queries early, which counts for more there than
-// the padding (40 rows, us, three slabs / four: 192 units x 400 tokens 32.5 / 27.7, 256 x 60 15.1 / 14.0, x 400 40.0 / 33.0, x 2000 106.9 / 95.3, 512 x 400
-// 76.0 / 63.4; not with a unit per CTA or less: 128 x 400 14.6 / 15.4).
+// Many units have a kernel of their own: those, and 33 to 48 rows with more units than SMs the one of four slabs.  What
+// helps there is its second query buffer, which three slabs have no register for (VShared); the fourth slab's two warps multiply
+// zeros, and its records are padding (40 rows, us, three slabs / four: 192 units x 400 tokens 32.5 / 27.7, 256 x 60 15.1 / 14.0, x 400
+// 40.0 / 33.0, x 2000 106.9 / 95.3, 512 x 400 76.0 / 63.4; not with a unit per CTA or less: 128 x 400 14.6 / 15.4).
 bool many_units(const specattn_verify_args& A, int n_sm) {
   const int rows = query_rows(A);
   return half_sm(A, n_sm) || (rows > 32 && rows <= 48 && static_cast<long long>(A.batch) * A.n_kv_heads > n_sm);

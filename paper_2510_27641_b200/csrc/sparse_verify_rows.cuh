@@ -13,8 +13,8 @@
 //       S[16 rows x 16 keys] = Q K^T per slab,      O^T[128 dims x 8 rows] += V^T P^T per 8 rows,
 //     where the accumulators of S are the B fragments of P^T as they lie, and the query rows are padded to eight instead
 //     of sixteen in the larger product: 80 MMAs per 16 keys at 20 rows instead of 96.
-// (20 rows, us, whole / half: 128 units x 2000 tokens, a call by itself, 41.4 / 36.6; 80 x 400 11.6 / 11.1; 256 x 400
-// 26.0 / 15.5, x 3000 89.7 / 72.4, 512 x 400 45.6 / 38.3.  Not for more rows: 28, 128 x 400 13.0 / 14.7; the same warps in
+// (20 rows, us, whole / half: 128 units x 2053 tokens, a call by itself, 43.3 / 36.4; 80 x 400 11.5 / 11.0; 256 x 400 26.1 / 15.4, x
+// 2000 65.6 / 49.2, 512 x 400 45.7 / 37.3; the rule and its limits: half_sm.  Not for more rows: 28, 128 x 400 13.0 / 14.7; the same warps in
 // whole-SM CTAs, 40 rows, 128 x 400 14.6 / 13.1, but 256 x 60 15.2 / 18.1, and 160 x 315 at 56 rows 30.4 / 36.4, since
 // an end of a unit costs more.  Nor for few units, which get more parts each: 24 rows, 64 x 1228 16.4 / 19.1.)
 #pragma once
